@@ -214,7 +214,9 @@ int clbm_set_launch(clbm_handle h, int block_x, int block_y, int npt);
  * cascaded collision (Sec. 3.1 sets all to 1; Sec. 5 notes that tuning them
  * can improve stability).  omega[k] is omega_(9+k); each must lie in (0, 2).
  * omega_9 also scales the isotropic part of the strain rate that sets
- * omega_nu.  Takes effect from the next step.  Not for a lattice in a batch
+ * omega_nu.  Takes effect from the next step.  Lattices whose rates are not
+ * all 1 run the plain one-node-per-thread kernel whatever launch shape is set
+ * (its block is kept).  Not for a lattice in a batch
  * (CLBM_ERR_ARG: detach it first).  Errors: CLBM_ERR_ARG. */
 int clbm_set_rates(clbm_handle h, const double omega[10]);
 

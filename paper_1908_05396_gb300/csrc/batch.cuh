@@ -37,7 +37,7 @@ struct LatDesc {
 // step_kernel.  Source offsets are formed from compile-time direction
 // constants right before each load, so no per-direction table is held in
 // registers.
-template <typename S, typename R, bool FORCE>
+template <typename S, typename R, bool FORCE, bool UNIT>
 __device__ __forceinline__ void batch_node(const LatDesc<R>& L, const S* __restrict__ src,
                                            S* __restrict__ dst, int x, int y, int z,
                                            unsigned step, NodeOut<R>& o) {
@@ -71,7 +71,7 @@ __device__ __forceinline__ void batch_node(const LatDesc<R>& L, const S* __restr
     pull_face<S, R>(src, L.qstride, L.nx, L.ny, L.nz, pitch, plane, L.facebits, x, y, z, i,
                     L.lidc, d);
   }
-  collide<R, FORCE, pair_out<S>(), log2_scale<S>()>(L.C, d, o);
+  collide<R, FORCE, pair_out<S>(), log2_scale<S>(), UNIT>(L.C, d, o);
   if constexpr (std::is_same<S, __half>::value) {
     if (L.sround) {  // as step_f16sr.cu: two directions per stochastic conversion
       uint32_t state = sr_seed(uint32_t(i), step);
@@ -91,7 +91,7 @@ __device__ __forceinline__ void batch_node(const LatDesc<R>& L, const S* __restr
 
 // One node of the batched step in the F16R form (defined with the other F16R
 // kernels, the only translation unit that instantiates the batch with REF).
-template <bool FORCE>
+template <bool FORCE, bool UNIT>
 __device__ void batch_node_ref(const LatDesc<float>& L, int parity, int x, int y, int z,
                                unsigned step, NodeOut<float>& o);
 
@@ -103,19 +103,19 @@ __host__ __device__ __forceinline__ unsigned tile_word(int tx, int ty, int tz) {
 // The tile loop of the batched step.  get(li) returns lattice li's
 // descriptor from the translation unit's __constant__ table, so ptxas can
 // reload its fields where it needs them instead of holding them in registers.
-template <typename S, typename R, bool CHECK, bool FORCE, bool REF, typename Get>
+template <typename S, typename R, bool CHECK, bool FORCE, bool REF, bool UNIT, typename Get>
 __device__ __forceinline__ void batch_tiles(Get get, const int* __restrict__ owner,
                                             const unsigned* __restrict__ coord,
                                             BatchHeader* hdr, int parity, double* acc, int zc) {
-  // tiles [0, ntiles0) belong to lattices without force, [ntiles0, ntiles) with
-  // F16R and F16S (whose lattices may round stochastically): this chain's
+  // F16R and F16S (whose lattices may round stochastically): this group's
   // step count, advanced at the end of each of its launches by the launch's
   // last CTA
+  constexpr int GROUP = (FORCE ? 2 : 0) + (UNIT ? 0 : 1);
   constexpr bool STEPS = REF || std::is_same<S, __half>::value;
   const unsigned bstep =
-      STEPS ? *reinterpret_cast<volatile const unsigned*>(&hdr->step[FORCE ? 1 : 0]) : 0u;
-  const int t0 = FORCE ? hdr->ntiles0 : 0;
-  const int t1 = FORCE ? hdr->ntiles : hdr->ntiles0;
+      STEPS ? *reinterpret_cast<volatile const unsigned*>(&hdr->step[GROUP]) : 0u;
+  const int t0 = GROUP ? hdr->tile_end[GROUP ? GROUP - 1 : 0] : 0;
+  const int t1 = hdr->tile_end[GROUP];
   const int nlat = hdr->nlat;
   // The next tile's table entries are loaded while this tile collides, so a
   // tile starts with one dependent round trip (descriptor) instead of two.
@@ -161,8 +161,8 @@ __device__ __forceinline__ void batch_tiles(Get get, const int* __restrict__ own
     for (int z = tz * zc; z < z1; ++z) {
       if (active) {
         NodeOut<R> o;
-        if constexpr (REF) batch_node_ref<FORCE>(L, parity, x, y, z, bstep + L.step_offset, o);
-        else batch_node<S, R, FORCE>(L, src, dst, x, y, z, bstep + L.step_offset, o);
+        if constexpr (REF) batch_node_ref<FORCE, UNIT>(L, parity, x, y, z, bstep + L.step_offset, o);
+        else batch_node<S, R, FORCE, UNIT>(L, src, dst, x, y, z, bstep + L.step_offset, o);
         if (CHECK) {
           R* up = static_cast<R*>(L.uprev);
           const int64_t nst = int64_t(L.plane) * L.nz;
@@ -199,9 +199,9 @@ __device__ __forceinline__ void batch_tiles(Get get, const int* __restrict__ own
     __syncthreads();
     if (threadIdx.x == 0 && threadIdx.y == 0) {
       __threadfence();
-      if (atomicAdd(&hdr->done[FORCE ? 1 : 0], 1) == int(gridDim.x) - 1) {
-        atomicExch(&hdr->done[FORCE ? 1 : 0], 0);
-        atomicAdd(&hdr->step[FORCE ? 1 : 0], 1u);
+      if (atomicAdd(&hdr->done[GROUP], 1) == int(gridDim.x) - 1) {
+        atomicExch(&hdr->done[GROUP], 0);
+        atomicAdd(&hdr->step[GROUP], 1u);
       }
     }
   }
@@ -248,39 +248,40 @@ void fill_desc_t(void* out, double lam, const Geom& g, const PhysParams& P, cons
 #define CLBM_DEFINE_BATCH(SUFFIX, S, R, REF)                                                   \
   namespace clbm {                                                                             \
   __constant__ LatDesc<R> c_lat_##SUFFIX[BATCH_CONST_BYTES / sizeof(LatDesc<R>)];              \
-  template <bool CHECK, bool CAP, bool FORCE>                                                  \
+  template <bool CHECK, bool CAP, bool FORCE, bool UNIT>                                       \
   __global__ void __launch_bounds__(256, CAP ? 4 : 1)                                          \
       batch_kernel_##SUFFIX(int base, const int* __restrict__ owner,                           \
                             const unsigned* __restrict__ coord, BatchHeader* hdr, int parity,  \
                             double* acc, int zc) {                                             \
-    batch_tiles<S, R, CHECK, FORCE, REF>(                                                      \
+    batch_tiles<S, R, CHECK, FORCE, REF, UNIT>(                                                \
         [base](int li) -> const LatDesc<R>& { return c_lat_##SUFFIX[base + li]; }, owner,      \
         coord, hdr, parity, acc, zc);                                                          \
   }                                                                                            \
   cudaError_t launch_batch_##SUFFIX(int base, const int* owner, const unsigned* coord,         \
                                     const void* hdr, int parity, bool check, double* acc,      \
-                                    int zc, dim3 block, int grid, cudaStream_t st,             \
+                                    int zc, dim3 block, int grid, bool rates, cudaStream_t st, \
                                     cudaStream_t stf) {                                         \
     BatchHeader* H = static_cast<BatchHeader*>(const_cast<void*>(hdr));                        \
     const bool cap = grid < 0;                                                                 \
     if (cap) grid = -grid;                                                                     \
     /* tiles without force on st, tiles with force on stf (an empty range exits at once) */   \
-    if (check) {                                                                               \
-      if (cap) {                                                                               \
-        batch_kernel_##SUFFIX<true, true, false><<<grid, block, 0, st>>>(base, owner, coord, H, parity, acc, zc); \
-        batch_kernel_##SUFFIX<true, true, true><<<grid, block, 0, stf>>>(base, owner, coord, H, parity, acc, zc); \
-      } else {                                                                                 \
-        batch_kernel_##SUFFIX<true, false, false><<<grid, block, 0, st>>>(base, owner, coord, H, parity, acc, zc); \
-        batch_kernel_##SUFFIX<true, false, true><<<grid, block, 0, stf>>>(base, owner, coord, H, parity, acc, zc); \
-      }                                                                                        \
-    } else {                                                                                   \
-      if (cap) {                                                                               \
-        batch_kernel_##SUFFIX<false, true, false><<<grid, block, 0, st>>>(base, owner, coord, H, parity, acc, zc); \
-        batch_kernel_##SUFFIX<false, true, true><<<grid, block, 0, stf>>>(base, owner, coord, H, parity, acc, zc); \
-      } else {                                                                                 \
-        batch_kernel_##SUFFIX<false, false, false><<<grid, block, 0, st>>>(base, owner, coord, H, parity, acc, zc); \
-        batch_kernel_##SUFFIX<false, false, true><<<grid, block, 0, stf>>>(base, owner, coord, H, parity, acc, zc); \
-      }                                                                                        \
+    auto k0 = check ? (cap ? batch_kernel_##SUFFIX<true, true, false, true>                    \
+                           : batch_kernel_##SUFFIX<true, false, false, true>)                  \
+                    : (cap ? batch_kernel_##SUFFIX<false, true, false, true>                   \
+                           : batch_kernel_##SUFFIX<false, false, false, true>);                \
+    auto k1 = check ? (cap ? batch_kernel_##SUFFIX<true, true, true, true>                     \
+                           : batch_kernel_##SUFFIX<true, false, true, true>)                   \
+                    : (cap ? batch_kernel_##SUFFIX<false, true, true, true>                    \
+                           : batch_kernel_##SUFFIX<false, false, true, true>);                 \
+    k0<<<grid, block, 0, st>>>(base, owner, coord, H, parity, acc, zc);                        \
+    k1<<<grid, block, 0, stf>>>(base, owner, coord, H, parity, acc, zc);                       \
+    if (rates) { /* some lattice has other rates omega_9..18: their tiles */                   \
+      auto r0 = check ? batch_kernel_##SUFFIX<true, false, false, false>                       \
+                      : batch_kernel_##SUFFIX<false, false, false, false>;                     \
+      auto r1 = check ? batch_kernel_##SUFFIX<true, false, true, false>                        \
+                      : batch_kernel_##SUFFIX<false, false, true, false>;                      \
+      r0<<<grid, block, 0, st>>>(base, owner, coord, H, parity, acc, zc);                      \
+      r1<<<grid, block, 0, stf>>>(base, owner, coord, H, parity, acc, zc);                     \
     }                                                                                          \
     return cudaGetLastError();                                                                 \
   }                                                                                            \

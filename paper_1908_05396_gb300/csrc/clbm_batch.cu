@@ -68,6 +68,7 @@ struct clbm_batch_ctx {
   int blocks_per_sm = 8;
   bool cap = true;                    // register-capped kernel variant
   int sms = 1;
+  bool rates = false;                 // some attached lattice has rates omega_9..18 other than 1
   int mode = 0;                       // 0: persistent kernel; 1: one launch per lattice
   dim3 pl_block{32, 2, 1};            // mode 1: block of every lattice's step kernel
   int pl_npt = 5;                     // mode 1: 1, or 5 for the register-capped kernel
@@ -183,16 +184,16 @@ cudaError_t launch(clbm_batch_ctx* b, bool check) {
   switch (b->dtype) {
     case CLBM_F64:
       return launch_batch_f64(b->desc_base, b->d_owner, b->d_coord, b->d_hdr, b->parity, check,
-                              b->d_acc, b->zc, b->block, grid, b->stream, sf);
+                              b->d_acc, b->zc, b->block, grid, b->rates, b->stream, sf);
     case CLBM_F32:
       return launch_batch_f32(b->desc_base, b->d_owner, b->d_coord, b->d_hdr, b->parity, check,
-                              b->d_acc, b->zc, b->block, grid, b->stream, sf);
+                              b->d_acc, b->zc, b->block, grid, b->rates, b->stream, sf);
     case CLBM_F16R:
       return launch_batch_f16r(b->desc_base, b->d_owner, b->d_coord, b->d_hdr, b->parity, check,
-                               b->d_acc, b->zc, b->block, grid, b->stream, sf);
+                               b->d_acc, b->zc, b->block, grid, b->rates, b->stream, sf);
     default:
       return launch_batch_f16(b->desc_base, b->d_owner, b->d_coord, b->d_hdr, b->parity, check,
-                              b->d_acc, b->zc, b->block, grid, b->stream, sf);
+                              b->d_acc, b->zc, b->block, grid, b->rates, b->stream, sf);
   }
 }
 
@@ -315,16 +316,20 @@ cudaError_t launch_lattices(clbm_batch_ctx* b, bool check, int flip) {
 // Rebuild and upload the tables from the attached lattices' current state.
 int upload(clbm_batch_ctx* b) {
   BCK(b, cudaStreamSynchronize(b->stream));  // staging buffers and tables are free
-  int ntiles = 0, nlat = 0, ntiles0 = 0;
+  int ntiles = 0, nlat = 0;
+  int tile_end[BATCH_GROUPS] = {};
   b->h_owner.clear();
   b->h_coord.clear();
   char* stage = static_cast<char*>(b->h_stage);
-  // lattices without body force first, then those with: two launches
-  for (int pass = 0; pass < 2; ++pass) {
+  // lattices without body force first, then those with; in each, the unit
+  // rates omega_9..18 first, then others: a launch each
+  for (int pass = 0; pass < BATCH_GROUPS; ++pass) {
     for (int s = 0; s < b->capacity; ++s) {
       clbm_ctx* h = b->slots[s];
       // in-place lattices (mode 1 only) have no place in the tile tables
-      if (!h || h->in_place || (h->P.has_force != 0) != (pass == 1)) continue;
+      if (!h || h->in_place ||
+          (h->P.has_force ? 2 : 0) + (unit_rates(h->P) ? 0 : 1) != pass)
+        continue;
       const int threads = int(b->block.x * b->block.y);
       const int tw = tile_width(h->g.nx, int(h->elem), int(b->block.x), threads);
       int twl = 0;
@@ -348,7 +353,12 @@ int upload(clbm_batch_ctx* b) {
       ntiles += tx * ty * tz;
       ++nlat;
     }
-    if (pass == 0) ntiles0 = ntiles;
+    tile_end[pass] = ntiles;
+  }
+  const bool rates = tile_end[1] > tile_end[0] || tile_end[3] > tile_end[2];
+  if (rates != b->rates) {
+    b->rates = rates;
+    drop_graph(b);  // the graph has, or lacks, the launches of the other rates
   }
   if (ntiles > b->owner_cap) {
     if (b->d_owner) BCK(b, cudaFree(b->d_owner));
@@ -362,7 +372,12 @@ int upload(clbm_batch_ctx* b) {
     drop_graph(b);  // the graph holds the old table address
   }
   const unsigned st0 = unsigned(uint64_t(b->steps));
-  BatchHeader hdr{nlat, ntiles, ntiles0, 0, {st0, st0}, {0, 0}};
+  BatchHeader hdr{};
+  hdr.nlat = nlat;
+  for (int k = 0; k < BATCH_GROUPS; ++k) {
+    hdr.tile_end[k] = tile_end[k];
+    hdr.step[k] = st0;
+  }
   if (nlat) BCK(b, upload_desc(b->dtype, stage, b->desc_base, nlat));
   if (ntiles) {
     BCK(b, cudaMemcpy(b->d_owner, b->h_owner.data(), size_t(ntiles) * sizeof(int),

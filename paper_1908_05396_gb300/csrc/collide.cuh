@@ -11,6 +11,7 @@
 #pragma once
 
 #include "d3q19.cuh"
+#include "log_table.h"
 #include "v2.cuh"
 
 namespace clbm {
@@ -20,22 +21,26 @@ namespace clbm {
 template <typename R> struct ScalarOf { using type = R; };
 template <> struct ScalarOf<V2> { using type = float; };
 
+// Constants of the FP64 step of the omega solve.
+template <typename R> struct SolveConst64 {};
+template <> struct SolveConst64<double> {
+  double clog;      // log(3 K) + (n-1)/2 log 9
+  double eh, nm1;   // (n - 1) / 2, n - 1 (power-law index n)
+  double tlo, thi;  // 3 nu_min, 3 nu_max (clamp of 1/w - 1/2)
+};
+
 // Per-lattice constants of the collision, in the math precision R.
 template <typename R>
-struct CollideConst {
+struct CollideConst : SolveConst64<R> {
   R rho0;
-  R F[3];        // body force
   R rhoS;        // lam rho0 and lam F: rest density and force of deviations
   R FS[3];       //   carried scaled by lam (FP16 storage: lam = 1024; else 1)
-  R K3;          // 3 K (K = mu_p, consistency coefficient, Eq. 5)
-  R logK3;       // log(3 K)
-  R log2K3;      // log2(3 K)
-  R n;           // power-law index
-  R rn;          // 1 / n
-  R ehalf;       // (n - 1) / 2
-  R ylo, yhi;    // log(3 nu_min), log(3 nu_max): clamp of y = log(1/w - 1/2)
-  R ylo2, yhi2;  // the same clamp in base 2
+  R r30;         // rhoS / 3
+  R K3;          // 3 K lam (K = mu_p, consistency coefficient, Eq. 5)
   R nu_min, nu_max;
+  // FP32 solve of every form: n, 1/n, (n-1)/2, log2(3 K lam) + (n-1)/2 log2 9,
+  // the clamp of y = log2(1/w - 1/2), lower bound of the invariant g2
+  float n, rn, ehalf, clog2, ylo2, yhi2, g2lo;
   int newtonian; // n == 1: omega_nu has a closed form
   int has_force;
   // The rates omega_9..18 enter only as factors of their own relaxation
@@ -43,8 +48,8 @@ struct CollideConst {
   // rate), and omega_9 scales the isotropic part of the strain rate.  They
   // are folded into the brackets' constants: c9 = -omega_9/126,
   // c10..c15 = omega_j/8, c16 = omega_16/12, c17 = omega_17/24,
-  // c18 = omega_18/8, cB = 6 omega_9^2 (unit rates give the constants of the
-  // printed forms exactly).
+  // c18 = omega_18/8, cB = omega_9^2 / 6 (unit rates give the constants of
+  // the printed forms exactly).
   R c9, c10, c11, c12, c13, c14, c15, c16, c17, c18, cB;
 };
 
@@ -71,137 +76,203 @@ template <typename R> __device__ __forceinline__ R rlg2(R x);
 template <> __device__ __forceinline__ float rlg2<float>(float x) { return lg2f(x); }
 template <typename R> __device__ __forceinline__ R rex2(R x);
 template <> __device__ __forceinline__ float rex2<float>(float x) { return ex2f(x); }
-template <typename R> __device__ __forceinline__ R rdiv(R a, R b);
-template <> __device__ __forceinline__ float rdiv<float>(float a, float b) { return __fdividef(a, b); }
-template <> __device__ __forceinline__ double rdiv<double>(double a, double b) { return a / b; }
-
-// Reciprocal: fast approximate (MUFU based, ~1 ulp) in FP32, IEEE in FP64.
+// Reciprocal on the special-function unit (1 ulp) in FP32; rcp64 in FP64.
+__device__ __forceinline__ float rcpf(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
 template <typename R> __device__ __forceinline__ R rrcp(R x);
-template <> __device__ __forceinline__ float rrcp<float>(float x) { return __fdividef(1.0f, x); }
-template <> __device__ __forceinline__ double rrcp<double>(double x) { return 1.0 / x; }
-
+template <> __device__ __forceinline__ float rrcp<float>(float x) { return rcpf(x); }
 template <> __device__ __forceinline__ V2 rlg2<V2>(V2 x) { return V2(lg2f(x.v.x), lg2f(x.v.y)); }
 template <> __device__ __forceinline__ V2 rex2<V2>(V2 x) { return V2(ex2f(x.v.x), ex2f(x.v.y)); }
-template <> __device__ __forceinline__ V2 rdiv<V2>(V2 a, V2 b) {
-  return V2(__fdividef(a.v.x, b.v.x), __fdividef(a.v.y, b.v.y));
-}
-template <> __device__ __forceinline__ V2 rrcp<V2>(V2 x) {
-  return V2(__fdividef(1.0f, x.v.x), __fdividef(1.0f, x.v.y));
-}
+template <> __device__ __forceinline__ V2 rrcp<V2>(V2 x) { return V2(rcpf(x.v.x), rcpf(x.v.y)); }
 
+// A product that the compiler may not fuse into a later sum.  The unit-rate
+// collision and the solve below spell out every fused multiply-add, so that
+// one node and a packed pair of nodes, in any kernel, round alike.
+__device__ __forceinline__ float mulr(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mulr(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ V2 mulr(V2 a, V2 b) { return a * b; }
+
+// Lower bound of the shear-rate invariant inside the logarithm.
 template <typename R> __device__ __forceinline__ R tiny();
 template <> __device__ __forceinline__ float tiny<float>() { return 1e-36f; }
 template <> __device__ __forceinline__ double tiny<double>() { return 1e-300; }
 template <> __device__ __forceinline__ V2 tiny<V2>() { return V2(1e-36f); }
 
 // Starting point of the solve below.  Without the bulk part B, the unknown
-// z = 1/omega - 1/2 = 3 nu solves z (z + 1/2)^(n-1) = P with
-// log2 P = log2(3K/rho) + (n-1)/2 log2 A, whose two asymptotes are
-// z = P^(1/n) (z >> 1/2) and z = 2^(n-1) P (z << 1/2); they meet at z = 1/2,
-// where log2 P = -n.  The guess takes the asymptote of its side (with A + B
-// for A), which three Newton steps then take to the FP32 rounding level
-// over the workloads' range of n, K and shear rate.
+// z = 1/omega - 1/2 = 3 nu solves z (z + 1/2)^(n-1) = P, whose two asymptotes
+// are z = P^(1/n) (z >> 1/2) and z = 2^(n-1) P (z << 1/2); they meet at
+// z = 1/2, where log2 P = -n.  The guess takes the asymptote of its side
+// (with A + B for A), which three Newton steps then take to the FP32 rounding
+// level over the workloads' range of n, K and shear rate.
 __device__ __forceinline__ float regime_guess(float lp, float n, float rn) {
-  return lp > -n ? lp * rn : lp + (n - 1.0f);
+  return lp > -n ? mulr(lp, rn) : lp + (n - 1.0f);
 }
 __device__ __forceinline__ V2 regime_guess(V2 lp, float n, float rn) {
   return V2(regime_guess(lp.v.x, n, rn), regime_guess(lp.v.y, n, rn));
 }
 
-// Newton iterations on y = log2(1/omega - 1/2) for
-//   G(y) = y - log2(3K/rho) - (n-1)/2 log2(omega(y)^2 A + B) = 0,
+// The solve for omega_nu, on y = log2(1/omega - 1/2):
+//   G(y) = y - c - (n-1)/2 log2(g2),  g2 = omega(y)^2 A + B,
 // i.e. 1/omega - 1/2 = 3 nu with nu = (K/rho) gamma_dot^(n-1) (Eq. 6,
-// Eq. localvarationsrelaxationtimes) and gamma_dot^2 = omega^2 A + B: the
-// omega part of the strain rate of Eq. strainratetensor is traceless, so its
-// invariant (Eq. shearrateexpression) is quadratic in omega.
-// dG/dy = 1 + (n-1) r tau omega with r = omega^2 A / gamma_dot^2 and
-// tau omega in (0, 1) (the base of the logarithm cancels), so G is
+// Eq. localvarationsrelaxationtimes) and gamma_dot^2 = (9 / rho^2) g2 (see
+// strain_AB): the omega part of the strain rate of Eq. strainratetensor is
+// traceless, so its invariant (Eq. shearrateexpression) is quadratic in
+// omega.  The factor 9 / rho^2 sits in c = log2(3 K) + (n-1)/2 log2 9 - n log2 rho.
+// dG/dy = 1 + (n-1) r s with r = omega^2 A / g2 and s = tau omega
+// = 1 - omega/2 in (0, 1) (the base of the logarithm cancels), so G is
 // increasing with slope between min(n, 1) and max(n, 1) and has one root;
 // projecting each iterate onto [ylo, yhi] makes the iteration land on the
-// clamp when the root lies beyond it.
+// clamp when the root lies beyond it.  The step G / (dG/dy) is taken as
+// G g2 / (g2 + (n-1) omega^2 A s): one reciprocal.
 template <typename R>
-__device__ __forceinline__ R newton_y2(R y, R c, R ehalf, R nm1, R A, R B, R ylo, R yhi,
+__device__ __forceinline__ R newton_y2(R y, R c, R ehalf, R nm1, R A, R B, R ylo, R yhi, R lo,
                                        int iters) {
 #pragma unroll 1
   for (int it = 0; it < iters; ++it) {
-    R tau = rex2<R>(y);
-    R w = rrcp<R>(tau + R(0.5));
-    R wwA = w * w * A;
-    R g2 = fmax(wwA + B, tiny<R>());
-    R G = (y - c) - ehalf * rlg2<R>(g2);
-    R dG = R(1) + nm1 * rdiv<R>(wwA, g2) * (tau * w);
-    y = fmin(fmax(y - rdiv<R>(G, dG), ylo), yhi);
+    const R w = rrcp<R>(rex2<R>(y) + R(0.5f));
+    const R wwA = mulr(mulr(w, w), A);
+    const R g2 = fmax(wwA + B, lo);
+    const R G = fma(-ehalf, rlg2<R>(g2), y - c);
+    const R den = fma(nm1, mulr(wwA, fma(R(-0.5f), w, R(1.0f))), g2);
+    y = fmin(fmax(fma(-mulr(G, g2), rrcp<R>(den), y), ylo), yhi);
   }
   return y;
 }
 
-// omega_nu from A and B (see above); writes |gamma_dot| at that omega.
+// omega_nu from rho (scaled by lam), its reciprocal and A, B of strain_AB.
 // FP32 (one node or a pair): the regime guess and three Newton steps reach
 // the FP32 rounding level.
 template <typename R>
-__device__ __forceinline__ R omega_nu(const CollideConst<float>& C, R rho, R rinv, R A, R B,
-                                      R* gd) {
-  R w;
+__device__ __forceinline__ R solve_y2(const float n, const float rn, const float ehalf,
+                                      const float clog2, const float ylo2, const float yhi2,
+                                      const float lo, R rho, R A, R B) {
+  const R c = fma(R(-n), rlg2<R>(rho), R(clog2));
+  const R lp = fma(R(ehalf), rlg2<R>(fmax(A + B, R(lo))), c);
+  const R y = fmin(fmax(regime_guess(lp, n, rn), R(ylo2)), R(yhi2));
+  return newton_y2<R>(y, c, R(ehalf), R(n - 1.0f), A, B, R(ylo2), R(yhi2), R(lo), 3);
+}
+template <typename R>
+__device__ __forceinline__ R omega_nu(const CollideConst<float>& C, R rho, R rinv, R A, R B) {
   if (C.newtonian) {
-    R nu = fmin(fmax(R(C.K3 * (1.0f / 3.0f)) * rinv, R(C.nu_min)), R(C.nu_max));
-    w = rrcp<R>(R(3.0f) * nu + R(0.5f));
-  } else {
-    const R c = R(C.log2K3) - rlg2<R>(rho);
-    const R lp = c + R(C.ehalf) * rlg2<R>(fmax(A + B, tiny<R>()));
-    R y0 = regime_guess(lp, C.n, C.rn);
-    y0 = fmin(fmax(y0, R(C.ylo2)), R(C.yhi2));
-    const R y = newton_y2<R>(y0, c, R(C.ehalf), R(C.n - 1.0f), A, B, R(C.ylo2), R(C.yhi2), 3);
-    w = rrcp<R>(rex2<R>(y) + R(0.5f));
+    const R nu = fmin(fmax(mulr(R(C.K3 * (1.0f / 3.0f)), rinv), R(C.nu_min)), R(C.nu_max));
+    return rrcp<R>(fma(R(3.0f), nu, R(0.5f)));
   }
-  *gd = sqrt(fmax(w * w * A + B, R(0.0f)));
-  return w;
+  const R y = solve_y2<R>(C.n, C.rn, C.ehalf, C.clog2, C.ylo2, C.yhi2, C.g2lo, rho, A, B);
+  return rrcp<R>(rex2<R>(y) + R(0.5f));
 }
 
-// FP64: the FP32 solve, then one Halley step in FP64 on the natural-log
-// y = log(1/omega - 1/2).  Halley's step converges cubically, so from the
-// FP32 estimate (relative error ~1e-5) it lands at the FP64 rounding level.
-// With s = tau omega and r as above,
+// ---- FP64 helpers -----------------------------------------------------------
+// FP64 arithmetic runs at 1/64 of the FP32 rate on this part and bounds the
+// FP64 step, so the solve spends as few FP64 instructions as it can: seeds
+// come from FP32, and conversions between the types are integer operations
+// on the bit patterns (the hardware's conversions share the FP64 rate).
+
+// A normal float as a double, exactly (zero comes out as 2^-127).
+__device__ __forceinline__ double widen(float x) {
+  const unsigned b = __float_as_uint(x);
+  const unsigned hi = ((b & 0x7fffffffu) >> 3) + 0x38000000u;
+  return __hiloint2double(int(hi | (b & 0x80000000u)), int(b << 29));
+}
+
+// A non-negative double truncated to float; zero and values below 2^-125 give 2^-125.
+__device__ __forceinline__ float narrow(double x) {
+  const int hi = __double2hiint(x);
+  const unsigned lo = unsigned(__double2loint(x));
+  return hi < 0x38200000 ? 2.3509887e-38f
+                         : __uint_as_float((unsigned(hi - 0x38000000) << 3) | (lo >> 29));
+}
+
+// 1/x for normal x: the FP32 reciprocal of the mantissa as the seed r0, then
+// r0 (1 + e + e^2) with e = 1 - x r0 (the cubically convergent iteration):
+// the seed's 2^-22 leaves 2^-66, below the rounding of the last operation.
+__device__ __forceinline__ double rcp64(double x) {
+  const int hi = __double2hiint(x);
+  const unsigned lo = unsigned(__double2loint(x));
+  const float m = __uint_as_float(0x3f800000u | ((unsigned(hi) & 0xfffffu) << 3) | (lo >> 29));
+  const unsigned s = __float_as_uint(rcpf(m));
+  // exponent of the seed minus that of x, and the sign of x
+  const int e = (hi & 0x7ff00000) - 0x3ff00000;
+  const double r0 = __hiloint2double(
+      (int((s >> 3) + 0x38000000u) - e) | (hi & int(0x80000000u)), int(s << 29));
+  const double d = fma(-x, r0, 1.0);
+  return fma(r0, fma(d, d, d), r0);
+}
+
+template <> __device__ __forceinline__ double rrcp<double>(double x) { return rcp64(x); }
+
+// Natural logarithm of a positive normal x, as (exponent, log of the mantissa)
+// with x = 2^ex z: z = 1 + i/128 to within 1/256, and with the table's c near
+// 1/z, log z = -log c + log1p(r), r = z c - 1, |r| < 2^-8 (P. T. P. Tang,
+// ACM TOMS 16(4), 1990).  The series to r^6 leaves r^7/7 < 2^-58.
+__device__ __forceinline__ double log_mant(double x, int& ex) {
+  const int hi = __double2hiint(x) + 0x1000;
+  ex = (hi >> 20) - 1023;
+  const double z = __hiloint2double(__double2hiint(x) - (ex << 20), __double2loint(x));
+  const double2 t = __ldg(&LOG_TAB[(hi >> 13) & 127]);
+  const double r = fma(z, t.x, -1.0);
+  double p = fma(r, -1.0 / 6.0, 0.2);
+  p = fma(r, p, -0.25);
+  p = fma(r, p, 1.0 / 3.0);
+  p = fma(r, p, -0.5);
+  return t.y + fma(mulr(r, r), p, r);
+}
+
+// FP64: the FP32 solve gives tau0 = 1/omega - 1/2 to about 1e-6, taken as the
+// exact value of a float; one Halley step in FP64 on y = log tau then lands
+// at the FP64 rounding level (it converges cubically).  With g2, r and s as
+// above at tau0, and G = log(tau0 rho) - log(3 K) - (n-1)/2 log(9 g2 / rho^2)
+// (two logarithms, each by log_mant),
 //   G'  = 1 + (n-1) r s,
 //   G'' = (n-1) [s omega r / 2 - 2 r (1 - r) s^2]
-// (from d(tau omega)/dy = tau omega^2 / 2 and dr/dy = -2 r (1 - r) s), and
-// the step is dy = -2 G G' / (2 G'^2 - G G'').  tau = exp(y) is then carried
-// to the new y by exp(dy) = 1 + dy + dy^2/2 + dy^3/6 (|dy| ~ 1e-5, so the
-// omitted terms lie below 1e-20), or set to 3 nu exactly on a clamp.
+// (from ds/dy = tau omega^2 / 2 and dr/dy = -2 r (1 - r) s), and the step is
+// dy = d1 (1 - d1 G'' / (2 G')) with d1 = -G/G'.  The correction of the second
+// factor is of the order of dy, so it needs FP32 only.  tau is carried to the new y
+// by exp(dy) = 1 + dy + dy^2/2 + dy^3/6.
 __device__ __forceinline__ double omega_nu(const CollideConst<double>& C, double rho,
-                                           double rinv, double A, double B, double* gd) {
-  double w;
+                                           double rinv, double A, double B) {
   if (C.newtonian) {
-    double nu = fmin(fmax(C.K3 * (1.0 / 3.0) * rinv, C.nu_min), C.nu_max);
-    w = 1.0 / (3.0 * nu + 0.5);
-  } else {
-    const float rf = float(rho), Af = float(A), Bf = float(B);
-    const float cf = float(C.log2K3) - lg2f(rf);
-    const float lp = cf + float(C.ehalf) * lg2f(fmaxf(Af + Bf, 1e-36f));
-    float yf = regime_guess(lp, float(C.n), float(C.rn));
-    yf = fminf(fmaxf(yf, float(C.ylo2)), float(C.yhi2));
-    yf = newton_y2<float>(yf, cf, float(C.ehalf), float(C.n) - 1.0f, Af, Bf, float(C.ylo2),
-                          float(C.yhi2), 3);
-    const double y0 = fmin(fmax(double(yf) * 0.69314718055994530942, C.ylo), C.yhi);
-    const double tau = exp(y0);
-    const double w0 = 1.0 / (tau + 0.5);
-    const double wwA = w0 * w0 * A;
-    const double g2 = fmax(wwA + B, 1e-300);
-    const double nm1 = C.n - 1.0;
-    const double G = (y0 - (C.logK3 - log(rho))) - C.ehalf * log(g2);
-    const double r = wwA / g2;
-    const double sw = tau * w0;
-    const double G1 = 1.0 + nm1 * r * sw;
-    const double G2 = nm1 * (sw * (0.5 * w0) * r - 2.0 * r * (1.0 - r) * sw * sw);
-    const double dy = -2.0 * G * G1 / (2.0 * G1 * G1 - G * G2);
-    const double y1 = y0 + dy;
-    double tau1;
-    if (y1 <= C.ylo) tau1 = 3.0 * C.nu_min;
-    else if (y1 >= C.yhi) tau1 = 3.0 * C.nu_max;
-    else tau1 = tau + tau * (dy * (1.0 + dy * (0.5 + dy * (1.0 / 6.0))));
-    w = 1.0 / (tau1 + 0.5);
+    const double nu = fmin(fmax(mulr(C.K3 * (1.0 / 3.0), rinv), C.nu_min), C.nu_max);
+    return rcp64(fma(3.0, nu, 0.5));
   }
-  *gd = sqrt(fmax(w * w * A + B, 0.0));
-  return w;
+  const float Af = narrow(A), Bf = narrow(B);
+  const float yf = solve_y2<float>(C.n, C.rn, C.ehalf, C.clog2, C.ylo2, C.yhi2, C.g2lo,
+                                   narrow(rho), Af, Bf);
+  const double tau = widen(ex2f(yf));
+  const double w = rcp64(tau + 0.5);
+  const double wwA = mulr(mulr(w, w), A);
+  double g2 = wwA + B;
+  if (g2 < 1e-300) g2 = 1e-300;
+  int e1, e2;
+  const double l1 = log_mant(mulr(tau, rho), e1);
+  const double l2 = log_mant(mulr(mulr(rinv, rinv), g2), e2);
+  const double LN2 = 0.69314718055994530942;
+  const double L1 = fma(widen(float(e1)), LN2, l1), L2 = fma(widen(float(e2)), LN2, l2);
+  const double G = fma(-C.eh, L2, L1 - C.clog);
+  const double s = fma(-0.5, w, 1.0);
+  const double den = fma(C.nm1, mulr(wwA, s), g2);
+  const double d1 = mulr(-mulr(G, g2), rcp64(den));  // -G / G'
+  const float wf = narrow(w), sf = narrow(s), nm1 = C.n - 1.0f;
+  const float rf = fminf(narrow(wwA) * rcpf(narrow(g2)), 1.0f);
+  const float G1 = 1.0f + nm1 * rf * sf;
+  const float G2 = nm1 * (0.5f * sf * wf * rf - 2.0f * rf * (1.0f - rf) * sf * sf);
+  // the magnitude of d1 with its sign; |d1| is large only when the root lies
+  // beyond a clamp, where the sign of dy decides
+  const float d1f = copysignf(narrow(fabs(d1)), __uint_as_float(unsigned(__double2hiint(d1))));
+  const float h = fminf(fmaxf(-0.5f * G2 * rcpf(G1) * d1f, -0.25f), 0.25f);
+  const double dy = fma(d1, widen(h), d1);
+  double t1 = fma(tau, mulr(dy, fma(dy, fma(dy, 1.0 / 6.0, 0.5), 1.0)), tau);
+  if (t1 < C.tlo) t1 = C.tlo;
+  else if (t1 > C.thi) t1 = C.thi;
+  return rcp64(t1 + 0.5);
+}
+
+// |gamma_dot| at the solved omega.
+template <typename R>
+__device__ __forceinline__ R shear_rate(R rinv, R w, R A, R B) {
+  return mulr(mulr(R(3), rinv), sqrt(fma(mulr(w, w), A, B)));
 }
 
 // ---- pair space -------------------------------------------------------------
@@ -480,20 +551,21 @@ constexpr bool add_K_g_source() {
 static_assert(add_K_g_is_K(), "the additive back-transform must add the columns of K");
 static_assert(add_K_g_source(), "the additive back-transform must add the body-force source");
 
-// gamma_dot^2 = omega^2 A + B from Eq. strainratetensor (bulk rate omega_9)
-// and Eq. shearrateexpression, for the non-equilibrium moments m^(1)_4..9
-// (Sec. 3.2): with q = 1/(2 rho), the traceless part gives
-// A = 12 q^2 [m7^2 - m7 m8 + m8^2 + 3 (m4^2 + m5^2 + m6^2)] and the
-// isotropic part B = 6 omega_9^2 q^2 m9^2.
+// gamma_dot^2 = (9 / rho^2) (omega^2 A + B) from Eq. strainratetensor (bulk
+// rate omega_9) and Eq. shearrateexpression, for the non-equilibrium moments
+// m^(1)_4..9 (Sec. 3.2): the traceless part gives
+// A = (m7^2 - m7 m8 + m8^2) / 3 + m4^2 + m5^2 + m6^2 and the isotropic part
+// B = omega_9^2 m9^2 / 6.
 template <typename R, typename T>
-__device__ __forceinline__ void strain_AB(const CollideConst<T>& C, R rinv, R m4, R m5, R m6,
-                                          R m7, R m8, R m9, R& A, R& B) {
-  const R q2 = R(0.25) * rinv * rinv;
-  A = R(12) * q2 * (m7 * m7 - m7 * m8 + m8 * m8 + R(3) * (m4 * m4 + m5 * m5 + m6 * m6));
-  B = R(C.cB) * q2 * m9 * m9;  // 6 omega_9^2 q^2 m9^2
+__device__ __forceinline__ void strain_AB(const CollideConst<T>& C, R m4, R m5, R m6, R m7, R m8,
+                                          R m9, R& A, R& B) {
+  const R d = fma(m7, m7 - m8, mulr(m8, m8));
+  A = fma(R(1.0 / 3.0), d, fma(m4, m4, fma(m5, m5, mulr(m6, m6))));
+  B = mulr(mulr(R(C.cB), m9), m9);
 }
 
-// Collide one node.  d[19] holds the pre-collision deviations on entry and
+// Collide one node with any relaxation rates omega_9..18 (collide_unit below
+// takes the unit rates of Sec. 3.1).  d[19] holds the pre-collision deviations on entry and
 // the post-collision deviations f~ - w rho0 on return.
 // PAIR_OUT selects how the populations are written back: rebuilt from the
 // pair values (fewer registers: the 19 inputs are dead after the pair values
@@ -510,9 +582,9 @@ __device__ __forceinline__ void strain_AB(const CollideConst<T>& C, R rinv, R m4
 // of m^(1)/rho, the omega solve of 3K/rho), so the scaled populations come
 // out exactly as lam times the unscaled ones up to rounding, and only rho
 // is unscaled for the output.
-template <typename R, bool FORCE, bool PAIR_OUT = false, int LOG2LAM = 0>
-__device__ __forceinline__ void collide(const CollideConst<typename ScalarOf<R>::type>& C,
-                                        R (&d)[Q], NodeOut<R>& out) {
+template <typename R, bool FORCE, bool PAIR_OUT, int LOG2LAM>
+__device__ __forceinline__ void collide_rates(const CollideConst<typename ScalarOf<R>::type>& C,
+                                              R (&d)[Q], NodeOut<R>& out) {
   using T = typename ScalarOf<R>::type;
   // ---- mass and momentum (Eqs. hydrodynamicfields1/2) -------------------
   static_assert(cx(1) == 1 && cy(3) == 1 && cz(5) == 1 && cx(7) == 1 && cy(7) == 1 &&
@@ -561,9 +633,8 @@ __device__ __forceinline__ void collide(const CollideConst<typename ScalarOf<R>:
   const R m9 = (Dxx + Dyy + Dzz) - drho - rho * (ux2 + uy2 + uz2);
 
   R A, B;
-  strain_AB(C, rinv, m4, m5, m6, m7, m8, m9, A, B);
-  R gd;
-  const R w = omega_nu(C, rho, rinv, A, B, &gd);
+  strain_AB(C, m4, m5, m6, m7, m8, m9, A, B);
+  const R w = omega_nu(C, rho, rinv, A, B);
 
   // ---- change of moments, Eqs. collisionkernelg4..g18 --------------------
   // omega_4..8 = w (Sec. 3.1); omega_9..18 from the constants above (1 in Sec. 3.1).
@@ -655,7 +726,272 @@ __device__ __forceinline__ void collide(const CollideConst<typename ScalarOf<R>:
   out.ux = ux;
   out.uy = uy;
   out.uz = uz;
-  out.gamma_dot = gd;
+  out.gamma_dot = shear_rate(rinv, w, A, B);
+}
+
+// Collide one node with the rates omega_9..18 = 1 of Sec. 3.1, the default.
+//
+// With unit rates every third- and fourth-order central moment relaxes to its
+// attractor in one step (Eqs. centralmomentrelaxation,
+// discretecentralmomentattractors), so the post-collision raw moments follow
+// from rho, u and the relaxed second-order central moments alone, and the
+// brackets of g^_10..g^_18 need not be formed.  With J = rho u, the
+// non-equilibrium moments m_ij = k'_ij - J_i u_j (m^(1)_4..6 of Sec. 3.2),
+// s_i = D_ii - J_i u_i, their trace part m9 = s_x + s_y + s_z - (rho - rho0)
+// (m^(1)_9) and traceless parts e_i = s_i - (s_x + s_y + s_z)/3 (m^(1)_7 and
+// m^(1)_8 are differences of them):
+//   c_ij  = (1 - omega) m_ij                 relaxed central moments, order 2
+//   c_ii  = rho/3 + a_i, a_i = (1 - omega) e_i    (the trace relaxes fully)
+//   k_ii  = c_ii + J_i u_i                   raw
+//   k_iij = 2 u_i c_ij + u_j k_ii            raw, order 3 (central: 0)
+//   k_iijj = c*_iijj + u_i^2 k_jj + u_j^2 c_ii + 4 u_i u_j c_ij
+//            with the attractor c*_iijj = (rho/3 + a_i)(rho/3 + a_j)/rho,
+// each taken relative to the rest state so that rho0/3 and rho0/9 cancel
+// analytically.  The gamma_dot invariant of strain_AB is
+// A = (e_x^2 + e_y^2 + e_z^2)/2 + m_xy^2 + m_xz^2 + m_yz^2, B = m9^2 / 6.
+// Against collide_rates with the same rates this takes 232 FP operations per
+// node instead of 424 (pair output; 240 instead of 475 with one correction
+// per population), counted with every possible multiply-add fused.  What it
+// gave: the FP64 step is bound by the FP64 pipe and went from 2030 to 978 us
+// on 128^3 (with the solve above); on 256^3 FP32 went from 431 to 379 us a
+// step (6.7 TB/s), F16S from 395 to 323 and F16R from 792 to 753 us, and no
+// register-capped FP32 or FP16 kernel spills any more.
+//
+// PAIR_OUT, LOG2LAM and the body force's symmetric split are as in
+// collide_rates.  With PAIR_OUT the populations are rebuilt from the raw
+// moments; without it the moments' increments are added to the populations,
+// one correction each.
+template <typename R, bool FORCE, bool PAIR_OUT, int LOG2LAM>
+__device__ __forceinline__ void collide_unit(const CollideConst<typename ScalarOf<R>::type>& C,
+                                             R (&d)[Q], NodeOut<R>& out) {
+  using T = typename ScalarOf<R>::type;
+  const Pairs<R> p = to_pairs(d);
+  // ---- mass, momentum, second moments (Eqs. hydrodynamicfields1/2) --------
+  const R Dxx = p.sAx + (p.Dxxyy + p.Dxxzz), Dyy = p.sAy + (p.Dxxyy + p.Dyyzz),
+          Dzz = p.sAz + (p.Dxxzz + p.Dyyzz);
+  const R drho = (p.d0 + Dxx) + ((p.sAy + p.sAz) + p.Dyyzz);
+  const R jx = p.tAx + (p.Dxyy + p.Dxzz), jy = p.tAy + (p.Dxxy + p.Dyzz),
+          jz = p.tAz + (p.Dxxz + p.Dyyz);
+  const R rho = R(C.rhoS) + drho;
+  const R rinv = rrcp<R>(rho);
+  R Jx = jx, Jy = jy, Jz = jz;
+  if (FORCE) {
+    // rho u = j + F/2
+    Jx = jx + R(T(0.5) * C.FS[0]);
+    Jy = jy + R(T(0.5) * C.FS[1]);
+    Jz = jz + R(T(0.5) * C.FS[2]);
+  }
+  const R ux = mulr(Jx, rinv), uy = mulr(Jy, rinv), uz = mulr(Jz, rinv);
+  // half of the source S before the collision: S_ii = 2 u_i F_i, S_ij = u_i F_j + u_j F_i
+  R Fx(0), Fy(0), Fz(0), hFx(0), hFy(0), hFz(0);
+  R hxx = Dxx, hyy = Dyy, hzz = Dzz, hxy = p.Dxy, hxz = p.Dxz, hyz = p.Dyz;
+  if (FORCE) {
+    Fx = R(C.FS[0]), Fy = R(C.FS[1]), Fz = R(C.FS[2]);
+    hFx = R(T(0.5) * C.FS[0]), hFy = R(T(0.5) * C.FS[1]), hFz = R(T(0.5) * C.FS[2]);
+    hxx = fma(ux, Fx, hxx);
+    hyy = fma(uy, Fy, hyy);
+    hzz = fma(uz, Fz, hzz);
+    hxy = fma(ux, hFy, fma(uy, hFx, hxy));
+    hxz = fma(ux, hFz, fma(uz, hFx, hxz));
+    hyz = fma(uy, hFz, fma(uz, hFy, hyz));
+  }
+  // ---- non-equilibrium second moments -------------------------------------
+  const R third = R(T(1.0 / 3.0));
+  const R sx = fma(-Jx, ux, hxx), sy = fma(-Jy, uy, hyy), sz = fma(-Jz, uz, hzz);
+  const R mxy = fma(-Jx, uy, hxy), mxz = fma(-Jx, uz, hxz), myz = fma(-Jy, uz, hyz);
+  const R tr = (sx + sy) + sz;
+  const R m9 = tr - drho;
+  const R ex = fma(-third, tr, sx), ey = fma(-third, tr, sy), ez = fma(-third, tr, sz);
+  const R A = fma(R(T(0.5)), fma(ex, ex, fma(ey, ey, mulr(ez, ez))),
+                  fma(mxy, mxy, fma(mxz, mxz, mulr(myz, myz))));
+  const R B = mulr(mulr(R(T(1.0 / 6.0)), m9), m9);
+  const R w = omega_nu(C, rho, rinv, A, B);
+
+  // ---- relaxed second moments ------------------------------------------------
+  const R wm = R(T(1.0)) - w;
+  const R cxy = mulr(wm, mxy), cxz = mulr(wm, mxz), cyz = mulr(wm, myz);
+  const R ax = mulr(wm, ex), ay = mulr(wm, ey), az = mulr(wm, ez);
+  const R dr3 = mulr(third, drho);
+  const R zx = ax + dr3, zy = ay + dr3, zz = az + dr3;
+  const R Exx = fma(Jx, ux, zx), Eyy = fma(Jy, uy, zy), Ezz = fma(Jz, uz, zz);
+  const R r30 = R(C.r30);
+  const R kxx = Exx + r30, kyy = Eyy + r30, kzz = Ezz + r30;
+  const R cxx = zx + r30, cyy = zy + r30;
+
+  if constexpr (PAIR_OUT) {
+    // a quarter of every plane moment: the populations of a plane are sums
+    // and differences of the four quarters (plane_out)
+    const R q4 = R(T(0.25)), h2 = R(T(0.5));
+    const R qx = mulr(q4, ux), qy = mulr(q4, uy), qz = mulr(q4, uz);
+    const R hx = mulr(h2, ux), hy = mulr(h2, uy), hz = mulr(h2, uz);
+    R oxyy = mulr(qx, kyy), oxzz = mulr(qx, kzz), oxxy = mulr(qy, kxx), oyzz = mulr(qy, kzz),
+      oxxz = mulr(qz, kxx), oyyz = mulr(qz, kyy);
+    R ddr = mulr(R(T(1.0 / 36.0)), drho);
+    R pxy = fma(Jx, qy, mulr(q4, cxy)), pxz = fma(Jx, qz, mulr(q4, cxz)),
+      pyz = fma(Jy, qz, mulr(q4, cyz));
+    R fExx = Exx, fEyy = Eyy, fEzz = Ezz;
+    R gx = mulr(h2, jx), gy = mulr(h2, jy), gz = mulr(h2, jz);
+    if (FORCE) {
+      // the other half of the source
+      const R fx = R(T(C.FS[0]) * T(1.0 / 24.0)), fy = R(T(C.FS[1]) * T(1.0 / 24.0)),
+              fz = R(T(C.FS[2]) * T(1.0 / 24.0));
+      oxyy = fma(qx, kyy, fx);
+      oxzz = fma(qx, kzz, fx);
+      oxxy = fma(qy, kxx, fy);
+      oyzz = fma(qy, kzz, fy);
+      oxxz = fma(qz, kxx, fz);
+      oyyz = fma(qz, kyy, fz);
+      pxy = fma(qx, hFy, fma(qy, hFx, pxy));
+      pxz = fma(qx, hFz, fma(qz, hFx, pxz));
+      pyz = fma(qy, hFz, fma(qz, hFy, pyz));
+      fExx = fma(ux, Fx, fExx);
+      fEyy = fma(uy, Fy, fEyy);
+      fEzz = fma(uz, Fz, fEzz);
+      gx = fma(h2, jx, hFx);
+      gy = fma(h2, jy, hFy);
+      gz = fma(h2, jz, hFz);
+      ddr = fma(R(T(1.0 / 12.0)), fma(ux, Fx, fma(uy, Fy, mulr(uz, Fz))), ddr);
+    }
+    oxyy = fma(hy, cxy, oxyy);
+    oxzz = fma(hz, cxz, oxzz);
+    oxxy = fma(hx, cxy, oxxy);
+    oyzz = fma(hz, cyz, oyzz);
+    oxxz = fma(hx, cxz, oxxz);
+    oyyz = fma(hy, cyz, oyyz);
+    // attractors: a quarter of (rho/3 + a_i)(rho/3 + a_j)/rho - rho0/9
+    const R qr = mulr(q4, rinv), tw = R(T(1.0 / 12.0));
+    const R by = fma(ay, qr, tw), bz = fma(az, qr, tw);
+    const R ty = fma(tw, ay, ddr), tz = fma(tw, az, ddr);
+    R fxy = fma(ax, by, ty), fxz = fma(ax, bz, tz), fyz = fma(ay, bz, tz);
+    const R qxx = mulr(qx, ux), qyy = mulr(qy, uy), qzz = mulr(qz, uz);
+    fxy = fma(mulr(ux, uy), cxy, fma(qyy, cxx, fma(qxx, kyy, fxy)));
+    fxz = fma(mulr(ux, uz), cxz, fma(qzz, cxx, fma(qxx, kzz, fxz)));
+    fyz = fma(mulr(uy, uz), cyz, fma(qzz, cyy, fma(qyy, kzz, fyz)));
+    if (FORCE) {
+      const R e8 = R(T(-0.125));
+      fxy = fma(e8, mulr(uz, Fz), fxy);
+      fxz = fma(e8, mulr(uy, Fy), fxz);
+      fyz = fma(e8, mulr(ux, Fx), fyz);
+    }
+    const R m2 = R(T(-2.0));
+    const R fs = fxy + fxz;
+    d[0] = fma(R(T(4.0)), fs + fyz, drho - ((fExx + fEyy) + fEzz));
+    {
+      const R hs = fma(m2, fs, mulr(h2, fExx)), ht = fma(m2, oxyy + oxzz, gx);
+      d[1] = hs + ht;
+      d[2] = hs - ht;
+    }
+    {
+      const R hs = fma(m2, fxy + fyz, mulr(h2, fEyy)), ht = fma(m2, oxxy + oyzz, gy);
+      d[3] = hs + ht;
+      d[4] = hs - ht;
+    }
+    {
+      const R hs = fma(m2, fxz + fyz, mulr(h2, fEzz)), ht = fma(m2, oxxz + oyyz, gz);
+      d[5] = hs + ht;
+      d[6] = hs - ht;
+    }
+    auto plane = [](R f, R pr, R oi, R oj, R& Pp, R& Pm, R& Mp, R& Mm) {
+      const R a = f + pr, b = f - pr, c = oi + oj, e = oi - oj;
+      Pp = a + c;
+      Pm = a - c;
+      Mp = b + e;
+      Mm = b - e;
+    };
+    plane(fxy, pxy, oxyy, oxxy, d[7], d[10], d[9], d[8]);
+    plane(fxz, pxz, oxzz, oxxz, d[11], d[14], d[13], d[12]);
+    plane(fyz, pyz, oyzz, oyyz, d[15], d[18], d[17], d[16]);
+  } else {
+    // increments of the moments (with the whole source S): n, r of order 2,
+    // t of order 3, q of order 4
+    const R nw = -w;
+    R nxy = mulr(nw, mxy), nxz = mulr(nw, mxz), nyz = mulr(nw, myz);
+    const R m93 = mulr(third, m9);
+    R rx = fma(nw, ex, -m93), ry = fma(nw, ey, -m93), rz = fma(nw, ez, -m93);
+    const R tux = ux + ux, tuy = uy + uy, tuz = uz + uz;
+    R bx = -p.Dxyy, cx_ = -p.Dxzz, by_ = -p.Dxxy, cy_ = -p.Dyzz, bz_ = -p.Dxxz, cz_ = -p.Dyyz;
+    R dr9 = mulr(R(T(1.0 / 9.0)), drho);
+    if (FORCE) {
+      const R fx = R(T(C.FS[0]) * T(1.0 / 6.0)), fy = R(T(C.FS[1]) * T(1.0 / 6.0)),
+              fz = R(T(C.FS[2]) * T(1.0 / 6.0));
+      bx = fx - p.Dxyy;
+      cx_ = fx - p.Dxzz;
+      by_ = fy - p.Dxxy;
+      cy_ = fy - p.Dyzz;
+      bz_ = fz - p.Dxxz;
+      cz_ = fz - p.Dyyz;
+      nxy = fma(ux, Fy, fma(uy, Fx, nxy));
+      nxz = fma(ux, Fz, fma(uz, Fx, nxz));
+      nyz = fma(uy, Fz, fma(uz, Fy, nyz));
+      const R two = R(T(2.0));
+      const R wx = mulr(ux, Fx), wy = mulr(uy, Fy), wz = mulr(uz, Fz);
+      rx = fma(two, wx, rx);
+      ry = fma(two, wy, ry);
+      rz = fma(two, wz, rz);
+      dr9 = fma(third, (wx + wy) + wz, dr9);
+    }
+    const R txyy = fma(tuy, cxy, fma(ux, kyy, bx)), txzz = fma(tuz, cxz, fma(ux, kzz, cx_));
+    const R txxy = fma(tux, cxy, fma(uy, kxx, by_)), tyzz = fma(tuz, cyz, fma(uy, kzz, cy_));
+    const R txxz = fma(tux, cxz, fma(uz, kxx, bz_)), tyyz = fma(tuy, cyz, fma(uz, kyy, cz_));
+    const R by = fma(ay, rinv, third), bz = fma(az, rinv, third);
+    const R ty = fma(third, ay, dr9), tz = fma(third, az, dr9);
+    const R ux2 = mulr(ux, ux), uy2 = mulr(uy, uy), uz2 = mulr(uz, uz);
+    R qxy = fma(ax, by, ty - p.Dxxyy), qxz = fma(ax, bz, tz - p.Dxxzz),
+      qyz = fma(ay, bz, tz - p.Dyyzz);
+    qxy = fma(mulr(tux, tuy), cxy, fma(uy2, cxx, fma(ux2, kyy, qxy)));
+    qxz = fma(mulr(tux, tuz), cxz, fma(uz2, cxx, fma(ux2, kzz, qxz)));
+    qyz = fma(mulr(tuy, tuz), cyz, fma(uz2, cyy, fma(uy2, kzz, qyz)));
+    if (FORCE) {
+      const R h2 = R(T(-0.5));
+      qxy = fma(h2, mulr(uz, Fz), qxy);
+      qxz = fma(h2, mulr(uy, Fy), qxz);
+      qyz = fma(h2, mulr(ux, Fx), qyz);
+    }
+    const R qs = qxy + qxz, half = R(T(0.5));
+    d[0] = d[0] + ((qs + qyz) - ((rx + ry) + rz));
+    {
+      const R e = rx - qs;
+      const R o = FORCE ? Fx - (txyy + txzz) : -(txyy + txzz);
+      d[1] = fma(half, e + o, d[1]);
+      d[2] = fma(half, e - o, d[2]);
+    }
+    {
+      const R e = ry - (qxy + qyz);
+      const R o = FORCE ? Fy - (txxy + tyzz) : -(txxy + tyzz);
+      d[3] = fma(half, e + o, d[3]);
+      d[4] = fma(half, e - o, d[4]);
+    }
+    {
+      const R e = rz - (qxz + qyz);
+      const R o = FORCE ? Fz - (txxz + tyyz) : -(txxz + tyyz);
+      d[5] = fma(half, e + o, d[5]);
+      d[6] = fma(half, e - o, d[6]);
+    }
+    auto plane = [](R q, R n, R ti, R tj, R& Pp, R& Pm, R& Mp, R& Mm) {
+      const R a = q + n, b = q - n, c = ti + tj, e = ti - tj, f = R(T(0.25));
+      Pp = fma(f, a + c, Pp);
+      Pm = fma(f, a - c, Pm);
+      Mp = fma(f, b + e, Mp);
+      Mm = fma(f, b - e, Mm);
+    };
+    plane(qxy, nxy, txyy, txxy, d[7], d[10], d[9], d[8]);
+    plane(qxz, nxz, txzz, txxz, d[11], d[14], d[13], d[12]);
+    plane(qyz, nyz, tyzz, tyyz, d[15], d[18], d[17], d[16]);
+  }
+  if constexpr (LOG2LAM != 0) out.rho = mulr(rho, R(T(1.0 / double(1 << LOG2LAM))));
+  else out.rho = rho;
+  out.ux = ux;
+  out.uy = uy;
+  out.uz = uz;
+  out.gamma_dot = shear_rate(rinv, w, A, B);
+}
+
+// UNIT: the rates omega_9..18 are all 1 (PhysParams::unit_rates).
+template <typename R, bool FORCE, bool PAIR_OUT, int LOG2LAM, bool UNIT>
+__device__ __forceinline__ void collide(const CollideConst<typename ScalarOf<R>::type>& C,
+                                        R (&d)[Q], NodeOut<R>& out) {
+  if constexpr (UNIT) collide_unit<R, FORCE, PAIR_OUT, LOG2LAM>(C, d, out);
+  else collide_rates<R, FORCE, PAIR_OUT, LOG2LAM>(C, d, out);
 }
 
 }  // namespace clbm

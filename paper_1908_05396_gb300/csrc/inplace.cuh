@@ -111,7 +111,8 @@ __device__ __forceinline__ void aa_lid_fix(int x, int y, int z, int nx, int ny, 
 // step (srcq[q] = A + q qs, dstq[q] = A + opp(q) qs); a.src is the buffer A.
 // Nodes off the y and z faces take the direct path (the x-face lanes fix
 // their crossing directions); nodes on a y or z face resolve every direction.
-template <typename S, typename R, int LIN, bool FORCE, bool CHECK, bool CAP>
+// UNIT as in step_kernel.
+template <typename S, typename R, int LIN, bool FORCE, bool CHECK, bool CAP, bool UNIT>
 __global__ void __launch_bounds__(256, CAP ? 4 : 1) step_aa_kernel(const StepArgs<S, R> a) {
   pdl_enter();
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -155,7 +156,7 @@ __global__ void __launch_bounds__(256, CAP ? 4 : 1) step_aa_kernel(const StepArg
                        a.lidc, d);
     }
     NodeOut<R> o;
-    collide<R, FORCE, pair_out<S>(), log2_scale<S>()>(a.C, d, o);
+    collide<R, FORCE, pair_out<S>(), log2_scale<S>(), UNIT>(a.C, d, o);
     if (LIN == 1) {
 #pragma unroll
       for (int q = 0; q < Q; ++q) a.dstq[q][i] = Codec<S, R>::enc(d[q], R(1));
@@ -206,13 +207,12 @@ __global__ void __launch_bounds__(256, CAP ? 4 : 1) step_aa_kernel(const StepArg
 // rho, u and |gamma_dot| of the next collision, from either layout.
 template <typename S, typename R, int L, bool FORCE>
 __global__ void __launch_bounds__(256) fields_aa_kernel(const S* __restrict__ A, Geom g,
-                                                        PhysParams P, double* rho, double* u,
-                                                        double* gd) {
+                                                        CollideConst<R> C, double* rho,
+                                                        double* u, double* gd) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z;
   if (x >= g.nx || y >= g.ny) return;
-  const CollideConst<R> C = make_const<R>(P, double(1 << log2_scale<S>()));
   R lidc[Q];
 #pragma unroll
   for (int q = 0; q < Q; ++q)
@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(256) fields_aa_kernel(const S* __restrict__ A,
   aa_read<S, R, L>(A, g.qstride, x, y, z, i, g.nx, g.ny, g.nz, g.pitch, int(g.plane), g.facebits,
                    lidc, d);
   NodeOut<R> o;
-  collide<R, FORCE, pair_out<S>(), log2_scale<S>()>(C, d, o);
+  collide<R, FORCE, pair_out<S>(), log2_scale<S>(), false>(C, d, o);
   const int64_t N = int64_t(g.nx) * g.ny * g.nz;
   const int64_t k = (int64_t(z) * g.ny + y) * g.nx + x;
   if (rho) rho[k] = double(o.rho);
@@ -313,19 +313,20 @@ cudaError_t launch_step_aa_t(void* buf, const Geom& g, const PhysParams& P, cons
   a.cb = cb;
   const bool cap = (npt & 4) != 0;
   const dim3 grid((g.nx + block.x - 1) / block.x, (g.ny + block.y - 1) / block.y, g.nz);
-  cudaError_t e = cudaSuccess;
-#define CLBM_AA_LAUNCH(L, F, C_)                                                                \
-  e = cap ? pdl_launch(step_aa_kernel<S, R, L, F, C_, true>, grid, block, st, a)                \
-          : pdl_launch(step_aa_kernel<S, R, L, F, C_, false>, grid, block, st, a)
+  void (*kernel)(const StepArgs<S, R>) = nullptr;
+#define CLBM_AA(L, F, C_)                                              \
+  kernel = !unit_rates(P) ? step_aa_kernel<S, R, L, F, C_, false, false> \
+           : cap          ? step_aa_kernel<S, R, L, F, C_, true, true>   \
+                          : step_aa_kernel<S, R, L, F, C_, false, true>
   if (layout == 0) {
-    if (P.has_force) { if (check) CLBM_AA_LAUNCH(0, true, true); else CLBM_AA_LAUNCH(0, true, false); }
-    else { if (check) CLBM_AA_LAUNCH(0, false, true); else CLBM_AA_LAUNCH(0, false, false); }
+    if (P.has_force) { if (check) CLBM_AA(0, true, true); else CLBM_AA(0, true, false); }
+    else { if (check) CLBM_AA(0, false, true); else CLBM_AA(0, false, false); }
   } else {
-    if (P.has_force) { if (check) CLBM_AA_LAUNCH(1, true, true); else CLBM_AA_LAUNCH(1, true, false); }
-    else { if (check) CLBM_AA_LAUNCH(1, false, true); else CLBM_AA_LAUNCH(1, false, false); }
+    if (P.has_force) { if (check) CLBM_AA(1, true, true); else CLBM_AA(1, true, false); }
+    else { if (check) CLBM_AA(1, false, true); else CLBM_AA(1, false, false); }
   }
-#undef CLBM_AA_LAUNCH
-  return e != cudaSuccess ? e : cudaGetLastError();
+#undef CLBM_AA
+  return pdl_launch(kernel, grid, block, st, a);
 }
 
 template <typename S, typename R>
@@ -334,12 +335,13 @@ cudaError_t launch_fields_aa_t(const void* buf, const Geom& g, const PhysParams&
   const dim3 block(32, 4);
   const dim3 grid((g.nx + 31) / 32, (g.ny + 3) / 4, g.nz);
   const S* A = static_cast<const S*>(buf);
+  const CollideConst<R> C = make_const<R>(P, double(1 << log2_scale<S>()));
   if (layout == 0) {
-    if (P.has_force) fields_aa_kernel<S, R, 0, true><<<grid, block, 0, st>>>(A, g, P, rho, u, gd);
-    else fields_aa_kernel<S, R, 0, false><<<grid, block, 0, st>>>(A, g, P, rho, u, gd);
+    if (P.has_force) fields_aa_kernel<S, R, 0, true><<<grid, block, 0, st>>>(A, g, C, rho, u, gd);
+    else fields_aa_kernel<S, R, 0, false><<<grid, block, 0, st>>>(A, g, C, rho, u, gd);
   } else {
-    if (P.has_force) fields_aa_kernel<S, R, 1, true><<<grid, block, 0, st>>>(A, g, P, rho, u, gd);
-    else fields_aa_kernel<S, R, 1, false><<<grid, block, 0, st>>>(A, g, P, rho, u, gd);
+    if (P.has_force) fields_aa_kernel<S, R, 1, true><<<grid, block, 0, st>>>(A, g, C, rho, u, gd);
+    else fields_aa_kernel<S, R, 1, false><<<grid, block, 0, st>>>(A, g, C, rho, u, gd);
   }
   return cudaGetLastError();
 }

@@ -58,32 +58,35 @@ __host__ __device__ constexpr bool pair_out() {
 }
 
 // Collision constants for deviations carried scaled by lam (a power of two;
-// see collide): the rest density and the force of the scaled moments, and
-// 3K, log(3K) so that nu and the omega solve come out unscaled.
+// see collide_rates): the rest density and the force of the scaled moments, and
+// 3K and its logarithm so that nu and the omega solve come out unscaled.
 template <typename R>
-__host__ __device__ __forceinline__ CollideConst<R> make_const(const PhysParams& P,
-                                                             double lam = 1.0) {
+inline CollideConst<R> make_const(const PhysParams& P, double lam = 1.0) {
+  const double L2E = 1.4426950408889634074;
   CollideConst<R> C;
   C.rho0 = R(P.rho0);
   C.rhoS = R(lam * P.rho0);
-  C.FS[0] = R(lam * P.F[0]);
-  C.FS[1] = R(lam * P.F[1]);
-  C.FS[2] = R(lam * P.F[2]);
-  C.F[0] = R(P.F[0]);
-  C.F[1] = R(P.F[1]);
-  C.F[2] = R(P.F[2]);
+  C.r30 = R(lam * P.rho0 / 3.0);
+  for (int a = 0; a < 3; ++a) C.FS[a] = R(lam * P.F[a]);
   C.K3 = R(3.0 * P.K * lam);
-  C.logK3 = R(P.logK3 + log(lam));
-  C.log2K3 = R(P.logK3 * 1.4426950408889634074 + log2(lam));
-  C.n = R(P.n);
-  C.rn = R(1.0 / P.n);
-  C.ehalf = R(0.5 * (P.n - 1.0));
-  C.ylo = R(P.ylo);
-  C.yhi = R(P.yhi);
-  C.ylo2 = R(P.ylo * 1.4426950408889634074);
-  C.yhi2 = R(P.yhi * 1.4426950408889634074);
   C.nu_min = R(P.nu_min);
   C.nu_max = R(P.nu_max);
+  const double clog = P.logK3 + log(lam) + 0.5 * (P.n - 1.0) * log(9.0);
+  if constexpr (std::is_same<R, double>::value) {
+    C.clog = clog;
+    C.eh = 0.5 * (P.n - 1.0);
+    C.nm1 = P.n - 1.0;
+    C.tlo = 3.0 * P.nu_min;
+    C.thi = 3.0 * P.nu_max;
+  }
+  C.n = float(P.n);
+  C.rn = float(1.0 / P.n);
+  C.ehalf = float(0.5 * (P.n - 1.0));
+  C.clog2 = float(clog * L2E);
+  C.ylo2 = float(P.ylo * L2E);
+  C.yhi2 = float(P.yhi * L2E);
+  // the invariant carries lam^2: the same shear rate for every scale
+  C.g2lo = float(1e-36 * lam * lam);
   C.newtonian = P.newtonian;
   C.has_force = P.has_force;
   const double* w = P.omega_high;  // omega_9 .. omega_18
@@ -97,7 +100,7 @@ __host__ __device__ __forceinline__ CollideConst<R> make_const(const PhysParams&
   C.c16 = R(w[7] / 12.0);
   C.c17 = R(w[8] / 24.0);
   C.c18 = R(0.125 * w[9]);
-  C.cB = R(6.0 * w[0] * w[0]);
+  C.cB = R(w[0] * w[0] / 6.0);
   return C;
 }
 
@@ -289,7 +292,8 @@ inline cudaError_t pdl_launch_smem(void (*kernel)(KArgs...), dim3 grid, dim3 blo
 #else
   cfg.numAttrs = 1;
 #endif
-  return cudaLaunchKernelEx(&cfg, kernel, args...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 template <typename... KArgs, typename... Args>
 inline cudaError_t pdl_launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t st,
@@ -306,7 +310,9 @@ inline cudaError_t pdl_launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, c
 // CAP = true caps registers so that four 256-thread (or eight 128-thread)
 // blocks fit on an SM: more warps to hide DRAM latency, at the risk of
 // spills; the autotuner decides.
-template <typename S, typename R, bool FORCE, bool CHECK, bool CAP>
+// UNIT: relaxation rates omega_9..18 all 1 (collide_unit); lattices with other
+// rates have no register-capped variant.
+template <typename S, typename R, bool FORCE, bool CHECK, bool CAP, bool UNIT>
 __global__ void __launch_bounds__(256, CAP ? 4 : 1) step_kernel(const StepArgs<S, R> a) {
   pdl_enter();
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -328,7 +334,7 @@ __global__ void __launch_bounds__(256, CAP ? 4 : 1) step_kernel(const StepArgs<S
                       i, a.lidc, d);
     }
     NodeOut<R> o;
-    collide<R, FORCE, pair_out<S>(), log2_scale<S>()>(a.C, d, o);
+    collide<R, FORCE, pair_out<S>(), log2_scale<S>(), UNIT>(a.C, d, o);
 #pragma unroll
     for (int q = 0; q < Q; ++q) a.dstq[q][i] = Codec<S, R>::enc(d[q], R(1));
     if (CHECK) {
@@ -415,7 +421,7 @@ __global__ void __launch_bounds__(128, CAP ? 4 : 1) step2_kernel(const StepArgs<
       for (int q = 0; q < Q; ++q) d[q] = V2(dA[q], dB[q]);
     }
     NodeOut<V2> o;
-    collide<V2, FORCE, pair_out<S>(), log2_scale<S>()>(a.C, d, o);
+    collide<V2, FORCE, pair_out<S>(), log2_scale<S>(), true>(a.C, d, o);
 #pragma unroll
     for (int q = 0; q < Q; ++q) a.dstq[q][iA] = Codec<S, float>::enc(lane0(d[q]), 1.0f);
     if (activeB) {
@@ -459,19 +465,18 @@ __global__ void __launch_bounds__(128, CAP ? 4 : 1) step2_kernel(const StepArgs<
 // Macroscopic fields of the current state (pull + moments + omega solve).
 template <typename S, typename R, bool FORCE>
 __global__ void __launch_bounds__(256) fields_kernel(const S* __restrict__ src, Geom g,
-                                                     PhysParams P, double* rho,
+                                                     CollideConst<R> C, double* rho,
                                                      double* u, double* gd) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z;
   if (x >= g.nx || y >= g.ny) return;
   const double lam = double(1 << log2_scale<S>());
-  const CollideConst<R> C = make_const<R>(P, lam);
   const int64_t i = int64_t(z) * g.plane + int64_t(y) * g.pitch + x;
   R d[Q];
   pull<S, R>(src, g, x, y, z, i, R(lam), d);
   NodeOut<R> o;
-  collide<R, FORCE, pair_out<S>(), log2_scale<S>()>(C, d, o);
+  collide<R, FORCE, pair_out<S>(), log2_scale<S>(), false>(C, d, o);
   const int64_t N = int64_t(g.nx) * g.ny * g.nz;
   const int64_t k = (int64_t(z) * g.ny + y) * g.nx + x;
   if (rho) rho[k] = double(o.rho);
@@ -485,25 +490,24 @@ __global__ void __launch_bounds__(256) fields_kernel(const S* __restrict__ src, 
 
 // Collide M independent nodes given as plain FP64 populations [q][node].
 template <typename S, typename R, bool FORCE>
-__global__ void collide_nodes_kernel(PhysParams P, const double* __restrict__ fin,
+__global__ void collide_nodes_kernel(CollideConst<R> C, double rho0, const double* __restrict__ fin,
                                      double* __restrict__ fout, double* rho,
                                      double* u, double* gd, int64_t M) {
   const int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (k >= M) return;
   const double lam = double(1 << log2_scale<S>());
-  const CollideConst<R> C = make_const<R>(P, lam);
   R d[Q];
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
-    const R dev = R((fin[q * M + k] - wt<double>(q) * P.rho0) * lam);
+    const R dev = R((fin[q * M + k] - wt<double>(q) * rho0) * lam);
     d[q] = Codec<S, R>::dec(Codec<S, R>::enc(dev, R(lam)), R(lam));
   }
   NodeOut<R> o;
-  collide<R, FORCE, pair_out<S>(), log2_scale<S>()>(C, d, o);
+  collide<R, FORCE, pair_out<S>(), log2_scale<S>(), true>(C, d, o);
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
     const R st = Codec<S, R>::dec(Codec<S, R>::enc(d[q], R(lam)), R(lam));
-    fout[q * M + k] = double(st) / lam + wt<double>(q) * P.rho0;
+    fout[q * M + k] = double(st) / lam + wt<double>(q) * rho0;
   }
   if (rho) rho[k] = double(o.rho);
   if (u) {
@@ -518,21 +522,19 @@ __global__ void collide_nodes_kernel(PhysParams P, const double* __restrict__ fi
 // density and non-equilibrium moments m^(1)_4..9 ([6][node], FP64), solved
 // in the math precision R exactly as the collision does.
 template <typename R>
-__global__ void omega_nodes_kernel(PhysParams P, const double* __restrict__ rho_in,
+__global__ void omega_nodes_kernel(CollideConst<R> C, const double* __restrict__ rho_in,
                                    const double* __restrict__ m, double* omega, double* gd,
                                    int64_t M) {
   const int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (k >= M) return;
-  const CollideConst<R> C = make_const<R>(P);
   const R rho = R(rho_in[k]);
   const R rinv = rrcp<R>(rho);
   R A, B;
-  strain_AB(C, rinv, R(m[k]), R(m[M + k]), R(m[2 * M + k]), R(m[3 * M + k]), R(m[4 * M + k]),
+  strain_AB(C, R(m[k]), R(m[M + k]), R(m[2 * M + k]), R(m[3 * M + k]), R(m[4 * M + k]),
             R(m[5 * M + k]), A, B);
-  R g;
-  const R w = omega_nu(C, rho, rinv, A, B, &g);
+  const R w = omega_nu(C, rho, rinv, A, B);
   omega[k] = double(w);
-  if (gd) gd[k] = double(g);
+  if (gd) gd[k] = double(shear_rate(rinv, w, A, B));
 }
 
 // Stored populations <-> plain FP64 f in the unpadded layout [q][z][y][x].
@@ -608,44 +610,49 @@ cudaError_t launch_step_t(const void* src, void* dst, const Geom& g, const PhysP
   // TMA_NPT + 32 v the TMA-staged kernel of shape v (check steps take the
   // plain kernel with the same block).
   if constexpr (std::is_same<R, float>::value && !std::is_same<S, double>::value) {
-    if ((npt & TMA_NPT) && !check)
+    if ((npt & TMA_NPT) && !check && unit_rates(P))
       return launch_step_tma<S>(a, src, g, P.has_force != 0, npt >> 5, cb.flag + 1, st);
   }
   const bool cap = (npt & 4) != 0;
   npt &= 3;
-#define CLBM_STEP_LAUNCH(KERNEL, GRID, ...)                                                 \
-  do {                                                                                     \
-    if (P.has_force) {                                                                     \
-      if (check) {                                                                         \
-        if (cap) e_ = pdl_launch(KERNEL<__VA_ARGS__, true, true, true>, GRID, block, st, a);         \
-        else e_ = pdl_launch(KERNEL<__VA_ARGS__, true, true, false>, GRID, block, st, a);            \
-      } else {                                                                             \
-        if (cap) e_ = pdl_launch(KERNEL<__VA_ARGS__, true, false, true>, GRID, block, st, a);        \
-        else e_ = pdl_launch(KERNEL<__VA_ARGS__, true, false, false>, GRID, block, st, a);           \
-      }                                                                                    \
-    } else {                                                                               \
-      if (check) {                                                                         \
-        if (cap) e_ = pdl_launch(KERNEL<__VA_ARGS__, false, true, true>, GRID, block, st, a);        \
-        else e_ = pdl_launch(KERNEL<__VA_ARGS__, false, true, false>, GRID, block, st, a);           \
-      } else {                                                                             \
-        if (cap) e_ = pdl_launch(KERNEL<__VA_ARGS__, false, false, true>, GRID, block, st, a);       \
-        else e_ = pdl_launch(KERNEL<__VA_ARGS__, false, false, false>, GRID, block, st, a);          \
-      }                                                                                    \
-    }                                                                                      \
-  } while (0)
+  const dim3 grid((g.nx + block.x - 1) / block.x, (g.ny + block.y - 1) / block.y, g.nz);
+  const int fc = (P.has_force ? 2 : 0) + (check ? 1 : 0);
+  void (*kernel)(const StepArgs<S, R>) = nullptr;
+  if (!unit_rates(P)) {
+    kernel = fc == 3   ? step_kernel<S, R, true, true, false, false>
+             : fc == 2 ? step_kernel<S, R, true, false, false, false>
+             : fc == 1 ? step_kernel<S, R, false, true, false, false>
+                       : step_kernel<S, R, false, false, false, false>;
+    return pdl_launch(kernel, grid, block, st, a);
+  }
   if constexpr (std::is_same<R, float>::value) {
     if (npt == 2) {
-      dim3 grid2((g.nx + block.x - 1) / block.x, (g.ny + 2 * block.y - 1) / (2 * block.y), g.nz);
-      cudaError_t e_ = cudaSuccess;
-      CLBM_STEP_LAUNCH(step2_kernel, grid2, S);
-      return e_ != cudaSuccess ? e_ : cudaGetLastError();
+      const dim3 grid2((g.nx + block.x - 1) / block.x, (g.ny + 2 * block.y - 1) / (2 * block.y),
+                       g.nz);
+      if (cap)
+        kernel = fc == 3   ? step2_kernel<S, true, true, true>
+                 : fc == 2 ? step2_kernel<S, true, false, true>
+                 : fc == 1 ? step2_kernel<S, false, true, true>
+                           : step2_kernel<S, false, false, true>;
+      else
+        kernel = fc == 3   ? step2_kernel<S, true, true, false>
+                 : fc == 2 ? step2_kernel<S, true, false, false>
+                 : fc == 1 ? step2_kernel<S, false, true, false>
+                           : step2_kernel<S, false, false, false>;
+      return pdl_launch(kernel, grid2, block, st, a);
     }
   }
-  dim3 grid((g.nx + block.x - 1) / block.x, (g.ny + block.y - 1) / block.y, g.nz);
-  cudaError_t e_ = cudaSuccess;
-  CLBM_STEP_LAUNCH(step_kernel, grid, S, R);
-#undef CLBM_STEP_LAUNCH
-  return e_ != cudaSuccess ? e_ : cudaGetLastError();
+  if (cap)
+    kernel = fc == 3   ? step_kernel<S, R, true, true, true, true>
+             : fc == 2 ? step_kernel<S, R, true, false, true, true>
+             : fc == 1 ? step_kernel<S, R, false, true, true, true>
+                       : step_kernel<S, R, false, false, true, true>;
+  else
+    kernel = fc == 3   ? step_kernel<S, R, true, true, false, true>
+             : fc == 2 ? step_kernel<S, R, true, false, false, true>
+             : fc == 1 ? step_kernel<S, R, false, true, false, true>
+                       : step_kernel<S, R, false, false, false, true>;
+  return pdl_launch(kernel, grid, block, st, a);
 }
 
 template <typename S, typename R>
@@ -654,8 +661,9 @@ cudaError_t launch_fields_t(const void* src, const Geom& g, const PhysParams& P,
   dim3 block(32, 4);
   dim3 grid((g.nx + 31) / 32, (g.ny + 3) / 4, g.nz);
   const S* s = static_cast<const S*>(src);
-  if (P.has_force) fields_kernel<S, R, true><<<grid, block, 0, st>>>(s, g, P, rho, u, gd);
-  else fields_kernel<S, R, false><<<grid, block, 0, st>>>(s, g, P, rho, u, gd);
+  const CollideConst<R> C = make_const<R>(P, double(1 << log2_scale<S>()));
+  if (P.has_force) fields_kernel<S, R, true><<<grid, block, 0, st>>>(s, g, C, rho, u, gd);
+  else fields_kernel<S, R, false><<<grid, block, 0, st>>>(s, g, C, rho, u, gd);
   return cudaGetLastError();
 }
 
@@ -665,8 +673,11 @@ cudaError_t launch_collide_nodes_t(const PhysParams& P, const double* fin, doubl
                                    cudaStream_t st) {
   const int b = 128;
   const unsigned grid = unsigned((M + b - 1) / b);
-  if (P.has_force) collide_nodes_kernel<S, R, true><<<grid, b, 0, st>>>(P, fin, fout, rho, u, gd, M);
-  else collide_nodes_kernel<S, R, false><<<grid, b, 0, st>>>(P, fin, fout, rho, u, gd, M);
+  const CollideConst<R> C = make_const<R>(P, double(1 << log2_scale<S>()));
+  if (P.has_force)
+    collide_nodes_kernel<S, R, true><<<grid, b, 0, st>>>(C, P.rho0, fin, fout, rho, u, gd, M);
+  else
+    collide_nodes_kernel<S, R, false><<<grid, b, 0, st>>>(C, P.rho0, fin, fout, rho, u, gd, M);
   return cudaGetLastError();
 }
 
@@ -674,7 +685,7 @@ template <typename R>
 cudaError_t launch_omega_nodes_t(const PhysParams& P, const double* rho, const double* m,
                                  double* omega, double* gd, int64_t M, cudaStream_t st) {
   const int b = 128;
-  omega_nodes_kernel<R><<<unsigned((M + b - 1) / b), b, 0, st>>>(P, rho, m, omega, gd, M);
+  omega_nodes_kernel<R><<<unsigned((M + b - 1) / b), b, 0, st>>>(make_const<R>(P), rho, m, omega, gd, M);
   return cudaGetLastError();
 }
 

@@ -56,6 +56,13 @@ struct PhysParams {
   double omega_high[10] = {1, 1, 1, 1, 1, 1, 1, 1, 1, 1};
 };
 
+// Whether the rates omega_9 .. omega_18 are all 1 (Sec. 3.1, the default).
+inline bool unit_rates(const PhysParams& P) {
+  for (double w : P.omega_high)
+    if (w != 1.0) return false;
+  return true;
+}
+
 // Work buffers of a check step.
 struct CheckBufs {
   void* uprev;      // 3 x (plane * nz) velocities of the previous check, math type
@@ -100,19 +107,21 @@ void set_unbound_error(const char* msg);
 // Batched step (batch.cuh): descriptors are opaque bytes to the host code.
 // The unforced and the forced lattices form two independent chains of
 // launches (on two streams), so each chain counts its own steps.
+// Each chain steps its lattices in two groups with a kernel each: those with
+// the unit rates omega_9..18, then those with other rates.
+constexpr int BATCH_GROUPS = 4;  // 2 * forced + (other rates)
 struct BatchHeader {
   int nlat;
-  int ntiles;   // all tiles
-  int ntiles0;  // tiles of lattices without force (they come first)
+  int tile_end[BATCH_GROUPS];  // the tiles of group k end here (and begin where group k-1's end)
   int err;      // set by the kernel if a tile's descriptor fails its checks
-  unsigned step[2];  // steps done by the unforced [0] / forced [1] chain (F16R: each
-                     // lattice's step is its chain's count plus an offset)
-  int done[2];       // F16R: CTAs of that chain's current launch that finished
+  unsigned step[BATCH_GROUPS];  // steps done by that group's launches (F16R: each
+                                // lattice's step is its group's count plus an offset)
+  int done[BATCH_GROUPS];       // F16R: CTAs of that group's current launch that finished
 };
 #define CLBM_DECLARE_BATCH(SUFFIX)                                                              \
   cudaError_t launch_batch_##SUFFIX(int base, const int* owner, const unsigned* coord,         \
                                     const void* hdr, int parity, bool check, double* acc,       \
-                                    int zc, dim3 block, int grid, cudaStream_t st,              \
+                                    int zc, dim3 block, int grid, bool rates, cudaStream_t st,  \
                                     cudaStream_t st_forced);                                    \
   size_t desc_size_##SUFFIX();                                                                  \
   int desc_capacity_##SUFFIX();                                                                 \

@@ -53,21 +53,20 @@ cudaError_t scratch_address(int dev, double** out) {
 template <typename S, typename R, bool FORCE>
 __global__ void __launch_bounds__(256) step_partials_kernel(const S* __restrict__ src,
                                                             S* __restrict__ dst, Geom g,
-                                                            PhysParams P, R* uprev,
+                                                            CollideConst<R> C, R* uprev,
                                                             double* partials) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z;
   const bool active = x < g.nx && y < g.ny;
   const double lam = double(1 << log2_scale<S>());
-  const CollideConst<R> C = make_const<R>(P, lam);
   double v[4] = {0.0, 0.0, 0.0, 0.0};
   if (active) {
     const int64_t i = int64_t(z) * g.plane + int64_t(y) * g.pitch + x;
     R d[Q];
     pull<S, R>(src, g, x, y, z, i, R(lam), d);
     NodeOut<R> o;
-    collide<R, FORCE, pair_out<S>(), log2_scale<S>()>(C, d, o);
+    collide<R, FORCE, pair_out<S>(), log2_scale<S>(), true>(C, d, o);
 #pragma unroll
     for (int q = 0; q < Q; ++q) dst[q * g.qstride + i] = Codec<S, R>::enc(d[q], R(lam));
     const int64_t nst = g.plane * g.nz;
@@ -80,7 +79,7 @@ __global__ void __launch_bounds__(256) step_partials_kernel(const S* __restrict_
     v[0] = ex * ex + ey * ey + ez * ez;
     v[1] = double(o.ux) * double(o.ux) + double(o.uy) * double(o.uy) +
            double(o.uz) * double(o.uz);
-    v[2] = double(o.rho) - double(P.rho0);
+    v[2] = double(o.rho) - double(C.rho0);
     const double chk = double(o.rho) + double(o.ux) + double(o.uy) + double(o.uz);
     v[3] = (!(chk == chk) || !(fabs(chk) < 1e30) ||
             !(double(o.rho) > 0.5 && double(o.rho) < 2.0)) ? 1.0 : 0.0;
@@ -143,10 +142,12 @@ cudaError_t launch_noalloc(const void* src, void* dst, const Geom& g, const Phys
   const S* s = static_cast<const S*>(src);
   S* d = static_cast<S*>(dst);
   R* up = static_cast<R*>(uprev);
+  const CollideConst<R> C = make_const<R>(P, double(1 << log2_scale<S>()));
+  // the entry point takes the unit rates omega_9..18 only
   if (P.has_force)
-    step_partials_kernel<S, R, true><<<grid, block, 0, st>>>(s, d, g, P, up, partials);
+    step_partials_kernel<S, R, true><<<grid, block, 0, st>>>(s, d, g, C, up, partials);
   else
-    step_partials_kernel<S, R, false><<<grid, block, 0, st>>>(s, d, g, P, up, partials);
+    step_partials_kernel<S, R, false><<<grid, block, 0, st>>>(s, d, g, C, up, partials);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   finish_kernel<<<1, 256, 0, st>>>(partials, int(grid.x * grid.y * grid.z), stats);

@@ -132,7 +132,7 @@ __device__ __forceinline__ void pull_face_ref(const __half* __restrict__ src,
   }
 }
 
-template <bool FORCE, bool CHECK, bool CAP>
+template <bool FORCE, bool CHECK, bool CAP, bool UNIT>
 __global__ void __launch_bounds__(256, CAP ? 4 : 1) step_ref_kernel(const StepArgs<__half, float> a,
                                                                     const RefArgs r) {
   pdl_enter();
@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(256, CAP ? 4 : 1) step_ref_kernel(const StepAr
                     x, y, z, i, a.lidc, d);
     }
     NodeOut<float> o;
-    collide<float, FORCE, !FORCE, LOG2LAM>(a.C, d, o);
+    collide<float, FORCE, !FORCE, LOG2LAM, UNIT>(a.C, d, o);
     Ref4 rr;
     r.ref_dst[i] = ref_make(o.rho - rho0, o.rho, o.ux, o.uy, o.uz, rr);
     store_sr([&](int q) -> __half& { return a.dstq[q][i]; }, d, rr, sr_seed(uint32_t(i), r.step));
@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(256) fields_ref_kernel(const __half* __restric
   pull_face_ref(src, ref, g.qstride, g.nx, g.ny, g.nz, g.pitch, int(g.plane), g.facebits, x, y,
                 z, i, lidc, d);
   NodeOut<float> o;
-  collide<float, FORCE, !FORCE, LOG2LAM>(C, d, o);
+  collide<float, FORCE, !FORCE, LOG2LAM, false>(C, d, o);
   const int64_t N = int64_t(g.nx) * g.ny * g.nz;
   const int64_t k = (int64_t(z) * g.ny + y) * g.nx + x;
   if (rho) rho[k] = double(o.rho);
@@ -305,7 +305,7 @@ __global__ void collide_nodes_ref_kernel(CollideConst<float> C, const double* __
     d[q] = dec16(enc16(float((fin[q * M + k] - wt<double>(q) * rho0) * double(LAM)) - t)) + t;
   }
   NodeOut<float> o;
-  collide<float, FORCE, !FORCE, LOG2LAM>(C, d, o);
+  collide<float, FORCE, !FORCE, LOG2LAM, true>(C, d, o);
   ref_make(o.rho - rho0, o.rho, o.ux, o.uy, o.uz, rr);
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
@@ -333,7 +333,7 @@ void lid_table(const Geom& g, float* out) {
 
 // One node of the batched step in the F16R form: the same pull, references
 // and collision as step_ref_kernel.
-template <bool FORCE>
+template <bool FORCE, bool UNIT>
 __device__ void batch_node_ref(const LatDesc<float>& L, int parity, int x, int y, int z,
                                unsigned step, NodeOut<float>& o) {
   const __half* src = static_cast<const __half*>(L.buf[parity]);
@@ -374,7 +374,7 @@ __device__ void batch_node_ref(const LatDesc<float>& L, int parity, int x, int y
     pull_face_ref(src, rs, L.qstride, L.nx, L.ny, L.nz, pitch, plane, L.facebits, x, y, z, i,
                   L.lidc, d);
   }
-  collide<float, FORCE, !FORCE, LOG2LAM>(L.C, d, o);
+  collide<float, FORCE, !FORCE, LOG2LAM, UNIT>(L.C, d, o);
   Ref4 rr;
   rd[i] = ref_make(o.rho - rho0, o.rho, o.ux, o.uy, o.uz, rr);
   store_sr([&](int q) -> __half& { return dst[q * qs + i]; }, d, rr, sr_seed(uint32_t(i), step));
@@ -413,21 +413,20 @@ cudaError_t launch_step_f16r(const void* src, void* dst, const void* ref_src, vo
   a.cb = cb;
   const bool cap = (npt & 4) != 0;
   dim3 grid((g.nx + block.x - 1) / block.x, (g.ny + block.y - 1) / block.y, g.nz);
-  cudaError_t e_ = cudaSuccess;
-#define CLBM_REF_LAUNCH(F, C_)                                                                  \
-  do {                                                                                         \
-    if (cap) e_ = pdl_launch(step_ref_kernel<F, C_, true>, grid, block, st, a, r);            \
-    else e_ = pdl_launch(step_ref_kernel<F, C_, false>, grid, block, st, a, r);               \
-  } while (0)
+  void (*kernel)(const StepArgs<__half, float>, const RefArgs) = nullptr;
+#define CLBM_REF(F, C_)                                            \
+  kernel = !unit_rates(P) ? step_ref_kernel<F, C_, false, false>   \
+           : cap          ? step_ref_kernel<F, C_, true, true>     \
+                          : step_ref_kernel<F, C_, false, true>
   if (P.has_force) {
-    if (check) CLBM_REF_LAUNCH(true, true);
-    else CLBM_REF_LAUNCH(true, false);
+    if (check) CLBM_REF(true, true);
+    else CLBM_REF(true, false);
   } else {
-    if (check) CLBM_REF_LAUNCH(false, true);
-    else CLBM_REF_LAUNCH(false, false);
+    if (check) CLBM_REF(false, true);
+    else CLBM_REF(false, false);
   }
-#undef CLBM_REF_LAUNCH
-  return e_ != cudaSuccess ? e_ : cudaGetLastError();
+#undef CLBM_REF
+  return pdl_launch(kernel, grid, block, st, a, r);
 }
 
 cudaError_t launch_fields_f16r(const void* src, const void* ref, const Geom& g,

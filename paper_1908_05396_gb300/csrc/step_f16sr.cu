@@ -15,7 +15,7 @@
 namespace clbm {
 namespace {
 
-template <bool FORCE, bool CHECK, bool CAP>
+template <bool FORCE, bool CHECK, bool CAP, bool UNIT>
 __global__ void __launch_bounds__(256, CAP ? 4 : 1) step_sr_kernel(const StepArgs<__half, float> a,
                                                                    unsigned step) {
   pdl_enter();
@@ -38,7 +38,7 @@ __global__ void __launch_bounds__(256, CAP ? 4 : 1) step_sr_kernel(const StepArg
                                x, y, z, i, a.lidc, d);
     }
     NodeOut<float> o;
-    collide<float, FORCE, pair_out<__half>(), log2_scale<__half>()>(a.C, d, o);
+    collide<float, FORCE, pair_out<__half>(), log2_scale<__half>(), UNIT>(a.C, d, o);
     // the deviations are carried scaled by 1024, as they are stored
     uint32_t state = sr_seed(uint32_t(i), step);
 #pragma unroll
@@ -109,21 +109,20 @@ cudaError_t launch_step_f16sr(const void* src, void* dst, const Geom& g, const P
   const unsigned sstep = unsigned(uint64_t(step));
   const bool cap = (npt & 4) != 0;
   dim3 grid((g.nx + block.x - 1) / block.x, (g.ny + block.y - 1) / block.y, g.nz);
-  cudaError_t e_ = cudaSuccess;
-#define CLBM_SR_LAUNCH(F, C_)                                                                  \
-  do {                                                                                        \
-    if (cap) e_ = pdl_launch(step_sr_kernel<F, C_, true>, grid, block, st, a, sstep);         \
-    else e_ = pdl_launch(step_sr_kernel<F, C_, false>, grid, block, st, a, sstep);            \
-  } while (0)
+  void (*kernel)(const StepArgs<__half, float>, unsigned) = nullptr;
+#define CLBM_SR(F, C_)                                            \
+  kernel = !unit_rates(P) ? step_sr_kernel<F, C_, false, false>   \
+           : cap          ? step_sr_kernel<F, C_, true, true>     \
+                          : step_sr_kernel<F, C_, false, true>
   if (P.has_force) {
-    if (check) CLBM_SR_LAUNCH(true, true);
-    else CLBM_SR_LAUNCH(true, false);
+    if (check) CLBM_SR(true, true);
+    else CLBM_SR(true, false);
   } else {
-    if (check) CLBM_SR_LAUNCH(false, true);
-    else CLBM_SR_LAUNCH(false, false);
+    if (check) CLBM_SR(false, true);
+    else CLBM_SR(false, false);
   }
-#undef CLBM_SR_LAUNCH
-  return e_ != cudaSuccess ? e_ : cudaGetLastError();
+#undef CLBM_SR
+  return pdl_launch(kernel, grid, block, st, a, sstep);
 }
 
 }  // namespace clbm

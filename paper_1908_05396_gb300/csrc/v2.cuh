@@ -9,6 +9,7 @@
 namespace clbm {
 
 // Keep the scalar overloads visible next to the V2 ones below.
+using ::fma;
 using ::fmax;
 using ::fmin;
 using ::sqrt;
