@@ -73,15 +73,8 @@ __device__ __forceinline__ void batch_node(const LatDesc<R>& L, const S* __restr
   }
   collide<R, FORCE, pair_out<S>(), log2_scale<S>(), UNIT>(L.C, d, o);
   if constexpr (std::is_same<S, __half>::value) {
-    if (L.sround) {  // as step_f16sr.cu: two directions per stochastic conversion
-      uint32_t state = sr_seed(uint32_t(i), step);
-#pragma unroll
-      for (int q = 0; q < Q; q += 2) {
-        __half hi, lo;
-        enc16_sr2(d[q], q + 1 < Q ? d[q + 1 < Q ? q + 1 : q] : 0.0f, state, hi, lo);
-        dst[q * qs + i] = hi;
-        if (q + 1 < Q) dst[(q + 1 < Q ? q + 1 : q) * qs + i] = lo;
-      }
+    if (L.sround) {
+      store_sr1([&](int q) { return dst + (q * qs + i); }, d, uint32_t(i), step);
       return;
     }
   }
@@ -89,11 +82,53 @@ __device__ __forceinline__ void batch_node(const LatDesc<R>& L, const S* __restr
   for (int q = 0; q < Q; ++q) dst[q * qs + i] = Codec<S, R>::enc(d[q], R(1));
 }
 
-// One node of the batched step in the F16R form (defined with the other F16R
-// kernels, the only translation unit that instantiates the batch with REF).
-template <bool FORCE, bool UNIT>
+// One node of the batched step in the F16R form, any rates (defined with the
+// other F16R kernels, the only translation unit that instantiates the batch
+// with REF).
+template <bool FORCE>
 __device__ void batch_node_ref(const LatDesc<float>& L, int parity, int x, int y, int z,
                                unsigned step, NodeOut<float>& o);
+
+// A pair's upwind values in a lattice of the batch (see LonePair).
+struct BatchPair {
+  const LatDesc<float>& L;
+  const __half* src;  // the pair's own value of direction 0
+  const uint2* ref;
+  int qs;
+  __device__ __forceinline__ const __half* up(int q) const {
+    return src + (q * qs - (cz(q) * L.plane + cy(q) * L.pitch + cx(q)));
+  }
+  __device__ __forceinline__ const __half* own(int q) const { return src + q * qs; }
+  __device__ __forceinline__ int nx() const { return L.nx; }
+  __device__ __forceinline__ int ny() const { return L.ny; }
+  __device__ __forceinline__ int nz() const { return L.nz; }
+  __device__ __forceinline__ int pitch() const { return L.pitch; }
+  __device__ __forceinline__ int plane() const { return L.plane; }
+  __device__ __forceinline__ unsigned faces() const { return L.facebits; }
+  __device__ __forceinline__ float lid(int q) const { return L.lidc[q]; }
+};
+
+// Two nodes along x of the batched step of an FP16 form: the pull, collision
+// and store of step_pair_kernel.
+template <bool FORCE, bool REF>
+__device__ __forceinline__ void batch_pair(const LatDesc<float>& L, int parity, int x, int y, int z,
+                                           unsigned step, NodeOut<V2>& o) {
+  const int i = z * L.plane + y * L.pitch + x, qs = int(L.qstride);
+  const __half* src = static_cast<const __half*>(L.buf[parity]) + i;
+  __half* out = static_cast<__half*>(const_cast<void*>(L.buf[parity ^ 1])) + i;
+  const uint2* rs = REF ? static_cast<const uint2*>(L.ref[parity]) + i : nullptr;
+  uint2* rd = REF ? static_cast<uint2*>(const_cast<void*>(L.ref[parity ^ 1])) + i : nullptr;
+  V2 d[Q];
+  pull_pair<REF>(BatchPair{L, src, rs, qs}, x, y, z, d);
+  collide_pair<REF, FORCE>(L.C, d, o);
+  auto dst = [&](int q) { return out + q * qs; };
+  if constexpr (REF) {
+    store_pair<PAIR_REF>(L.C, d, o, dst, rd, i, step);
+  } else {
+    if (L.sround) store_pair<PAIR_SR>(L.C, d, o, dst, rd, i, step);
+    else store_pair<PAIR_RN>(L.C, d, o, dst, rd, i, step);
+  }
+}
 
 // tile word: x tile (8 bits) | y tile (12 bits) | z chunk (12 bits)
 __host__ __device__ __forceinline__ unsigned tile_word(int tx, int ty, int tz) {
@@ -110,6 +145,7 @@ __device__ __forceinline__ void batch_tiles(Get get, const int* __restrict__ own
   // F16R and F16S (whose lattices may round stochastically): this group's
   // step count, advanced at the end of each of its launches by the launch's
   // last CTA
+  constexpr bool PAIR = UNIT && std::is_same<S, __half>::value;
   constexpr int GROUP = (FORCE ? 2 : 0) + (UNIT ? 0 : 1);
   constexpr bool STEPS = REF || std::is_same<S, __half>::value;
   const unsigned bstep =
@@ -145,9 +181,10 @@ __device__ __forceinline__ void batch_tiles(Get get, const int* __restrict__ own
       continue;
     }
     // the block's threads in row order over a tile of 2^tw_log2 x (threads
-    // >> tw_log2) nodes (the tile width is chosen per lattice)
+    // >> tw_log2) nodes, or node pairs (the tile width is chosen per lattice)
     const int lin = int(threadIdx.y * blockDim.x + threadIdx.x);
-    const int x = (tx << L.tw_log2) + (lin & ((1 << L.tw_log2) - 1));
+    const int xt = (tx << L.tw_log2) + (lin & ((1 << L.tw_log2) - 1));
+    const int x = PAIR ? 2 * xt : xt;
     const int y = ty * (int(blockDim.x * blockDim.y) >> L.tw_log2) + (lin >> L.tw_log2);
     const S* src = static_cast<const S*>(L.buf[parity]);
     S* dst = static_cast<S*>(const_cast<void*>(L.buf[parity ^ 1]));
@@ -160,8 +197,16 @@ __device__ __forceinline__ void batch_tiles(Get get, const int* __restrict__ own
 #pragma unroll 1
     for (int z = tz * zc; z < z1; ++z) {
       if (active) {
+        if constexpr (PAIR) {
+          NodeOut<V2> o;
+          batch_pair<FORCE, REF>(L, parity, x, y, z, bstep + L.step_offset, o);
+          if (CHECK)
+            check_pair(o, L.C.rho0, static_cast<float*>(L.uprev), int64_t(L.plane) * L.nz,
+                       z * L.plane + y * L.pitch + x, x + 1 < L.nx, du2, uu, dr, bad);
+          continue;
+        }
         NodeOut<R> o;
-        if constexpr (REF) batch_node_ref<FORCE, UNIT>(L, parity, x, y, z, bstep + L.step_offset, o);
+        if constexpr (REF) batch_node_ref<FORCE>(L, parity, x, y, z, bstep + L.step_offset, o);
         else batch_node<S, R, FORCE, UNIT>(L, src, dst, x, y, z, bstep + L.step_offset, o);
         if (CHECK) {
           R* up = static_cast<R*>(L.uprev);
@@ -207,6 +252,25 @@ __device__ __forceinline__ void batch_tiles(Get get, const int* __restrict__ own
   }
 }
 
+// Blocks of 256 threads per SM that the batch kernel is compiled for: 64
+// registers when capped, what it likes when not; kernels that step two nodes
+// per thread have one variant (launched for both).
+template <typename S>
+constexpr int batch_min_blocks(bool cap, bool unit, bool ref, bool force) {
+  return std::is_same<S, __half>::value && unit ? pair_min_blocks(ref, force) : cap ? 4 : 1;
+}
+
+// The grid of a persistent launch: per_sm blocks per SM, but no more than fit
+// at once (a block beyond them would start its share of the tiles only when
+// another has finished all of its own).
+inline int batch_grid(const void* kernel, dim3 block, int per_sm, int sms) {
+  int fit = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, kernel, int(block.x * block.y), 0) !=
+          cudaSuccess || fit < 1)
+    return per_sm * sms;
+  return (per_sm < fit ? per_sm : fit) * sms;
+}
+
 // Bytes of __constant__ memory given to the descriptor table of one storage
 // form; batches reserve disjoint ranges of it.
 constexpr int BATCH_CONST_BYTES = 60 * 1024;
@@ -249,7 +313,7 @@ void fill_desc_t(void* out, double lam, const Geom& g, const PhysParams& P, cons
   namespace clbm {                                                                             \
   __constant__ LatDesc<R> c_lat_##SUFFIX[BATCH_CONST_BYTES / sizeof(LatDesc<R>)];              \
   template <bool CHECK, bool CAP, bool FORCE, bool UNIT>                                       \
-  __global__ void __launch_bounds__(256, CAP ? 4 : 1)                                          \
+  __global__ void __launch_bounds__(256, batch_min_blocks<S>(CAP, UNIT, REF, FORCE))           \
       batch_kernel_##SUFFIX(int base, const int* __restrict__ owner,                           \
                             const unsigned* __restrict__ coord, BatchHeader* hdr, int parity,  \
                             double* acc, int zc) {                                             \
@@ -259,12 +323,16 @@ void fill_desc_t(void* out, double lam, const Geom& g, const PhysParams& P, cons
   }                                                                                            \
   cudaError_t launch_batch_##SUFFIX(int base, const int* owner, const unsigned* coord,         \
                                     const void* hdr, int parity, bool check, double* acc,      \
-                                    int zc, dim3 block, int grid, bool rates, cudaStream_t st, \
-                                    cudaStream_t stf) {                                         \
+                                    int zc, dim3 block, int per_sm, bool cap, int sms,         \
+                                    bool rates, cudaStream_t st, cudaStream_t stf) {           \
     BatchHeader* H = static_cast<BatchHeader*>(const_cast<void*>(hdr));                        \
-    const bool cap = grid < 0;                                                                 \
-    if (cap) grid = -grid;                                                                     \
+    auto go = [&](void (*k)(int, const int*, const unsigned*, BatchHeader*, int, double*, int), \
+                  cudaStream_t s) {                                                            \
+      k<<<batch_grid(reinterpret_cast<const void*>(k), block, per_sm, sms), block, 0, s>>>(    \
+          base, owner, coord, H, parity, acc, zc);                                             \
+    };                                                                                         \
     /* tiles without force on st, tiles with force on stf (an empty range exits at once) */   \
+    if (std::is_same<S, __half>::value) cap = true;                                            \
     auto k0 = check ? (cap ? batch_kernel_##SUFFIX<true, true, false, true>                    \
                            : batch_kernel_##SUFFIX<true, false, false, true>)                  \
                     : (cap ? batch_kernel_##SUFFIX<false, true, false, true>                   \
@@ -273,15 +341,13 @@ void fill_desc_t(void* out, double lam, const Geom& g, const PhysParams& P, cons
                            : batch_kernel_##SUFFIX<true, false, true, true>)                   \
                     : (cap ? batch_kernel_##SUFFIX<false, true, true, true>                    \
                            : batch_kernel_##SUFFIX<false, false, true, true>);                 \
-    k0<<<grid, block, 0, st>>>(base, owner, coord, H, parity, acc, zc);                        \
-    k1<<<grid, block, 0, stf>>>(base, owner, coord, H, parity, acc, zc);                       \
+    go(k0, st);                                                                                \
+    go(k1, stf);                                                                               \
     if (rates) { /* some lattice has other rates omega_9..18: their tiles */                   \
-      auto r0 = check ? batch_kernel_##SUFFIX<true, false, false, false>                       \
-                      : batch_kernel_##SUFFIX<false, false, false, false>;                     \
-      auto r1 = check ? batch_kernel_##SUFFIX<true, false, true, false>                        \
-                      : batch_kernel_##SUFFIX<false, false, true, false>;                      \
-      r0<<<grid, block, 0, st>>>(base, owner, coord, H, parity, acc, zc);                      \
-      r1<<<grid, block, 0, stf>>>(base, owner, coord, H, parity, acc, zc);                     \
+      go(check ? batch_kernel_##SUFFIX<true, false, false, false>                              \
+               : batch_kernel_##SUFFIX<false, false, false, false>, st);                       \
+      go(check ? batch_kernel_##SUFFIX<true, false, true, false>                               \
+               : batch_kernel_##SUFFIX<false, false, true, false>, stf);                       \
     }                                                                                          \
     return cudaGetLastError();                                                                 \
   }                                                                                            \

@@ -179,21 +179,24 @@ bool any_sround(const clbm_batch_ctx* b) {
 // disjoint lattices, so between fork_streams(b, 2) and join_streams(b, 2) they
 // run concurrently, each chain in step order.
 cudaError_t launch(clbm_batch_ctx* b, bool check) {
-  const int grid = b->blocks_per_sm * b->sms * (b->cap ? -1 : 1);
   const cudaStream_t sf = b->aux[0];
   switch (b->dtype) {
     case CLBM_F64:
       return launch_batch_f64(b->desc_base, b->d_owner, b->d_coord, b->d_hdr, b->parity, check,
-                              b->d_acc, b->zc, b->block, grid, b->rates, b->stream, sf);
+                              b->d_acc, b->zc, b->block, b->blocks_per_sm, b->cap, b->sms,
+                              b->rates, b->stream, sf);
     case CLBM_F32:
       return launch_batch_f32(b->desc_base, b->d_owner, b->d_coord, b->d_hdr, b->parity, check,
-                              b->d_acc, b->zc, b->block, grid, b->rates, b->stream, sf);
+                              b->d_acc, b->zc, b->block, b->blocks_per_sm, b->cap, b->sms,
+                              b->rates, b->stream, sf);
     case CLBM_F16R:
       return launch_batch_f16r(b->desc_base, b->d_owner, b->d_coord, b->d_hdr, b->parity, check,
-                               b->d_acc, b->zc, b->block, grid, b->rates, b->stream, sf);
+                               b->d_acc, b->zc, b->block, b->blocks_per_sm, b->cap, b->sms,
+                              b->rates, b->stream, sf);
     default:
       return launch_batch_f16(b->desc_base, b->d_owner, b->d_coord, b->d_hdr, b->parity, check,
-                              b->d_acc, b->zc, b->block, grid, b->rates, b->stream, sf);
+                              b->d_acc, b->zc, b->block, b->blocks_per_sm, b->cap, b->sms,
+                              b->rates, b->stream, sf);
   }
 }
 
@@ -331,11 +334,15 @@ int upload(clbm_batch_ctx* b) {
           (h->P.has_force ? 2 : 0) + (unit_rates(h->P) ? 0 : 1) != pass)
         continue;
       const int threads = int(b->block.x * b->block.y);
-      const int tw = tile_width(h->g.nx, int(h->elem), int(b->block.x), threads);
+      // FP16 forms with unit rates step two nodes along x per thread
+      const bool pair = h->elem == 2 && unit_rates(h->P);
+      const int tw = pair ? pair_width(h->g.nx, threads, int(b->block.x))
+                          : tile_width(h->g.nx, int(h->elem), int(b->block.x), threads);
       int twl = 0;
       while ((1 << twl) < tw) ++twl;
       const int th = threads / tw;
-      const int tx = (h->g.nx + tw - 1) / tw;
+      const int nodes_x = pair ? 2 * tw : tw;
+      const int tx = (h->g.nx + nodes_x - 1) / nodes_x;
       const int ty = (h->g.ny + th - 1) / th;
       const int tz = (h->g.nz + b->zc - 1) / b->zc;   // chunks of zc planes
       if (tx > 255 || ty > 4095 || tz > 4095)

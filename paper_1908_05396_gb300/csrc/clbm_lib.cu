@@ -480,7 +480,12 @@ int clbm_autotune(clbm_handle h, int steps, int* block_x, int* block_y, int* npt
   std::vector<Cand> cands;
   const int shapes[][2] = {{32, 1}, {32, 2}, {32, 4}, {32, 8}, {64, 1}, {64, 2}, {64, 4},
                            {128, 1}, {128, 2}, {256, 1}};
-  for (int capped = 0; capped <= 1; ++capped)
+  // FP16 forms with unit rates and two buffers: the pair kernel, which takes
+  // from the block its thread count only
+  const bool pair = h->elem == 2 && !h->in_place && unit_rates(h->P);
+  if (pair)
+    for (int t : {32, 64, 128, 256}) cands.push_back({32, t / 32, 1});
+  for (int capped = 0; capped <= 1 && !pair; ++capped)
     for (int np = 1; np <= ((h->dtype == CLBM_F64 || h->dtype == CLBM_F16R || h->in_place || h->sround) ? 1 : 2); ++np)
       for (auto& sh : shapes) {
         if (sh[0] * sh[1] > (np == 2 ? 128 : 256)) continue;
@@ -489,7 +494,7 @@ int clbm_autotune(clbm_handle h, int steps, int* block_x, int* block_y, int* npt
       }
   // a lattice narrower than a warp: blocks as wide as its tile width
   const int tw = tile_width(h->g.nx, int(h->elem), 32, 64);
-  if (tw < 32)
+  if (tw < 32 && !pair)
     for (int capped = 0; capped <= 1; ++capped)
       for (int t : {64, 128, 256}) cands.push_back({tw, t / tw, 1 + 4 * capped});
   // FP32 and FP16 storage: the TMA-staged kernel in each of its shapes

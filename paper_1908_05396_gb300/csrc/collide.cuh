@@ -133,10 +133,10 @@ __device__ __forceinline__ R newton_y2(R y, R c, R ehalf, R nm1, R A, R B, R ylo
 #pragma unroll 1
   for (int it = 0; it < iters; ++it) {
     const R w = rrcp<R>(rex2<R>(y) + R(0.5f));
-    const R wwA = mulr(mulr(w, w), A);
-    const R g2 = fmax(wwA + B, lo);
+    const R ww = mulr(w, w);
+    const R g2 = fmax(fma(ww, A, B), lo);
     const R G = fma(-ehalf, rlg2<R>(g2), y - c);
-    const R den = fma(nm1, mulr(wwA, fma(R(-0.5f), w, R(1.0f))), g2);
+    const R den = fma(nm1, mulr(mulr(ww, A), fma(R(-0.5f), w, R(1.0f))), g2);
     y = fmin(fmax(fma(-mulr(G, g2), rrcp<R>(den), y), ylo), yhi);
   }
   return y;
@@ -242,8 +242,8 @@ __device__ __forceinline__ double omega_nu(const CollideConst<double>& C, double
                                    narrow(rho), Af, Bf);
   const double tau = widen(ex2f(yf));
   const double w = rcp64(tau + 0.5);
-  const double wwA = mulr(mulr(w, w), A);
-  double g2 = wwA + B;
+  const double ww = mulr(w, w), wwA = mulr(ww, A);
+  double g2 = fma(ww, A, B);
   if (g2 < 1e-300) g2 = 1e-300;
   int e1, e2;
   const double l1 = log_mant(mulr(tau, rho), e1);
@@ -255,13 +255,15 @@ __device__ __forceinline__ double omega_nu(const CollideConst<double>& C, double
   const double den = fma(C.nm1, mulr(wwA, s), g2);
   const double d1 = mulr(-mulr(G, g2), rcp64(den));  // -G / G'
   const float wf = narrow(w), sf = narrow(s), nm1 = C.n - 1.0f;
-  const float rf = fminf(narrow(wwA) * rcpf(narrow(g2)), 1.0f);
-  const float G1 = 1.0f + nm1 * rf * sf;
-  const float G2 = nm1 * (0.5f * sf * wf * rf - 2.0f * rf * (1.0f - rf) * sf * sf);
+  const float rf = fminf(mulr(narrow(wwA), rcpf(narrow(g2))), 1.0f);
+  const float rs = mulr(rf, sf);
+  const float G1 = fma(nm1, rs, 1.0f);
+  // G'' = (n-1) r s [omega/2 - 2 (1 - r) s]
+  const float G2 = mulr(mulr(nm1, rs), fma(-2.0f * sf, 1.0f - rf, 0.5f * wf));
   // the magnitude of d1 with its sign; |d1| is large only when the root lies
   // beyond a clamp, where the sign of dy decides
   const float d1f = copysignf(narrow(fabs(d1)), __uint_as_float(unsigned(__double2hiint(d1))));
-  const float h = fminf(fmaxf(-0.5f * G2 * rcpf(G1) * d1f, -0.25f), 0.25f);
+  const float h = fminf(fmaxf(mulr(mulr(-0.5f * G2, rcpf(G1)), d1f), -0.25f), 0.25f);
   const double dy = fma(d1, widen(h), d1);
   double t1 = fma(tau, mulr(dy, fma(dy, fma(dy, 1.0 / 6.0, 0.5), 1.0)), tau);
   if (t1 < C.tlo) t1 = C.tlo;
@@ -812,7 +814,7 @@ __device__ __forceinline__ void collide_unit(const CollideConst<typename ScalarO
   const R cxy = mulr(wm, mxy), cxz = mulr(wm, mxz), cyz = mulr(wm, myz);
   const R ax = mulr(wm, ex), ay = mulr(wm, ey), az = mulr(wm, ez);
   const R dr3 = mulr(third, drho);
-  const R zx = ax + dr3, zy = ay + dr3, zz = az + dr3;
+  const R zx = fma(wm, ex, dr3), zy = fma(wm, ey, dr3), zz = fma(wm, ez, dr3);  // a_i + dr3
   const R Exx = fma(Jx, ux, zx), Eyy = fma(Jy, uy, zy), Ezz = fma(Jz, uz, zz);
   const R r30 = R(C.r30);
   const R kxx = Exx + r30, kyy = Eyy + r30, kzz = Ezz + r30;
@@ -902,10 +904,10 @@ __device__ __forceinline__ void collide_unit(const CollideConst<typename ScalarO
     plane(fxz, pxz, oxzz, oxxz, d[11], d[14], d[13], d[12]);
     plane(fyz, pyz, oyzz, oyyz, d[15], d[18], d[17], d[16]);
   } else {
-    // increments of the moments (with the whole source S): n, r of order 2,
-    // t of order 3, q of order 4
+    // increments of the moments (with the whole source S): n = -omega m + S and r
+    // of order 2, t of order 3, q of order 4
     const R nw = -w;
-    R nxy = mulr(nw, mxy), nxz = mulr(nw, mxz), nyz = mulr(nw, myz);
+    R nxy(0), nxz(0), nyz(0);  // the source's part of n (see plane)
     const R m93 = mulr(third, m9);
     R rx = fma(nw, ex, -m93), ry = fma(nw, ey, -m93), rz = fma(nw, ez, -m93);
     const R tux = ux + ux, tuy = uy + uy, tuz = uz + uz;
@@ -920,15 +922,13 @@ __device__ __forceinline__ void collide_unit(const CollideConst<typename ScalarO
       cy_ = fy - p.Dyzz;
       bz_ = fz - p.Dxxz;
       cz_ = fz - p.Dyyz;
-      nxy = fma(ux, Fy, fma(uy, Fx, nxy));
-      nxz = fma(ux, Fz, fma(uz, Fx, nxz));
-      nyz = fma(uy, Fz, fma(uz, Fy, nyz));
-      const R two = R(T(2.0));
-      const R wx = mulr(ux, Fx), wy = mulr(uy, Fy), wz = mulr(uz, Fz);
-      rx = fma(two, wx, rx);
-      ry = fma(two, wy, ry);
-      rz = fma(two, wz, rz);
-      dr9 = fma(third, (wx + wy) + wz, dr9);
+      nxy = fma(ux, Fy, fma(uy, Fx, mulr(nw, mxy)));
+      nxz = fma(ux, Fz, fma(uz, Fx, mulr(nw, mxz)));
+      nyz = fma(uy, Fz, fma(uz, Fy, mulr(nw, myz)));
+      rx = fma(tux, Fx, rx);
+      ry = fma(tuy, Fy, ry);
+      rz = fma(tuz, Fz, rz);
+      dr9 = fma(third, fma(ux, Fx, fma(uy, Fy, mulr(uz, Fz))), dr9);
     }
     const R txyy = fma(tuy, cxy, fma(ux, kyy, bx)), txzz = fma(tuz, cxz, fma(ux, kzz, cx_));
     const R txxy = fma(tux, cxy, fma(uy, kxx, by_)), tyzz = fma(tuz, cyz, fma(uy, kzz, cy_));
@@ -967,16 +967,17 @@ __device__ __forceinline__ void collide_unit(const CollideConst<typename ScalarO
       d[5] = fma(half, e + o, d[5]);
       d[6] = fma(half, e - o, d[6]);
     }
-    auto plane = [](R q, R n, R ti, R tj, R& Pp, R& Pm, R& Mp, R& Mm) {
-      const R a = q + n, b = q - n, c = ti + tj, e = ti - tj, f = R(T(0.25));
+    auto plane = [&](R q, R n, R m, R ti, R tj, R& Pp, R& Pm, R& Mp, R& Mm) {
+      const R a = FORCE ? q + n : fma(nw, m, q), b = FORCE ? q - n : fma(w, m, q);
+      const R c = ti + tj, e = ti - tj, f = R(T(0.25));
       Pp = fma(f, a + c, Pp);
       Pm = fma(f, a - c, Pm);
       Mp = fma(f, b + e, Mp);
       Mm = fma(f, b - e, Mm);
     };
-    plane(qxy, nxy, txyy, txxy, d[7], d[10], d[9], d[8]);
-    plane(qxz, nxz, txzz, txxz, d[11], d[14], d[13], d[12]);
-    plane(qyz, nyz, tyzz, tyyz, d[15], d[18], d[17], d[16]);
+    plane(qxy, nxy, mxy, txyy, txxy, d[7], d[10], d[9], d[8]);
+    plane(qxz, nxz, mxz, txzz, txxz, d[11], d[14], d[13], d[12]);
+    plane(qyz, nyz, myz, tyzz, tyyz, d[15], d[18], d[17], d[16]);
   }
   if constexpr (LOG2LAM != 0) out.rho = mulr(rho, R(T(1.0 / double(1 << LOG2LAM))));
   else out.rho = rho;

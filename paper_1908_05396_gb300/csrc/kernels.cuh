@@ -570,17 +570,20 @@ __global__ void import_kernel(const double* __restrict__ in, Geom g, double rho0
 
 #include "tma_step.cuh"
 #include "inplace.cuh"
+#include "pair.cuh"
 
 namespace clbm {
 
 // ---- host-side launchers, instantiated once per storage type --------------
+
+// The arguments of a two-buffer step from src to dst.
 template <typename S, typename R>
-cudaError_t launch_step_t(const void* src, void* dst, const Geom& g, const PhysParams& P,
-                          const CheckBufs& cb, bool check, dim3 block, int npt,
-                          cudaStream_t st) {
+StepArgs<S, R> step_args(const void* src, void* dst, const Geom& g, const PhysParams& P,
+                         const CheckBufs& cb) {
   StepArgs<S, R> a;
   const S* s = static_cast<const S*>(src);
   S* d = static_cast<S*>(dst);
+  const double lam = double(1 << log2_scale<S>());
   for (int q = 0; q < Q; ++q) {
     const int64_t off = int64_t(cz(q)) * g.plane + int64_t(cy(q)) * g.pitch + cx(q);
     // address arithmetic through integers: the shifted base may precede the
@@ -588,7 +591,7 @@ cudaError_t launch_step_t(const void* src, void* dst, const Geom& g, const PhysP
     a.srcq[q] = reinterpret_cast<const S*>(reinterpret_cast<uintptr_t>(s) +
                                             (int64_t(q) * g.qstride - off) * int64_t(sizeof(S)));
     a.dstq[q] = d + int64_t(q) * g.qstride;
-    a.lidc[q] = R(6.0 * wt<double>(q) * g.rho0 * double(1 << log2_scale<S>()) *
+    a.lidc[q] = R(6.0 * wt<double>(q) * g.rho0 * lam *
                   (cx(q) * g.U[0] + cy(q) * g.U[1] + cz(q) * g.U[2]));
   }
   a.src = s;
@@ -604,8 +607,16 @@ cudaError_t launch_step_t(const void* src, void* dst, const Geom& g, const PhysP
   // (the steps that write the lower-addressed of the two buffers) makes the
   // next step read those planes first, from L2.
   a.zrev = reinterpret_cast<uintptr_t>(dst) < reinterpret_cast<uintptr_t>(src) ? 1 : 0;
-  a.C = make_const<R>(P, double(1 << log2_scale<S>()));
+  a.C = make_const<R>(P, lam);
   a.cb = cb;
+  return a;
+}
+
+template <typename S, typename R>
+cudaError_t launch_step_t(const void* src, void* dst, const Geom& g, const PhysParams& P,
+                          const CheckBufs& cb, bool check, dim3 block, int npt,
+                          cudaStream_t st) {
+  StepArgs<S, R> a = step_args<S, R>(src, dst, g, P, cb);
   // npt: 1 or 2 nodes per thread; +4 selects the register-capped variant;
   // TMA_NPT + 32 v the TMA-staged kernel of shape v (check steps take the
   // plain kernel with the same block).
@@ -625,34 +636,44 @@ cudaError_t launch_step_t(const void* src, void* dst, const Geom& g, const PhysP
                        : step_kernel<S, R, false, false, false, false>;
     return pdl_launch(kernel, grid, block, st, a);
   }
-  if constexpr (std::is_same<R, float>::value) {
-    if (npt == 2) {
-      const dim3 grid2((g.nx + block.x - 1) / block.x, (g.ny + 2 * block.y - 1) / (2 * block.y),
-                       g.nz);
-      if (cap)
-        kernel = fc == 3   ? step2_kernel<S, true, true, true>
-                 : fc == 2 ? step2_kernel<S, true, false, true>
-                 : fc == 1 ? step2_kernel<S, false, true, true>
-                           : step2_kernel<S, false, false, true>;
-      else
-        kernel = fc == 3   ? step2_kernel<S, true, true, false>
-                 : fc == 2 ? step2_kernel<S, true, false, false>
-                 : fc == 1 ? step2_kernel<S, false, true, false>
-                           : step2_kernel<S, false, false, false>;
-      return pdl_launch(kernel, grid2, block, st, a);
-    }
-  }
-  if (cap)
+  if constexpr (std::is_same<S, __half>::value) {
+    if (npt == 2 || pair_pays(g, false))
+      return launch_step_pair<PAIR_RN>(a, PairExtra{}, P.has_force != 0, check, block, st);
     kernel = fc == 3   ? step_kernel<S, R, true, true, true, true>
              : fc == 2 ? step_kernel<S, R, true, false, true, true>
              : fc == 1 ? step_kernel<S, R, false, true, true, true>
                        : step_kernel<S, R, false, false, true, true>;
-  else
-    kernel = fc == 3   ? step_kernel<S, R, true, true, false, true>
-             : fc == 2 ? step_kernel<S, R, true, false, false, true>
-             : fc == 1 ? step_kernel<S, R, false, true, false, true>
-                       : step_kernel<S, R, false, false, false, true>;
-  return pdl_launch(kernel, grid, block, st, a);
+    return pdl_launch(kernel, grid, block, st, a);
+  } else {
+    if constexpr (std::is_same<R, float>::value) {
+      if (npt == 2) {
+        const dim3 grid2((g.nx + block.x - 1) / block.x,
+                         (g.ny + 2 * block.y - 1) / (2 * block.y), g.nz);
+        if (cap)
+          kernel = fc == 3   ? step2_kernel<S, true, true, true>
+                   : fc == 2 ? step2_kernel<S, true, false, true>
+                   : fc == 1 ? step2_kernel<S, false, true, true>
+                             : step2_kernel<S, false, false, true>;
+        else
+          kernel = fc == 3   ? step2_kernel<S, true, true, false>
+                   : fc == 2 ? step2_kernel<S, true, false, false>
+                   : fc == 1 ? step2_kernel<S, false, true, false>
+                             : step2_kernel<S, false, false, false>;
+        return pdl_launch(kernel, grid2, block, st, a);
+      }
+    }
+    if (cap)
+      kernel = fc == 3   ? step_kernel<S, R, true, true, true, true>
+               : fc == 2 ? step_kernel<S, R, true, false, true, true>
+               : fc == 1 ? step_kernel<S, R, false, true, true, true>
+                         : step_kernel<S, R, false, false, true, true>;
+    else
+      kernel = fc == 3   ? step_kernel<S, R, true, true, false, true>
+               : fc == 2 ? step_kernel<S, R, true, false, false, true>
+               : fc == 1 ? step_kernel<S, R, false, true, false, true>
+                         : step_kernel<S, R, false, false, false, true>;
+    return pdl_launch(kernel, grid, block, st, a);
+  }
 }
 
 template <typename S, typename R>

@@ -41,6 +41,39 @@ inline int tile_width(int nx, int elem, int bx, int threads) {
   return w;
 }
 
+// Whether a lattice of an FP16 form (ref: F16R) is stepped faster two nodes
+// per thread.  Below the line the GPU is not filled either way, and a step
+// takes the latency of one thread, which one node has less of: F16S 8.6 us
+// against 9.7 at 32^3, 9.7 and 10.1 at 48^3, but 11.2 and 10.4 at 56^3 and
+// 26.4 and 21.8 at 96^3; F16R, whose references the pair loads with half the
+// instructions, 9.0 against 11.8 at 32^3, but 10.7 and 10.0 at 40^3 and 38.3
+// and 35.0 at 96^3.  Both round alike, so the results do not depend on it.
+inline bool pair_pays(const Geom& g, bool ref) {
+  return int64_t(g.nx) * g.ny * g.nz >= (ref ? 48000 : 140000);
+}
+
+// Threads along x (two nodes each) for rows of nx nodes in blocks of
+// `threads` threads, at most `most`: the narrowest of 64, 32 and 16 whose
+// padded row is at least 1/8 shorter than the wider one's (16 pairs are two
+// sectors of FP16 values; narrower tiles of long rows multiply the memory
+// requests: 161-node rows took 73 us a step in tiles of 4 pairs and 44 in
+// tiles of 32), and 8 or 4 for rows that fit them whole, which would leave
+// half of a 16-wide tile idle.
+inline int pair_width(int nx, int threads, int most = 64) {
+  const int np = (nx + 1) / 2;
+  int w = 64;
+  while (w > 4 && (w > most || threads % w)) w /= 2;
+  for (int c = w / 2; c >= 4; c /= 2) {
+    if (c < 16) {
+      if (np <= c) w = c;
+      continue;
+    }
+    const int pw = (np + w - 1) / w * w, pc = (np + c - 1) / c * c;
+    if (8 * pc <= 7 * pw) w = c;
+  }
+  return w;
+}
+
 // Physical parameters of the collision (host precision; kernels convert).
 struct PhysParams {
   double rho0;
@@ -121,8 +154,8 @@ struct BatchHeader {
 #define CLBM_DECLARE_BATCH(SUFFIX)                                                              \
   cudaError_t launch_batch_##SUFFIX(int base, const int* owner, const unsigned* coord,         \
                                     const void* hdr, int parity, bool check, double* acc,       \
-                                    int zc, dim3 block, int grid, bool rates, cudaStream_t st,  \
-                                    cudaStream_t st_forced);                                    \
+                                    int zc, dim3 block, int per_sm, bool cap, int sms,          \
+                                    bool rates, cudaStream_t st, cudaStream_t st_forced);       \
   size_t desc_size_##SUFFIX();                                                                  \
   int desc_capacity_##SUFFIX();                                                                 \
   cudaError_t upload_desc_##SUFFIX(const void* host, int base, int n);                          \

@@ -33,23 +33,13 @@ constexpr int LOG2LAM = 10;  // log2 of the scale of the carried deviations
 constexpr float LAM = float(1 << LOG2LAM);
 static_assert(double(1 << LOG2LAM) == F16_SCALE, "one FP16 storage scale");
 
-struct Ref4 {
-  float dr, vx, vy, vz;  // lam (rho - rho0) and v = lam 3 rho u, as stored (FP16)
-};
-
-__device__ __forceinline__ Ref4 ref_load(const uint2* p) {
-  const uint2 v = *p;
-  const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&v.x));
-  const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&v.y));
-  return {a.x, a.y, b.x, b.y};
-}
-
 // The reference of a node with density rho = rho0 + drho and velocity u,
 // rounded to FP16 for storage; r receives the rounded values.
 __device__ __forceinline__ uint2 ref_make(float drho, float rho, float ux, float uy, float uz,
-                                          Ref4& r) {
-  const float r3 = (3.0f * LAM) * rho;
-  const __half2 a = __floats2half2_rn(LAM * drho, r3 * ux), b = __floats2half2_rn(r3 * uy, r3 * uz);
+                                          RefT<float>& r) {
+  const float r3 = mulr(3.0f * LAM, rho);
+  const __half2 a = __floats2half2_rn(mulr(LAM, drho), mulr(r3, ux)),
+                b = __floats2half2_rn(mulr(r3, uy), mulr(r3, uz));
   const float2 fa = __half22float2(a), fb = __half22float2(b);
   r = {fa.x, fa.y, fb.x, fb.y};
   uint2 v;
@@ -58,31 +48,13 @@ __device__ __forceinline__ uint2 ref_make(float drho, float rho, float ux, float
   return v;
 }
 
-// First-order equilibrium deviation of direction q about the reference,
-// lam w_q [drho + 3 rho (e_q . u)]: the stored v = lam 3 rho u saves the
-// product per direction.
-__device__ __forceinline__ float ref_term(int q, const Ref4& r) {
-  const float ev = float(cx(q)) * r.vx + float(cy(q)) * r.vy + float(cz(q)) * r.vz;
-  return wt<float>(q) * (r.dr + ev);
-}
-
 __device__ __forceinline__ float dec16(__half v) { return __half2float(v); }
 __device__ __forceinline__ __half enc16(float v) { return __float2half_rn(v); }
 
-// Store the 19 post-collision remainders of node i with stochastic rounding,
-// two directions per conversion.
-template <typename Dst>
-__device__ __forceinline__ void store_sr(Dst&& dst_q, const float (&d)[Q], const Ref4& rr,
-                                         uint32_t state) {
-#pragma unroll
-  for (int q = 0; q < Q; q += 2) {
-    const float a = d[q] - ref_term(q, rr);
-    const float b = q + 1 < Q ? d[q + 1] - ref_term(q + 1 < Q ? q + 1 : q, rr) : 0.0f;
-    __half hi, lo;
-    enc16_sr2(a, b, state, hi, lo);
-    dst_q(q) = hi;
-    if (q + 1 < Q) dst_q(q + 1) = lo;
-  }
+// v plus (sgn = 1) or minus (sgn = -1) the first-order equilibrium deviation
+// of direction q about the reference, lam w_q [drho + 3 rho (e_q . u)].
+__device__ __forceinline__ float plus_ref(float v, int q, const RefT<float>& r, float sgn = 1.0f) {
+  return fma(sgn * wt<float>(q), ref_sum(q, r), v);
 }
 
 struct RefArgs {
@@ -111,7 +83,7 @@ __device__ __forceinline__ void pull_face_ref(const __half* __restrict__ src,
     const bool oz = (cz(q) == 1 && fz0) || (cz(q) == -1 && fz1);
     const int up = i - (cz(q) * plane + cy(q) * pitch + cx(q));
     if (!(ox || oy || oz)) {
-      d[q] = dec16(sq[up]) + ref_term(q, ref_load(ref + up));
+      d[q] = plus_ref(dec16(sq[up]), q, ref1(ref + up));
       continue;
     }
     const int kx = ox ? int((fb >> (cx(q) == 1 ? 0 : 2)) & 3u) : int(BC_PERIODIC);
@@ -119,22 +91,22 @@ __device__ __forceinline__ void pull_face_ref(const __half* __restrict__ src,
     const int kz = oz ? int((fb >> (cz(q) == 1 ? 8 : 10)) & 3u) : int(BC_PERIODIC);
     if (kx != BC_PERIODIC || ky != BC_PERIODIC || kz != BC_PERIODIC) {
       const bool lid = kx == BC_LID || ky == BC_LID || kz == BC_LID;
-      const float v = dec16(src[int64_t(opp(q)) * qstride + i]) +
-                      ref_term(opp(q), ref_load(ref + i));
+      const float v = plus_ref(dec16(src[int64_t(opp(q)) * qstride + i]), opp(q), ref1(ref + i));
       d[q] = lid ? v + lidc[q] : v;
     } else {
       int j = up;
       if (ox) j += cx(q) == 1 ? nx : -nx;
       if (oy) j += cy(q) == 1 ? ny * pitch : -ny * pitch;
       if (oz) j += cz(q) == 1 ? nz * plane : -nz * plane;
-      d[q] = dec16(sq[j]) + ref_term(q, ref_load(ref + j));
+      d[q] = plus_ref(dec16(sq[j]), q, ref1(ref + j));
     }
   }
 }
 
-template <bool FORCE, bool CHECK, bool CAP, bool UNIT>
-__global__ void __launch_bounds__(256, CAP ? 4 : 1) step_ref_kernel(const StepArgs<__half, float> a,
-                                                                    const RefArgs r) {
+// One node per thread.
+template <bool FORCE, bool CHECK, bool UNIT>
+__global__ void __launch_bounds__(256) step_ref_kernel(const StepArgs<__half, float> a,
+                                                       const RefArgs r) {
   pdl_enter();
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
@@ -173,9 +145,9 @@ __global__ void __launch_bounds__(256, CAP ? 4 : 1) step_ref_kernel(const StepAr
             extra = k == BC_LID ? a.lidc[q] : 0.0f;
           }
         }
-        const Ref4 t = ref_load(rq);
-        const float ev = float(cx(q)) * t.vx + float(cy(q)) * t.vy + float(cz(q)) * t.vz;
-        d[q] = dec16(*pq) + wt<float>(q) * (t.dr + sgn * ev) + extra;
+        RefT<float> t = ref1(rq);
+        t = {t.dr, mulr(sgn, t.vx), mulr(sgn, t.vy), mulr(sgn, t.vz)};
+        d[q] = plus_ref(dec16(*pq), q, t) + extra;
       }
     } else {
       pull_face_ref(a.src, r.ref_src, a.qstride, a.nx, a.ny, a.nz, a.pitch, a.plane, a.facebits,
@@ -183,9 +155,11 @@ __global__ void __launch_bounds__(256, CAP ? 4 : 1) step_ref_kernel(const StepAr
     }
     NodeOut<float> o;
     collide<float, FORCE, !FORCE, LOG2LAM, UNIT>(a.C, d, o);
-    Ref4 rr;
+    RefT<float> rr;
     r.ref_dst[i] = ref_make(o.rho - rho0, o.rho, o.ux, o.uy, o.uz, rr);
-    store_sr([&](int q) -> __half& { return a.dstq[q][i]; }, d, rr, sr_seed(uint32_t(i), r.step));
+#pragma unroll
+    for (int q = 0; q < Q; ++q) d[q] = plus_ref(d[q], q, rr, -1.0f);
+    store_sr1([&](int q) { return a.dstq[q] + i; }, d, uint32_t(i), r.step);
     if (CHECK) {
       float* up = reinterpret_cast<float*>(a.cb.uprev);
       const int64_t nst = int64_t(a.plane) * a.nz;
@@ -247,7 +221,7 @@ __global__ void export_ref_kernel(const __half* __restrict__ src, const uint2* _
   const int64_t k = t - int64_t(q) * N;
   const int x = int(k % g.nx), y = int((k / g.nx) % g.ny), z = int(k / (int64_t(g.nx) * g.ny));
   const int64_t i = int64_t(z) * g.plane + int64_t(y) * g.pitch + x;
-  const float dev = dec16(src[q * g.qstride + i]) + ref_term(q, ref_load(ref + i));
+  const float dev = plus_ref(dec16(src[q * g.qstride + i]), q, ref1(ref + i));
   out[t] = double(dev) * (1.0 / double(LAM)) + wt<double>(q) * double(rho0);
 }
 
@@ -269,13 +243,13 @@ __global__ void import_ref_kernel(const double* __restrict__ in, Geom g, float r
     jy += cy(q) * f[q];
     jz += cz(q) * f[q];
   }
-  Ref4 rr;
+  RefT<float> rr;
   ref[i] = ref_make(float(rho - rho0), float(rho), float(jx / rho), float(jy / rho),
                     float(jz / rho), rr);
 #pragma unroll
   for (int q = 0; q < Q; ++q)
     dst[q * g.qstride + i] =
-        enc16(float((f[q] - wt<double>(q) * rho0) * double(LAM)) - ref_term(q, rr));
+        enc16(plus_ref(float((f[q] - wt<double>(q) * rho0) * double(LAM)), q, rr, -1.0f));
 }
 
 // M independent nodes: store (with its own reference), load, collide, store
@@ -296,22 +270,21 @@ __global__ void collide_nodes_ref_kernel(CollideConst<float> C, const double* __
     jy += cy(q) * v;
     jz += cz(q) * v;
   }
-  Ref4 rr;
+  RefT<float> rr;
   ref_make(float(r0 - rho0), float(r0), float(jx / r0), float(jy / r0), float(jz / r0), rr);
   float d[Q];
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
-    const float t = ref_term(q, rr);
-    d[q] = dec16(enc16(float((fin[q * M + k] - wt<double>(q) * rho0) * double(LAM)) - t)) + t;
+    const float dev = float((fin[q * M + k] - wt<double>(q) * rho0) * double(LAM));
+    d[q] = plus_ref(dec16(enc16(plus_ref(dev, q, rr, -1.0f))), q, rr);
   }
   NodeOut<float> o;
   collide<float, FORCE, !FORCE, LOG2LAM, true>(C, d, o);
   ref_make(o.rho - rho0, o.rho, o.ux, o.uy, o.uz, rr);
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
-    const float t = ref_term(q, rr);
-    fout[q * M + k] = double(dec16(enc16(d[q] - t)) + t) * (1.0 / double(LAM)) +
-                      wt<double>(q) * double(rho0);
+    const float dev = plus_ref(dec16(enc16(plus_ref(d[q], q, rr, -1.0f))), q, rr);
+    fout[q * M + k] = double(dev) * (1.0 / double(LAM)) + wt<double>(q) * double(rho0);
   }
   if (rho) rho[k] = double(o.rho);
   if (u) {
@@ -333,7 +306,7 @@ void lid_table(const Geom& g, float* out) {
 
 // One node of the batched step in the F16R form: the same pull, references
 // and collision as step_ref_kernel.
-template <bool FORCE, bool UNIT>
+template <bool FORCE>
 __device__ void batch_node_ref(const LatDesc<float>& L, int parity, int x, int y, int z,
                                unsigned step, NodeOut<float>& o) {
   const __half* src = static_cast<const __half*>(L.buf[parity]);
@@ -366,58 +339,44 @@ __device__ void batch_node_ref(const LatDesc<float>& L, int parity, int x, int y
           extra = k == BC_LID ? L.lidc[q] : 0.0f;
         }
       }
-      const Ref4 t = ref_load(rs + jr);
-      const float ev = float(cx(q)) * t.vx + float(cy(q)) * t.vy + float(cz(q)) * t.vz;
-      d[q] = dec16(src[j]) + wt<float>(q) * (t.dr + sgn * ev) + extra;
+      RefT<float> t = ref1(rs + jr);
+      t = {t.dr, mulr(sgn, t.vx), mulr(sgn, t.vy), mulr(sgn, t.vz)};
+      d[q] = plus_ref(dec16(src[j]), q, t) + extra;
     }
   } else {
     pull_face_ref(src, rs, L.qstride, L.nx, L.ny, L.nz, pitch, plane, L.facebits, x, y, z, i,
                   L.lidc, d);
   }
-  collide<float, FORCE, !FORCE, LOG2LAM, UNIT>(L.C, d, o);
-  Ref4 rr;
+  collide<float, FORCE, !FORCE, LOG2LAM, false>(L.C, d, o);
+  RefT<float> rr;
   rd[i] = ref_make(o.rho - rho0, o.rho, o.ux, o.uy, o.uz, rr);
-  store_sr([&](int q) -> __half& { return dst[q * qs + i]; }, d, rr, sr_seed(uint32_t(i), step));
+#pragma unroll
+  for (int q = 0; q < Q; ++q) d[q] = plus_ref(d[q], q, rr, -1.0f);
+  store_sr1([&](int q) { return dst + (q * qs + i); }, d, uint32_t(i), step);
 }
 
 cudaError_t launch_step_f16r(const void* src, void* dst, const void* ref_src, void* ref_dst,
                              const Geom& g, const PhysParams& P, const CheckBufs& cb, bool check,
                              dim3 block, int npt, int64_t step, cudaStream_t st) {
-  StepArgs<__half, float> a;
+  const StepArgs<__half, float> a = step_args<__half, float>(src, dst, g, P, cb);
+  const uint2* rs = static_cast<const uint2*>(ref_src);
+  uint2* rd = static_cast<uint2*>(ref_dst);
+  const bool unit = unit_rates(P);
+  if (unit && pair_pays(g, true))
+    return launch_step_pair<PAIR_REF>(a, PairExtra{rs, rd, unsigned(uint64_t(step))},
+                                      P.has_force != 0, check, block, st);
   RefArgs r;
   r.step = unsigned(uint64_t(step));
-  const __half* s = static_cast<const __half*>(src);
-  __half* d = static_cast<__half*>(dst);
-  const uint2* rs = static_cast<const uint2*>(ref_src);
+  r.ref_src = rs;
+  r.ref_dst = rd;
   for (int q = 0; q < Q; ++q) {
     const int64_t off = int64_t(cz(q)) * g.plane + int64_t(cy(q)) * g.pitch + cx(q);
-    a.srcq[q] = reinterpret_cast<const __half*>(reinterpret_cast<uintptr_t>(s) +
-                                                 (int64_t(q) * g.qstride - off) * 2);
-    a.dstq[q] = d + int64_t(q) * g.qstride;
     r.refq[q] = reinterpret_cast<const uint2*>(reinterpret_cast<uintptr_t>(rs) -
-                                                 off * int64_t(sizeof(uint2)));
+                                                off * int64_t(sizeof(uint2)));
   }
-  lid_table(g, a.lidc);
-  r.ref_src = rs;
-  r.ref_dst = static_cast<uint2*>(ref_dst);
-  a.zrev = reinterpret_cast<uintptr_t>(dst) < reinterpret_cast<uintptr_t>(src) ? 1 : 0;
-  a.src = s;
-  a.qstride = g.qstride;
-  a.nx = g.nx;
-  a.ny = g.ny;
-  a.nz = g.nz;
-  a.pitch = g.pitch;
-  a.plane = int(g.plane);
-  a.facebits = g.facebits;
-  a.C = make_const<float>(P, double(LAM));
-  a.cb = cb;
-  const bool cap = (npt & 4) != 0;
-  dim3 grid((g.nx + block.x - 1) / block.x, (g.ny + block.y - 1) / block.y, g.nz);
+  const dim3 grid((g.nx + block.x - 1) / block.x, (g.ny + block.y - 1) / block.y, g.nz);
   void (*kernel)(const StepArgs<__half, float>, const RefArgs) = nullptr;
-#define CLBM_REF(F, C_)                                            \
-  kernel = !unit_rates(P) ? step_ref_kernel<F, C_, false, false>   \
-           : cap          ? step_ref_kernel<F, C_, true, true>     \
-                          : step_ref_kernel<F, C_, false, true>
+#define CLBM_REF(F, C_) kernel = unit ? step_ref_kernel<F, C_, true> : step_ref_kernel<F, C_, false>
   if (P.has_force) {
     if (check) CLBM_REF(true, true);
     else CLBM_REF(true, false);

@@ -15,9 +15,10 @@
 namespace clbm {
 namespace {
 
-template <bool FORCE, bool CHECK, bool CAP, bool UNIT>
-__global__ void __launch_bounds__(256, CAP ? 4 : 1) step_sr_kernel(const StepArgs<__half, float> a,
-                                                                   unsigned step) {
+// One node per thread.
+template <bool FORCE, bool CHECK, bool UNIT>
+__global__ void __launch_bounds__(256) step_sr_kernel(const StepArgs<__half, float> a,
+                                                      unsigned step) {
   pdl_enter();
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
@@ -40,14 +41,7 @@ __global__ void __launch_bounds__(256, CAP ? 4 : 1) step_sr_kernel(const StepArg
     NodeOut<float> o;
     collide<float, FORCE, pair_out<__half>(), log2_scale<__half>(), UNIT>(a.C, d, o);
     // the deviations are carried scaled by 1024, as they are stored
-    uint32_t state = sr_seed(uint32_t(i), step);
-#pragma unroll
-    for (int q = 0; q < Q; q += 2) {
-      __half hi, lo;
-      enc16_sr2(d[q], q + 1 < Q ? d[q + 1 < Q ? q + 1 : q] : 0.0f, state, hi, lo);
-      a.dstq[q][i] = hi;
-      if (q + 1 < Q) a.dstq[q + 1 < Q ? q + 1 : q][i] = lo;
-    }
+    store_sr1([&](int q) { return a.dstq[q] + i; }, d, uint32_t(i), step);
     if (CHECK) {
       float* up = reinterpret_cast<float*>(a.cb.uprev);
       const int64_t nst = int64_t(a.plane) * a.nz;
@@ -75,45 +69,20 @@ __global__ void __launch_bounds__(256, CAP ? 4 : 1) step_sr_kernel(const StepArg
 
 }  // namespace
 
-// The arguments are those launch_step_t gives the F16S step kernel (upwind
-// base pointers, scaled lid terms and collision constants, the alternating
-// z sweep); npt 1 (plus 4: register-capped) is the only shape.
+// Lattices with the unit rates omega_9..18 take the pair kernel where it is
+// the faster one (pair_pays), the others one node per thread.
 cudaError_t launch_step_f16sr(const void* src, void* dst, const Geom& g, const PhysParams& P,
                               const CheckBufs& cb, bool check, dim3 block, int npt, int64_t step,
                               cudaStream_t st) {
-  StepArgs<__half, float> a;
-  const __half* s = static_cast<const __half*>(src);
-  __half* d = static_cast<__half*>(dst);
-  const double lam = double(1 << log2_scale<__half>());
-  for (int q = 0; q < Q; ++q) {
-    const int64_t off = int64_t(cz(q)) * g.plane + int64_t(cy(q)) * g.pitch + cx(q);
-    // the shifted base may precede the buffer; only base + i of a node in
-    // the box is dereferenced
-    a.srcq[q] = reinterpret_cast<const __half*>(reinterpret_cast<uintptr_t>(s) +
-                                                 (int64_t(q) * g.qstride - off) * 2);
-    a.dstq[q] = d + int64_t(q) * g.qstride;
-    a.lidc[q] = float(6.0 * wt<double>(q) * g.rho0 * lam *
-                      (cx(q) * g.U[0] + cy(q) * g.U[1] + cz(q) * g.U[2]));
-  }
-  a.src = s;
-  a.qstride = g.qstride;
-  a.nx = g.nx;
-  a.ny = g.ny;
-  a.nz = g.nz;
-  a.pitch = g.pitch;
-  a.plane = int(g.plane);
-  a.facebits = g.facebits;
-  a.zrev = reinterpret_cast<uintptr_t>(dst) < reinterpret_cast<uintptr_t>(src) ? 1 : 0;
-  a.C = make_const<float>(P, lam);
-  a.cb = cb;
+  const StepArgs<__half, float> a = step_args<__half, float>(src, dst, g, P, cb);
   const unsigned sstep = unsigned(uint64_t(step));
-  const bool cap = (npt & 4) != 0;
-  dim3 grid((g.nx + block.x - 1) / block.x, (g.ny + block.y - 1) / block.y, g.nz);
+  const bool unit = unit_rates(P);
+  if (unit && pair_pays(g, false))
+    return launch_step_pair<PAIR_SR>(a, PairExtra{nullptr, nullptr, sstep}, P.has_force != 0,
+                                     check, block, st);
+  const dim3 grid((g.nx + block.x - 1) / block.x, (g.ny + block.y - 1) / block.y, g.nz);
   void (*kernel)(const StepArgs<__half, float>, unsigned) = nullptr;
-#define CLBM_SR(F, C_)                                            \
-  kernel = !unit_rates(P) ? step_sr_kernel<F, C_, false, false>   \
-           : cap          ? step_sr_kernel<F, C_, true, true>     \
-                          : step_sr_kernel<F, C_, false, true>
+#define CLBM_SR(F, C_) kernel = unit ? step_sr_kernel<F, C_, true> : step_sr_kernel<F, C_, false>
   if (P.has_force) {
     if (check) CLBM_SR(true, true);
     else CLBM_SR(true, false);
