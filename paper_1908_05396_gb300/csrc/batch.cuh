@@ -44,29 +44,12 @@ __device__ __forceinline__ void batch_node(const LatDesc<R>& L, const S* __restr
   const int qs = int(L.qstride), plane = L.plane, pitch = L.pitch;
   const int i = z * plane + y * pitch + x;
   R d[Q];
-  if (y > 0 && y < L.ny - 1 && z > 0 && z < L.nz - 1) {
+  // as pull_node: warps off every face load directly
+  const bool inner = y > 0 && y < L.ny - 1 && z > 0 && z < L.nz - 1 && x > 0 && x < L.nx - 1;
+  if (__all_sync(__activemask(), inner)) {
 #pragma unroll
     for (int q = 0; q < Q; ++q)
       d[q] = Codec<S, R>::dec(src[q * qs + i - (cz(q) * plane + cy(q) * pitch + cx(q))], R(1));
-    if (x == 0 || x == L.nx - 1) {
-      const int kl = L.facebits & 3, kr = (L.facebits >> 2) & 3;
-#pragma unroll
-      for (int q = 1; q < Q; ++q) {
-        const int j = q * qs + i - (cz(q) * plane + cy(q) * pitch + cx(q));
-        if (cx(q) == 1 && x == 0) {
-          d[q] = kl == BC_PERIODIC
-                     ? Codec<S, R>::dec(src[j + L.nx], R(1))
-                     : Codec<S, R>::dec(src[opp(q) * qs + i], R(1)) +
-                           (kl == BC_LID ? L.lidc[q] : R(0));
-        }
-        if (cx(q) == -1 && x == L.nx - 1) {
-          d[q] = kr == BC_PERIODIC
-                     ? Codec<S, R>::dec(src[j - L.nx], R(1))
-                     : Codec<S, R>::dec(src[opp(q) * qs + i], R(1)) +
-                           (kr == BC_LID ? L.lidc[q] : R(0));
-        }
-      }
-    }
   } else {
     pull_face<S, R>(src, L.qstride, L.nx, L.ny, L.nz, pitch, plane, L.facebits, x, y, z, i,
                     L.lidc, d);

@@ -191,10 +191,7 @@ int clbm_create(const clbm_domain* d, double K, double n, const double U_lid[3],
   for (int a = 0; a < 3; ++a) g.U[a] = U[a];
   g.rho0 = rho0;
   fill_params(h->P, K, n, body_force, rho0, nu_min, nu_max, dtype);
-  h->block.x = d->nx <= 32 ? unsigned(tile_width(d->nx, int(h->elem), 32, 128))
-                           : d->nx <= 64 ? 64 : 128;
-  h->block.y = 128 / h->block.x;
-  h->block.z = 1;
+  h->block = default_block(d->nx, int(h->elem));
   h->npt = 1;  // the autotuner may switch to two nodes per thread
 
   auto cleanup = [&](int code, const std::string& m) {
@@ -478,8 +475,8 @@ int clbm_autotune(clbm_handle h, int steps, int* block_x, int* block_y, int* npt
   // whose kernel is compiled for 128), x extent at most the padded row.
   struct Cand { int bx, by, npt; };
   std::vector<Cand> cands;
-  const int shapes[][2] = {{32, 1}, {32, 2}, {32, 4}, {32, 8}, {64, 1}, {64, 2}, {64, 4},
-                           {128, 1}, {128, 2}, {256, 1}};
+  const int shapes[][2] = {{8, 4},  {8, 8},  {16, 2}, {16, 4}, {16, 8},  {32, 1}, {32, 2},
+                           {32, 4}, {32, 8}, {64, 1}, {64, 2}, {64, 4}, {128, 1}, {256, 1}};
   // FP16 forms with unit rates and two buffers: the pair kernel, which takes
   // from the block its thread count only
   const bool pair = h->elem == 2 && !h->in_place && unit_rates(h->P);

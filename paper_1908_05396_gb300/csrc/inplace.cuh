@@ -23,161 +23,80 @@
 
 namespace clbm {
 
-// Where the node at (x, y, z) crosses a face going one step along -e_q
-// (up = true, the upwind side) or +e_q (the downstream side): for each axis
-// whether it crosses, the kind of the crossed face, and the index shift that
-// wraps a periodic crossing.
-struct Crossing {
-  bool any, bounce, lid;
-  int wrap;  // index offset of the periodic wrap (when !bounce)
-};
-
-template <int q, bool UP>
-__device__ __forceinline__ Crossing crossing(int x, int y, int z, int nx, int ny, int nz,
-                                             int pitch, int plane, unsigned fb) {
-  constexpr int s = UP ? -1 : 1;                  // step along s * e_q
-  constexpr int ex = s * cx(q), ey = s * cy(q), ez = s * cz(q);
-  const bool ox = (ex == -1 && x == 0) || (ex == 1 && x == nx - 1);
-  const bool oy = (ey == -1 && y == 0) || (ey == 1 && y == ny - 1);
-  const bool oz = (ez == -1 && z == 0) || (ez == 1 && z == nz - 1);
-  // faces -x, +x, -y, +y, -z, +z: two bits each
-  const int kx = ox ? int((fb >> (ex == -1 ? 0 : 2)) & 3u) : int(BC_PERIODIC);
-  const int ky = oy ? int((fb >> (ey == -1 ? 4 : 6)) & 3u) : int(BC_PERIODIC);
-  const int kz = oz ? int((fb >> (ez == -1 ? 8 : 10)) & 3u) : int(BC_PERIODIC);
-  Crossing c;
-  c.any = ox || oy || oz;
-  c.bounce = kx != BC_PERIODIC || ky != BC_PERIODIC || kz != BC_PERIODIC;
-  c.lid = kx == BC_LID || ky == BC_LID || kz == BC_LID;
-  c.wrap = (ox ? -ex * nx : 0) + (oy ? -ey * ny * pitch : 0) + (oz ? -ez * nz * plane : 0);
-  return c;
-}
-
-// Pre-collision values of node i in layout L (any node, faces included).
-template <typename S, typename R, int L, int q>
-__device__ __forceinline__ R aa_read_one(const S* A, int64_t qs, int x, int y, int z, int i,
-                                         int nx, int ny, int nz, int pitch, int plane,
-                                         unsigned fb, R lid) {
-  const Crossing c = crossing<q, true>(x, y, z, nx, ny, nz, pitch, plane, fb);
-  if (L == 1) {  // streamed layout: own slot; bounced values get the lid term
-    const R v = Codec<S, R>::dec(A[q * qs + i], R(1));
-    return (c.any && c.bounce && c.lid) ? v + lid : v;
+// Pre-collision values of node i in layout L (any node, faces included).  As
+// in pull_face the face rules select addresses.
+template <typename S, typename R, int L>
+__device__ __forceinline__ void aa_read(const S* A, int64_t qs, int i, int pitch, int plane,
+                                        const Faces& f, const R* lidc, R (&d)[Q]) {
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    // streamed layout: the own slot; swapped layout: the upwind node's
+    // opposite slot, or the own slot q (bounce: f~_opp(q)(x) sits in slot
+    // opp(opp(q)) = q)
+    const bool own = L == 1 || (f.wall & up_faces(q)) != 0;
+    const int j = i - (cz(q) * plane + cy(q) * pitch + cx(q)) + up_wrap(f, q);
+    const S* p = A + (own ? int64_t(q) * qs : int64_t(opp(q)) * qs);
+    d[q] = Codec<S, R>::dec(p[own ? i : j], R(1));
+    if (f.lid & up_faces(q)) d[q] += lidc[q];  // (a lid always bounces)
   }
-  // swapped layout: the upwind node's opposite slot, or the own slot q
-  // (bounce: f~_opp(q)(x) sits in slot opp(opp(q)) = q)
-  if (c.any && c.bounce) {
-    const R v = Codec<S, R>::dec(A[q * qs + i], R(1));
-    return c.lid ? v + lid : v;
-  }
-  const int up = i - (cz(q) * plane + cy(q) * pitch + cx(q)) + (c.any ? c.wrap : 0);
-  return Codec<S, R>::dec(A[opp(q) * qs + up], R(1));
-}
-
-template <typename S, typename R, int L, int q = 0>
-__device__ __forceinline__ void aa_read(const S* A, int64_t qs, int x, int y, int z, int i,
-                                        int nx, int ny, int nz, int pitch, int plane,
-                                        unsigned fb, const R* lidc, R (&d)[Q]) {
-  d[q] = aa_read_one<S, R, L, q>(A, qs, x, y, z, i, nx, ny, nz, pitch, plane, fb, lidc[q]);
-  if constexpr (q + 1 < Q) aa_read<S, R, L, q + 1>(A, qs, x, y, z, i, nx, ny, nz, pitch, plane, fb, lidc, d);
 }
 
 // Post-collision values of node i written for the next layout: after a
 // neighbour step (layout 1) to the downstream node's slot q, or back into
 // the own opposite slot where the downstream side crosses a wall or the lid.
-template <typename S, typename R, int q = 0>
-__device__ __forceinline__ void aa_write_streamed(S* A, int64_t qs, int x, int y, int z, int i,
-                                                  int nx, int ny, int nz, int pitch, int plane,
-                                                  unsigned fb, const R (&d)[Q]) {
-  const Crossing c = crossing<q, false>(x, y, z, nx, ny, nz, pitch, plane, fb);
-  if (c.any && c.bounce) {
-    A[opp(q) * qs + i] = Codec<S, R>::enc(d[q], R(1));
-  } else {
-    const int dn = i + (cz(q) * plane + cy(q) * pitch + cx(q)) + (c.any ? c.wrap : 0);
-    A[q * qs + dn] = Codec<S, R>::enc(d[q], R(1));
+template <typename S, typename R>
+__device__ __forceinline__ void aa_write_streamed(S* A, int64_t qs, int i, int pitch, int plane,
+                                                  const Faces& f, const R (&d)[Q]) {
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    const bool bounce = (f.wall & up_faces(opp(q))) != 0;
+    const int j = i + (cz(q) * plane + cy(q) * pitch + cx(q)) + up_wrap(f, opp(q));
+    S* p = A + (bounce ? int64_t(opp(q)) * qs : int64_t(q) * qs);
+    p[bounce ? i : j] = Codec<S, R>::enc(d[q], R(1));
   }
-  if constexpr (q + 1 < Q) aa_write_streamed<S, R, q + 1>(A, qs, x, y, z, i, nx, ny, nz, pitch, plane, fb, d);
 }
 
-// Lid terms of the bounced values in the streamed layout (local step).
-template <typename S, typename R, int q = 1>
-__device__ __forceinline__ void aa_lid_fix(int x, int y, int z, int nx, int ny, int nz, int pitch,
-                                           int plane, unsigned fb, const R* lidc, R (&d)[Q]) {
-  const Crossing c = crossing<q, true>(x, y, z, nx, ny, nz, pitch, plane, fb);
-  if (c.any && c.bounce && c.lid) d[q] += lidc[q];
-  if constexpr (q + 1 < Q) aa_lid_fix<S, R, q + 1>(x, y, z, nx, ny, nz, pitch, plane, fb, lidc, d);
+// In-place update of node (x, y, z) with index i.  LIN is the layout the step
+// reads: 0 -> neighbour step (srcq[q] = A + opp(q) qs - off(q), dstq[q] =
+// A + q qs + off(q)), 1 -> local step (srcq[q] = A + q qs, dstq[q] = A +
+// opp(q) qs); a.src is the buffer A.  Nodes off the faces take the direct path.
+template <typename S, typename R, int LIN, bool FORCE, bool UNIT>
+__device__ __forceinline__ void aa_update(const StepArgs<S, R>& a, int x, int y, int z, int i,
+                                          NodeOut<R>& o) {
+  S* A = const_cast<S*>(a.src);
+  const bool inner = x > 0 && x < a.nx - 1 && y > 0 && y < a.ny - 1 && z > 0 && z < a.nz - 1;
+  const Faces f = faces_of(x, y, z, a.nx, a.ny, a.nz, a.pitch, a.plane, a.facebits);
+  R d[Q];
+  if (inner) {
+#pragma unroll
+    for (int q = 0; q < Q; ++q) d[q] = Codec<S, R>::dec(a.srcq[q][i], R(1));
+  } else {
+    aa_read<S, R, LIN>(A, a.qstride, i, a.pitch, a.plane, f, a.lidc, d);
+  }
+  collide<R, FORCE, pair_out<S>(), log2_scale<S>(), UNIT>(a.C, d, o);
+  if (LIN == 1 || inner) {
+#pragma unroll
+    for (int q = 0; q < Q; ++q) a.dstq[q][i] = Codec<S, R>::enc(d[q], R(1));
+  } else {
+    aa_write_streamed<S, R>(A, a.qstride, i, a.pitch, a.plane, f, d);
+  }
 }
 
-// One in-place step.  LIN is the layout the step reads: 0 -> neighbour step
-// (srcq[q] = A + opp(q) qs - off(q), dstq[q] = A + q qs + off(q)), 1 -> local
-// step (srcq[q] = A + q qs, dstq[q] = A + opp(q) qs); a.src is the buffer A.
-// Nodes off the y and z faces take the direct path (the x-face lanes fix
-// their crossing directions); nodes on a y or z face resolve every direction.
-// UNIT as in step_kernel.
+// One in-place step.  UNIT as in step_kernel.
 template <typename S, typename R, int LIN, bool FORCE, bool CHECK, bool CAP, bool UNIT>
 __global__ void __launch_bounds__(256, CAP ? 4 : 1) step_aa_kernel(const StepArgs<S, R> a) {
   pdl_enter();
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
-  const int z = a.zrev ? a.nz - 1 - int(blockIdx.z) : int(blockIdx.z);  // as step_kernel
+  const int z = blockIdx.z;
   const bool active = x < a.nx && y < a.ny;
   if (!CHECK && !active) return;
   double du2 = 0.0, uu = 0.0, dr = 0.0;
   int bad = 0;
   if (active) {
     const int i = z * a.plane + y * a.pitch + x;
-    S* A = const_cast<S*>(a.src);
-    const bool inyz = y > 0 && y < a.ny - 1 && z > 0 && z < a.nz - 1;
-    const bool xface = x == 0 || x == a.nx - 1;
-    const int kl = a.facebits & 3, kr = (a.facebits >> 2) & 3;
-    R d[Q];
-    if (LIN == 1) {
-#pragma unroll
-      for (int q = 0; q < Q; ++q) d[q] = Codec<S, R>::dec(a.srcq[q][i], R(1));
-      if (!inyz || xface)
-        aa_lid_fix<S, R>(x, y, z, a.nx, a.ny, a.nz, a.pitch, a.plane, a.facebits, a.lidc, d);
-    } else if (inyz) {
-#pragma unroll
-      for (int q = 0; q < Q; ++q) d[q] = Codec<S, R>::dec(a.srcq[q][i], R(1));
-      if (xface) {
-#pragma unroll
-        for (int q = 1; q < Q; ++q) {
-          const bool left = cx(q) == 1 && x == 0, right = cx(q) == -1 && x == a.nx - 1;
-          if (left || right) {
-            const int k = left ? kl : kr;
-            if (k == BC_PERIODIC)
-              d[q] = Codec<S, R>::dec(a.srcq[q][left ? i + a.nx : i - a.nx], R(1));
-            else
-              d[q] = Codec<S, R>::dec(A[q * a.qstride + i], R(1)) +
-                     (k == BC_LID ? a.lidc[q] : R(0));
-          }
-        }
-      }
-    } else {
-      aa_read<S, R, 0>(A, a.qstride, x, y, z, i, a.nx, a.ny, a.nz, a.pitch, a.plane, a.facebits,
-                       a.lidc, d);
-    }
     NodeOut<R> o;
-    collide<R, FORCE, pair_out<S>(), log2_scale<S>(), UNIT>(a.C, d, o);
-    if (LIN == 1) {
-#pragma unroll
-      for (int q = 0; q < Q; ++q) a.dstq[q][i] = Codec<S, R>::enc(d[q], R(1));
-    } else if (inyz) {
-#pragma unroll
-      for (int q = 0; q < Q; ++q) {
-        // downstream across an x face: wrap, or keep at the node (bounce)
-        const bool right = cx(q) == 1 && x == a.nx - 1, left = cx(q) == -1 && x == 0;
-        const S v = Codec<S, R>::enc(d[q], R(1));
-        if (right || left) {
-          const int k = right ? kr : kl;
-          if (k == BC_PERIODIC) a.dstq[q][right ? i - a.nx : i + a.nx] = v;
-          else A[opp(q) * a.qstride + i] = v;
-        } else {
-          a.dstq[q][i] = v;
-        }
-      }
-    } else {
-      aa_write_streamed<S, R>(A, a.qstride, x, y, z, i, a.nx, a.ny, a.nz, a.pitch, a.plane,
-                              a.facebits, d);
-    }
+    aa_update<S, R, LIN, FORCE, UNIT>(a, x, y, z, i, o);
     if (CHECK) {
       R* up = reinterpret_cast<R*>(a.cb.uprev);
       const int64_t nst = int64_t(a.plane) * a.nz;
@@ -220,8 +139,8 @@ __global__ void __launch_bounds__(256) fields_aa_kernel(const S* __restrict__ A,
                 (cx(q) * g.U[0] + cy(q) * g.U[1] + cz(q) * g.U[2]));
   const int i = z * int(g.plane) + y * g.pitch + x;
   R d[Q];
-  aa_read<S, R, L>(A, g.qstride, x, y, z, i, g.nx, g.ny, g.nz, g.pitch, int(g.plane), g.facebits,
-                   lidc, d);
+  aa_read<S, R, L>(A, g.qstride, i, g.pitch, int(g.plane),
+                   faces_of(x, y, z, g.nx, g.ny, g.nz, g.pitch, int(g.plane), g.facebits), lidc, d);
   NodeOut<R> o;
   collide<R, FORCE, pair_out<S>(), log2_scale<S>(), false>(C, d, o);
   const int64_t N = int64_t(g.nx) * g.ny * g.nz;
@@ -283,13 +202,13 @@ __global__ void import_aa_kernel(const double* __restrict__ in, Geom g, double r
 }
 
 // ---- host-side launchers ------------------------------------------------------
+// The arguments of a step that reads layout `layout` (all planes in ascending
+// order: an alternating sweep, either parity, measured 2 % slower here).
 template <typename S, typename R>
-cudaError_t launch_step_aa_t(void* buf, const Geom& g, const PhysParams& P, const CheckBufs& cb,
-                             bool check, dim3 block, int npt, int layout, cudaStream_t st) {
-  StepArgs<S, R> a;
-  S* A = static_cast<S*>(buf);
-  const uintptr_t base = reinterpret_cast<uintptr_t>(A);
-  a.zrev = 0;  // an alternating sweep (either parity) measured 2 % slower here
+StepArgs<S, R> aa_args(void* buf, const Geom& g, const PhysParams& P, const CheckBufs& cb,
+                       int layout) {
+  StepArgs<S, R> a = step_args<S, R>(buf, buf, g, P, cb);
+  const uintptr_t base = reinterpret_cast<uintptr_t>(buf);
   for (int q = 0; q < Q; ++q) {
     const int64_t off = int64_t(cz(q)) * g.plane + int64_t(cy(q)) * g.pitch + cx(q);
     // address arithmetic through integers: a shifted base may lie outside the
@@ -298,19 +217,14 @@ cudaError_t launch_step_aa_t(void* buf, const Geom& g, const PhysParams& P, cons
     const int64_t dq = layout == 0 ? int64_t(q) * g.qstride + off : int64_t(opp(q)) * g.qstride;
     a.srcq[q] = reinterpret_cast<const S*>(base + sq * int64_t(sizeof(S)));
     a.dstq[q] = reinterpret_cast<S*>(base + dq * int64_t(sizeof(S)));
-    a.lidc[q] = R(6.0 * wt<double>(q) * g.rho0 * double(1 << log2_scale<S>()) *
-                  (cx(q) * g.U[0] + cy(q) * g.U[1] + cz(q) * g.U[2]));
   }
-  a.src = A;
-  a.qstride = g.qstride;
-  a.nx = g.nx;
-  a.ny = g.ny;
-  a.nz = g.nz;
-  a.pitch = g.pitch;
-  a.plane = int(g.plane);
-  a.facebits = g.facebits;
-  a.C = make_const<R>(P, double(1 << log2_scale<S>()));
-  a.cb = cb;
+  return a;
+}
+
+template <typename S, typename R>
+cudaError_t launch_step_aa_t(void* buf, const Geom& g, const PhysParams& P, const CheckBufs& cb,
+                             bool check, dim3 block, int npt, int layout, cudaStream_t st) {
+  const StepArgs<S, R> a = aa_args<S, R>(buf, g, P, cb, layout);
   const bool cap = (npt & 4) != 0;
   const dim3 grid((g.nx + block.x - 1) / block.x, (g.ny + block.y - 1) / block.y, g.nz);
   void (*kernel)(const StepArgs<S, R>) = nullptr;

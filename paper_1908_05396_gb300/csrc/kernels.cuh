@@ -192,70 +192,84 @@ struct StepArgs {
   CheckBufs cb;
 };
 
+// The faces a node lies on.  Bits 0..5 stand for the faces -x, +x, -y, +y,
+// -z, +z: `wall` has those of the node's faces that are walls or lids, `lid`
+// the lids among them; wrap[k] is the index offset that brings a step across
+// face k back into the lattice when the node lies on that face (else 0).
+struct Faces {
+  unsigned wall, lid;
+  int wrap[6];
+};
+__device__ __forceinline__ Faces faces_of(int x, int y, int z, int nx, int ny, int nz, int pitch,
+                                          int plane, unsigned fb) {
+  const bool at[6] = {x == 0, x == nx - 1, y == 0, y == ny - 1, z == 0, z == nz - 1};
+  const int len[3] = {nx, ny * pitch, nz * plane};
+  Faces f;
+  f.wall = f.lid = 0u;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const unsigned kind = (fb >> (2 * k)) & 3u;
+    if (at[k] && kind != BC_PERIODIC) f.wall |= 1u << k;
+    if (at[k] && kind == BC_LID) f.lid |= 1u << k;
+    f.wrap[k] = at[k] ? (k & 1 ? -len[k / 2] : len[k / 2]) : 0;
+  }
+  return f;
+}
+// Faces that a step along -e_q (the upwind side) can cross; the downwind side
+// of q is the upwind side of opp(q).
+__host__ __device__ constexpr unsigned up_faces(int q) {
+  return (cx(q) == 1 ? 1u : cx(q) == -1 ? 2u : 0u) | (cy(q) == 1 ? 4u : cy(q) == -1 ? 8u : 0u) |
+         (cz(q) == 1 ? 16u : cz(q) == -1 ? 32u : 0u);
+}
+// Index offset of the periodic wrap of a step along -e_q.
+__device__ __forceinline__ int up_wrap(const Faces& f, int q) {
+  int w = 0;
+  if (cx(q)) w += f.wrap[cx(q) == 1 ? 0 : 1];
+  if (cy(q)) w += f.wrap[cy(q) == 1 ? 2 : 3];
+  if (cz(q)) w += f.wrap[cz(q) == 1 ? 4 : 5];
+  return w;
+}
+
 // Pull of all 19 directions into node (x, y, z) with index i, for a node on
-// any face.  A direction whose upwind node lies inside the lattice is loaded
-// as in the interior (its address is formed only then); the others follow the
-// face rules -- the periodic wrap along a periodic axis, or else (any crossed
-// wall or lid face) halfway bounce-back from the node's own opposite
-// population, plus the lid term when a crossed face is the lid.  With the directions unrolled, a warp on a face issues one load per
-// direction instead of a call with table lookups.
+// any face: the upwind node's value, across a periodic face the wrapped
+// node's, or, where any crossed face is a wall or the lid, halfway bounce-back
+// from the node's own opposite population, plus the lid term when a crossed
+// face is the lid.  The rule selects an address, so the 19 loads are issued
+// together; branching to a load per rule exposed their latency one after the
+// other, in a small lattice most of the step (32^3 F16S 8.3 us a step, 4.6
+// with the addresses selected, FP32 6.1 and 4.3) and in a large one the tail
+// that the face blocks formed (128^3 F16S 38.6 and 30.7, F16R 61 and 55, FP32
+// 53 and 50).
 template <typename S, typename R>
 __device__ __forceinline__ void pull_face(const S* __restrict__ src, int64_t qstride, int nx,
                                           int ny, int nz, int pitch, int plane, unsigned fb,
                                           int x, int y, int z, int i, const R* lidc, R (&d)[Q]) {
-  const bool fx0 = x == 0, fx1 = x == nx - 1, fy0 = y == 0, fy1 = y == ny - 1;
-  const bool fz0 = z == 0, fz1 = z == nz - 1;
+  const Faces f = faces_of(x, y, z, nx, ny, nz, pitch, plane, fb);
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
-    const S* sq = src + int64_t(q) * qstride;
-    const bool ox = (cx(q) == 1 && fx0) || (cx(q) == -1 && fx1);
-    const bool oy = (cy(q) == 1 && fy0) || (cy(q) == -1 && fy1);
-    const bool oz = (cz(q) == 1 && fz0) || (cz(q) == -1 && fz1);
-    const int up = i - (cz(q) * plane + cy(q) * pitch + cx(q));
-    if (!(ox || oy || oz)) {
-      d[q] = Codec<S, R>::dec(sq[up], R(1));
-      continue;
-    }
-    // kind of each crossed face (faces -x, +x, -y, +y, -z, +z, two bits each)
-    const int kx = ox ? int((fb >> (cx(q) == 1 ? 0 : 2)) & 3u) : int(BC_PERIODIC);
-    const int ky = oy ? int((fb >> (cy(q) == 1 ? 4 : 6)) & 3u) : int(BC_PERIODIC);
-    const int kz = oz ? int((fb >> (cz(q) == 1 ? 8 : 10)) & 3u) : int(BC_PERIODIC);
-    if (kx != BC_PERIODIC || ky != BC_PERIODIC || kz != BC_PERIODIC) {
-      const bool lid = kx == BC_LID || ky == BC_LID || kz == BC_LID;
-      const R v = Codec<S, R>::dec(src[int64_t(opp(q)) * qstride + i], R(1));
-      d[q] = lid ? v + lidc[q] : v;
-    } else {
-      int j = up;
-      if (ox) j += cx(q) == 1 ? nx : -nx;
-      if (oy) j += cy(q) == 1 ? ny * pitch : -ny * pitch;
-      if (oz) j += cz(q) == 1 ? nz * plane : -nz * plane;
-      d[q] = Codec<S, R>::dec(sq[j], R(1));
-    }
+    const bool bounce = (f.wall & up_faces(q)) != 0;
+    const int j = i - (cz(q) * plane + cy(q) * pitch + cx(q)) + up_wrap(f, q);
+    const S* p = src + (bounce ? int64_t(opp(q)) * qstride : int64_t(q) * qstride);
+    d[q] = Codec<S, R>::dec(p[bounce ? i : j], R(1));
+    if (f.lid & up_faces(q)) d[q] += lidc[q];
   }
 }
 
-// For a node off the y and z faces whose d[] holds the plain upwind values:
-// replace the directions that cross an x face (bounce-back with the lid term,
-// or the periodic wrap).  Only lanes at x = 0 or x = nx - 1 do any work.
+// Pull of node (x, y, z) with index i of a two-buffer lattice: a warp off
+// every face loads its 19 upwind values directly, any other goes through
+// pull_face as a whole (patching the lanes on an x face after direct loads
+// costs a second, dependent round of loads: 32^3 FP32 4.3 us a step against
+// 2.6, 128^3 50.4 against 48.4).
 template <typename S, typename R>
-__device__ __forceinline__ void xface_fix(const StepArgs<S, R>& a, int x, int i, R (&d)[Q]) {
-  if (x == 0 || x == a.nx - 1) {
-    const int kl = a.facebits & 3, kr = (a.facebits >> 2) & 3;
+__device__ __forceinline__ void pull_node(const StepArgs<S, R>& a, int x, int y, int z, int i,
+                                          R (&d)[Q]) {
+  const bool inner = y > 0 && y < a.ny - 1 && z > 0 && z < a.nz - 1 && x > 0 && x < a.nx - 1;
+  if (__all_sync(__activemask(), inner)) {
 #pragma unroll
-    for (int q = 1; q < Q; ++q) {
-      if (cx(q) == 1 && x == 0) {
-        d[q] = kl == BC_PERIODIC
-                   ? Codec<S, R>::dec(a.srcq[q][i + a.nx], R(1))
-                   : Codec<S, R>::dec(a.src[opp(q) * a.qstride + i], R(1)) +
-                         (kl == BC_LID ? a.lidc[q] : R(0));
-      }
-      if (cx(q) == -1 && x == a.nx - 1) {
-        d[q] = kr == BC_PERIODIC
-                   ? Codec<S, R>::dec(a.srcq[q][i - a.nx], R(1))
-                   : Codec<S, R>::dec(a.src[opp(q) * a.qstride + i], R(1)) +
-                         (kr == BC_LID ? a.lidc[q] : R(0));
-      }
-    }
+    for (int q = 0; q < Q; ++q) d[q] = Codec<S, R>::dec(a.srcq[q][i], R(1));
+  } else {
+    pull_face<S, R>(a.src, a.qstride, a.nx, a.ny, a.nz, a.pitch, a.plane, a.facebits, x, y, z, i,
+                    a.lidc, d);
   }
 }
 
@@ -301,10 +315,7 @@ inline cudaError_t pdl_launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, c
   return pdl_launch_smem(kernel, grid, block, 0, st, args...);
 }
 
-// One time step.  Warps off the y and z faces load all 19 upwind values
-// unconditionally and then, in the one or two lanes on an x face, replace the
-// five directions that come from outside the box; warps on a y or z face go
-// through pull_face.  CHECK = true also writes u into uprev (after reading
+// One time step.  CHECK = true also writes u into uprev (after reading
 // the previous check's value there) and reduces sum|u - uprev|^2, sum|u|^2,
 // sum(rho - rho0) and a divergence flag in FP64.
 // CAP = true caps registers so that four 256-thread (or eight 128-thread)
@@ -325,14 +336,7 @@ __global__ void __launch_bounds__(256, CAP ? 4 : 1) step_kernel(const StepArgs<S
   if (active) {
     const int i = z * a.plane + y * a.pitch + x;
     R d[Q];
-    if (y > 0 && y < a.ny - 1 && z > 0 && z < a.nz - 1) {
-#pragma unroll
-      for (int q = 0; q < Q; ++q) d[q] = Codec<S, R>::dec(a.srcq[q][i], R(1));
-      xface_fix(a, x, i, d);
-    } else {
-      pull_face<S, R>(a.src, a.qstride, a.nx, a.ny, a.nz, a.pitch, a.plane, a.facebits, x, y, z,
-                      i, a.lidc, d);
-    }
+    pull_node(a, x, y, z, i, d);
     NodeOut<R> o;
     collide<R, FORCE, pair_out<S>(), log2_scale<S>(), UNIT>(a.C, d, o);
 #pragma unroll
@@ -566,16 +570,6 @@ __global__ void import_kernel(const double* __restrict__ in, Geom g, double rho0
   dst[q * g.qstride + i] = Codec<S, double>::enc((in[t] - w * rho0) / inv_scale, inv_scale);
 }
 
-}  // namespace clbm
-
-#include "tma_step.cuh"
-#include "inplace.cuh"
-#include "pair.cuh"
-
-namespace clbm {
-
-// ---- host-side launchers, instantiated once per storage type --------------
-
 // The arguments of a two-buffer step from src to dst.
 template <typename S, typename R>
 StepArgs<S, R> step_args(const void* src, void* dst, const Geom& g, const PhysParams& P,
@@ -611,6 +605,16 @@ StepArgs<S, R> step_args(const void* src, void* dst, const Geom& g, const PhysPa
   a.cb = cb;
   return a;
 }
+
+}  // namespace clbm
+
+#include "tma_step.cuh"
+#include "inplace.cuh"
+#include "pair.cuh"
+
+namespace clbm {
+
+// ---- host-side launchers, instantiated once per storage type --------------
 
 template <typename S, typename R>
 cudaError_t launch_step_t(const void* src, void* dst, const Geom& g, const PhysParams& P,

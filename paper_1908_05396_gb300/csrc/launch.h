@@ -41,15 +41,29 @@ inline int tile_width(int nx, int elem, int bx, int threads) {
   return w;
 }
 
+// Block of a lone lattice's step kernel until it is tuned.  Tiles of 16 x 4
+// nodes (8 x 8 where that shortens the padded row by 1/8) beat rows of 32 to
+// 128 nodes at every size: the y neighbours' rows are found in L1 more often
+// and fewer warps hold face nodes or idle lanes (FP32 128^3 48.6 -> 47.3 us
+// a step, in place 58.5 -> 54.1, 80^3 15.4 -> 12.7, 40^3 5.2 -> 3.5).  FP64
+// is bound by the FP64 pipe, which a warp occupies whatever its idle lanes:
+// one warp per block, 8 x 4 (the finest spread over the SMs; 128^3 alike,
+// 80^3 304 -> 247 us, 48^3 78 -> 59, 36^3 58 -> 28).
+inline dim3 default_block(int nx, int elem) {
+  if (elem == 8) return nx <= 4 ? dim3(4, 8, 1) : dim3(8, 4, 1);
+  const int p16 = (nx + 15) / 16 * 16, p8 = (nx + 7) / 8 * 8;
+  return 8 * p8 <= 7 * p16 ? dim3(8, 8, 1) : dim3(16, 4, 1);
+}
+
 // Whether a lattice of an FP16 form (ref: F16R) is stepped faster two nodes
 // per thread.  Below the line the GPU is not filled either way, and a step
-// takes the latency of one thread, which one node has less of: F16S 8.6 us
-// against 9.7 at 32^3, 9.7 and 10.1 at 48^3, but 11.2 and 10.4 at 56^3 and
-// 26.4 and 21.8 at 96^3; F16R, whose references the pair loads with half the
-// instructions, 9.0 against 11.8 at 32^3, but 10.7 and 10.0 at 40^3 and 38.3
-// and 35.0 at 96^3.  Both round alike, so the results do not depend on it.
+// takes the latency of one thread, which one node has less of: F16S 2.8 us
+// against 4.0 at 32^3 and 3.5 against 3.9 at 40^3, but 5.7 and 5.0 at 48^3;
+// F16R 5.0 against 6.1 at 32^3 and 5.7 against 6.2 at 36^3, but 38 and 29 at
+// 96^3, where its reference loads count.  Both round alike, so the results
+// do not depend on the choice.
 inline bool pair_pays(const Geom& g, bool ref) {
-  return int64_t(g.nx) * g.ny * g.nz >= (ref ? 48000 : 140000);
+  return int64_t(g.nx) * g.ny * g.nz >= (ref ? 48000 : 100000);
 }
 
 // Threads along x (two nodes each) for rows of nx nodes in blocks of

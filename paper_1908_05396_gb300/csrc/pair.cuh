@@ -40,12 +40,12 @@ template <typename R>
 struct RefT {
   R dr, vx, vy, vz;
 };
-__device__ __forceinline__ RefT<float> ref1(const uint2* p) {
-  const uint2 v = *p;
+__device__ __forceinline__ RefT<float> ref_dec(uint2 v) {
   const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&v.x));
   const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&v.y));
   return {a.x, a.y, b.x, b.y};
 }
+__device__ __forceinline__ RefT<float> ref1(const uint2* p) { return ref_dec(*p); }
 // dr + e_q . v, the part of the reference term that w_q multiplies; the sums
 // are associated alike for a node and a pair, so that a reader forms the
 // value the writer subtracted.
@@ -168,50 +168,33 @@ __device__ __forceinline__ void pull_pair(const P& p, int x, int y, int z, V2 (&
     }
     return;
   }
-  const int n1 = x + 1 < nx ? 1 : 0;  // offset of the second node (0: it is padding)
-  const bool fy0 = y == 0, fy1 = y == p.ny() - 1, fz0 = z == 0, fz1 = z == p.nz() - 1;
+  // Rows on a y or z face: the rules select an address per direction (and
+  // node, where e_x != 0), so that all loads can be issued together (see
+  // pull_face).  A second node in the padding repeats the first.
+  const int n1 = x + 1 < nx ? 1 : 0;
+  const Faces fA = faces_of(x, y, z, nx, p.ny(), p.nz(), pitch, plane, fb);
+  const Faces fB = faces_of(x + n1, y, z, nx, p.ny(), p.nz(), pitch, plane, fb);
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
-    const bool oy = (cy(q) == 1 && fy0) || (cy(q) == -1 && fy1);
-    const bool oz = (cz(q) == 1 && fz0) || (cz(q) == -1 && fz1);
-    const int ky = oy ? int((fb >> (cy(q) == 1 ? 4 : 6)) & 3u) : int(BC_PERIODIC);
-    const int kz = oz ? int((fb >> (cz(q) == 1 ? 8 : 10)) & 3u) : int(BC_PERIODIC);
-    const bool oxA = (cx(q) == 1 && first) || (cx(q) == -1 && last && nr == 0);
-    const bool oxB = cx(q) == -1 && last && nr == 1;
-    const int kx = cx(q) == 1 ? kl : kr;
-    if (ky != BC_PERIODIC || kz != BC_PERIODIC) {
-      // a y or z wall: both nodes bounce; the lid rule where a lid is crossed
-      V2 v = ld2(p.own(opp(q)));
-      if (REF) {
-        const RefT<float> r0 = ref1(p.ref), r1 = ref1(p.ref + n1);
-        v = fma(V2(wt<float>(q)), V2(ref_sum(opp(q), r0), ref_sum(opp(q), r1)), v);
-      }
-      const bool lid = ky == BC_LID || kz == BC_LID;
-      if (lid || (oxA && kx == BC_LID)) set0(v, lane0(v) + p.lid(q));
-      if (lid || (oxB && kx == BC_LID)) set1(v, lane1(v) + p.lid(q));
-      d[q] = v;
-      continue;
+    const int off = cz(q) * plane + cy(q) * pitch + cx(q);
+    const bool bA = (fA.wall & up_faces(q)) != 0, bB = (fB.wall & up_faces(q)) != 0;
+    const __half *same = p.own(q), *anti = p.own(opp(q));
+    const int jA = bA ? 0 : up_wrap(fA, q) - off;
+    const int jB = cx(q) == 0 ? jA + n1 : bB ? n1 : up_wrap(fB, q) - off + n1;
+    V2 v;
+    if (cx(q) == 0) v = ld2((bA ? anti : same) + jA);
+    else v = V2(ld1((bA ? anti : same) + jA), ld1((bB ? anti : same) + jB));
+    if (REF) {
+      // a bounced value is decoded as opp(q): e_q . v changes sign
+      const V2 sgn(bA ? -1.0f : 1.0f, bB ? -1.0f : 1.0f);
+      const RefT<float> rA = ref1(p.ref + jA), rB = ref1(p.ref + jB);
+      const RefT<V2> r{V2(rA.dr, rB.dr), mulr(sgn, V2(rA.vx, rB.vx)), mulr(sgn, V2(rA.vy, rB.vy)),
+                       mulr(sgn, V2(rA.vz, rB.vz))};
+      v = fma(V2(wt<float>(q)), ref_sum(q, r), v);
     }
-    int j = 0;  // wrap along periodic y and z
-    if (oy) j += cy(q) == 1 ? p.ny() * pitch : -p.ny() * pitch;
-    if (oz) j += cz(q) == 1 ? p.nz() * plane : -p.nz() * plane;
-    const __half* u = p.up(q) + j;
-    const uint2* r = p.ref - (cz(q) * plane + cy(q) * pitch + cx(q)) + j;
-    const int dx = cx(q) == 1 ? nx : -nx;
-    float v0, v1;
-    if (cx(q) != 0 && oxA) {
-      v0 = xface_value<REF>(p, q, kx, 0, u, r, dx);
-    } else {
-      v0 = ld1(u);
-      if (REF) v0 = fma(wt<float>(q), ref_sum(q, ref1(r)), v0);
-    }
-    if (cx(q) != 0 && oxB) {
-      v1 = xface_value<REF>(p, q, kx, 1, u + 1, r + 1, dx);
-    } else {
-      v1 = n1 ? ld1(u + 1) : 0.0f;
-      if (REF && n1) v1 = fma(wt<float>(q), ref_sum(q, ref1(r + 1)), v1);
-    }
-    d[q] = V2(v0, v1);
+    if (fA.lid & up_faces(q)) set0(v, lane0(v) + p.lid(q));
+    if (fB.lid & up_faces(q)) set1(v, lane1(v) + p.lid(q));
+    d[q] = v;
   }
 }
 

@@ -73,34 +73,45 @@ __device__ __forceinline__ void pull_face_ref(const __half* __restrict__ src,
                                               int nx, int ny, int nz, int pitch, int plane,
                                               unsigned fb, int x, int y, int z, int i,
                                               const float* lidc, float (&d)[Q]) {
-  const bool fx0 = x == 0, fx1 = x == nx - 1, fy0 = y == 0, fy1 = y == ny - 1;
-  const bool fz0 = z == 0, fz1 = z == nz - 1;
+  const Faces f = faces_of(x, y, z, nx, ny, nz, pitch, plane, fb);
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
-    const __half* sq = src + int64_t(q) * qstride;
-    const bool ox = (cx(q) == 1 && fx0) || (cx(q) == -1 && fx1);
-    const bool oy = (cy(q) == 1 && fy0) || (cy(q) == -1 && fy1);
-    const bool oz = (cz(q) == 1 && fz0) || (cz(q) == -1 && fz1);
-    const int up = i - (cz(q) * plane + cy(q) * pitch + cx(q));
-    if (!(ox || oy || oz)) {
-      d[q] = plus_ref(dec16(sq[up]), q, ref1(ref + up));
-      continue;
-    }
-    const int kx = ox ? int((fb >> (cx(q) == 1 ? 0 : 2)) & 3u) : int(BC_PERIODIC);
-    const int ky = oy ? int((fb >> (cy(q) == 1 ? 4 : 6)) & 3u) : int(BC_PERIODIC);
-    const int kz = oz ? int((fb >> (cz(q) == 1 ? 8 : 10)) & 3u) : int(BC_PERIODIC);
-    if (kx != BC_PERIODIC || ky != BC_PERIODIC || kz != BC_PERIODIC) {
-      const bool lid = kx == BC_LID || ky == BC_LID || kz == BC_LID;
-      const float v = plus_ref(dec16(src[int64_t(opp(q)) * qstride + i]), opp(q), ref1(ref + i));
-      d[q] = lid ? v + lidc[q] : v;
-    } else {
-      int j = up;
-      if (ox) j += cx(q) == 1 ? nx : -nx;
-      if (oy) j += cy(q) == 1 ? ny * pitch : -ny * pitch;
-      if (oz) j += cz(q) == 1 ? nz * plane : -nz * plane;
-      d[q] = plus_ref(dec16(sq[j]), q, ref1(ref + j));
-    }
+    const bool bounce = (f.wall & up_faces(q)) != 0;
+    const int j = bounce ? i : i - (cz(q) * plane + cy(q) * pitch + cx(q)) + up_wrap(f, q);
+    const __half v = (src + (bounce ? int64_t(opp(q)) * qstride : int64_t(q) * qstride))[j];
+    // a bounced value is decoded as opp(q): e_q . v changes sign
+    const float sgn = bounce ? -1.0f : 1.0f;
+    RefT<float> t = ref1(ref + j);
+    t = {t.dr, mulr(sgn, t.vx), mulr(sgn, t.vy), mulr(sgn, t.vz)};
+    d[q] = plus_ref(dec16(v), q, t);
+    if (f.lid & up_faces(q)) d[q] += lidc[q];
   }
+}
+
+// Pull of node (x, y, z) with index i: warps off every face load directly.
+__device__ __forceinline__ void pull_node_ref(const StepArgs<__half, float>& a, const RefArgs& r,
+                                              int x, int y, int z, int i, float (&d)[Q]) {
+  const bool inner = y > 0 && y < a.ny - 1 && z > 0 && z < a.nz - 1 && x > 0 && x < a.nx - 1;
+  if (__all_sync(__activemask(), inner)) {
+#pragma unroll
+    for (int q = 0; q < Q; ++q) d[q] = plus_ref(dec16(a.srcq[q][i]), q, ref1(r.refq[q] + i));
+  } else {
+    pull_face_ref(a.src, r.ref_src, a.qstride, a.nx, a.ny, a.nz, a.pitch, a.plane, a.facebits, x,
+                  y, z, i, a.lidc, d);
+  }
+}
+
+// Collide the node and store it.
+template <bool FORCE, bool UNIT>
+__device__ __forceinline__ void collide_store_ref(const StepArgs<__half, float>& a,
+                                                  const RefArgs& r, int i, unsigned step,
+                                                  float (&d)[Q], NodeOut<float>& o) {
+  collide<float, FORCE, !FORCE, LOG2LAM, UNIT>(a.C, d, o);
+  RefT<float> rr;
+  r.ref_dst[i] = ref_make(o.rho - a.C.rho0, o.rho, o.ux, o.uy, o.uz, rr);
+#pragma unroll
+  for (int q = 0; q < Q; ++q) d[q] = plus_ref(d[q], q, rr, -1.0f);
+  store_sr1([&](int q) { return a.dstq[q] + i; }, d, uint32_t(i), step);
 }
 
 // One node per thread.
@@ -119,47 +130,9 @@ __global__ void __launch_bounds__(256) step_ref_kernel(const StepArgs<__half, fl
   if (active) {
     const int i = z * a.plane + y * a.pitch + x;
     float d[Q];
-    if (y > 0 && y < a.ny - 1 && z > 0 && z < a.nz - 1) {
-      // One population and one reference load per direction: a lane on an x
-      // face takes, for the five directions that come from outside, the
-      // periodic wrap or the halfway bounce-back from its own opposite
-      // population, decoded with its own reference (the term of opp(q) is
-      // w_q (dr - e_q.v)), plus the lid term -- a select of the addresses,
-      // so that every lane issues the same loads.
-      const bool fl = x == 0, fr = x == a.nx - 1;
-      const int kl = a.facebits & 3, kr = (a.facebits >> 2) & 3;
-#pragma unroll
-      for (int q = 0; q < Q; ++q) {
-        const __half* pq = a.srcq[q] + i;
-        const uint2* rq = r.refq[q] + i;
-        float sgn = 1.0f, extra = 0.0f;
-        if ((cx(q) == 1 && fl) || (cx(q) == -1 && fr)) {
-          const int k = cx(q) == 1 ? kl : kr;
-          if (k == BC_PERIODIC) {
-            pq += cx(q) == 1 ? a.nx : -a.nx;
-            rq += cx(q) == 1 ? a.nx : -a.nx;
-          } else {
-            pq = a.src + int64_t(opp(q)) * a.qstride + i;
-            rq = r.ref_src + i;
-            sgn = -1.0f;
-            extra = k == BC_LID ? a.lidc[q] : 0.0f;
-          }
-        }
-        RefT<float> t = ref1(rq);
-        t = {t.dr, mulr(sgn, t.vx), mulr(sgn, t.vy), mulr(sgn, t.vz)};
-        d[q] = plus_ref(dec16(*pq), q, t) + extra;
-      }
-    } else {
-      pull_face_ref(a.src, r.ref_src, a.qstride, a.nx, a.ny, a.nz, a.pitch, a.plane, a.facebits,
-                    x, y, z, i, a.lidc, d);
-    }
+    pull_node_ref(a, r, x, y, z, i, d);
     NodeOut<float> o;
-    collide<float, FORCE, !FORCE, LOG2LAM, UNIT>(a.C, d, o);
-    RefT<float> rr;
-    r.ref_dst[i] = ref_make(o.rho - rho0, o.rho, o.ux, o.uy, o.uz, rr);
-#pragma unroll
-    for (int q = 0; q < Q; ++q) d[q] = plus_ref(d[q], q, rr, -1.0f);
-    store_sr1([&](int q) { return a.dstq[q] + i; }, d, uint32_t(i), r.step);
+    collide_store_ref<FORCE, UNIT>(a, r, i, r.step, d, o);
     if (CHECK) {
       float* up = reinterpret_cast<float*>(a.cb.uprev);
       const int64_t nst = int64_t(a.plane) * a.nz;
@@ -295,6 +268,19 @@ __global__ void collide_nodes_ref_kernel(CollideConst<float> C, const double* __
   if (gd) gd[k] = double(o.gamma_dot);
 }
 
+RefArgs ref_args(const void* ref_src, void* ref_dst, const Geom& g, unsigned step) {
+  RefArgs r;
+  r.step = step;
+  r.ref_src = static_cast<const uint2*>(ref_src);
+  r.ref_dst = static_cast<uint2*>(ref_dst);
+  for (int q = 0; q < Q; ++q) {
+    const int64_t off = int64_t(cz(q)) * g.plane + int64_t(cy(q)) * g.pitch + cx(q);
+    r.refq[q] = reinterpret_cast<const uint2*>(reinterpret_cast<uintptr_t>(ref_src) -
+                                                off * int64_t(sizeof(uint2)));
+  }
+  return r;
+}
+
 // Lid terms of the bounce-back, in the scaled deviations.
 void lid_table(const Geom& g, float* out) {
   for (int q = 0; q < Q; ++q)
@@ -317,31 +303,12 @@ __device__ void batch_node_ref(const LatDesc<float>& L, int parity, int x, int y
   const int qs = int(L.qstride), plane = L.plane, pitch = L.pitch;
   const int i = z * plane + y * pitch + x;
   float d[Q];
-  if (y > 0 && y < L.ny - 1 && z > 0 && z < L.nz - 1) {
-    // as in step_ref_kernel: one load of each kind per direction, x faces
-    // by a select
-    const bool fl = x == 0, fr = x == L.nx - 1;
-    const int kl = L.facebits & 3, kr = (L.facebits >> 2) & 3;
+  const bool inner = y > 0 && y < L.ny - 1 && z > 0 && z < L.nz - 1 && x > 0 && x < L.nx - 1;
+  if (__all_sync(__activemask(), inner)) {
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
       const int up = i - (cz(q) * plane + cy(q) * pitch + cx(q));
-      int j = q * qs + up, jr = up;
-      float sgn = 1.0f, extra = 0.0f;
-      if ((cx(q) == 1 && fl) || (cx(q) == -1 && fr)) {
-        const int k = cx(q) == 1 ? kl : kr;
-        if (k == BC_PERIODIC) {
-          j += cx(q) == 1 ? L.nx : -L.nx;
-          jr += cx(q) == 1 ? L.nx : -L.nx;
-        } else {
-          j = opp(q) * qs + i;
-          jr = i;
-          sgn = -1.0f;
-          extra = k == BC_LID ? L.lidc[q] : 0.0f;
-        }
-      }
-      RefT<float> t = ref1(rs + jr);
-      t = {t.dr, mulr(sgn, t.vx), mulr(sgn, t.vy), mulr(sgn, t.vz)};
-      d[q] = plus_ref(dec16(src[j]), q, t) + extra;
+      d[q] = plus_ref(dec16(src[q * qs + up]), q, ref1(rs + up));
     }
   } else {
     pull_face_ref(src, rs, L.qstride, L.nx, L.ny, L.nz, pitch, plane, L.facebits, x, y, z, i,
@@ -365,15 +332,7 @@ cudaError_t launch_step_f16r(const void* src, void* dst, const void* ref_src, vo
   if (unit && pair_pays(g, true))
     return launch_step_pair<PAIR_REF>(a, PairExtra{rs, rd, unsigned(uint64_t(step))},
                                       P.has_force != 0, check, block, st);
-  RefArgs r;
-  r.step = unsigned(uint64_t(step));
-  r.ref_src = rs;
-  r.ref_dst = rd;
-  for (int q = 0; q < Q; ++q) {
-    const int64_t off = int64_t(cz(q)) * g.plane + int64_t(cy(q)) * g.pitch + cx(q);
-    r.refq[q] = reinterpret_cast<const uint2*>(reinterpret_cast<uintptr_t>(rs) -
-                                                off * int64_t(sizeof(uint2)));
-  }
+  const RefArgs r = ref_args(rs, rd, g, unsigned(uint64_t(step)));
   const dim3 grid((g.nx + block.x - 1) / block.x, (g.ny + block.y - 1) / block.y, g.nz);
   void (*kernel)(const StepArgs<__half, float>, const RefArgs) = nullptr;
 #define CLBM_REF(F, C_) kernel = unit ? step_ref_kernel<F, C_, true> : step_ref_kernel<F, C_, false>

@@ -30,14 +30,7 @@ __global__ void __launch_bounds__(256) step_sr_kernel(const StepArgs<__half, flo
   if (active) {
     const int i = z * a.plane + y * a.pitch + x;
     float d[Q];
-    if (y > 0 && y < a.ny - 1 && z > 0 && z < a.nz - 1) {
-#pragma unroll
-      for (int q = 0; q < Q; ++q) d[q] = Codec<__half, float>::dec(a.srcq[q][i], 1.0f);
-      xface_fix(a, x, i, d);
-    } else {
-      pull_face<__half, float>(a.src, a.qstride, a.nx, a.ny, a.nz, a.pitch, a.plane, a.facebits,
-                               x, y, z, i, a.lidc, d);
-    }
+    pull_node(a, x, y, z, i, d);
     NodeOut<float> o;
     collide<float, FORCE, pair_out<__half>(), log2_scale<__half>(), UNIT>(a.C, d, o);
     // the deviations are carried scaled by 1024, as they are stored

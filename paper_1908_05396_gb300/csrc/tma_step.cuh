@@ -32,7 +32,7 @@
 #include <mutex>
 
 // Included by kernels.cuh after the step kernels (StepArgs, pull_face,
-// xface_fix, collide, pdl_enter) and before the host launchers.
+// collide, pdl_enter) and before the host launchers.
 
 namespace clbm {
 
