@@ -178,11 +178,8 @@ typedef void (*clbm_free_fn)(void* ptr, size_t bytes, int device, void* stream, 
 int clbm_set_allocator(clbm_alloc_fn alloc_fn, clbm_free_fn free_fn, void* user);
 
 /* Pick the launch shape of h's step kernel by timing: thread-block shapes
- * from 32x1 to 256x1 (and, for a lattice narrower than a warp, blocks 8 or
- * 16 wide) and, for FP32, one or two nodes per
- * thread (two nodes are collided together with packed FP32 instructions),
- * with and without a 64-register cap; for the two-buffer FP16 forms the
- * block's thread count; for FP32 and F16S storage also the
+ * from 8x4 to 256x1 with and without a 64-register cap; for the two-buffer
+ * FP16 forms the block's thread count; for FP32 and F16S storage also the
  * TMA-staged kernel in each of its shapes (see clbm_set_launch).
  * Each candidate runs `steps` steps (<= 0 -> 10) after two warm-up steps,
  * timed with CUDA events on the handle's stream; the state is saved first
@@ -202,12 +199,12 @@ int clbm_autotune(clbm_handle h, int steps, int* block_x, int* block_y, int* npt
  * memory by TMA loads, in shape v (block, nodes per thread): v = 0: 64x4, 1;
  * v = 1: 128x2, 1; v = 2: 32x8, 1; v = 3: 64x4, 1 (three ring stages);
  * v = 4: 32x4, 1; v = 5: 64x2, 1; v = 6: 64x2, 2; v = 7: 32x4, 2; v = 8:
- * 64x2, 2 (four CTAs per SM); v = 9: 128x1, 2.  With two nodes an FP32
- * lattice's thread collides rows 2y and 2y+1 as a packed FP32 pair.  The FP16
- * forms choose one or two nodes per thread themselves by the lattice's size
- * (two along x; npt = 2 makes F16S take two), and of the block they then use
- * the thread count only; the choice does not change results.  For the TMA
- * kernel block_x x block_y must be that shape's.  Check steps run
+ * 64x2, 2 (four CTAs per SM); v = 9: 128x1, 2 (rows 2y and 2y+1); its
+ * block_x x block_y must be that shape's.  npt = 2 is a wish: FP32 lattices
+ * step one node per thread, which is the faster way at every size; the FP16
+ * forms choose one or two by the lattice's size (two along x; npt = 2 makes
+ * F16S take two) and of the block then use the thread count only.  Neither
+ * changes the results.  Check steps run
  * the plain kernel with the same block.  If a pipeline wait of that kernel
  * gives up (about one second; never expected), the next check makes
  * clbm_step / clbm_residual return CLBM_ERR_CUDA. */

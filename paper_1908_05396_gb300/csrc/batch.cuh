@@ -172,8 +172,7 @@ __device__ __forceinline__ void batch_tiles(Get get, const int* __restrict__ own
     const S* src = static_cast<const S*>(L.buf[parity]);
     S* dst = static_cast<S*>(const_cast<void*>(L.buf[parity ^ 1]));
     const bool active = x < L.nx && y < L.ny;
-    double du2 = 0.0, uu = 0.0, dr = 0.0;
-    int bad = 0;
+    CheckSums sums;
     // the tile's zc planes: the per-tile work (table entries, descriptor,
     // checks, the check-step reductions) is shared by zc nodes per thread
     const int z1 = min(tz * zc + zc, L.nz);
@@ -184,41 +183,23 @@ __device__ __forceinline__ void batch_tiles(Get get, const int* __restrict__ own
           NodeOut<V2> o;
           batch_pair<FORCE, REF>(L, parity, x, y, z, bstep + L.step_offset, o);
           if (CHECK)
-            check_pair(o, L.C.rho0, static_cast<float*>(L.uprev), int64_t(L.plane) * L.nz,
-                       z * L.plane + y * L.pitch + x, x + 1 < L.nx, du2, uu, dr, bad);
+            check_pair(sums, o, L.C.rho0,
+                       static_cast<float*>(L.uprev) + (z * L.plane + y * L.pitch + x),
+                       int64_t(L.plane) * L.nz, x + 1 < L.nx);
           continue;
         }
         NodeOut<R> o;
         if constexpr (REF) batch_node_ref<FORCE>(L, parity, x, y, z, bstep + L.step_offset, o);
         else batch_node<S, R, FORCE, UNIT>(L, src, dst, x, y, z, bstep + L.step_offset, o);
-        if (CHECK) {
-          R* up = static_cast<R*>(L.uprev);
-          const int64_t nst = int64_t(L.plane) * L.nz;
-          const int64_t i = int64_t(z) * L.plane + int64_t(y) * L.pitch + x;
-          const R px = up[i], py = up[nst + i], pz = up[2 * nst + i];
-          up[i] = o.ux;
-          up[nst + i] = o.uy;
-          up[2 * nst + i] = o.uz;
-          const double ex = double(o.ux) - double(px), ey = double(o.uy) - double(py),
-                       ez = double(o.uz) - double(pz);
-          du2 += ex * ex + ey * ey + ez * ez;
-          uu += double(o.ux) * double(o.ux) + double(o.uy) * double(o.uy) +
-                double(o.uz) * double(o.uz);
-          dr += double(o.rho) - double(L.C.rho0);
-          const double chk = double(o.rho) + double(o.ux) + double(o.uy) + double(o.uz);
-          bad |= !(chk == chk) || !(fabs(chk) < 1e30) ||
-                 !(double(o.rho) > 0.5 && double(o.rho) < 2.0);
-        }
+        if (CHECK)
+          check_node(sums, o.rho, o.ux, o.uy, o.uz, L.C.rho0,
+                     static_cast<R*>(L.uprev) + (z * L.plane + y * L.pitch + x),
+                     int64_t(L.plane) * L.nz);
       }
     }
     if (CHECK) {
-      __shared__ double smem[32];
-      double* a = acc + 4 * L.slot;
-      block_sum_add(du2, &a[0], smem);
-      block_sum_add(uu, &a[1], smem);
-      block_sum_add(dr, &a[2], smem);
-      if (__syncthreads_or(bad) && threadIdx.x == 0 && threadIdx.y == 0)
-        atomicOr(reinterpret_cast<int*>(&a[3]), 1);
+      double* a = acc + 4 * BATCH_ROWS * L.slot;
+      block_sums(sums, a + 4 * (t & (BATCH_ROWS - 1)), reinterpret_cast<int*>(a + 3));
     }
   }
   if constexpr (STEPS) {

@@ -51,7 +51,7 @@ struct clbm_batch_ctx {
   unsigned* d_coord = nullptr;        // tile -> packed tile coordinates
   int owner_cap = 0;
   BatchHeader* d_hdr = nullptr;
-  double* d_acc = nullptr;            // capacity x 4
+  double* d_acc = nullptr;            // capacity x BATCH_ROWS x 4
   double* h_acc = nullptr;            // pinned copy
   void* h_stage = nullptr;            // pinned staging of descriptors
   std::vector<int> h_owner;
@@ -96,6 +96,11 @@ int bfail(clbm_batch_ctx* b, int code, const std::string& m) {
       return bfail(b, e_ == cudaErrorMemoryAllocation ? CLBM_ERR_OOM : CLBM_ERR_CUDA,        \
                    std::string(#expr) + ": " + cudaGetErrorString(e_));                      \
   } while (0)
+
+// Bytes of the check sums of all slots.
+size_t acc_bytes(const clbm_batch_ctx* b) {
+  return size_t(b->capacity) * BATCH_ROWS * 4 * sizeof(double);
+}
 
 size_t desc_size(clbm_dtype t) {
   return t == CLBM_F64   ? desc_size_f64()
@@ -273,8 +278,8 @@ cudaError_t launch_lattices(clbm_batch_ctx* b, bool check, int flip) {
   for (int s = 0; s < b->capacity; ++s) {
     clbm_ctx* h = b->slots[size_t(s)];
     if (!h) continue;
-    double* acc = b->d_acc + 4 * size_t(s);
-    CheckBufs cb{h->uprev, acc, reinterpret_cast<int*>(acc + 3)};
+    double* acc = b->d_acc + 4 * BATCH_ROWS * size_t(s);
+    CheckBufs cb{h->uprev, acc, reinterpret_cast<int*>(acc + 3), BATCH_ROWS};
     const cudaStream_t st = pl_stream(b, b->stream_of[size_t(s)]);
     // the lattice's own block: the tile width of the persistent kernel's rule
     const int threads = int(b->pl_block.x * b->pl_block.y);
@@ -417,7 +422,7 @@ void advance(clbm_batch_ctx* b, int64_t n) {
 
 int one_step(clbm_batch_ctx* b) {
   const bool check = ((b->steps + 1) % b->check_interval) == 0;
-  if (check) BCK(b, cudaMemsetAsync(b->d_acc, 0, size_t(b->capacity) * 4 * sizeof(double), b->stream));
+  if (check) BCK(b, cudaMemsetAsync(b->d_acc, 0, acc_bytes(b), b->stream));
   if (b->mode == 1) {
     BCK(b, fork_streams(b, b->pl_streams));
     BCK(b, launch_lattices(b, check, 0));
@@ -429,7 +434,7 @@ int one_step(clbm_batch_ctx* b) {
   }
   b->parity ^= 1;
   if (check) {
-    BCK(b, cudaMemcpyAsync(b->h_acc, b->d_acc, size_t(b->capacity) * 4 * sizeof(double),
+    BCK(b, cudaMemcpyAsync(b->h_acc, b->d_acc, acc_bytes(b),
                            cudaMemcpyDeviceToHost, b->stream));
     BCK(b, cudaEventRecord(b->check_done, b->stream));
     for (int s = 0; s < b->capacity; ++s)
@@ -448,20 +453,20 @@ int capture(clbm_batch_ctx* b) {
   if (b->mode == 1) {
     // Only the last step's check writes the sums: clear them up front, so
     // that the streams stay forked for the whole interval.
-    e = cudaMemsetAsync(b->d_acc, 0, size_t(b->capacity) * 4 * sizeof(double), b->stream);
+    e = cudaMemsetAsync(b->d_acc, 0, acc_bytes(b), b->stream);
     if (e == cudaSuccess) e = fork_streams(b, b->pl_streams);
     for (int k = 0; k < b->check_interval && e == cudaSuccess; ++k)
       e = launch_lattices(b, k == b->check_interval - 1, k & 1);
     if (e == cudaSuccess) e = join_streams(b, b->pl_streams);
     if (e == cudaSuccess)
-      e = cudaMemcpyAsync(b->h_acc, b->d_acc, size_t(b->capacity) * 4 * sizeof(double),
+      e = cudaMemcpyAsync(b->h_acc, b->d_acc, acc_bytes(b),
                           cudaMemcpyDeviceToHost, b->stream);
     if (e == cudaSuccess) e = cudaEventRecord(b->check_done, b->stream);
   }
   if (b->mode == 0) {
     // as in mode 1: the sums are cleared up front, so that the two chains stay
     // forked for the whole interval
-    e = cudaMemsetAsync(b->d_acc, 0, size_t(b->capacity) * 4 * sizeof(double), b->stream);
+    e = cudaMemsetAsync(b->d_acc, 0, acc_bytes(b), b->stream);
     if (e == cudaSuccess) e = fork_streams(b, 2);
     const int keep = b->parity;
     for (int k = 0; k < b->check_interval && e == cudaSuccess; ++k) {
@@ -471,7 +476,7 @@ int capture(clbm_batch_ctx* b) {
     b->parity = keep;
     if (e == cudaSuccess) e = join_streams(b, 2);
     if (e == cudaSuccess)
-      e = cudaMemcpyAsync(b->h_acc, b->d_acc, size_t(b->capacity) * 4 * sizeof(double),
+      e = cudaMemcpyAsync(b->h_acc, b->d_acc, acc_bytes(b),
                           cudaMemcpyDeviceToHost, b->stream);
     if (e == cudaSuccess) e = cudaEventRecord(b->check_done, b->stream);
   }
@@ -493,7 +498,11 @@ bool valid(const clbm_batch_ctx* b) { return b && b->d_desc; }
 // this batch), mass, divergence flag, steps.
 void slot_stats(const clbm_batch_ctx* b, int slot, double* residual, double* mass,
                 int* diverged, int64_t* steps) {
-  const double* a = b->h_acc + 4 * slot;
+  // BATCH_ROWS rows of sums; the flag sits in the first row's fourth entry
+  const double* rows = b->h_acc + 4 * BATCH_ROWS * size_t(slot);
+  double a[4] = {0.0, 0.0, 0.0, rows[3]};
+  for (int r = 0; r < BATCH_ROWS; ++r)
+    for (int k = 0; k < 3; ++k) a[k] += rows[4 * r + k];
   const clbm_ctx* h = b->slots[size_t(slot)];
   if (residual) {
     if (b->slot_checks[size_t(slot)] < 2) *residual = INFINITY;
@@ -562,12 +571,12 @@ int clbm_batch_create(clbm_dtype dtype, int capacity, int check_interval, void* 
   }
   if (e == cudaSuccess) e = cudaMalloc(&b->d_desc, 256);
   if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&b->d_hdr), sizeof(BatchHeader));
-  if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&b->d_acc), size_t(capacity) * 4 * sizeof(double));
-  if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&b->h_acc), size_t(capacity) * 4 * sizeof(double));
+  if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&b->d_acc), acc_bytes(b));
+  if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&b->h_acc), acc_bytes(b));
   if (e == cudaSuccess) e = cudaMallocHost(&b->h_stage, size_t(capacity) * b->desc_bytes);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->check_done, cudaEventDisableTiming);
   if (e == cudaSuccess) e = ensure_streams(b, 2);  // the forced lattices' chain
-  if (e == cudaSuccess) std::memset(b->h_acc, 0, size_t(capacity) * 4 * sizeof(double));
+  if (e == cudaSuccess) std::memset(b->h_acc, 0, acc_bytes(b));
   if (e != cudaSuccess) {
     std::string m = std::string("clbm_batch_create: ") + cudaGetErrorString(e);
     clbm_batch_destroy(b);

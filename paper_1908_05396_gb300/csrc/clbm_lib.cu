@@ -85,7 +85,7 @@ void dev_free(clbm_ctx* h, void* p, size_t bytes) {
 int64_t round_up(int64_t v, int64_t m) { return (v + m - 1) / m * m; }
 
 cudaError_t dispatch_step(clbm_ctx* h, bool check) {
-  CheckBufs cb{h->uprev, h->acc, h->flag};
+  CheckBufs cb{h->uprev, h->acc, h->flag, CHECK_ROWS};
   if (h->in_place) {
     const int npt = h->npt & 4 ? 5 : 1;
     switch (h->dtype) {
@@ -108,6 +108,14 @@ cudaError_t dispatch_step(clbm_ctx* h, bool check) {
                                  h->stream);
       return launch_step_f16(src, dst, h->g, h->P, cb, check, h->block, h->npt, h->stream);
   }
+}
+
+// Sum k of the last completed check step: 0 sum|u - u_prev|^2, 1 sum|u|^2,
+// 2 sum(rho - rho0).
+double check_sum(const clbm_ctx* h, int k) {
+  double s = 0.0;
+  for (int r = 0; r < CHECK_ROWS; ++r) s += h->host[4 * r + k];
+  return s;
 }
 
 // After a step: the other buffer holds the state, or (in place) the buffer
@@ -231,13 +239,12 @@ int clbm_create(const clbm_domain* d, double K, double n, const double U_lid[3],
   }
   rc = dev_alloc(h, &h->uprev, h->uprev_bytes, "velocity buffer");
   if (rc != CLBM_OK) return cleanup(rc, "clbm_create");
-  // acc: 3 FP64 sums, then the divergence flag and the TMA error word
-  rc = dev_alloc(h, reinterpret_cast<void**>(&h->acc), 4 * sizeof(double), "reduction buffer");
+  rc = dev_alloc(h, reinterpret_cast<void**>(&h->acc), CHECK_BYTES, "reduction buffer");
   if (rc != CLBM_OK) return cleanup(rc, "clbm_create");
-  h->flag = reinterpret_cast<int*>(h->acc + 3);
-  e = cudaMallocHost(&h->host, 4 * sizeof(double));
+  h->flag = reinterpret_cast<int*>(h->acc + 4 * CHECK_ROWS);
+  e = cudaMallocHost(&h->host, CHECK_BYTES);
   if (e != cudaSuccess) return cleanup(CLBM_ERR_OOM, "pinned buffer allocation failed");
-  std::memset(h->host, 0, 4 * sizeof(double));
+  std::memset(h->host, 0, CHECK_BYTES);
   e = cudaEventCreateWithFlags(&h->check_done, cudaEventDisableTiming);
   if (e != cudaSuccess) return cleanup(CLBM_ERR_CUDA, cudaGetErrorString(e));
   // Rest state: stored deviation f - w rho0 = 0 (all-zero bits in every form).
@@ -246,7 +253,7 @@ int clbm_create(const clbm_domain* d, double K, double n, const double U_lid[3],
     if (e != cudaSuccess) return cleanup(CLBM_ERR_CUDA, cudaGetErrorString(e));
   }
   e = cudaMemsetAsync(h->uprev, 0, 3 * size_t(g.plane) * g.nz * h->rsize, h->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(h->acc, 0, 4 * sizeof(double), h->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(h->acc, 0, CHECK_BYTES, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return cleanup(CLBM_ERR_CUDA, cudaGetErrorString(e));
   *out = h;
@@ -261,20 +268,19 @@ int clbm_step(clbm_handle h, int64_t nsteps) {
   const int64_t every = h->dom.check_interval;
   for (int64_t s = 0; s < nsteps; ++s) {
     const bool check = ((h->steps + 1) % every) == 0;
-    if (check) CK(h, cudaMemsetAsync(h->acc, 0, 3 * sizeof(double), h->stream));
+    if (check) CK(h, cudaMemsetAsync(h->acc, 0, CHECK_SUMS_BYTES, h->stream));
     CK(h, dispatch_step(h, check));
     advance_state(h);
     h->steps += 1;
     if (check) {
       h->checks += 1;
-      CK(h, cudaMemcpyAsync(h->host, h->acc, 4 * sizeof(double), cudaMemcpyDeviceToHost,
-                            h->stream));
+      CK(h, cudaMemcpyAsync(h->host, h->acc, CHECK_BYTES, cudaMemcpyDeviceToHost, h->stream));
       CK(h, cudaEventRecord(h->check_done, h->stream));
     }
   }
   if (!h->diverged && h->checks > 0 && cudaEventQuery(h->check_done) == cudaSuccess) {
     int f[2] = {0, 0};
-    std::memcpy(f, &h->host[3], sizeof(f));
+    std::memcpy(f, &h->host[4 * CHECK_ROWS], sizeof(f));
     h->diverged = f[0] != 0;
     h->pipeline_err = h->pipeline_err || f[1] != 0;
   }
@@ -346,13 +352,13 @@ int clbm_residual(clbm_handle h, double* out) {
   CK(h, cudaStreamSynchronize(h->stream));
   if (h->checks < 2) {
     *out = INFINITY;
-  } else if (!(h->host[1] > 0.0)) {
-    *out = h->host[0] == 0.0 ? 0.0 : INFINITY;   // fluid at rest
   } else {
-    *out = std::sqrt(h->host[0]) / (double(h->dom.check_interval) * std::sqrt(h->host[1]));
+    const double du2 = check_sum(h, 0), uu = check_sum(h, 1);
+    if (!(uu > 0.0)) *out = du2 == 0.0 ? 0.0 : INFINITY;  // fluid at rest
+    else *out = std::sqrt(du2) / (double(h->dom.check_interval) * std::sqrt(uu));
   }
   int f[2] = {0, 0};
-  std::memcpy(f, &h->host[3], sizeof(f));
+  std::memcpy(f, &h->host[4 * CHECK_ROWS], sizeof(f));
   h->diverged = h->diverged || f[0] != 0;
   h->pipeline_err = h->pipeline_err || f[1] != 0;
   if (h->pipeline_err)
@@ -368,7 +374,7 @@ int clbm_mass(clbm_handle h, double* out) {
   CK(h, cudaStreamSynchronize(h->stream));
   if (h->checks < 1) return fail(h, CLBM_ERR_ARG, "no check step has run yet");
   const double N = double(h->g.nx) * h->g.ny * h->g.nz;
-  *out = N * h->g.rho0 + h->host[2];
+  *out = N * h->g.rho0 + check_sum(h, 2);
   return CLBM_OK;
 }
 
@@ -483,12 +489,10 @@ int clbm_autotune(clbm_handle h, int steps, int* block_x, int* block_y, int* npt
   if (pair)
     for (int t : {32, 64, 128, 256}) cands.push_back({32, t / 32, 1});
   for (int capped = 0; capped <= 1 && !pair; ++capped)
-    for (int np = 1; np <= ((h->dtype == CLBM_F64 || h->dtype == CLBM_F16R || h->in_place || h->sround) ? 1 : 2); ++np)
-      for (auto& sh : shapes) {
-        if (sh[0] * sh[1] > (np == 2 ? 128 : 256)) continue;
-        if (sh[0] > 32 && sh[0] > h->g.pitch) continue;
-        cands.push_back({sh[0], sh[1], np + 4 * capped});
-      }
+    for (auto& sh : shapes) {
+      if (sh[0] > 32 && sh[0] > h->g.pitch) continue;
+      cands.push_back({sh[0], sh[1], 1 + 4 * capped});
+    }
   // a lattice narrower than a warp: blocks as wide as its tile width
   const int tw = tile_width(h->g.nx, int(h->elem), 32, 64);
   if (tw < 32 && !pair)
@@ -645,7 +649,7 @@ int clbm_destroy(clbm_handle h) {
     dev_free(h, h->ref[b], h->ref_bytes);
   }
   dev_free(h, h->uprev, h->uprev_bytes);
-  dev_free(h, h->acc, 4 * sizeof(double));
+  dev_free(h, h->acc, CHECK_BYTES);
   if (h->host) cudaFreeHost(h->host);
   if (h->check_done) cudaEventDestroy(h->check_done);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);

@@ -177,6 +177,16 @@ __device__ __forceinline__ double widen(float x) {
   return __hiloint2double(int(hi | (b & 0x80000000u)), int(b << 29));
 }
 
+// double(x) for the FP64 sums and outputs of the FP32-math forms: integer
+// operations for zero and normal values, the hardware's conversion otherwise.
+__device__ __forceinline__ double to64(double x) { return x; }
+__device__ __forceinline__ double to64(float x) {
+  const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+  if (m - 0x00800000u < 0x7f000000u) return widen(x);
+  if (m == 0u) return __hiloint2double(int(b), 0);
+  return double(x);
+}
+
 // A non-negative double truncated to float; zero and values below 2^-125 give 2^-125.
 __device__ __forceinline__ float narrow(double x) {
   const int hi = __double2hiint(x);
@@ -985,6 +995,49 @@ __device__ __forceinline__ void collide_unit(const CollideConst<typename ScalarO
   out.uy = uy;
   out.uz = uz;
   out.gamma_dot = shear_rate(rinv, w, A, B);
+}
+
+// rho, u and, when want_gd, |gamma_dot| of a node without colliding it, for
+// any rates (only omega_9 enters).  d holds the pre-collision deviations.
+template <typename R, bool FORCE, int LOG2LAM>
+__device__ __forceinline__ void node_fields(const CollideConst<R>& C, const R (&d)[Q],
+                                            bool want_gd, NodeOut<R>& out) {
+  const Pairs<R> p = to_pairs(d);
+  const R Dxx = p.sAx + (p.Dxxyy + p.Dxxzz), Dyy = p.sAy + (p.Dxxyy + p.Dyyzz),
+          Dzz = p.sAz + (p.Dxxzz + p.Dyyzz);
+  const R drho = (p.d0 + Dxx) + ((p.sAy + p.sAz) + p.Dyyzz);
+  R Jx = p.tAx + (p.Dxyy + p.Dxzz), Jy = p.tAy + (p.Dxxy + p.Dyzz),
+    Jz = p.tAz + (p.Dxxz + p.Dyyz);
+  const R rho = C.rhoS + drho;
+  const R rinv = rrcp<R>(rho);
+  if (FORCE) {
+    Jx = Jx + R(0.5) * C.FS[0];
+    Jy = Jy + R(0.5) * C.FS[1];
+    Jz = Jz + R(0.5) * C.FS[2];
+  }
+  const R ux = mulr(Jx, rinv), uy = mulr(Jy, rinv), uz = mulr(Jz, rinv);
+  if (LOG2LAM != 0) out.rho = mulr(rho, R(1.0 / double(1 << LOG2LAM)));
+  else out.rho = rho;
+  out.ux = ux;
+  out.uy = uy;
+  out.uz = uz;
+  if (!want_gd) return;
+  R hxx = Dxx, hyy = Dyy, hzz = Dzz, hxy = p.Dxy, hxz = p.Dxz, hyz = p.Dyz;
+  if (FORCE) {  // half of the source, as in collide_unit
+    const R hFx = R(0.5) * C.FS[0], hFy = R(0.5) * C.FS[1], hFz = R(0.5) * C.FS[2];
+    hxx = fma(ux, C.FS[0], hxx);
+    hyy = fma(uy, C.FS[1], hyy);
+    hzz = fma(uz, C.FS[2], hzz);
+    hxy = fma(ux, hFy, fma(uy, hFx, hxy));
+    hxz = fma(ux, hFz, fma(uz, hFx, hxz));
+    hyz = fma(uy, hFz, fma(uz, hFy, hyz));
+  }
+  const R sx = fma(-Jx, ux, hxx), sy = fma(-Jy, uy, hyy), sz = fma(-Jz, uz, hzz);
+  const R tr = (sx + sy) + sz;
+  R A, B;
+  strain_AB(C, fma(-Jx, uy, hxy), fma(-Jx, uz, hxz), fma(-Jy, uz, hyz), sx - sy, sx - sz,
+            tr - drho, A, B);
+  out.gamma_dot = shear_rate(rinv, omega_nu(C, rho, rinv, A, B), A, B);
 }
 
 // UNIT: the rates omega_9..18 are all 1 (PhysParams::unit_rates).

@@ -29,9 +29,11 @@ struct clbm_ctx {
   bool sround = false;   // F16S: stores rounded stochastically (step_f16sr.cu)
   int layout = 0;        // in place: the layout the buffer holds (0 swapped, 1 streamed)
   void* uprev = nullptr;
-  double* acc = nullptr; // device: 3 doubles, then the int flag and the TMA error word
+  // device: CHECK_ROWS rows of 4 doubles (three sums of a check step each), then
+  // the int flag and the TMA error word; host: its pinned copy
+  double* acc = nullptr;
   int* flag = nullptr;
-  double* host = nullptr; // pinned: acc[3], flag as double
+  double* host = nullptr;
   cudaEvent_t check_done = nullptr;
   cudaStream_t stream = nullptr;
   bool own_stream = false;
@@ -51,6 +53,9 @@ struct clbm_ctx {
 };
 
 namespace clbm {
+constexpr size_t CHECK_SUMS_BYTES = size_t(CHECK_ROWS) * 4 * sizeof(double);
+constexpr size_t CHECK_BYTES = CHECK_SUMS_BYTES + sizeof(double);  // and the two flag words
+
 // Queue one step of a handle (clbm_lib.cu).
 cudaError_t handle_dispatch_step(clbm_ctx* h, bool check);
 }  // namespace clbm

@@ -91,67 +91,33 @@ __global__ void __launch_bounds__(256, CAP ? 4 : 1) step_aa_kernel(const StepArg
   const int z = blockIdx.z;
   const bool active = x < a.nx && y < a.ny;
   if (!CHECK && !active) return;
-  double du2 = 0.0, uu = 0.0, dr = 0.0;
-  int bad = 0;
+  CheckSums sums;
   if (active) {
     const int i = z * a.plane + y * a.pitch + x;
     NodeOut<R> o;
     aa_update<S, R, LIN, FORCE, UNIT>(a, x, y, z, i, o);
-    if (CHECK) {
-      R* up = reinterpret_cast<R*>(a.cb.uprev);
-      const int64_t nst = int64_t(a.plane) * a.nz;
-      const R px = up[i], py = up[nst + i], pz = up[2 * nst + i];
-      up[i] = o.ux;
-      up[nst + i] = o.uy;
-      up[2 * nst + i] = o.uz;
-      const double ex = double(o.ux) - double(px), ey = double(o.uy) - double(py),
-                   ez = double(o.uz) - double(pz);
-      du2 = ex * ex + ey * ey + ez * ez;
-      uu = double(o.ux) * double(o.ux) + double(o.uy) * double(o.uy) +
-           double(o.uz) * double(o.uz);
-      dr = double(o.rho) - double(a.C.rho0);
-      const double chk = double(o.rho) + double(o.ux) + double(o.uy) + double(o.uz);
-      bad = !(chk == chk) || !(fabs(chk) < 1e30) || !(double(o.rho) > 0.5 && double(o.rho) < 2.0);
-    }
+    if (CHECK)
+      check_node(sums, o.rho, o.ux, o.uy, o.uz, a.C.rho0, static_cast<R*>(a.cb.uprev) + i,
+                 int64_t(a.plane) * a.nz);
   }
-  if (CHECK) {
-    __shared__ double smem[32];
-    block_sum_add(du2, &a.cb.acc[0], smem);
-    block_sum_add(uu, &a.cb.acc[1], smem);
-    block_sum_add(dr, &a.cb.acc[2], smem);
-    if (__syncthreads_or(bad) && threadIdx.x == 0 && threadIdx.y == 0) atomicOr(a.cb.flag, 1);
-  }
+  if (CHECK) block_sums(sums, check_row(a.cb), a.cb.flag);
 }
 
 // rho, u and |gamma_dot| of the next collision, from either layout.
 template <typename S, typename R, int L, bool FORCE>
-__global__ void __launch_bounds__(256) fields_aa_kernel(const S* __restrict__ A, Geom g,
-                                                        CollideConst<R> C, double* rho,
-                                                        double* u, double* gd) {
+__global__ void __launch_bounds__(256) fields_aa_kernel(const StepArgs<S, R> a,
+                                                        const FieldsOut f) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z;
-  if (x >= g.nx || y >= g.ny) return;
-  R lidc[Q];
-#pragma unroll
-  for (int q = 0; q < Q; ++q)
-    lidc[q] = R(6.0 * wt<double>(q) * g.rho0 * double(1 << log2_scale<S>()) *
-                (cx(q) * g.U[0] + cy(q) * g.U[1] + cz(q) * g.U[2]));
-  const int i = z * int(g.plane) + y * g.pitch + x;
+  if (x >= a.nx || y >= a.ny) return;
+  const int i = z * a.plane + y * a.pitch + x;
   R d[Q];
-  aa_read<S, R, L>(A, g.qstride, i, g.pitch, int(g.plane),
-                   faces_of(x, y, z, g.nx, g.ny, g.nz, g.pitch, int(g.plane), g.facebits), lidc, d);
+  aa_read<S, R, L>(a.src, a.qstride, i, a.pitch, a.plane,
+                   faces_of(x, y, z, a.nx, a.ny, a.nz, a.pitch, a.plane, a.facebits), a.lidc, d);
   NodeOut<R> o;
-  collide<R, FORCE, pair_out<S>(), log2_scale<S>(), false>(C, d, o);
-  const int64_t N = int64_t(g.nx) * g.ny * g.nz;
-  const int64_t k = (int64_t(z) * g.ny + y) * g.nx + x;
-  if (rho) rho[k] = double(o.rho);
-  if (u) {
-    u[k] = double(o.ux);
-    u[N + k] = double(o.uy);
-    u[2 * N + k] = double(o.uz);
-  }
-  if (gd) gd[k] = double(o.gamma_dot);
+  node_fields<R, FORCE, log2_scale<S>()>(a.C, d, f.gd != nullptr, o);
+  write_fields(f, o, a.nx, a.ny, a.nz, x, y, z);
 }
 
 // The post-collision populations f~_q(x) (the state the two-buffer form
@@ -248,14 +214,14 @@ cudaError_t launch_fields_aa_t(const void* buf, const Geom& g, const PhysParams&
                                double* rho, double* u, double* gd, cudaStream_t st) {
   const dim3 block(32, 4);
   const dim3 grid((g.nx + 31) / 32, (g.ny + 3) / 4, g.nz);
-  const S* A = static_cast<const S*>(buf);
-  const CollideConst<R> C = make_const<R>(P, double(1 << log2_scale<S>()));
+  const StepArgs<S, R> a = step_args<S, R>(buf, nullptr, g, P, CheckBufs{});
+  const FieldsOut f{rho, u, gd};
   if (layout == 0) {
-    if (P.has_force) fields_aa_kernel<S, R, 0, true><<<grid, block, 0, st>>>(A, g, C, rho, u, gd);
-    else fields_aa_kernel<S, R, 0, false><<<grid, block, 0, st>>>(A, g, C, rho, u, gd);
+    if (P.has_force) fields_aa_kernel<S, R, 0, true><<<grid, block, 0, st>>>(a, f);
+    else fields_aa_kernel<S, R, 0, false><<<grid, block, 0, st>>>(a, f);
   } else {
-    if (P.has_force) fields_aa_kernel<S, R, 1, true><<<grid, block, 0, st>>>(A, g, C, rho, u, gd);
-    else fields_aa_kernel<S, R, 1, false><<<grid, block, 0, st>>>(A, g, C, rho, u, gd);
+    if (P.has_force) fields_aa_kernel<S, R, 1, true><<<grid, block, 0, st>>>(a, f);
+    else fields_aa_kernel<S, R, 1, false><<<grid, block, 0, st>>>(a, f);
   }
   return cudaGetLastError();
 }

@@ -104,69 +104,76 @@ inline CollideConst<R> make_const(const PhysParams& P, double lam = 1.0) {
   return C;
 }
 
-// Pull the 19 pre-collision deviations of node (x, y, z).
-template <typename S, typename R>
-__device__ __forceinline__ void pull(const S* __restrict__ src, const Geom& g,
-                                     int x, int y, int z, int64_t i, R lam,
-                                     R (&d)[Q]) {
-  const bool interior = x > 0 && x < g.nx - 1 && y > 0 && y < g.ny - 1 &&
-                        z > 0 && z < g.nz - 1;
-  if (interior) {
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      const int64_t off = int64_t(cz(q)) * g.plane + int64_t(cy(q)) * g.pitch + cx(q);
-      d[q] = Codec<S, R>::dec(src[q * g.qstride + i - off], lam);
-    }
-    return;
-  }
-#pragma unroll
-  for (int q = 0; q < Q; ++q) {
-    int s[3] = {x - cx(q), y - cy(q), z - cz(q)};
-    const int n3[3] = {g.nx, g.ny, g.nz};
-    bool bounce = false, lid = false;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      if (s[a] < 0 || s[a] >= n3[a]) {
-        const int kind = (g.facebits >> (2 * (2 * a + (s[a] < 0 ? 0 : 1)))) & 3;
-        if (kind == BC_PERIODIC) {
-          s[a] += (s[a] < 0) ? n3[a] : -n3[a];
-        } else {
-          bounce = true;
-          lid = lid || kind == BC_LID;
-        }
-      }
-    }
-    if (bounce) {
-      // Halfway bounce-back f_q(x) = f~_opp(q)(x); a lid adds
-      // 6 w_q rho0 (e_q . U), which is the same for deviations.
-      R v = Codec<S, R>::dec(src[opp(q) * g.qstride + i], lam);
-      if (lid)
-        v += lam * R(6) * wt<R>(q) * R(g.rho0) *
-             (R(cx(q)) * R(g.U[0]) + R(cy(q)) * R(g.U[1]) + R(cz(q)) * R(g.U[2]));
-      d[q] = v;
-    } else {
-      const int64_t j = int64_t(s[2]) * g.plane + int64_t(s[1]) * g.pitch + s[0];
-      d[q] = Codec<S, R>::dec(src[q * g.qstride + j], lam);
-    }
-  }
+// ---- check-step sums ----------------------------------------------------------
+// FP64 instructions run at 1/64 of the FP32 rate, so a check step spends as few
+// as it can: conversions are integer operations (to64), the finiteness test is
+// made in the math type, and a warp's three sums share their reduction steps.
+// The blocks' sums go to CheckBufs::rows rows, so that no address takes more
+// than a few hundred atomic additions.  With one row, a tree per sum and the
+// hardware's conversions a check step of 128^3 took 247 us in FP32, 211 in F16S
+// and 162 in F16R, against 100, 76 and 88 now (a plain step: 47, 31 and 56).
+
+// A node's part of the sums over the lattice, in FP64: sum|u - u_prev|^2,
+// sum|u|^2, sum(rho - rho0), and whether the node diverged.
+struct CheckSums {
+  double du2 = 0.0, uu = 0.0, dr = 0.0;
+  int bad = 0;
+};
+
+// Adds a node with the results (rho, u); up points at the node's x velocity of
+// the previous check (components nst apart), which is replaced.
+template <typename R>
+__device__ __forceinline__ void check_node(CheckSums& s, R rho, R ux, R uy, R uz, R rho0, R* up,
+                                           int64_t nst) {
+  const R px = up[0], py = up[nst], pz = up[2 * nst];
+  up[0] = ux;
+  up[nst] = uy;
+  up[2 * nst] = uz;
+  const double x = to64(ux), y = to64(uy), z = to64(uz);
+  const double ex = x - to64(px), ey = y - to64(py), ez = z - to64(pz);
+  s.du2 = fma(ex, ex, fma(ey, ey, fma(ez, ez, s.du2)));
+  s.uu = fma(x, x, fma(y, y, fma(z, z, s.uu)));
+  s.dr += to64(rho) - to64(rho0);
+  s.bad |= !(rho > R(0.5) && rho < R(2.0)) || !(fabs(ux) < R(1e30)) || !(fabs(uy) < R(1e30)) ||
+           !(fabs(uz) < R(1e30));
 }
 
-// Block-wide FP64 sum of v, added atomically to *acc by one thread.
-__device__ __forceinline__ void block_sum_add(double v, double* acc, double* smem) {
+// The warp's three sums: du2 in lane 0, uu in lane 16, dr in lane 8.  The
+// first two exchanges each fold two quantities into the halves of the warp.
+__device__ __forceinline__ double warp_sums(const CheckSums& s) {
+  constexpr unsigned ALL = 0xffffffffu;
+  const int lane = int(threadIdx.x + threadIdx.y * blockDim.x) & 31;
+  const bool h = lane & 16, o = lane & 8;
+  const double a = (h ? s.uu : s.du2) + __shfl_xor_sync(ALL, h ? s.du2 : s.uu, 16);
+  const double b = s.dr + __shfl_xor_sync(ALL, s.dr, 16);
+  double c = (o ? b : a) + __shfl_xor_sync(ALL, o ? a : b, 8);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  const int lane = (threadIdx.y * blockDim.x + threadIdx.x) & 31;
-  const int warp = (threadIdx.y * blockDim.x + threadIdx.x) >> 5;
-  const int nwarp = (blockDim.x * blockDim.y + 31) >> 5;
-  if (lane == 0) smem[warp] = v;
-  __syncthreads();
-  if (warp == 0) {
-    v = (lane < nwarp) ? smem[lane] : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) atomicAdd(acc, v);
+  for (int k = 4; k > 0; k >>= 1) c += __shfl_xor_sync(ALL, c, k);
+  return c;
+}
+
+// Adds the block's sums to a row of acc (4 doubles a row: the three sums) and
+// raises the flag if a node diverged.  Called by every thread of the block.
+__device__ __forceinline__ void block_sums(const CheckSums& s, double* row, int* flag) {
+  __shared__ double sm[8][3];
+  const int t = int(threadIdx.x + threadIdx.y * blockDim.x), lane = t & 31, warp = t >> 5;
+  const double v = warp_sums(s);
+  if (lane == 0) sm[warp][0] = v;
+  if (lane == 16) sm[warp][1] = v;
+  if (lane == 8) sm[warp][2] = v;
+  const int bad = __syncthreads_or(s.bad);
+  if (t < 3) {
+    double a = sm[0][t];
+    for (int w = 1; w < int(blockDim.x * blockDim.y) >> 5; ++w) a += sm[w][t];
+    atomicAdd(row + t, a);
   }
+  if (t == 0 && bad) atomicOr(flag, 1);
   __syncthreads();
+}
+// The row of a block of a lone lattice's check step.
+__device__ __forceinline__ double* check_row(const CheckBufs& cb) {
+  const unsigned blk = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+  return cb.acc + 4 * (blk & unsigned(cb.rows - 1));
 }
 
 // ---- the fused step ---------------------------------------------------------
@@ -331,8 +338,7 @@ __global__ void __launch_bounds__(256, CAP ? 4 : 1) step_kernel(const StepArgs<S
   const int z = a.zrev ? a.nz - 1 - int(blockIdx.z) : int(blockIdx.z);
   const bool active = x < a.nx && y < a.ny;
   if (!CHECK && !active) return;
-  double du2 = 0.0, uu = 0.0, dr = 0.0;
-  int bad = 0;
+  CheckSums sums;
   if (active) {
     const int i = z * a.plane + y * a.pitch + x;
     R d[Q];
@@ -341,155 +347,44 @@ __global__ void __launch_bounds__(256, CAP ? 4 : 1) step_kernel(const StepArgs<S
     collide<R, FORCE, pair_out<S>(), log2_scale<S>(), UNIT>(a.C, d, o);
 #pragma unroll
     for (int q = 0; q < Q; ++q) a.dstq[q][i] = Codec<S, R>::enc(d[q], R(1));
-    if (CHECK) {
-      R* up = reinterpret_cast<R*>(a.cb.uprev);
-      const int64_t nst = int64_t(a.plane) * a.nz;
-      const R px = up[i], py = up[nst + i], pz = up[2 * nst + i];
-      up[i] = o.ux;
-      up[nst + i] = o.uy;
-      up[2 * nst + i] = o.uz;
-      const double ex = double(o.ux) - double(px), ey = double(o.uy) - double(py),
-                   ez = double(o.uz) - double(pz);
-      du2 = ex * ex + ey * ey + ez * ez;
-      uu = double(o.ux) * double(o.ux) + double(o.uy) * double(o.uy) +
-           double(o.uz) * double(o.uz);
-      dr = double(o.rho) - double(a.C.rho0);
-      const double chk = double(o.rho) + double(o.ux) + double(o.uy) + double(o.uz);
-      bad = !(chk == chk) || !(fabs(chk) < 1e30) || !(double(o.rho) > 0.5 && double(o.rho) < 2.0);
-    }
+    if (CHECK)
+      check_node(sums, o.rho, o.ux, o.uy, o.uz, a.C.rho0, static_cast<R*>(a.cb.uprev) + i,
+                 int64_t(a.plane) * a.nz);
   }
-  if (CHECK) {
-    __shared__ double smem[32];
-    block_sum_add(du2, &a.cb.acc[0], smem);
-    block_sum_add(uu, &a.cb.acc[1], smem);
-    block_sum_add(dr, &a.cb.acc[2], smem);
-    if (__syncthreads_or(bad) && threadIdx.x == 0 && threadIdx.y == 0) atomicOr(a.cb.flag, 1);
-  }
+  if (CHECK) block_sums(sums, check_row(a.cb), a.cb.flag);
 }
 
-// Two nodes per thread, rows y and y + 1 at the same (x, z), collided as a
-// pair with packed FP32 arithmetic (R = V2).  Loads and stores stay 32-bit
-// per row, so every warp access still covers 32 consecutive x.  Both nodes
-// share x, so the x-face replacement is the same for the pair; a pair that
-// touches a y or z face pulls node by node through pull_face.
-template <typename S, bool FORCE, bool CHECK, bool CAP>
-__global__ void __launch_bounds__(128, CAP ? 4 : 1) step2_kernel(const StepArgs<S, float> a) {
-  pdl_enter();
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = 2 * (blockIdx.y * blockDim.y + threadIdx.y);
-  const int z = blockIdx.z;
-  const bool activeA = x < a.nx && y < a.ny;
-  const bool activeB = activeA && y + 1 < a.ny;
-  if (!CHECK && !activeA) return;
-  double du2 = 0.0, uu = 0.0, dr = 0.0;
-  int bad = 0;
-  if (activeA) {
-    const int iA = z * a.plane + y * a.pitch + x;
-    const int iB = activeB ? iA + a.pitch : iA;
-    V2 d[Q];
-    if (y > 0 && y + 1 < a.ny - 1 && z > 0 && z < a.nz - 1) {
-#pragma unroll
-      for (int q = 0; q < Q; ++q)
-        d[q] = V2(Codec<S, float>::dec(a.srcq[q][iA], 1.0f),
-                  Codec<S, float>::dec(a.srcq[q][iB], 1.0f));
-      if (x == 0 || x == a.nx - 1) {
-        const int kl = a.facebits & 3, kr = (a.facebits >> 2) & 3;
-#pragma unroll
-        for (int q = 1; q < Q; ++q) {
-          if (cx(q) == 1 && x == 0) {
-            d[q] = kl == BC_PERIODIC
-                       ? V2(Codec<S, float>::dec(a.srcq[q][iA + a.nx], 1.0f),
-                            Codec<S, float>::dec(a.srcq[q][iB + a.nx], 1.0f))
-                       : V2(Codec<S, float>::dec(a.src[opp(q) * a.qstride + iA], 1.0f),
-                            Codec<S, float>::dec(a.src[opp(q) * a.qstride + iB], 1.0f)) +
-                             V2(kl == BC_LID ? a.lidc[q] : 0.0f);
-          }
-          if (cx(q) == -1 && x == a.nx - 1) {
-            d[q] = kr == BC_PERIODIC
-                       ? V2(Codec<S, float>::dec(a.srcq[q][iA - a.nx], 1.0f),
-                            Codec<S, float>::dec(a.srcq[q][iB - a.nx], 1.0f))
-                       : V2(Codec<S, float>::dec(a.src[opp(q) * a.qstride + iA], 1.0f),
-                            Codec<S, float>::dec(a.src[opp(q) * a.qstride + iB], 1.0f)) +
-                             V2(kr == BC_LID ? a.lidc[q] : 0.0f);
-          }
-        }
-      }
-    } else {
-      const int yB = activeB ? y + 1 : y;
-      float dA[Q], dB[Q];
-      pull_face<S, float>(a.src, a.qstride, a.nx, a.ny, a.nz, a.pitch, a.plane, a.facebits, x, y,
-                          z, iA, a.lidc, dA);
-      pull_face<S, float>(a.src, a.qstride, a.nx, a.ny, a.nz, a.pitch, a.plane, a.facebits, x, yB,
-                          z, iB, a.lidc, dB);
-#pragma unroll
-      for (int q = 0; q < Q; ++q) d[q] = V2(dA[q], dB[q]);
-    }
-    NodeOut<V2> o;
-    collide<V2, FORCE, pair_out<S>(), log2_scale<S>(), true>(a.C, d, o);
-#pragma unroll
-    for (int q = 0; q < Q; ++q) a.dstq[q][iA] = Codec<S, float>::enc(lane0(d[q]), 1.0f);
-    if (activeB) {
-#pragma unroll
-      for (int q = 0; q < Q; ++q) a.dstq[q][iB] = Codec<S, float>::enc(lane1(d[q]), 1.0f);
-    }
-    if (CHECK) {
-      float* up = reinterpret_cast<float*>(a.cb.uprev);
-      const int64_t nst = int64_t(a.plane) * a.nz;
-      const float ux[2] = {lane0(o.ux), lane1(o.ux)}, uy[2] = {lane0(o.uy), lane1(o.uy)},
-                  uz[2] = {lane0(o.uz), lane1(o.uz)}, rh[2] = {lane0(o.rho), lane1(o.rho)};
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        if (k == 1 && !activeB) break;
-        const int i = k == 0 ? iA : iB;
-        const float px = up[i], py = up[nst + i], pz = up[2 * nst + i];
-        up[i] = ux[k];
-        up[nst + i] = uy[k];
-        up[2 * nst + i] = uz[k];
-        const double ex = double(ux[k]) - double(px), ey = double(uy[k]) - double(py),
-                     ez = double(uz[k]) - double(pz);
-        du2 += ex * ex + ey * ey + ez * ez;
-        uu += double(ux[k]) * double(ux[k]) + double(uy[k]) * double(uy[k]) +
-              double(uz[k]) * double(uz[k]);
-        dr += double(rh[k]) - double(a.C.rho0);
-        const double chk = double(rh[k]) + double(ux[k]) + double(uy[k]) + double(uz[k]);
-        bad |= !(chk == chk) || !(fabs(chk) < 1e30) ||
-               !(double(rh[k]) > 0.5 && double(rh[k]) < 2.0);
-      }
-    }
+// Output arrays of the macroscopic fields, unpadded [z][y][x]; any may be null.
+struct FieldsOut {
+  double *rho, *u, *gd;
+};
+template <typename R>
+__device__ __forceinline__ void write_fields(const FieldsOut& f, const NodeOut<R>& o, int nx,
+                                             int ny, int nz, int x, int y, int z) {
+  const int64_t N = int64_t(nx) * ny * nz;
+  const int64_t k = (int64_t(z) * ny + y) * nx + x;
+  if (f.rho) f.rho[k] = to64(o.rho);
+  if (f.u) {
+    f.u[k] = to64(o.ux);
+    f.u[N + k] = to64(o.uy);
+    f.u[2 * N + k] = to64(o.uz);
   }
-  if (CHECK) {
-    __shared__ double smem[32];
-    block_sum_add(du2, &a.cb.acc[0], smem);
-    block_sum_add(uu, &a.cb.acc[1], smem);
-    block_sum_add(dr, &a.cb.acc[2], smem);
-    if (__syncthreads_or(bad) && threadIdx.x == 0 && threadIdx.y == 0) atomicOr(a.cb.flag, 1);
-  }
+  if (f.gd) f.gd[k] = to64(o.gamma_dot);
 }
 
-// Macroscopic fields of the current state (pull + moments + omega solve).
+// Macroscopic fields of the current state (pull + moments + omega solve, the
+// last only for |gamma_dot|).
 template <typename S, typename R, bool FORCE>
-__global__ void __launch_bounds__(256) fields_kernel(const S* __restrict__ src, Geom g,
-                                                     CollideConst<R> C, double* rho,
-                                                     double* u, double* gd) {
+__global__ void __launch_bounds__(256) fields_kernel(const StepArgs<S, R> a, const FieldsOut f) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z;
-  if (x >= g.nx || y >= g.ny) return;
-  const double lam = double(1 << log2_scale<S>());
-  const int64_t i = int64_t(z) * g.plane + int64_t(y) * g.pitch + x;
+  if (x >= a.nx || y >= a.ny) return;
   R d[Q];
-  pull<S, R>(src, g, x, y, z, i, R(lam), d);
+  pull_node(a, x, y, z, z * a.plane + y * a.pitch + x, d);
   NodeOut<R> o;
-  collide<R, FORCE, pair_out<S>(), log2_scale<S>(), false>(C, d, o);
-  const int64_t N = int64_t(g.nx) * g.ny * g.nz;
-  const int64_t k = (int64_t(z) * g.ny + y) * g.nx + x;
-  if (rho) rho[k] = double(o.rho);
-  if (u) {
-    u[k] = double(o.ux);
-    u[N + k] = double(o.uy);
-    u[2 * N + k] = double(o.uz);
-  }
-  if (gd) gd[k] = double(o.gamma_dot);
+  node_fields<R, FORCE, log2_scale<S>()>(a.C, d, f.gd != nullptr, o);
+  write_fields(f, o, a.nx, a.ny, a.nz, x, y, z);
 }
 
 // Collide M independent nodes given as plain FP64 populations [q][node].
@@ -649,23 +544,6 @@ cudaError_t launch_step_t(const void* src, void* dst, const Geom& g, const PhysP
                        : step_kernel<S, R, false, false, true, true>;
     return pdl_launch(kernel, grid, block, st, a);
   } else {
-    if constexpr (std::is_same<R, float>::value) {
-      if (npt == 2) {
-        const dim3 grid2((g.nx + block.x - 1) / block.x,
-                         (g.ny + 2 * block.y - 1) / (2 * block.y), g.nz);
-        if (cap)
-          kernel = fc == 3   ? step2_kernel<S, true, true, true>
-                   : fc == 2 ? step2_kernel<S, true, false, true>
-                   : fc == 1 ? step2_kernel<S, false, true, true>
-                             : step2_kernel<S, false, false, true>;
-        else
-          kernel = fc == 3   ? step2_kernel<S, true, true, false>
-                   : fc == 2 ? step2_kernel<S, true, false, false>
-                   : fc == 1 ? step2_kernel<S, false, true, false>
-                             : step2_kernel<S, false, false, false>;
-        return pdl_launch(kernel, grid2, block, st, a);
-      }
-    }
     if (cap)
       kernel = fc == 3   ? step_kernel<S, R, true, true, true, true>
                : fc == 2 ? step_kernel<S, R, true, false, true, true>
@@ -683,12 +561,12 @@ cudaError_t launch_step_t(const void* src, void* dst, const Geom& g, const PhysP
 template <typename S, typename R>
 cudaError_t launch_fields_t(const void* src, const Geom& g, const PhysParams& P, double* rho,
                             double* u, double* gd, cudaStream_t st) {
-  dim3 block(32, 4);
-  dim3 grid((g.nx + 31) / 32, (g.ny + 3) / 4, g.nz);
-  const S* s = static_cast<const S*>(src);
-  const CollideConst<R> C = make_const<R>(P, double(1 << log2_scale<S>()));
-  if (P.has_force) fields_kernel<S, R, true><<<grid, block, 0, st>>>(s, g, C, rho, u, gd);
-  else fields_kernel<S, R, false><<<grid, block, 0, st>>>(s, g, C, rho, u, gd);
+  const dim3 block(32, 4);
+  const dim3 grid((g.nx + 31) / 32, (g.ny + 3) / 4, g.nz);
+  const StepArgs<S, R> a = step_args<S, R>(src, nullptr, g, P, CheckBufs{});
+  const FieldsOut f{rho, u, gd};
+  if (P.has_force) fields_kernel<S, R, true><<<grid, block, 0, st>>>(a, f);
+  else fields_kernel<S, R, false><<<grid, block, 0, st>>>(a, f);
   return cudaGetLastError();
 }
 

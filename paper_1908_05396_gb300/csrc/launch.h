@@ -113,9 +113,12 @@ inline bool unit_rates(const PhysParams& P) {
 // Work buffers of a check step.
 struct CheckBufs {
   void* uprev;      // 3 x (plane * nz) velocities of the previous check, math type
-  double* acc;      // [0] sum|u-uprev|^2, [1] sum|u|^2, [2] sum(rho - rho0)
+  double* acc;      // rows of 4: sum|u-uprev|^2, sum|u|^2, sum(rho - rho0), unused
   int* flag;        // [0] divergence flag, [1] set when a TMA pipeline wait gave up
+  int rows = 1;     // rows of acc, a power of two, that the blocks spread over
 };
+constexpr int CHECK_ROWS = 64;  // of a lone lattice
+constexpr int BATCH_ROWS = 8;   // of each lattice in a batch
 
 // TMA-staged FP32 / FP16 step (tma_step.cuh): npt = TMA_NPT + 32 v selects
 // shape v, whose block must be tma_bx(v) x tma_by(v).

@@ -47,110 +47,81 @@ cudaError_t scratch_address(int dev, double** out) {
   return cudaSuccess;
 }
 
-// The fused step of step_kernel<..., CHECK = true>, with each block writing
-// its partial sums (sum|u - uprev|^2, sum|u|^2, sum(rho - rho0), divergence)
-// to its own slot of the scratch array instead of adding them atomically.
+// The check step of step_kernel, with each block writing its partial sums
+// (sum|u - uprev|^2, sum|u|^2, sum(rho - rho0), divergence) to its own slot of
+// the scratch array instead of adding them atomically.
 template <typename S, typename R, bool FORCE>
-__global__ void __launch_bounds__(256) step_partials_kernel(const S* __restrict__ src,
-                                                            S* __restrict__ dst, Geom g,
-                                                            CollideConst<R> C, R* uprev,
+__global__ void __launch_bounds__(256) step_partials_kernel(const StepArgs<S, R> a,
                                                             double* partials) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z;
-  const bool active = x < g.nx && y < g.ny;
-  const double lam = double(1 << log2_scale<S>());
-  double v[4] = {0.0, 0.0, 0.0, 0.0};
-  if (active) {
-    const int64_t i = int64_t(z) * g.plane + int64_t(y) * g.pitch + x;
+  CheckSums sums;
+  if (x < a.nx && y < a.ny) {
+    const int i = z * a.plane + y * a.pitch + x;
     R d[Q];
-    pull<S, R>(src, g, x, y, z, i, R(lam), d);
+    pull_node(a, x, y, z, i, d);
     NodeOut<R> o;
-    collide<R, FORCE, pair_out<S>(), log2_scale<S>(), true>(C, d, o);
+    collide<R, FORCE, pair_out<S>(), log2_scale<S>(), true>(a.C, d, o);
 #pragma unroll
-    for (int q = 0; q < Q; ++q) dst[q * g.qstride + i] = Codec<S, R>::enc(d[q], R(lam));
-    const int64_t nst = g.plane * g.nz;
-    const R px = uprev[i], py = uprev[nst + i], pz = uprev[2 * nst + i];
-    uprev[i] = o.ux;
-    uprev[nst + i] = o.uy;
-    uprev[2 * nst + i] = o.uz;
-    const double ex = double(o.ux) - double(px), ey = double(o.uy) - double(py),
-                 ez = double(o.uz) - double(pz);
-    v[0] = ex * ex + ey * ey + ez * ez;
-    v[1] = double(o.ux) * double(o.ux) + double(o.uy) * double(o.uy) +
-           double(o.uz) * double(o.uz);
-    v[2] = double(o.rho) - double(C.rho0);
-    const double chk = double(o.rho) + double(o.ux) + double(o.uy) + double(o.uz);
-    v[3] = (!(chk == chk) || !(fabs(chk) < 1e30) ||
-            !(double(o.rho) > 0.5 && double(o.rho) < 2.0)) ? 1.0 : 0.0;
+    for (int q = 0; q < Q; ++q) a.dstq[q][i] = Codec<S, R>::enc(d[q], R(1));
+    check_node(sums, o.rho, o.ux, o.uy, o.uz, a.C.rho0, static_cast<R*>(a.cb.uprev) + i,
+               int64_t(a.plane) * a.nz);
   }
-  // Fixed-order block reduction (warp shuffles, then warp 0), so that the
-  // result does not depend on scheduling.
-  __shared__ double sm[4][32];
+  // Fixed-order block reduction, so that the result does not depend on
+  // scheduling.
+  __shared__ double sm[8][3];
   const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-  const int lane = tid & 31, warp = tid >> 5, nwarp = (blockDim.x * blockDim.y + 31) >> 5;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    double a = v[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-    if (lane == 0) sm[k][warp] = a;
-  }
-  __syncthreads();
-  if (warp == 0) {
+  const int lane = tid & 31, warp = tid >> 5, nwarp = int(blockDim.x * blockDim.y) >> 5;
+  const double v = warp_sums(sums);
+  if (lane == 0) sm[warp][0] = v;
+  if (lane == 16) sm[warp][1] = v;
+  if (lane == 8) sm[warp][2] = v;
+  const int bad = __syncthreads_or(sums.bad);
+  if (tid < 4) {
+    double t = tid < 3 ? sm[0][tid < 3 ? tid : 0] : double(bad != 0);
+    for (int w = 1; w < nwarp && tid < 3; ++w) t += sm[w][tid];
     const int64_t b = (int64_t(blockIdx.z) * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      double a = lane < nwarp ? sm[k][lane] : 0.0;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-      if (lane == 0) partials[b * 4 + k] = a;
-    }
+    partials[b * 4 + tid] = t;
   }
 }
 
 // Second pass: one block sums the nblocks partials in a fixed order and
-// writes the four results (the divergence entry as 0 or 1).
-__global__ void __launch_bounds__(256) finish_kernel(const double* __restrict__ partials,
-                                                     int nblocks, double* stats) {
-  __shared__ double sm[4][256];
+// writes the four results (the divergence entry as 0 or 1).  Thread t takes
+// entry t & 3 of every 256th block's partials, so that a warp reads whole
+// lines; four sums a thread keep its loads in flight.
+constexpr int FINISH_THREADS = 1024;
+__global__ void __launch_bounds__(FINISH_THREADS) finish_kernel(
+    const double* __restrict__ partials, int nblocks, double* stats) {
+  __shared__ double sm[FINISH_THREADS];
+  const int t = int(threadIdx.x), n = 4 * nblocks;
   double a[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
+  for (int b = t; b < n; b += 4 * FINISH_THREADS)
 #pragma unroll
-    for (int k = 0; k < 4; ++k) a[k] += partials[int64_t(b) * 4 + k];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) sm[k][threadIdx.x] = a[k];
+    for (int k = 0; k < 4; ++k)
+      if (b + k * FINISH_THREADS < n) a[k] += partials[b + k * FINISH_THREADS];
+  sm[t] = (a[0] + a[1]) + (a[2] + a[3]);
   __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (int(threadIdx.x) < s)
-#pragma unroll
-      for (int k = 0; k < 4; ++k) sm[k][threadIdx.x] += sm[k][threadIdx.x + s];
+  for (int s = FINISH_THREADS / 2; s >= 4; s >>= 1) {
+    if (t < s) sm[t] += sm[t + s];
     __syncthreads();
   }
-  if (threadIdx.x == 0) {
-    stats[0] = sm[0][0];
-    stats[1] = sm[1][0];
-    stats[2] = sm[2][0];
-    stats[3] = sm[3][0] > 0.0 ? 1.0 : 0.0;
-  }
+  if (t < 4) stats[t] = t < 3 ? sm[t] : (sm[t] > 0.0 ? 1.0 : 0.0);
 }
 
 template <typename S, typename R>
 cudaError_t launch_noalloc(const void* src, void* dst, const Geom& g, const PhysParams& P,
                            void* uprev, double* partials, double* stats, dim3 grid, dim3 block,
                            cudaStream_t st) {
-  const S* s = static_cast<const S*>(src);
-  S* d = static_cast<S*>(dst);
-  R* up = static_cast<R*>(uprev);
-  const CollideConst<R> C = make_const<R>(P, double(1 << log2_scale<S>()));
-  // the entry point takes the unit rates omega_9..18 only
-  if (P.has_force)
-    step_partials_kernel<S, R, true><<<grid, block, 0, st>>>(s, d, g, C, up, partials);
-  else
-    step_partials_kernel<S, R, false><<<grid, block, 0, st>>>(s, d, g, C, up, partials);
+  CheckBufs cb{};
+  cb.uprev = uprev;
+  // (dense rows; the entry point takes the unit rates omega_9..18 only)
+  StepArgs<S, R> a = step_args<S, R>(src, dst, g, P, cb);
+  if (P.has_force) step_partials_kernel<S, R, true><<<grid, block, 0, st>>>(a, partials);
+  else step_partials_kernel<S, R, false><<<grid, block, 0, st>>>(a, partials);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  finish_kernel<<<1, 256, 0, st>>>(partials, int(grid.x * grid.y * grid.z), stats);
+  finish_kernel<<<1, FINISH_THREADS, 0, st>>>(partials, int(grid.x * grid.y * grid.z), stats);
   return cudaGetLastError();
 }
 

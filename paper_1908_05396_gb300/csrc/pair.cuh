@@ -9,7 +9,7 @@
 //     3.8), and index and face logic is shared by two nodes;
 //   - the two values of a direction with e_x = 0, and every stored value,
 //     are one aligned 32-bit access and one conversion instruction.
-// Rows y and y + 1 as the pair (the FP32 form's step2_kernel) keep every
+// Rows y and y + 1 as the pair (the first attempt, for FP32 too) keep every
 // 16-bit access and lose most of this.
 // Measured, one node per thread -> pairs, us a step: F16S 323 -> 233 on 256^3
 // (5.5 TB/s) and 49.8 -> 38.6 on 128^3; F16R 753 -> 418 and 95 -> 61, whose
@@ -267,30 +267,11 @@ __device__ __forceinline__ void store_pair(const CollideConst<float>& C, V2 (&d)
   }
 }
 
-// Check-step sums of the pair (see step_kernel): u into uprev after reading
-// the previous check's, sum|u - uprev|^2, sum|u|^2, sum(rho - rho0) and the
-// divergence flag.  n1: the second node exists.
-__device__ __forceinline__ void check_pair(const NodeOut<V2>& o, float rho0, float* up,
-                                           int64_t nst, int i, bool n1, double& du2, double& uu,
-                                           double& dr, int& bad) {
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    if (k == 1 && !n1) break;
-    const float ux = k ? lane1(o.ux) : lane0(o.ux), uy = k ? lane1(o.uy) : lane0(o.uy),
-                uz = k ? lane1(o.uz) : lane0(o.uz), rho = k ? lane1(o.rho) : lane0(o.rho);
-    float* u = up + i + k;
-    const float px = u[0], py = u[nst], pz = u[2 * nst];
-    u[0] = ux;
-    u[nst] = uy;
-    u[2 * nst] = uz;
-    const double ex = double(ux) - double(px), ey = double(uy) - double(py),
-                 ez = double(uz) - double(pz);
-    du2 += ex * ex + ey * ey + ez * ez;
-    uu += double(ux) * double(ux) + double(uy) * double(uy) + double(uz) * double(uz);
-    dr += double(rho) - double(rho0);
-    const double chk = double(rho) + double(ux) + double(uy) + double(uz);
-    bad |= !(chk == chk) || !(fabs(chk) < 1e30) || !(double(rho) > 0.5 && double(rho) < 2.0);
-  }
+// The pair's part of the check-step sums; n1: the second node exists.
+__device__ __forceinline__ void check_pair(CheckSums& s, const NodeOut<V2>& o, float rho0,
+                                           float* up, int64_t nst, bool n1) {
+  check_node(s, lane0(o.rho), lane0(o.ux), lane0(o.uy), lane0(o.uz), rho0, up, nst);
+  if (n1) check_node(s, lane1(o.rho), lane1(o.ux), lane1(o.uy), lane1(o.uz), rho0, up + 1, nst);
 }
 
 // F16R: reference buffers of a lone step; step: the lattice's steps done
@@ -311,8 +292,7 @@ __global__ void __launch_bounds__(256, pair_min_blocks(FORM == PAIR_REF, FORCE))
   const int z = a.zrev ? a.nz - 1 - int(blockIdx.z) : int(blockIdx.z);
   const bool active = x < a.nx && y < a.ny;
   if (!CHECK && !active) return;
-  double du2 = 0.0, uu = 0.0, dr = 0.0;
-  int bad = 0;
+  CheckSums sums;
   if (active) {
     const int i = z * a.plane + y * a.pitch + x;
     V2 d[Q];
@@ -323,16 +303,10 @@ __global__ void __launch_bounds__(256, pair_min_blocks(FORM == PAIR_REF, FORCE))
     store_pair<FORM>(a.C, d, o, [&](int q) { return a.dstq[q] + i; },
                      FORM == PAIR_REF ? e.ref_dst + i : nullptr, i, e.step);
     if (CHECK)
-      check_pair(o, a.C.rho0, static_cast<float*>(a.cb.uprev), int64_t(a.plane) * a.nz, i,
-                 x + 1 < a.nx, du2, uu, dr, bad);
+      check_pair(sums, o, a.C.rho0, static_cast<float*>(a.cb.uprev) + i, int64_t(a.plane) * a.nz,
+                 x + 1 < a.nx);
   }
-  if (CHECK) {
-    __shared__ double smem[32];
-    block_sum_add(du2, &a.cb.acc[0], smem);
-    block_sum_add(uu, &a.cb.acc[1], smem);
-    block_sum_add(dr, &a.cb.acc[2], smem);
-    if (__syncthreads_or(bad) && threadIdx.x == 0 && threadIdx.y == 0) atomicOr(a.cb.flag, 1);
-  }
+  if (CHECK) block_sums(sums, check_row(a.cb), a.cb.flag);
 }
 
 template <int FORM>

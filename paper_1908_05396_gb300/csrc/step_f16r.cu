@@ -124,65 +124,32 @@ __global__ void __launch_bounds__(256) step_ref_kernel(const StepArgs<__half, fl
   const int z = a.zrev ? a.nz - 1 - int(blockIdx.z) : int(blockIdx.z);  // as step_kernel
   const bool active = x < a.nx && y < a.ny;
   if (!CHECK && !active) return;
-  const float rho0 = a.C.rho0;
-  double du2 = 0.0, uu = 0.0, dr = 0.0;
-  int bad = 0;
+  CheckSums sums;
   if (active) {
     const int i = z * a.plane + y * a.pitch + x;
     float d[Q];
     pull_node_ref(a, r, x, y, z, i, d);
     NodeOut<float> o;
     collide_store_ref<FORCE, UNIT>(a, r, i, r.step, d, o);
-    if (CHECK) {
-      float* up = reinterpret_cast<float*>(a.cb.uprev);
-      const int64_t nst = int64_t(a.plane) * a.nz;
-      const float px = up[i], py = up[nst + i], pz = up[2 * nst + i];
-      up[i] = o.ux;
-      up[nst + i] = o.uy;
-      up[2 * nst + i] = o.uz;
-      const double ex = double(o.ux) - double(px), ey = double(o.uy) - double(py),
-                   ez = double(o.uz) - double(pz);
-      du2 = ex * ex + ey * ey + ez * ez;
-      uu = double(o.ux) * double(o.ux) + double(o.uy) * double(o.uy) + double(o.uz) * double(o.uz);
-      dr = double(o.rho) - double(rho0);
-      const double chk = double(o.rho) + double(o.ux) + double(o.uy) + double(o.uz);
-      bad = !(chk == chk) || !(fabs(chk) < 1e30) || !(double(o.rho) > 0.5 && double(o.rho) < 2.0);
-    }
+    if (CHECK)
+      check_node(sums, o.rho, o.ux, o.uy, o.uz, a.C.rho0, static_cast<float*>(a.cb.uprev) + i,
+                 int64_t(a.plane) * a.nz);
   }
-  if (CHECK) {
-    __shared__ double smem[32];
-    block_sum_add(du2, &a.cb.acc[0], smem);
-    block_sum_add(uu, &a.cb.acc[1], smem);
-    block_sum_add(dr, &a.cb.acc[2], smem);
-    if (__syncthreads_or(bad) && threadIdx.x == 0 && threadIdx.y == 0) atomicOr(a.cb.flag, 1);
-  }
+  if (CHECK) block_sums(sums, check_row(a.cb), a.cb.flag);
 }
 
 template <bool FORCE>
-__global__ void __launch_bounds__(256) fields_ref_kernel(const __half* __restrict__ src,
-                                                         const uint2* __restrict__ ref, Geom g,
-                                                         CollideConst<float> C,
-                                                         const float* __restrict__ lidc,
-                                                         double* rho, double* u, double* gd) {
+__global__ void __launch_bounds__(256) fields_ref_kernel(const StepArgs<__half, float> a,
+                                                         const RefArgs r, const FieldsOut f) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z;
-  if (x >= g.nx || y >= g.ny) return;
-  const int i = z * int(g.plane) + y * g.pitch + x;
+  if (x >= a.nx || y >= a.ny) return;
   float d[Q];
-  pull_face_ref(src, ref, g.qstride, g.nx, g.ny, g.nz, g.pitch, int(g.plane), g.facebits, x, y,
-                z, i, lidc, d);
+  pull_node_ref(a, r, x, y, z, z * a.plane + y * a.pitch + x, d);
   NodeOut<float> o;
-  collide<float, FORCE, !FORCE, LOG2LAM, false>(C, d, o);
-  const int64_t N = int64_t(g.nx) * g.ny * g.nz;
-  const int64_t k = (int64_t(z) * g.ny + y) * g.nx + x;
-  if (rho) rho[k] = double(o.rho);
-  if (u) {
-    u[k] = double(o.ux);
-    u[N + k] = double(o.uy);
-    u[2 * N + k] = double(o.uz);
-  }
-  if (gd) gd[k] = double(o.gamma_dot);
+  node_fields<float, FORCE, LOG2LAM>(a.C, d, f.gd != nullptr, o);
+  write_fields(f, o, a.nx, a.ny, a.nz, x, y, z);
 }
 
 __global__ void export_ref_kernel(const __half* __restrict__ src, const uint2* __restrict__ ref,
@@ -281,11 +248,17 @@ RefArgs ref_args(const void* ref_src, void* ref_dst, const Geom& g, unsigned ste
   return r;
 }
 
-// Lid terms of the bounce-back, in the scaled deviations.
-void lid_table(const Geom& g, float* out) {
-  for (int q = 0; q < Q; ++q)
-    out[q] = float(6.0 * double(LAM) * wt<double>(q) * g.rho0 *
-                   (cx(q) * g.U[0] + cy(q) * g.U[1] + cz(q) * g.U[2]));
+RefArgs ref_args(const uint2* ref_src, uint2* ref_dst, const Geom& g, unsigned step) {
+  RefArgs r;
+  r.step = step;
+  r.ref_src = ref_src;
+  r.ref_dst = ref_dst;
+  for (int q = 0; q < Q; ++q) {
+    const int64_t off = int64_t(cz(q)) * g.plane + int64_t(cy(q)) * g.pitch + cx(q);
+    r.refq[q] = reinterpret_cast<const uint2*>(reinterpret_cast<uintptr_t>(ref_src) -
+                                                off * int64_t(sizeof(uint2)));
+  }
+  return r;
 }
 
 }  // namespace
@@ -350,24 +323,14 @@ cudaError_t launch_step_f16r(const void* src, void* dst, const void* ref_src, vo
 cudaError_t launch_fields_f16r(const void* src, const void* ref, const Geom& g,
                                const PhysParams& P, double* rho, double* u, double* gd,
                                cudaStream_t st) {
-  float lid[Q];
-  lid_table(g, lid);
-  float* dlid = nullptr;
-  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&dlid), sizeof(lid), st);
-  if (e != cudaSuccess) return e;
-  e = cudaMemcpyAsync(dlid, lid, sizeof(lid), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) {
-    dim3 block(32, 4);
-    dim3 grid((g.nx + 31) / 32, (g.ny + 3) / 4, g.nz);
-    const CollideConst<float> C = make_const<float>(P, double(LAM));
-    const __half* s = static_cast<const __half*>(src);
-    const uint2* r = static_cast<const uint2*>(ref);
-    if (P.has_force) fields_ref_kernel<true><<<grid, block, 0, st>>>(s, r, g, C, dlid, rho, u, gd);
-    else fields_ref_kernel<false><<<grid, block, 0, st>>>(s, r, g, C, dlid, rho, u, gd);
-    e = cudaGetLastError();
-  }
-  cudaFreeAsync(dlid, st);
-  return e;
+  const dim3 block(32, 4);
+  const dim3 grid((g.nx + 31) / 32, (g.ny + 3) / 4, g.nz);
+  const StepArgs<__half, float> a = step_args<__half, float>(src, nullptr, g, P, CheckBufs{});
+  const RefArgs r = ref_args(static_cast<const uint2*>(ref), nullptr, g, 0u);
+  const FieldsOut f{rho, u, gd};
+  if (P.has_force) fields_ref_kernel<true><<<grid, block, 0, st>>>(a, r, f);
+  else fields_ref_kernel<false><<<grid, block, 0, st>>>(a, r, f);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_export_f16r(const void* src, const void* ref, const Geom& g, double rho0,

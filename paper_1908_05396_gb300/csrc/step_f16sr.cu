@@ -25,8 +25,7 @@ __global__ void __launch_bounds__(256) step_sr_kernel(const StepArgs<__half, flo
   const int z = a.zrev ? a.nz - 1 - int(blockIdx.z) : int(blockIdx.z);
   const bool active = x < a.nx && y < a.ny;
   if (!CHECK && !active) return;
-  double du2 = 0.0, uu = 0.0, dr = 0.0;
-  int bad = 0;
+  CheckSums sums;
   if (active) {
     const int i = z * a.plane + y * a.pitch + x;
     float d[Q];
@@ -35,29 +34,11 @@ __global__ void __launch_bounds__(256) step_sr_kernel(const StepArgs<__half, flo
     collide<float, FORCE, pair_out<__half>(), log2_scale<__half>(), UNIT>(a.C, d, o);
     // the deviations are carried scaled by 1024, as they are stored
     store_sr1([&](int q) { return a.dstq[q] + i; }, d, uint32_t(i), step);
-    if (CHECK) {
-      float* up = reinterpret_cast<float*>(a.cb.uprev);
-      const int64_t nst = int64_t(a.plane) * a.nz;
-      const float px = up[i], py = up[nst + i], pz = up[2 * nst + i];
-      up[i] = o.ux;
-      up[nst + i] = o.uy;
-      up[2 * nst + i] = o.uz;
-      const double ex = double(o.ux) - double(px), ey = double(o.uy) - double(py),
-                   ez = double(o.uz) - double(pz);
-      du2 = ex * ex + ey * ey + ez * ez;
-      uu = double(o.ux) * double(o.ux) + double(o.uy) * double(o.uy) + double(o.uz) * double(o.uz);
-      dr = double(o.rho) - double(a.C.rho0);
-      const double chk = double(o.rho) + double(o.ux) + double(o.uy) + double(o.uz);
-      bad = !(chk == chk) || !(fabs(chk) < 1e30) || !(double(o.rho) > 0.5 && double(o.rho) < 2.0);
-    }
+    if (CHECK)
+      check_node(sums, o.rho, o.ux, o.uy, o.uz, a.C.rho0, static_cast<float*>(a.cb.uprev) + i,
+                 int64_t(a.plane) * a.nz);
   }
-  if (CHECK) {
-    __shared__ double smem[32];
-    block_sum_add(du2, &a.cb.acc[0], smem);
-    block_sum_add(uu, &a.cb.acc[1], smem);
-    block_sum_add(dr, &a.cb.acc[2], smem);
-    if (__syncthreads_or(bad) && threadIdx.x == 0 && threadIdx.y == 0) atomicOr(a.cb.flag, 1);
-  }
+  if (CHECK) block_sums(sums, check_row(a.cb), a.cb.flag);
 }
 
 }  // namespace

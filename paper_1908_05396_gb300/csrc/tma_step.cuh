@@ -164,7 +164,7 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 
 // NP = 1: one node per thread (BX x BY threads).  NP = 2: BX x BY/2 threads,
 // each owning rows 2 ty and 2 ty + 1 of the tile at the same x, collided as a
-// pair with packed FP32 arithmetic (V2), as in step2_kernel.
+// pair with packed FP32 arithmetic (V2).
 template <typename S, int BX, int BY, int NP, int NST, int MINB, bool FORCE>
 __global__ void __launch_bounds__(BX * BY / NP, MINB)
     step_tma_kernel(const __grid_constant__ CUtensorMap mapA,
