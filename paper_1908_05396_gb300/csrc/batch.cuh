@@ -103,14 +103,8 @@ __device__ __forceinline__ void batch_pair(const LatDesc<float>& L, int parity, 
   uint2* rd = REF ? static_cast<uint2*>(const_cast<void*>(L.ref[parity ^ 1])) + i : nullptr;
   V2 d[Q];
   pull_pair<REF>(BatchPair{L, src, rs, qs}, x, y, z, d);
-  collide_pair<REF, FORCE>(L.C, d, o);
-  auto dst = [&](int q) { return out + q * qs; };
-  if constexpr (REF) {
-    store_pair<PAIR_REF>(L.C, d, o, dst, rd, i, step);
-  } else {
-    if (L.sround) store_pair<PAIR_SR>(L.C, d, o, dst, rd, i, step);
-    else store_pair<PAIR_RN>(L.C, d, o, dst, rd, i, step);
-  }
+  collide_pair<REF, FORCE>(L.C, d, o, rd);
+  store_pair(d, REF || L.sround != 0, [&](int q) { return out + q * qs; }, i, step);
 }
 
 // tile word: x tile (8 bits) | y tile (12 bits) | z chunk (12 bits)
@@ -218,10 +212,10 @@ __device__ __forceinline__ void batch_tiles(Get get, const int* __restrict__ own
 
 // Blocks of 256 threads per SM that the batch kernel is compiled for: 64
 // registers when capped, what it likes when not; kernels that step two nodes
-// per thread have one variant (launched for both).
+// per thread have one variant (launched for both) with 80, or 128, registers.
 template <typename S>
-constexpr int batch_min_blocks(bool cap, bool unit, bool ref, bool force) {
-  return std::is_same<S, __half>::value && unit ? pair_min_blocks(ref, force) : cap ? 4 : 1;
+constexpr int batch_min_blocks(bool cap, bool unit, bool ref) {
+  return std::is_same<S, __half>::value && unit ? pair_min_blocks(ref) : cap ? 4 : 1;
 }
 
 // The grid of a persistent launch: per_sm blocks per SM, but no more than fit
@@ -277,7 +271,7 @@ void fill_desc_t(void* out, double lam, const Geom& g, const PhysParams& P, cons
   namespace clbm {                                                                             \
   __constant__ LatDesc<R> c_lat_##SUFFIX[BATCH_CONST_BYTES / sizeof(LatDesc<R>)];              \
   template <bool CHECK, bool CAP, bool FORCE, bool UNIT>                                       \
-  __global__ void __launch_bounds__(256, batch_min_blocks<S>(CAP, UNIT, REF, FORCE))           \
+  __global__ void __launch_bounds__(256, batch_min_blocks<S>(CAP, UNIT, REF))                  \
       batch_kernel_##SUFFIX(int base, const int* __restrict__ owner,                           \
                             const unsigned* __restrict__ coord, BatchHeader* hdr, int parity,  \
                             double* acc, int zc) {                                             \

@@ -10,6 +10,8 @@
 // of order 1, and the FP64 form computes the same expressions.
 #pragma once
 
+#include <type_traits>
+
 #include "d3q19.cuh"
 #include "log_table.h"
 #include "v2.cuh"
@@ -741,6 +743,16 @@ __device__ __forceinline__ void collide_rates(const CollideConst<typename Scalar
   out.gamma_dot = shear_rate(rinv, w, A, B);
 }
 
+// The reference of the F16R form: lam (rho - rho0) and lam 3 rho u of a node,
+// as stored.  Its first-order equilibrium w_q [dr + e_q . v] has the moments
+// dr (mass), v/3 (momentum), dr/3 (each D_ii), v_i/9 (D_ijj) and dr/9 (D_iijj).
+template <typename R>
+struct RefT {
+  R dr, vx, vy, vz;
+};
+// collide_unit without a reference to subtract.
+struct NoRef {};
+
 // Collide one node with the rates omega_9..18 = 1 of Sec. 3.1, the default.
 //
 // With unit rates every third- and fourth-order central moment relaxes to its
@@ -773,10 +785,16 @@ __device__ __forceinline__ void collide_rates(const CollideConst<typename Scalar
 // collide_rates.  With PAIR_OUT the populations are rebuilt from the raw
 // moments; without it the moments' increments are added to the populations,
 // one correction each.
-template <typename R, bool FORCE, bool PAIR_OUT, int LOG2LAM>
+// With a function for `ref` (PAIR_OUT, no force) the post-collision deviations
+// come out less the first-order equilibrium of the reference ref(out): taken
+// off the moments, that costs a dozen operations instead of one or two and a
+// multiply-add per population.
+template <typename R, bool FORCE, bool PAIR_OUT, int LOG2LAM, typename Ref = NoRef>
 __device__ __forceinline__ void collide_unit(const CollideConst<typename ScalarOf<R>::type>& C,
-                                             R (&d)[Q], NodeOut<R>& out) {
+                                             R (&d)[Q], NodeOut<R>& out, Ref ref = Ref{}) {
   using T = typename ScalarOf<R>::type;
+  constexpr bool REF = !std::is_same<Ref, NoRef>::value;
+  static_assert(!REF || (PAIR_OUT && !FORCE), "references are taken off rebuilt populations");
   const Pairs<R> p = to_pairs(d);
   // ---- mass, momentum, second moments (Eqs. hydrodynamicfields1/2) --------
   const R Dxx = p.sAx + (p.Dxxyy + p.Dxxzz), Dyy = p.sAy + (p.Dxxyy + p.Dyyzz),
@@ -794,6 +812,11 @@ __device__ __forceinline__ void collide_unit(const CollideConst<typename ScalarO
     Jz = jz + R(T(0.5) * C.FS[2]);
   }
   const R ux = mulr(Jx, rinv), uy = mulr(Jy, rinv), uz = mulr(Jz, rinv);
+  if constexpr (LOG2LAM != 0) out.rho = mulr(rho, R(T(1.0 / double(1 << LOG2LAM))));
+  else out.rho = rho;
+  out.ux = ux;
+  out.uy = uy;
+  out.uz = uz;
   // half of the source S before the collision: S_ii = 2 u_i F_i, S_ij = u_i F_j + u_j F_i
   R Fx(0), Fy(0), Fz(0), hFx(0), hFy(0), hFz(0);
   R hxx = Dxx, hyy = Dyy, hzz = Dzz, hxy = p.Dxy, hxz = p.Dxz, hyz = p.Dyz;
@@ -841,8 +864,27 @@ __device__ __forceinline__ void collide_unit(const CollideConst<typename ScalarO
     R ddr = mulr(R(T(1.0 / 36.0)), drho);
     R pxy = fma(Jx, qy, mulr(q4, cxy)), pxz = fma(Jx, qz, mulr(q4, cxz)),
       pyz = fma(Jy, qz, mulr(q4, cyz));
-    R fExx = Exx, fEyy = Eyy, fEzz = Ezz;
+    R fExx = Exx, fEyy = Eyy, fEzz = Ezz, fdr = drho;
     R gx = mulr(h2, jx), gy = mulr(h2, jy), gz = mulr(h2, jz);
+    if constexpr (REF) {
+      const RefT<R> r = ref(out);
+      const R m6 = R(T(-1.0 / 6.0)), m36 = R(T(-1.0 / 36.0));
+      fdr = drho - r.dr;
+      ddr = fma(m36, r.dr, ddr);
+      fExx = fma(-third, r.dr, Exx);
+      fEyy = fma(-third, r.dr, Eyy);
+      fEzz = fma(-third, r.dr, Ezz);
+      gx = fma(m6, r.vx, gx);
+      gy = fma(m6, r.vy, gy);
+      gz = fma(m6, r.vz, gz);
+      const R vx = mulr(m36, r.vx), vy = mulr(m36, r.vy), vz = mulr(m36, r.vz);
+      oxyy = fma(qx, kyy, vx);
+      oxzz = fma(qx, kzz, vx);
+      oxxy = fma(qy, kxx, vy);
+      oyzz = fma(qy, kzz, vy);
+      oxxz = fma(qz, kxx, vz);
+      oyyz = fma(qz, kyy, vz);
+    }
     if (FORCE) {
       // the other half of the source
       const R fx = R(T(C.FS[0]) * T(1.0 / 24.0)), fy = R(T(C.FS[1]) * T(1.0 / 24.0)),
@@ -887,7 +929,7 @@ __device__ __forceinline__ void collide_unit(const CollideConst<typename ScalarO
     }
     const R m2 = R(T(-2.0));
     const R fs = fxy + fxz;
-    d[0] = fma(R(T(4.0)), fs + fyz, drho - ((fExx + fEyy) + fEzz));
+    d[0] = fma(R(T(4.0)), fs + fyz, fdr - ((fExx + fEyy) + fEzz));
     {
       const R hs = fma(m2, fs, mulr(h2, fExx)), ht = fma(m2, oxyy + oxzz, gx);
       d[1] = hs + ht;
@@ -989,11 +1031,6 @@ __device__ __forceinline__ void collide_unit(const CollideConst<typename ScalarO
     plane(qxz, nxz, mxz, txzz, txxz, d[11], d[14], d[13], d[12]);
     plane(qyz, nyz, myz, tyzz, tyyz, d[15], d[18], d[17], d[16]);
   }
-  if constexpr (LOG2LAM != 0) out.rho = mulr(rho, R(T(1.0 / double(1 << LOG2LAM))));
-  else out.rho = rho;
-  out.ux = ux;
-  out.uy = uy;
-  out.uz = uz;
   out.gamma_dot = shear_rate(rinv, w, A, B);
 }
 

@@ -12,10 +12,11 @@
 // Rows y and y + 1 as the pair (the first attempt, for FP32 too) keep every
 // 16-bit access and lose most of this.
 // Measured, one node per thread -> pairs, us a step: F16S 323 -> 233 on 256^3
-// (5.5 TB/s) and 49.8 -> 38.6 on 128^3; F16R 753 -> 418 and 95 -> 61, whose
-// 19 reference loads a node become 9.5 and whose reference terms are packed.
-// DRAM latency and the drain between dependent steps bound it now (128^3:
-// issue slots 49 % busy).
+// and 49.8 -> 38.6 on 128^3 (224, 5.7 TB/s, and 30 with the face rules as address
+// selects); F16R 753 -> 340 and 95 -> 47, whose 19 reference loads a node
+// become 9.5 and whose reference is taken off the moments instead of 19
+// populations.  DRAM latency and the drain between dependent steps bound F16S
+// now; F16R still issues 500 instructions a node.
 //
 // Included by kernels.cuh (StepArgs, codecs, pdl_launch).
 #pragma once
@@ -35,11 +36,7 @@ __device__ __forceinline__ void set0(V2& v, float f) { v.v.x = f; }
 __device__ __forceinline__ void set1(V2& v, float f) { v.v.y = f; }
 
 // ---- F16R references -----------------------------------------------------
-// (dr, v) of a node: lam (rho - rho0) and lam 3 rho u, as stored (FP16).
-template <typename R>
-struct RefT {
-  R dr, vx, vy, vz;
-};
+// (dr, v) of a node (RefT), stored as four FP16 values.
 __device__ __forceinline__ RefT<float> ref_dec(uint2 v) {
   const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&v.x));
   const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&v.y));
@@ -83,88 +80,142 @@ struct LonePair {
   __device__ __forceinline__ float lid(int q) const { return a.lidc[q]; }
 };
 
-// One direction of one node that crosses an x face (and no y or z wall):
-// the periodic wrap (dx nodes along x from the node's plain upwind value at
-// u, reference at r), or halfway bounce-back from the node's own opposite
-// value, plus the lid term.
-template <bool REF, typename P>
-__device__ __forceinline__ float xface_value(const P& p, int q, int k, int n, const __half* u,
-                                             const uint2* r, int dx) {
-  if (k == BC_PERIODIC) {
-    float v = ld1(u + dx);
-    if (REF) v = fma(wt<float>(q), ref_sum(q, ref1(r + dx)), v);
-    return v;
+// The pre-collision deviations of the pair (x, x + 1) in a row off the y and
+// z faces.  XF: some pair of the warp holds x = 0 or x = nx - 1; the nodes
+// there take the directions from outside by the face rules of pull_face, each
+// by a select of the address (values and references), in the same round of
+// loads.
+template <bool REF, bool XF, typename P>
+__device__ __forceinline__ void pull_row(const P& p, int x, V2 (&d)[Q]) {
+  const int nx = p.nx(), pitch = p.pitch(), plane = p.plane();
+  const unsigned fb = p.faces();
+  const int kl = int(fb & 3u), kr = int((fb >> 2) & 3u);
+  // the pair's first node is at x = 0 (fl); its first (f0) or second (f1) node at x = nx - 1
+  const bool fl = XF && x == 0, f0 = XF && x + 1 == nx, f1 = XF && x + 2 == nx;
+  const bool bl = fl && kl != BC_PERIODIC, b0 = f0 && kr != BC_PERIODIC,
+             b1 = f1 && kr != BC_PERIODIC;
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    const __half* u = p.up(q);
+    if (cx(q) == 0) {
+      d[q] = ld2(u);
+      continue;
+    }
+    const __half *u0 = u, *u1 = u + 1;
+    if (XF) {
+      const __half* own = p.own(opp(q));
+      if (cx(q) == 1) {
+        if (fl) u0 += nx;  // the periodic wrap
+        if (bl) u0 = own;  // halfway bounce-back
+      } else {
+        if (f0) u0 -= nx;
+        if (b0) u0 = own;
+        if (f1) u1 -= nx;
+        if (b1) u1 = own + 1;
+      }
+    }
+    d[q] = V2(ld1(u0), ld1(u1));
   }
-  float v = ld1(p.own(opp(q)) + n);
-  if (REF) v = fma(wt<float>(q), ref_sum(opp(q), ref1(p.ref + n)), v);
-  return k == BC_LID ? v + p.lid(q) : v;
+  if (REF) {
+    // Columns of upwind nodes (e_y, e_z), each one 128-bit reference load for
+    // the pair's own x and, where the column's directions have e_x != 0, a
+    // 64-bit load on either side.  A bounced value is decoded with the node's
+    // own reference as opp(q): e_q . v changes sign.
+    const float gl = bl ? -1.0f : 1.0f, g0 = b0 ? -1.0f : 1.0f, g1 = b1 ? -1.0f : 1.0f;
+#pragma unroll
+    for (int c = 0; c < Q; ++c) {
+      if (cx(c) != 0) continue;
+      const uint2* rc = p.ref - (cz(c) * plane + cy(c) * pitch);
+      const uint4 w = *reinterpret_cast<const uint4*>(rc);
+      const RefT<float> a = ref_dec(make_uint2(w.x, w.y)), b = ref_dec(make_uint2(w.z, w.w));
+      const RefT<V2> r{V2(a.dr, b.dr), V2(a.vx, b.vx), V2(a.vy, b.vy), V2(a.vz, b.vz)};
+      const V2 s = ref_sum(c, r);
+      d[c] = fma(V2(wt<float>(c)), s, d[c]);
+      if (cy(c) != 0 && cz(c) != 0) continue;
+      // left (x - 1) and right (x + 2, and where the pair's first node is the
+      // last of the row, x + 1) neighbours, or what stands in for them
+      const uint2 *rl = rc - 1, *rr = rc + 2;
+      if (XF) {
+        if (fl) rl = bl ? p.ref : rl + nx;
+        if (f1) rr = b1 ? p.ref + 1 : rr - nx;
+        if (f0) rr = b0 ? p.ref : rc + 1 - nx;
+      }
+      RefT<float> l = ref1(rl), n = ref1(rr);
+      float s1 = lane1(s), x1 = lane1(r.vx);
+      if (XF) {
+        const float gr = g0 * g1;  // (at most one of the two is -1)
+        l = {l.dr, mulr(gl, l.vx), mulr(gl, l.vy), mulr(gl, l.vz)};
+        n = {n.dr, mulr(gr, n.vx), mulr(gr, n.vy), mulr(gr, n.vz)};
+      }
+      const float sl = ref_sum(c, l), sn = ref_sum(c, n);
+      if (XF && f0) {  // the first node's e_x = -1 value comes from `n`
+        s1 = sn;
+        x1 = n.vx;
+      }
+#pragma unroll
+      for (int q = 1; q < Q; ++q) {
+        if (cy(q) != cy(c) || cz(q) != cz(c) || cx(q) == 0) continue;
+        // e_x = 1: upwind nodes x - 1, x; e_x = -1: x + 1, x + 2
+        const V2 t = cx(q) == 1 ? V2(sl, lane0(s)) + V2(l.vx, lane0(r.vx))
+                                : V2(s1, sn) - V2(x1, n.vx);
+        d[q] = fma(V2(wt<float>(q)), t, d[q]);
+      }
+    }
+  }
+  if (XF && ((fl && kl == BC_LID) || ((f0 || f1) && kr == BC_LID))) {
+#pragma unroll
+    for (int q = 1; q < Q; ++q) {
+      if (cx(q) == 1 && fl && kl == BC_LID) set0(d[q], lane0(d[q]) + p.lid(q));
+      if (cx(q) == -1 && f0 && kr == BC_LID) set0(d[q], lane0(d[q]) + p.lid(q));
+      if (cx(q) == -1 && f1 && kr == BC_LID) set1(d[q], lane1(d[q]) + p.lid(q));
+    }
+  }
 }
 
-// The pre-collision deviations of the pair (x, x + 1) in row (y, z).  Rows off
-// the y and z faces load every direction unconditionally and then replace, in
-// the threads that hold x = 0 or x = nx - 1, the five directions that come
-// from outside; rows on a y or z face resolve each direction.  When nx is odd
-// the last pair's second node lies in the row's padding: it is computed from
-// whatever is there and stored there.
+// F16S: replace the directions that cross an x face after the direct loads.  A
+// second round of loads in the threads at x = 0 and x = nx - 1, yet cheaper
+// than selecting addresses in all of the warp's (128^3: 30.0 us a step against
+// 31.7); F16R, whose patch would load and decode references again, is faster
+// the other way (61 and 49 us).
+template <typename P>
+__device__ __forceinline__ void xface_patch(const P& p, int x, V2 (&d)[Q]) {
+  const int nx = p.nx();
+  const int kl = int(p.faces() & 3u), kr = int((p.faces() >> 2) & 3u);
+  if (x == 0) {
+#pragma unroll
+    for (int q = 1; q < Q; ++q) {
+      if (cx(q) != 1) continue;
+      const float v = ld1(kl == BC_PERIODIC ? p.up(q) + nx : p.own(opp(q)));
+      set0(d[q], kl == BC_LID ? v + p.lid(q) : v);
+    }
+  }
+  if (x + 2 >= nx) {
+    const int n = nx - 1 - x;  // which node of the pair is at nx - 1
+#pragma unroll
+    for (int q = 1; q < Q; ++q) {
+      if (cx(q) != -1) continue;
+      float v = ld1(kr == BC_PERIODIC ? p.up(q) + n - nx : p.own(opp(q)) + n);
+      if (kr == BC_LID) v += p.lid(q);
+      if (n == 0) set0(d[q], v);
+      else set1(d[q], v);
+    }
+  }
+}
+
+// The pre-collision deviations of the pair (x, x + 1) in row (y, z).  When nx
+// is odd the last pair's second node lies in the row's padding: it is computed
+// from whatever is there and stored there.
 template <bool REF, typename P>
 __device__ __forceinline__ void pull_pair(const P& p, int x, int y, int z, V2 (&d)[Q]) {
   const int nx = p.nx(), pitch = p.pitch(), plane = p.plane();
   const unsigned fb = p.faces();
-  const int kl = int(fb & 3u), kr = int((fb >> 2) & 3u);
-  const bool first = x == 0, last = x + 2 >= nx;   // the pair holds x = 0 / x = nx - 1
-  const int nr = nx - 1 - x;                        // which node is at nx - 1
   if (y > 0 && y < p.ny() - 1 && z > 0 && z < p.nz() - 1) {
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      const __half* u = p.up(q);
-      if (cx(q) == 0) d[q] = ld2(u);
-      else d[q] = V2(ld1(u), ld1(u + 1));
-    }
-    if (REF) {
-      // Columns of upwind nodes (e_y, e_z), each one 128-bit reference load
-      // for the pair's own x and, where the column's directions have e_x != 0,
-      // a 64-bit load on either side.
-#pragma unroll
-      for (int c = 0; c < Q; ++c) {
-        if (cx(c) != 0) continue;
-        const uint2* rc = p.ref - (cz(c) * plane + cy(c) * pitch);
-        const uint4 w = *reinterpret_cast<const uint4*>(rc);
-        const float2 a0 = __half22float2(*reinterpret_cast<const __half2*>(&w.x));
-        const float2 b0 = __half22float2(*reinterpret_cast<const __half2*>(&w.y));
-        const float2 a1 = __half22float2(*reinterpret_cast<const __half2*>(&w.z));
-        const float2 b1 = __half22float2(*reinterpret_cast<const __half2*>(&w.w));
-        const RefT<V2> r{V2(a0.x, a1.x), V2(a0.y, a1.y), V2(b0.x, b1.x), V2(b0.y, b1.y)};
-        const V2 s = ref_sum(c, r);
-        d[c] = fma(V2(wt<float>(c)), s, d[c]);
-        if (cy(c) != 0 && cz(c) != 0) continue;
-        const float sl = ref_sum(c, ref1(rc - 1)), sr = ref_sum(c, ref1(rc + 2));
-        const float xl = ref1(rc - 1).vx, xr = ref1(rc + 2).vx;
-#pragma unroll
-        for (int q = 1; q < Q; ++q) {
-          if (cy(q) != cy(c) || cz(q) != cz(c) || cx(q) == 0) continue;
-          // e_x = 1: upwind nodes x - 1, x; e_x = -1: x + 1, x + 2
-          const V2 t = cx(q) == 1 ? V2(sl, lane0(s)) + V2(xl, lane0(r.vx))
-                                  : V2(lane1(s), sr) - V2(lane1(r.vx), xr);
-          d[q] = fma(V2(wt<float>(q)), t, d[q]);
-        }
-      }
-    }
-    if (first) {
-#pragma unroll
-      for (int q = 1; q < Q; ++q)
-        if (cx(q) == 1)
-          set0(d[q], xface_value<REF>(p, q, kl, 0, p.up(q),
-                                      p.ref - (cz(q) * plane + cy(q) * pitch + 1), nx));
-    }
-    if (last) {
-#pragma unroll
-      for (int q = 1; q < Q; ++q)
-        if (cx(q) == -1) {
-          const float v = xface_value<REF>(p, q, kr, nr, p.up(q) + nr,
-                                           p.ref - (cz(q) * plane + cy(q) * pitch - 1) + nr, -nx);
-          if (nr == 0) set0(d[q], v);
-          else set1(d[q], v);
-        }
+    if constexpr (REF) {
+      if (__any_sync(__activemask(), x == 0 || x + 2 >= nx)) pull_row<true, true>(p, x, d);
+      else pull_row<true, false>(p, x, d);
+    } else {
+      pull_row<false, false>(p, x, d);
+      xface_patch(p, x, d);
     }
     return;
   }
@@ -206,10 +257,10 @@ enum { PAIR_RN = 0, PAIR_SR = 1, PAIR_REF = 2 };
 __device__ __forceinline__ void st2(__half* p, __half2 v) { *reinterpret_cast<__half2*>(p) = v; }
 
 // The reference of the pair's nodes from density rho = rho0 + drho and
-// velocity u: rounded to FP16, stored by one 128-bit access; r receives the
+// velocity u: rounded to FP16 and stored by one 128-bit access; returns the
 // rounded values.
-__device__ __forceinline__ void ref_store2(uint2* p, const NodeOut<V2>& o, float rho0, float lam,
-                                           RefT<V2>& r) {
+__device__ __forceinline__ RefT<V2> ref_store2(uint2* p, const NodeOut<V2>& o, float rho0,
+                                               float lam) {
   const V2 r3 = mulr(V2(3.0f * lam), o.rho);
   const V2 dr = mulr(V2(lam), o.rho - V2(rho0));
   const V2 vx = mulr(r3, o.ux), vy = mulr(r3, o.uy), vz = mulr(r3, o.uz);
@@ -225,46 +276,53 @@ __device__ __forceinline__ void ref_store2(uint2* p, const NodeOut<V2>& o, float
   *reinterpret_cast<uint4*>(p) = w;
   const float2 fa0 = __half22float2(a0), fb0 = __half22float2(b0), fa1 = __half22float2(a1),
                fb1 = __half22float2(b1);
-  r = {V2(fa0.x, fa1.x), V2(fa0.y, fa1.y), V2(fb0.x, fb1.x), V2(fb0.y, fb1.y)};
+  return {V2(fa0.x, fa1.x), V2(fa0.y, fa1.y), V2(fb0.x, fb1.x), V2(fb0.y, fb1.y)};
 }
 
-// Blocks of 256 threads per SM the pair kernels are compiled for: at most 80
-// registers a thread, which all but the forced F16R kernels (one correction
-// per population: all 19 inputs live to the end) hold without spills in the
-// steps between checks; those take up to 128.
-constexpr int pair_min_blocks(bool ref, bool force) { return ref && force ? 2 : 3; }
+// Blocks of 256 threads per SM the pair kernels are compiled for: up to 80
+// registers a thread, for F16R up to 128, which it needs to hold a column's
+// references without spills (256^3: 340 us a step, against 352 with 80 and 373
+// with 64 registers; F16S with 64 ran at 227 against 224 us there and 31.5
+// against 30.0 on 128^3, its stochastic form 243 against 237).
+constexpr int pair_min_blocks(bool ref) { return ref ? 2 : 3; }
 
-// Collide the pair.  F16R with a body force takes one correction per
-// population (see step_f16r.cu).
+// Collide the pair and leave in d what is stored: the deviations, or (REF) the
+// remainders after the reference, which goes to rdst.  F16R with a body force
+// takes one correction per population (see step_f16r.cu).
 template <bool REF, bool FORCE>
 __device__ __forceinline__ void collide_pair(const CollideConst<float>& C, V2 (&d)[Q],
-                                             NodeOut<V2>& o) {
-  collide<V2, FORCE, !REF || !FORCE, log2_scale<__half>(), true>(C, d, o);
+                                             NodeOut<V2>& o, uint2* rdst) {
+  constexpr int L = log2_scale<__half>();
+  constexpr float LAM = float(1 << L);
+  if constexpr (!REF) {
+    collide_unit<V2, FORCE, true, L>(C, d, o);
+  } else if constexpr (FORCE) {
+    collide_unit<V2, true, false, L>(C, d, o);
+    const RefT<V2> r = ref_store2(rdst, o, C.rho0, LAM);
+#pragma unroll
+    for (int q = 0; q < Q; ++q) d[q] = fma(V2(-wt<float>(q)), ref_sum(q, r), d[q]);
+  } else {
+    collide_unit<V2, false, true, L>(
+        C, d, o, [&](const NodeOut<V2>& n) { return ref_store2(rdst, n, C.rho0, LAM); });
+  }
 }
 
-// Store the pair: dst(q) is its slot of direction q, rdst its reference slot
-// (PAIR_REF), i the index of its first node, step the lattice's steps done
-// before this one (the random bits depend on these two and the direction
-// only, so a lattice alone and in a batch rounds alike).
-template <int FORM, typename Dst>
-__device__ __forceinline__ void store_pair(const CollideConst<float>& C, V2 (&d)[Q],
-                                           const NodeOut<V2>& o, Dst&& dst, uint2* rdst, int i,
+// Store the pair: dst(q) is its slot of direction q, i the index of its first
+// node, step the lattice's steps done before this one (the random bits depend
+// on these two and the direction only, so a lattice alone and in a batch
+// rounds alike); sr: stochastic rounding.
+template <typename Dst>
+__device__ __forceinline__ void store_pair(const V2 (&d)[Q], bool sr, Dst&& dst, int i,
                                            unsigned step) {
-  if constexpr (FORM == PAIR_RN) {
+  if (!sr) {
 #pragma unroll
     for (int q = 0; q < Q; ++q) st2(dst(q), __float22half2_rn(d[q].v));
-  } else {
-    if constexpr (FORM == PAIR_REF) {
-      RefT<V2> r;
-      ref_store2(rdst, o, C.rho0, float(1 << log2_scale<__half>()), r);
-#pragma unroll
-      for (int q = 0; q < Q; ++q) d[q] = fma(V2(-wt<float>(q)), ref_sum(q, r), d[q]);
-    }
-    uint32_t state = sr_seed(uint32_t(i), step);
-#pragma unroll
-    for (int q = 0; q < Q; ++q)
-      *reinterpret_cast<uint32_t*>(dst(q)) = enc16_sr2(lane0(d[q]), lane1(d[q]), state);
+    return;
   }
+  uint32_t state = sr_seed(uint32_t(i), step);
+#pragma unroll
+  for (int q = 0; q < Q; ++q)
+    *reinterpret_cast<uint32_t*>(dst(q)) = enc16_sr2(lane0(d[q]), lane1(d[q]), state);
 }
 
 // The pair's part of the check-step sums; n1: the second node exists.
@@ -284,7 +342,7 @@ struct PairExtra {
 
 // One time step of a lone lattice; the block is pair_width() threads along x.
 template <int FORM, bool FORCE, bool CHECK>
-__global__ void __launch_bounds__(256, pair_min_blocks(FORM == PAIR_REF, FORCE))
+__global__ void __launch_bounds__(256, pair_min_blocks(FORM == PAIR_REF))
     step_pair_kernel(const StepArgs<__half, float> a, const PairExtra e) {
   pdl_enter();
   const int x = 2 * int(blockIdx.x * blockDim.x + threadIdx.x);
@@ -299,9 +357,8 @@ __global__ void __launch_bounds__(256, pair_min_blocks(FORM == PAIR_REF, FORCE))
     NodeOut<V2> o;
     const LonePair p{a, FORM == PAIR_REF ? e.ref_src + i : nullptr, i};
     pull_pair<FORM == PAIR_REF>(p, x, y, z, d);
-    collide_pair<FORM == PAIR_REF, FORCE>(a.C, d, o);
-    store_pair<FORM>(a.C, d, o, [&](int q) { return a.dstq[q] + i; },
-                     FORM == PAIR_REF ? e.ref_dst + i : nullptr, i, e.step);
+    collide_pair<FORM == PAIR_REF, FORCE>(a.C, d, o, e.ref_dst + i);
+    store_pair(d, FORM != PAIR_RN, [&](int q) { return a.dstq[q] + i; }, i, e.step);
     if (CHECK)
       check_pair(sums, o, a.C.rho0, static_cast<float*>(a.cb.uprev) + i, int64_t(a.plane) * a.nz,
                  x + 1 < a.nx);

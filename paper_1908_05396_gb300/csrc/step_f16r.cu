@@ -101,16 +101,24 @@ __device__ __forceinline__ void pull_node_ref(const StepArgs<__half, float>& a, 
   }
 }
 
-// Collide the node and store it.
+// Collide the node and store it (as collide_pair and store_pair).
 template <bool FORCE, bool UNIT>
 __device__ __forceinline__ void collide_store_ref(const StepArgs<__half, float>& a,
                                                   const RefArgs& r, int i, unsigned step,
                                                   float (&d)[Q], NodeOut<float>& o) {
-  collide<float, FORCE, !FORCE, LOG2LAM, UNIT>(a.C, d, o);
-  RefT<float> rr;
-  r.ref_dst[i] = ref_make(o.rho - a.C.rho0, o.rho, o.ux, o.uy, o.uz, rr);
+  auto reference = [&](const NodeOut<float>& n) {
+    RefT<float> t;
+    r.ref_dst[i] = ref_make(n.rho - a.C.rho0, n.rho, n.ux, n.uy, n.uz, t);
+    return t;
+  };
+  if constexpr (UNIT && !FORCE) {
+    collide_unit<float, false, true, LOG2LAM>(a.C, d, o, reference);
+  } else {
+    collide<float, FORCE, !FORCE, LOG2LAM, UNIT>(a.C, d, o);
+    const RefT<float> t = reference(o);
 #pragma unroll
-  for (int q = 0; q < Q; ++q) d[q] = plus_ref(d[q], q, rr, -1.0f);
+    for (int q = 0; q < Q; ++q) d[q] = plus_ref(d[q], q, t, -1.0f);
+  }
   store_sr1([&](int q) { return a.dstq[q] + i; }, d, uint32_t(i), step);
 }
 
