@@ -29,6 +29,7 @@ struct LatDesc {
   int slot;            // row of this lattice in the batch's reduction array
   unsigned step_offset;  // lattice steps minus batch steps (seeds stochastic rounding)
   int sround;            // F16S: stores rounded stochastically
+  int threads;           // threads per block the tiles were cut for; 0: not usable
   R lidc[Q];
   CollideConst<R> C;
 };
@@ -143,16 +144,14 @@ __device__ __forceinline__ void batch_tiles(Get get, const int* __restrict__ own
       w_next = coord[t + gridDim.x];
     }
     const int tx = int(w & 0xffu), ty = int((w >> 8) & 0xfffu), tz = int(w >> 20);
-    // Self-check of the tables before any access through them.
+    // Self-check of the tables before any access through them.  What does not
+    // depend on the tile was checked when the descriptor was filled
+    // (usable_desc), which leaves `threads` 0 otherwise.
     bool ok = li >= 0 && li < nlat;
     const LatDesc<R>& L = get(ok ? li : 0);
     if (ok)
-      ok = L.buf[0] != nullptr && L.buf[1] != nullptr && tx < L.tiles_x && ty < L.tiles_y &&
-           L.tw_log2 >= 0 && L.tw_log2 <= 10 && (1 << L.tw_log2) <= int(blockDim.x * blockDim.y) &&
-           (int(blockDim.x * blockDim.y) & ((1 << L.tw_log2) - 1)) == 0 &&
-           zc >= 1 && tz * zc < L.nz && L.pitch >= L.nx && L.plane == L.pitch * L.ny &&
-           L.qstride >= int64_t(L.plane) * L.nz && 19 * L.qstride < (int64_t(1) << 31) &&
-           (L.C.has_force != 0) == FORCE && (!REF || (L.ref[0] != nullptr && L.ref[1] != nullptr));
+      ok = L.threads == int(blockDim.x * blockDim.y) && tx < L.tiles_x && ty < L.tiles_y &&
+           zc >= 1 && tz * zc < L.nz && (L.C.has_force != 0) == FORCE;
     if (!ok) {  // block-uniform: skip the tile, report it
       if (threadIdx.x == 0 && threadIdx.y == 0) atomicOr(&hdr->err, 1);
       continue;
@@ -233,12 +232,22 @@ inline int batch_grid(const void* kernel, dim3 block, int per_sm, int sms) {
 // form; batches reserve disjoint ranges of it.
 constexpr int BATCH_CONST_BYTES = 60 * 1024;
 
+// Whether a descriptor is consistent, for blocks of `threads` threads.
+template <typename R>
+bool usable_desc(const LatDesc<R>& L, int threads, bool ref) {
+  return L.buf[0] && L.buf[1] && L.tw_log2 >= 0 && L.tw_log2 <= 10 &&
+         (1 << L.tw_log2) <= threads && threads % (1 << L.tw_log2) == 0 && L.pitch >= L.nx &&
+         L.plane == L.pitch * L.ny && L.qstride >= int64_t(L.plane) * L.nz &&
+         19 * L.qstride < (int64_t(1) << 31) && (!ref || (L.ref[0] && L.ref[1]));
+}
+
 // Host-side fill of one descriptor (constants converted once, in double).
 template <typename R>
 void fill_desc_t(void* out, double lam, const Geom& g, const PhysParams& P, const void* cur,
                  const void* other,
                  const void* ref_cur, const void* ref_other, void* uprev, int tiles_x,
-                 int tiles_y, int tw_log2, int slot, unsigned step_offset) {
+                 int tiles_y, int tw_log2, int slot, unsigned step_offset, int threads,
+                 bool ref) {
   LatDesc<R> L{};
   L.buf[0] = cur;
   L.buf[1] = other;
@@ -262,6 +271,7 @@ void fill_desc_t(void* out, double lam, const Geom& g, const PhysParams& P, cons
     L.lidc[q] = R(6.0 * wt<double>(q) * g.rho0 * lam *
                   (cx(q) * g.U[0] + cy(q) * g.U[1] + cz(q) * g.U[2]));
   L.C = make_const<R>(P, lam);
+  L.threads = usable_desc(L, threads, ref) ? threads : 0;
   *static_cast<LatDesc<R>*>(out) = L;
 }
 
@@ -313,10 +323,11 @@ void fill_desc_t(void* out, double lam, const Geom& g, const PhysParams& P, cons
   int desc_capacity_##SUFFIX() { return int(BATCH_CONST_BYTES / sizeof(LatDesc<R>)); }         \
   void fill_desc_##SUFFIX(void* out, const Geom& g, const PhysParams& P, const void* cur,        \
                           const void* other, const void* ref_cur, const void* ref_other,       \
-                          void* uprev, int tx, int ty, int twl, int slot, unsigned so) {       \
+                          void* uprev, int tx, int ty, int twl, int slot, unsigned so,         \
+                          int threads) {                                                       \
     /* FP16 storage (F16S, F16R) carries its deviations scaled by 1024 */                    \
     fill_desc_t<R>(out, double(1 << log2_scale<S>()), g, P, cur, other, ref_cur,             \
-                   ref_other, uprev, tx, ty, twl, slot, so);                                   \
+                   ref_other, uprev, tx, ty, twl, slot, so, threads, REF);                     \
   }                                                                                            \
   void desc_set_sround_##SUFFIX(void* out, int on) {                                           \
     static_cast<LatDesc<R>*>(out)->sround = on;                                                \

@@ -152,20 +152,20 @@ cudaError_t upload_desc(clbm_dtype t, const void* host, int base, int n) {
 }
 
 void fill_desc(clbm_dtype t, void* out, const clbm_ctx* h, int tx, int ty, int twl, int slot,
-               unsigned so) {
+               unsigned so, int threads) {
   const void* cur = h->buf[h->cur];
   const void* other = h->buf[1 - h->cur];
   // F16R: the reference moments travel with their population buffers
   const void* rcur = h->ref[h->cur];
   const void* rother = h->ref[1 - h->cur];
   if (t == CLBM_F64)
-    fill_desc_f64(out, h->g, h->P, cur, other, rcur, rother, h->uprev, tx, ty, twl, slot, so);
+    fill_desc_f64(out, h->g, h->P, cur, other, rcur, rother, h->uprev, tx, ty, twl, slot, so, threads);
   else if (t == CLBM_F32)
-    fill_desc_f32(out, h->g, h->P, cur, other, rcur, rother, h->uprev, tx, ty, twl, slot, so);
+    fill_desc_f32(out, h->g, h->P, cur, other, rcur, rother, h->uprev, tx, ty, twl, slot, so, threads);
   else if (t == CLBM_F16R)
-    fill_desc_f16r(out, h->g, h->P, cur, other, rcur, rother, h->uprev, tx, ty, twl, slot, so);
+    fill_desc_f16r(out, h->g, h->P, cur, other, rcur, rother, h->uprev, tx, ty, twl, slot, so, threads);
   else {
-    fill_desc_f16(out, h->g, h->P, cur, other, rcur, rother, h->uprev, tx, ty, twl, slot, so);
+    fill_desc_f16(out, h->g, h->P, cur, other, rcur, rother, h->uprev, tx, ty, twl, slot, so, threads);
     desc_set_sround_f16(out, h->sround ? 1 : 0);
   }
 }
@@ -355,7 +355,7 @@ int upload(clbm_batch_ctx* b) {
       // the lattice's step count minus the batch's: the kernels add the
       // batch's device-side count to recover the lattice's own
       const unsigned so = unsigned(uint64_t(h->steps) - uint64_t(b->steps));
-      fill_desc(b->dtype, stage + size_t(nlat) * b->desc_bytes, h, tx, ty, twl, s, so);
+      fill_desc(b->dtype, stage + size_t(nlat) * b->desc_bytes, h, tx, ty, twl, s, so, threads);
       for (int kz = 0; kz < tz; ++kz)
         for (int ky = 0; ky < ty; ++ky)
           for (int kx = 0; kx < tx; ++kx) {
@@ -527,6 +527,8 @@ int check_tables(clbm_batch_ctx* b) {
 }
 
 }  // namespace
+
+cudaStream_t clbm::batch_stream(clbm_batch b) { return b->stream; }
 
 extern "C" {
 
@@ -760,7 +762,7 @@ int clbm_batch_autotune(clbm_batch b, int steps, int* block_x, int* block_y, int
   const int64_t bsteps0 = b->steps;
   const dim3 block0 = b->block;
   const int zc0 = b->zc, bps0 = b->blocks_per_sm;
-  const int shapes[][2] = {{32, 2}, {32, 4}, {32, 8}, {64, 2}, {64, 4}, {128, 1}, {128, 2}};
+  const int shapes[][2] = {{16, 4}, {16, 8}, {32, 2}, {32, 4}, {32, 8}, {64, 4}};
   const int zcs[] = {1, 2, 4};
   const int bpss[] = {4, 6, 8};
   const bool cap0 = b->cap;
@@ -814,7 +816,7 @@ int clbm_batch_autotune(clbm_batch b, int steps, int* block_x, int* block_y, int
   // lattice): block x kernel variant x streams.
   int bmode = 0, pbx = 32, pby = 2, pnpt = 5, pst = 4;
   if (b->dtype != CLBM_F16R && !any_sround(b)) {
-    const int pshapes[][2] = {{32, 2}, {32, 4}, {64, 2}};
+    const int pshapes[][2] = {{16, 4}, {32, 2}, {32, 4}};
     const int pnpts[] = {5, 1};
     const int pstreams[] = {2, 4, 8};
     if (err == cudaSuccess) err = ensure_streams(b, 8);

@@ -48,14 +48,67 @@ clbm_alloc_fn g_alloc_fn = nullptr;
 clbm_free_fn g_free_fn = nullptr;
 void* g_alloc_user = nullptr;
 
-// A long-lived device buffer of h, from its allocator or cudaMalloc.
+// Pinned copies of the check sums (CHECK_BYTES each): the first 64 lattices of
+// the process share one pinned slab, because a cudaMallocHost and cudaFreeHost
+// pair costs 0.33 ms, as much as the rest of a small lattice's creation.
+// Slots are handed back at destruction; the slab (130 KB) stays.
+constexpr int PINNED_SLOTS = 64;
+constexpr size_t PINNED_STRIDE = (CHECK_BYTES + 63) / 64 * 64;
+std::mutex g_pinned_mu;
+char* g_pinned = nullptr;
+bool g_pinned_used[PINNED_SLOTS] = {};
+
+double* pinned_take() {
+  {
+    std::lock_guard<std::mutex> lk(g_pinned_mu);
+    if (!g_pinned) {
+      void* p = nullptr;
+      if (cudaHostAlloc(&p, PINNED_SLOTS * PINNED_STRIDE, cudaHostAllocPortable) == cudaSuccess)
+        g_pinned = static_cast<char*>(p);
+      else
+        cudaGetLastError();
+    }
+    for (int k = 0; g_pinned && k < PINNED_SLOTS; ++k)
+      if (!g_pinned_used[k]) {
+        g_pinned_used[k] = true;
+        return reinterpret_cast<double*>(g_pinned + size_t(k) * PINNED_STRIDE);
+      }
+  }
+  void* p = nullptr;
+  return cudaMallocHost(&p, CHECK_BYTES) == cudaSuccess ? static_cast<double*>(p) : nullptr;
+}
+
+void pinned_give(double* p) {
+  if (!p) return;
+  {
+    std::lock_guard<std::mutex> lk(g_pinned_mu);
+    const char* c = reinterpret_cast<const char*>(p);
+    if (g_pinned && c >= g_pinned && c < g_pinned + PINNED_SLOTS * PINNED_STRIDE) {
+      g_pinned_used[size_t(c - g_pinned) / PINNED_STRIDE] = false;
+      return;
+    }
+  }
+  cudaFreeHost(p);
+}
+
+size_t dev_round(size_t bytes) { return (bytes + 255) / 256 * 256; }
+
+// A long-lived device buffer of h, from its allocator or its one cudaMalloc
+// block (each cudaMalloc and cudaFree pair costs 0.14 ms, and a lattice has
+// four to six buffers).
 int dev_alloc(clbm_ctx* h, void** p, size_t bytes, const char* what) {
   *p = nullptr;
   if (!h->alloc_fn) {
-    if (cudaMalloc(p, bytes) != cudaSuccess) {
-      *p = nullptr;
-      return fail(h, CLBM_ERR_OOM, std::string(what) + " allocation failed");
+    if (!h->slab) {
+      void* b = nullptr;
+      if (cudaMalloc(&b, h->slab_bytes) != cudaSuccess)
+        return fail(h, CLBM_ERR_OOM, std::string(what) + " allocation failed");
+      h->slab = static_cast<char*>(b);
     }
+    if (h->slab_used + dev_round(bytes) > h->slab_bytes)
+      return fail(h, CLBM_ERR_OOM, std::string(what) + ": beyond the lattice's allocation");
+    *p = h->slab + h->slab_used;
+    h->slab_used += dev_round(bytes);
     return CLBM_OK;
   }
   void* q = h->alloc_fn(bytes, h->device, h->stream, h->alloc_user);
@@ -71,9 +124,7 @@ int dev_alloc(clbm_ctx* h, void** p, size_t bytes, const char* what) {
 }
 
 void dev_free(clbm_ctx* h, void* p, size_t bytes) {
-  if (!p) return;
-  if (h->free_fn) h->free_fn(p, bytes, h->device, h->stream, h->alloc_user);
-  else cudaFree(p);
+  if (p && h->free_fn) h->free_fn(p, bytes, h->device, h->stream, h->alloc_user);
 }
 
 #define CK(h, expr)                                   \
@@ -224,12 +275,15 @@ int clbm_create(const clbm_domain* d, double K, double n, const double U_lid[3],
   }
   h->pop_bytes = pop_bytes;
   h->uprev_bytes = 3 * size_t(g.plane) * g.nz * h->rsize;
+  h->ref_bytes = dtype == CLBM_F16R ? f16r_ref_bytes(g.plane * g.nz) : 0;
+  const size_t nbuf = h->in_place ? 1 : 2;
+  h->slab_bytes = nbuf * (dev_round(pop_bytes) + dev_round(h->ref_bytes)) +
+                   dev_round(h->uprev_bytes) + dev_round(CHECK_BYTES);
   int rc = CLBM_OK;
   for (int b = 0; b < (h->in_place ? 1 : 2) && rc == CLBM_OK; ++b)
     rc = dev_alloc(h, &h->buf[b], pop_bytes, "population buffer");
   if (rc != CLBM_OK) return cleanup(rc, "clbm_create");
   if (dtype == CLBM_F16R) {
-    h->ref_bytes = f16r_ref_bytes(g.plane * g.nz);
     for (int b = 0; b < 2 && rc == CLBM_OK; ++b) {
       rc = dev_alloc(h, &h->ref[b], h->ref_bytes, "reference buffer");
       if (rc == CLBM_OK && cudaMemsetAsync(h->ref[b], 0, h->ref_bytes, h->stream) != cudaSuccess)
@@ -242,8 +296,8 @@ int clbm_create(const clbm_domain* d, double K, double n, const double U_lid[3],
   rc = dev_alloc(h, reinterpret_cast<void**>(&h->acc), CHECK_BYTES, "reduction buffer");
   if (rc != CLBM_OK) return cleanup(rc, "clbm_create");
   h->flag = reinterpret_cast<int*>(h->acc + 4 * CHECK_ROWS);
-  e = cudaMallocHost(&h->host, CHECK_BYTES);
-  if (e != cudaSuccess) return cleanup(CLBM_ERR_OOM, "pinned buffer allocation failed");
+  h->host = pinned_take();
+  if (!h->host) return cleanup(CLBM_ERR_OOM, "pinned buffer allocation failed");
   std::memset(h->host, 0, CHECK_BYTES);
   e = cudaEventCreateWithFlags(&h->check_done, cudaEventDisableTiming);
   if (e != cudaSuccess) return cleanup(CLBM_ERR_CUDA, cudaGetErrorString(e));
@@ -412,8 +466,6 @@ static int state_io(clbm_handle h, double* out, const double* in) {
       case CLBM_F32: e = launch_export_aa_f32(h->buf[0], h->g, h->g.rho0, isc, h->layout, dev, h->stream); break;
       default: e = launch_export_aa_f16(h->buf[0], h->g, h->g.rho0, isc, h->layout, dev, h->stream); break;
     }
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(out, dev, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
   } else {
     switch (h->dtype) {
       case CLBM_F64: e = launch_export_f64(h->buf[h->cur], h->g, h->g.rho0, isc, dev, h->stream); break;
@@ -423,9 +475,9 @@ static int state_io(clbm_handle h, double* out, const double* in) {
         break;
       default: e = launch_export_f16(h->buf[h->cur], h->g, h->g.rho0, isc, dev, h->stream); break;
     }
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(out, dev, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
   }
+  if (out && e == cudaSuccess)
+    e = cudaMemcpyAsync(out, dev, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
   cudaFreeAsync(dev, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   CK(h, e);
@@ -650,7 +702,8 @@ int clbm_destroy(clbm_handle h) {
   }
   dev_free(h, h->uprev, h->uprev_bytes);
   dev_free(h, h->acc, CHECK_BYTES);
-  if (h->host) cudaFreeHost(h->host);
+  if (h->slab) cudaFree(h->slab);
+  pinned_give(h->host);
   if (h->check_done) cudaEventDestroy(h->check_done);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
   delete h;

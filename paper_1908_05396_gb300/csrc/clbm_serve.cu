@@ -19,6 +19,7 @@
 #include <cstring>
 #include <deque>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <string>
@@ -50,10 +51,20 @@ struct Active {
   int since_best = 0;
 };
 
+// Host memory of one request's fields: rho, u and gamma_dot, 5 N values.
+struct FieldsBuf {
+  std::unique_ptr<double[]> v;
+  size_t n = 0;
+};
+
 struct Done {
   clbm_result res;
-  std::vector<double> rho, u, gd;
+  FieldsBuf fields;
 };
+
+// Released fields kept for later requests, up to this many bytes: a copy into
+// memory that was touched before runs at 180 GB/s, into new pages at 20.
+constexpr size_t SPARE_BYTES = size_t(512) << 20;
 
 }  // namespace
 
@@ -73,6 +84,8 @@ struct clbm_server_ctx {
   std::deque<Pending> queue;
   std::vector<Active> active;
   std::map<int64_t, Done> done;
+  std::vector<FieldsBuf> spare;     // released fields (at most SPARE_BYTES)
+  size_t spare_bytes = 0;
   double used = 0;
   bool stop = false;
   int64_t next_id = 1;
@@ -95,6 +108,37 @@ int sfail(clbm_server_ctx* s, int code, const std::string& m) {
   if (s) s->err = m;
   clbm::set_unbound_error(m.c_str());
   return code;
+}
+
+// Memory for n values: a spare buffer at most twice as large, or a new one.
+FieldsBuf take_fields(clbm_server_ctx* s, size_t n) {
+  size_t best = s->spare.size();
+  for (size_t k = 0; k < s->spare.size(); ++k)
+    if (s->spare[k].n >= n && s->spare[k].n <= 2 * n &&
+        (best == s->spare.size() || s->spare[k].n < s->spare[best].n))
+      best = k;
+  FieldsBuf f;
+  if (best < s->spare.size()) {
+    f = std::move(s->spare[best]);
+    s->spare.erase(s->spare.begin() + long(best));
+    s->spare_bytes -= f.n * sizeof(double);
+    return f;
+  }
+  // (cleared: touching new pages here is cheaper than inside the copy)
+  f.v.reset(new (std::nothrow) double[n]());
+  f.n = f.v ? n : 0;
+  return f;
+}
+
+void give_fields(clbm_server_ctx* s, FieldsBuf f) {
+  if (!f.v || s->spare_bytes + f.n * sizeof(double) > SPARE_BYTES) return;
+  const size_t bytes = f.n * sizeof(double);
+  try {
+    s->spare.push_back(std::move(f));
+    s->spare_bytes += bytes;
+  } catch (const std::bad_alloc&) {
+    // not kept
+  }
 }
 
 // Device bytes of one lattice of this form (two population buffers, the
@@ -124,14 +168,12 @@ void finish(clbm_server_ctx* s, Active& a, int status, double R, double mass, in
   d.res.N = int64_t(a.req.dom.nx) * a.req.dom.ny * a.req.dom.nz;
   if (a.req.keep_fields && a.h && status != CLBM_SOLVE_ERROR) {
     const size_t N = size_t(d.res.N);
-    d.rho.resize(N);
-    d.u.resize(3 * N);
-    d.gd.resize(N);
-    if (clbm_fields(a.h, d.rho.data(), d.u.data(), d.gd.data()) != CLBM_OK) {
+    d.fields = take_fields(s, 5 * N);
+    double* f = d.fields.v.get();
+    if (!f || clbm_fields(a.h, f, f + N, f + 4 * N) != CLBM_OK) {
       d.res.status = CLBM_SOLVE_ERROR;
-      d.rho.clear();
-      d.u.clear();
-      d.gd.clear();
+      give_fields(s, std::move(d.fields));
+      d.fields = FieldsBuf{};
     }
   }
   if (a.h) clbm_destroy(a.h);  // leaves the batch, frees its memory
@@ -171,7 +213,8 @@ void worker_loop(clbm_server_ctx* s) {
       a.bytes = size_t(need);
       clbm_domain dom = p.req.dom;
       dom.check_interval = s->check_interval;
-      dom.stream = nullptr;
+      // the lattice is only ever stepped by the batch
+      dom.stream = clbm::batch_stream(s->batch);
       dom.in_place = 0;   // the batched step works on two buffers
       int rc = clbm_create(&dom, p.req.K, p.req.n, p.req.U_lid, p.req.body_force, s->dtype, &a.h);
       if (rc == CLBM_OK && s->sround) rc = clbm_set_rounding(a.h, CLBM_ROUND_STOCHASTIC);
@@ -344,17 +387,22 @@ int clbm_server_fields(clbm_server s, int64_t id, double* rho, double* u, double
   auto it = s->done.find(id);
   if (it == s->done.end()) return sfail(s, CLBM_ERR_ARG, "unknown or unfinished request");
   const Done& d = it->second;
-  if (d.rho.empty()) return sfail(s, CLBM_ERR_ARG, "request was not submitted with keep_fields");
-  if (rho) std::memcpy(rho, d.rho.data(), d.rho.size() * sizeof(double));
-  if (u) std::memcpy(u, d.u.data(), d.u.size() * sizeof(double));
-  if (gamma_dot) std::memcpy(gamma_dot, d.gd.data(), d.gd.size() * sizeof(double));
+  const double* f = d.fields.v.get();
+  if (!f) return sfail(s, CLBM_ERR_ARG, "request was not submitted with keep_fields");
+  const size_t N = size_t(d.res.N);
+  if (rho) std::memcpy(rho, f, N * sizeof(double));
+  if (u) std::memcpy(u, f + N, 3 * N * sizeof(double));
+  if (gamma_dot) std::memcpy(gamma_dot, f + 4 * N, N * sizeof(double));
   return CLBM_OK;
 }
 
 int clbm_server_release(clbm_server s, int64_t id) {
   if (!valid(s)) return sfail(s, CLBM_ERR_ARG, "invalid server");
   std::lock_guard<std::mutex> lk(s->mu);
-  if (!s->done.erase(id)) return sfail(s, CLBM_ERR_ARG, "unknown or unfinished request");
+  auto it = s->done.find(id);
+  if (it == s->done.end()) return sfail(s, CLBM_ERR_ARG, "unknown or unfinished request");
+  give_fields(s, std::move(it->second.fields));
+  s->done.erase(it);
   return CLBM_OK;
 }
 

@@ -49,6 +49,9 @@ struct clbm_ctx {
   clbm_free_fn free_fn = nullptr;
   void* alloc_user = nullptr;
   size_t pop_bytes = 0, ref_bytes = 0, uprev_bytes = 0;  // sizes handed to free_fn
+  // without an external allocator: one device allocation holds every buffer
+  char* slab = nullptr;
+  size_t slab_used = 0, slab_bytes = 0;
   std::string err;
 };
 
@@ -58,4 +61,6 @@ constexpr size_t CHECK_BYTES = CHECK_SUMS_BYTES + sizeof(double);  // and the tw
 
 // Queue one step of a handle (clbm_lib.cu).
 cudaError_t handle_dispatch_step(clbm_ctx* h, bool check);
+// The stream of a batch (clbm_batch.cu).
+cudaStream_t batch_stream(clbm_batch b);
 }  // namespace clbm

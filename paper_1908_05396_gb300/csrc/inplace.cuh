@@ -125,46 +125,40 @@ __global__ void __launch_bounds__(256) fields_aa_kernel(const StepArgs<S, R> a,
 // layout 1 holds them at the downstream node, or at the node itself in the
 // opposite slot where the downstream side is a wall or the lid.
 template <typename S>
-__global__ void export_aa_kernel(const S* __restrict__ A, Geom g, double rho0, double inv_scale,
-                                 int layout, double* __restrict__ out) {
-  const int64_t N = int64_t(g.nx) * g.ny * g.nz;
-  const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (t >= N * Q) return;
-  const int q = int(t / N);
-  const int64_t k = t - int64_t(q) * N;
-  const int x = int(k % g.nx), y = int((k / g.nx) % g.ny), z = int(k / (int64_t(g.nx) * g.ny));
-  const int64_t i = int64_t(z) * g.plane + int64_t(y) * g.pitch + x;
-  int64_t j = int64_t(c_opp[q]) * g.qstride + i;  // layout 0, or a bounced value
-  if (layout == 1) {
-    const int ex = c_ex[q], ey = c_ey[q], ez = c_ez[q];
-    const bool ox = (ex == -1 && x == 0) || (ex == 1 && x == g.nx - 1);
-    const bool oy = (ey == -1 && y == 0) || (ey == 1 && y == g.ny - 1);
-    const bool oz = (ez == -1 && z == 0) || (ez == 1 && z == g.nz - 1);
-    const int kx = ox ? int((g.facebits >> (ex == -1 ? 0 : 2)) & 3u) : int(BC_PERIODIC);
-    const int ky = oy ? int((g.facebits >> (ey == -1 ? 4 : 6)) & 3u) : int(BC_PERIODIC);
-    const int kz = oz ? int((g.facebits >> (ez == -1 ? 8 : 10)) & 3u) : int(BC_PERIODIC);
-    if (kx == BC_PERIODIC && ky == BC_PERIODIC && kz == BC_PERIODIC) {
-      const int xd = ox ? x + ex - ex * g.nx : x + ex, yd = oy ? y + ey - ey * g.ny : y + ey,
-                zd = oz ? z + ez - ez * g.nz : z + ez;
-      j = int64_t(q) * g.qstride + int64_t(zd) * g.plane + int64_t(yd) * g.pitch + xd;
-    }
+__global__ void __launch_bounds__(128) export_aa_kernel(const S* __restrict__ A, Geom g,
+                                                        double rho0, double inv_scale, int layout,
+                                                        double* __restrict__ out) {
+  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
+  const int z = blockIdx.z;
+  if (x >= g.nx || y >= g.ny) return;
+  const int64_t N = int64_t(g.nx) * g.ny * g.nz, k = (int64_t(z) * g.ny + y) * g.nx + x;
+  const int pitch = g.pitch, plane = int(g.plane), i = z * plane + y * pitch + x;
+  const Faces f = faces_of(x, y, z, g.nx, g.ny, g.nz, pitch, plane, g.facebits);
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    // the opposite slot: layout 0, or a value bounced downstream
+    const bool own = layout == 0 || (f.wall & up_faces(opp(q))) != 0;
+    const int j = i + (cz(q) * plane + cy(q) * pitch + cx(q)) + up_wrap(f, opp(q));
+    const S v = (A + (own ? opp(q) : q) * g.qstride)[own ? i : j];
+    out[q * N + k] =
+        double(Codec<S, double>::dec(v, inv_scale)) * inv_scale + wt<double>(q) * rho0;
   }
-  out[t] = double(Codec<S, double>::dec(A[j], inv_scale)) * inv_scale + wt<double>(q) * rho0;
 }
 
 // Import a state f~ into layout 0.
 template <typename S>
-__global__ void import_aa_kernel(const double* __restrict__ in, Geom g, double rho0,
-                                 double inv_scale, S* __restrict__ A) {
-  const int64_t N = int64_t(g.nx) * g.ny * g.nz;
-  const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (t >= N * Q) return;
-  const int q = int(t / N);
-  const int64_t k = t - int64_t(q) * N;
-  const int x = int(k % g.nx), y = int((k / g.nx) % g.ny), z = int(k / (int64_t(g.nx) * g.ny));
+__global__ void __launch_bounds__(128) import_aa_kernel(const double* __restrict__ in, Geom g,
+                                                        double rho0, double scale,
+                                                        S* __restrict__ A) {
+  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
+  const int z = blockIdx.z;
+  if (x >= g.nx || y >= g.ny) return;
+  const int64_t N = int64_t(g.nx) * g.ny * g.nz, k = (int64_t(z) * g.ny + y) * g.nx + x;
   const int64_t i = int64_t(z) * g.plane + int64_t(y) * g.pitch + x;
-  A[int64_t(c_opp[q]) * g.qstride + i] =
-      Codec<S, double>::enc((in[t] - wt<double>(q) * rho0) / inv_scale, inv_scale);
+#pragma unroll
+  for (int q = 0; q < Q; ++q)
+    A[opp(q) * g.qstride + i] =
+        Codec<S, double>::enc((in[q * N + k] - wt<double>(q) * rho0) * scale, scale);
 }
 
 // ---- host-side launchers ------------------------------------------------------
@@ -229,20 +223,18 @@ cudaError_t launch_fields_aa_t(const void* buf, const Geom& g, const PhysParams&
 template <typename S>
 cudaError_t launch_export_aa_t(const void* buf, const Geom& g, double rho0, double inv_scale,
                                int layout, double* out, cudaStream_t st) {
-  const int64_t total = int64_t(g.nx) * g.ny * g.nz * Q;
-  const int b = 256;
-  export_aa_kernel<S><<<unsigned((total + b - 1) / b), b, 0, st>>>(
-      static_cast<const S*>(buf), g, rho0, inv_scale, layout, out);
+  const dim3 grid((g.nx + 31) / 32, (g.ny + 3) / 4, g.nz);
+  export_aa_kernel<S><<<grid, dim3(32, 4), 0, st>>>(static_cast<const S*>(buf), g, rho0,
+                                                    inv_scale, layout, out);
   return cudaGetLastError();
 }
 
 template <typename S>
 cudaError_t launch_import_aa_t(const double* in, const Geom& g, double rho0, double inv_scale,
                                void* buf, cudaStream_t st) {
-  const int64_t total = int64_t(g.nx) * g.ny * g.nz * Q;
-  const int b = 256;
-  import_aa_kernel<S><<<unsigned((total + b - 1) / b), b, 0, st>>>(in, g, rho0, inv_scale,
-                                                                   static_cast<S*>(buf));
+  const dim3 grid((g.nx + 31) / 32, (g.ny + 3) / 4, g.nz);
+  import_aa_kernel<S><<<grid, dim3(32, 4), 0, st>>>(in, g, rho0, 1.0 / inv_scale,
+                                                    static_cast<S*>(buf));
   return cudaGetLastError();
 }
 

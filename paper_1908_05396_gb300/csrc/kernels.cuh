@@ -177,12 +177,6 @@ __device__ __forceinline__ double* check_row(const CheckBufs& cb) {
 }
 
 // ---- the fused step ---------------------------------------------------------
-// Direction tables for the general pull, where the direction is a run-time value.
-static __constant__ signed char c_ex[Q] = {0, 1, -1, 0, 0, 0, 0, 1, -1, 1, -1, 1, -1, 1, -1, 0, 0, 0, 0};
-static __constant__ signed char c_ey[Q] = {0, 0, 0, 1, -1, 0, 0, 1, 1, -1, -1, 0, 0, 0, 0, 1, -1, 1, -1};
-static __constant__ signed char c_ez[Q] = {0, 0, 0, 0, 0, 1, -1, 0, 0, 0, 0, 1, 1, -1, -1, 1, 1, -1, -1};
-static __constant__ signed char c_opp[Q] = {0, 2, 1, 4, 3, 6, 5, 10, 9, 8, 7, 14, 13, 12, 11, 18, 17, 16, 15};
-
 // Everything one step launch needs, precomputed on the host in the math
 // precision R (no double arithmetic is left in the FP32 kernels).
 template <typename S, typename R>
@@ -436,33 +430,37 @@ __global__ void omega_nodes_kernel(CollideConst<R> C, const double* __restrict__
   if (gd) gd[k] = double(shear_rate(rinv, w, A, B));
 }
 
-// Stored populations <-> plain FP64 f in the unpadded layout [q][z][y][x].
+// Stored populations <-> plain FP64 f in the unpadded layout [q][z][y][x]: one
+// thread per node, all directions (one per population spent four 64-bit
+// divisions on its place, and the import a fifth on the scale, a power of two).
 template <typename S>
-__global__ void export_kernel(const S* __restrict__ src, Geom g, double rho0,
-                              double inv_scale, double* __restrict__ out) {
-  const int64_t N = int64_t(g.nx) * g.ny * g.nz;
-  const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (t >= N * Q) return;
-  const int q = int(t / N);
-  const int64_t k = t - int64_t(q) * N;
-  const int x = int(k % g.nx), y = int((k / g.nx) % g.ny), z = int(k / (int64_t(g.nx) * g.ny));
+__global__ void __launch_bounds__(128) export_kernel(const S* __restrict__ src, Geom g,
+                                                     double rho0, double inv_scale,
+                                                     double* __restrict__ out) {
+  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
+  const int z = blockIdx.z;
+  if (x >= g.nx || y >= g.ny) return;
+  const int64_t N = int64_t(g.nx) * g.ny * g.nz, k = (int64_t(z) * g.ny + y) * g.nx + x;
   const int64_t i = int64_t(z) * g.plane + int64_t(y) * g.pitch + x;
-  const double w = wt<double>(q);
-  out[t] = double(Codec<S, double>::dec(src[q * g.qstride + i], inv_scale)) * inv_scale + w * rho0;
+#pragma unroll
+  for (int q = 0; q < Q; ++q)
+    out[q * N + k] = double(Codec<S, double>::dec(src[q * g.qstride + i], inv_scale)) * inv_scale +
+                     wt<double>(q) * rho0;
 }
 
 template <typename S>
-__global__ void import_kernel(const double* __restrict__ in, Geom g, double rho0,
-                              double inv_scale, S* __restrict__ dst) {
-  const int64_t N = int64_t(g.nx) * g.ny * g.nz;
-  const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (t >= N * Q) return;
-  const int q = int(t / N);
-  const int64_t k = t - int64_t(q) * N;
-  const int x = int(k % g.nx), y = int((k / g.nx) % g.ny), z = int(k / (int64_t(g.nx) * g.ny));
+__global__ void __launch_bounds__(128) import_kernel(const double* __restrict__ in, Geom g,
+                                                     double rho0, double scale,
+                                                     S* __restrict__ dst) {
+  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
+  const int z = blockIdx.z;
+  if (x >= g.nx || y >= g.ny) return;
+  const int64_t N = int64_t(g.nx) * g.ny * g.nz, k = (int64_t(z) * g.ny + y) * g.nx + x;
   const int64_t i = int64_t(z) * g.plane + int64_t(y) * g.pitch + x;
-  const double w = wt<double>(q);
-  dst[q * g.qstride + i] = Codec<S, double>::enc((in[t] - w * rho0) / inv_scale, inv_scale);
+#pragma unroll
+  for (int q = 0; q < Q; ++q)
+    dst[q * g.qstride + i] =
+        Codec<S, double>::enc((in[q * N + k] - wt<double>(q) * rho0) * scale, scale);
 }
 
 // The arguments of a two-buffer step from src to dst.
@@ -592,23 +590,23 @@ cudaError_t launch_omega_nodes_t(const PhysParams& P, const double* rho, const d
   return cudaGetLastError();
 }
 
+inline dim3 node_grid(const Geom& g) {
+  return dim3((g.nx + 31) / 32, (g.ny + 3) / 4, g.nz);
+}
+
 template <typename S>
 cudaError_t launch_export_t(const void* src, const Geom& g, double rho0, double inv_scale,
                             double* out, cudaStream_t st) {
-  const int64_t total = int64_t(g.nx) * g.ny * g.nz * Q;
-  const int b = 256;
-  export_kernel<S><<<unsigned((total + b - 1) / b), b, 0, st>>>(static_cast<const S*>(src), g,
-                                                                 rho0, inv_scale, out);
+  export_kernel<S><<<node_grid(g), dim3(32, 4), 0, st>>>(static_cast<const S*>(src), g, rho0,
+                                                         inv_scale, out);
   return cudaGetLastError();
 }
 
 template <typename S>
 cudaError_t launch_import_t(const double* in, const Geom& g, double rho0, double inv_scale,
                             void* dst, cudaStream_t st) {
-  const int64_t total = int64_t(g.nx) * g.ny * g.nz * Q;
-  const int b = 256;
-  import_kernel<S><<<unsigned((total + b - 1) / b), b, 0, st>>>(in, g, rho0, inv_scale,
-                                                                 static_cast<S*>(dst));
+  import_kernel<S><<<node_grid(g), dim3(32, 4), 0, st>>>(in, g, rho0, 1.0 / inv_scale,
+                                                         static_cast<S*>(dst));
   return cudaGetLastError();
 }
 

@@ -179,7 +179,7 @@ struct BatchHeader {
   void fill_desc_##SUFFIX(void* out, const Geom& g, const PhysParams& P, const void* cur,       \
                           const void* other, const void* ref_cur, const void* ref_other,      \
                           void* uprev, int tx, int ty, int tw_log2, int slot,               \
-                          unsigned step_offset);
+                          unsigned step_offset, int threads);
 CLBM_DECLARE_BATCH(f64)
 CLBM_DECLARE_BATCH(f32)
 CLBM_DECLARE_BATCH(f16)
