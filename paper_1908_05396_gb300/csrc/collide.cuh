@@ -197,6 +197,16 @@ __device__ __forceinline__ float narrow(double x) {
                          : __uint_as_float((unsigned(hi - 0x38000000) << 3) | (lo >> 29));
 }
 
+// The same for either sign.
+__device__ __forceinline__ float narrow_signed(double x) {
+  return copysignf(narrow(fabs(x)), __uint_as_float(unsigned(__double2hiint(x))));
+}
+
+// Comparison of two doubles, the second positive, by their bit patterns.
+__device__ __forceinline__ bool below(double x, double bound) {
+  return __double_as_longlong(x) < __double_as_longlong(bound);
+}
+
 // 1/x for normal x: the FP32 reciprocal of the mantissa as the seed r0, then
 // r0 (1 + e + e^2) with e = 1 - x r0 (the cubically convergent iteration):
 // the seed's 2^-22 leaves 2^-66, below the rounding of the last operation.
@@ -216,20 +226,21 @@ __device__ __forceinline__ double rcp64(double x) {
 template <> __device__ __forceinline__ double rrcp<double>(double x) { return rcp64(x); }
 
 // Natural logarithm of a positive normal x, as (exponent, log of the mantissa)
-// with x = 2^ex z: z = 1 + i/128 to within 1/256, and with the table's c near
-// 1/z, log z = -log c + log1p(r), r = z c - 1, |r| < 2^-8 (P. T. P. Tang,
-// ACM TOMS 16(4), 1990).  The series to r^6 leaves r^7/7 < 2^-58.
+// with x = 2^ex z: z = 1 + i/1024 to within 1/2048, and with the table's c
+// near 1/z, log z = -log c + log1p(r), r = z c - 1, |r| < 2^-10.9 (P. T. P.
+// Tang, ACM TOMS 16(4), 1990).  Of log1p(r) = r - r^2/2 + r^3/3 - r^4/4 + r^5/5
+// (what is left out is below 2^-68) the terms from r^3 on are below 2^-34, so
+// FP32 gives them to 2^-58: five FP64 instructions where a table of 128 and
+// an FP64 series took nine.
 __device__ __forceinline__ double log_mant(double x, int& ex) {
-  const int hi = __double2hiint(x) + 0x1000;
+  const int hi = __double2hiint(x) + 0x200;
   ex = (hi >> 20) - 1023;
   const double z = __hiloint2double(__double2hiint(x) - (ex << 20), __double2loint(x));
-  const double2 t = __ldg(&LOG_TAB[(hi >> 13) & 127]);
+  const double2 t = __ldg(&LOG_TAB[(hi >> 10) & 1023]);
   const double r = fma(z, t.x, -1.0);
-  double p = fma(r, -1.0 / 6.0, 0.2);
-  p = fma(r, p, -0.25);
-  p = fma(r, p, 1.0 / 3.0);
-  p = fma(r, p, -0.5);
-  return t.y + fma(mulr(r, r), p, r);
+  const float f = narrow_signed(r), f2 = mulr(f, f);
+  const float c = mulr(mulr(f2, f), fma(f, fma(f, 0.2f, -0.25f), 1.0f / 3.0f));
+  return t.y + (fma(-0.5, mulr(r, r), r) + widen(c));
 }
 
 // FP64: the FP32 solve gives tau0 = 1/omega - 1/2 to about 1e-6, taken as the
@@ -241,8 +252,8 @@ __device__ __forceinline__ double log_mant(double x, int& ex) {
 //   G'' = (n-1) [s omega r / 2 - 2 r (1 - r) s^2]
 // (from ds/dy = tau omega^2 / 2 and dr/dy = -2 r (1 - r) s), and the step is
 // dy = d1 (1 - d1 G'' / (2 G')) with d1 = -G/G'.  The correction of the second
-// factor is of the order of dy, so it needs FP32 only.  tau is carried to the new y
-// by exp(dy) = 1 + dy + dy^2/2 + dy^3/6.
+// factor is of the order of dy, so it needs FP32 only; tau is carried to the
+// new y by exp(dy) = 1 + dy + dy^2/2 + dy^3/6, whose terms beyond d1 likewise.
 __device__ __forceinline__ double omega_nu(const CollideConst<double>& C, double rho,
                                            double rinv, double A, double B) {
   if (C.newtonian) {
@@ -256,7 +267,7 @@ __device__ __forceinline__ double omega_nu(const CollideConst<double>& C, double
   const double w = rcp64(tau + 0.5);
   const double ww = mulr(w, w), wwA = mulr(ww, A);
   double g2 = fma(ww, A, B);
-  if (g2 < 1e-300) g2 = 1e-300;
+  if (below(g2, 1e-300)) g2 = 1e-300;
   int e1, e2;
   const double l1 = log_mant(mulr(tau, rho), e1);
   const double l2 = log_mant(mulr(mulr(rinv, rinv), g2), e2);
@@ -272,14 +283,16 @@ __device__ __forceinline__ double omega_nu(const CollideConst<double>& C, double
   const float G1 = fma(nm1, rs, 1.0f);
   // G'' = (n-1) r s [omega/2 - 2 (1 - r) s]
   const float G2 = mulr(mulr(nm1, rs), fma(-2.0f * sf, 1.0f - rf, 0.5f * wf));
-  // the magnitude of d1 with its sign; |d1| is large only when the root lies
-  // beyond a clamp, where the sign of dy decides
-  const float d1f = copysignf(narrow(fabs(d1)), __uint_as_float(unsigned(__double2hiint(d1))));
+  // tau1 = tau exp(dy), dy = d1 (1 + h): what exp(dy) - 1 has beyond d1 is of
+  // the order of d1^2, so FP32 gives it.  |d1| is large only when the root
+  // lies beyond a clamp, where the sign of dy decides.
+  const float d1f = narrow_signed(d1);
   const float h = fminf(fmaxf(mulr(mulr(-0.5f * G2, rcpf(G1)), d1f), -0.25f), 0.25f);
-  const double dy = fma(d1, widen(h), d1);
-  double t1 = fma(tau, mulr(dy, fma(dy, fma(dy, 1.0 / 6.0, 0.5), 1.0)), tau);
-  if (t1 < C.tlo) t1 = C.tlo;
-  else if (t1 > C.thi) t1 = C.thi;
+  const float dyf = fma(d1f, h, d1f);
+  const float rest = fma(d1f, h, mulr(mulr(dyf, dyf), fma(dyf, 1.0f / 6.0f, 0.5f)));
+  double t1 = fma(tau, d1 + widen(rest), tau);
+  if (below(t1, C.tlo)) t1 = C.tlo;
+  else if (below(C.thi, t1)) t1 = C.thi;
   return rcp64(t1 + 0.5);
 }
 
@@ -854,16 +867,16 @@ __device__ __forceinline__ void collide_unit(const CollideConst<typename ScalarO
   const R cxx = zx + r30, cyy = zy + r30;
 
   if constexpr (PAIR_OUT) {
-    // a quarter of every plane moment: the populations of a plane are sums
-    // and differences of the four quarters (plane_out)
+    // a quarter of every plane moment (but for the products k_ij): the
+    // populations of a plane are sums and differences of the four quarters
+    // (plane_out)
     const R q4 = R(T(0.25)), h2 = R(T(0.5));
     const R qx = mulr(q4, ux), qy = mulr(q4, uy), qz = mulr(q4, uz);
     const R hx = mulr(h2, ux), hy = mulr(h2, uy), hz = mulr(h2, uz);
     R oxyy = mulr(qx, kyy), oxzz = mulr(qx, kzz), oxxy = mulr(qy, kxx), oyzz = mulr(qy, kzz),
       oxxz = mulr(qz, kxx), oyyz = mulr(qz, kyy);
     R ddr = mulr(R(T(1.0 / 36.0)), drho);
-    R pxy = fma(Jx, qy, mulr(q4, cxy)), pxz = fma(Jx, qz, mulr(q4, cxz)),
-      pyz = fma(Jy, qz, mulr(q4, cyz));
+    R pxy = fma(Jx, uy, cxy), pxz = fma(Jx, uz, cxz), pyz = fma(Jy, uz, cyz);  // raw k_ij
     R fExx = Exx, fEyy = Eyy, fEzz = Ezz, fdr = drho;
     R gx = mulr(h2, jx), gy = mulr(h2, jy), gz = mulr(h2, jz);
     if constexpr (REF) {
@@ -895,9 +908,9 @@ __device__ __forceinline__ void collide_unit(const CollideConst<typename ScalarO
       oyzz = fma(qy, kzz, fy);
       oxxz = fma(qz, kxx, fz);
       oyyz = fma(qz, kyy, fz);
-      pxy = fma(qx, hFy, fma(qy, hFx, pxy));
-      pxz = fma(qx, hFz, fma(qz, hFx, pxz));
-      pyz = fma(qy, hFz, fma(qz, hFy, pyz));
+      pxy = fma(ux, hFy, fma(uy, hFx, pxy));
+      pxz = fma(ux, hFz, fma(uz, hFx, pxz));
+      pyz = fma(uy, hFz, fma(uz, hFy, pyz));
       fExx = fma(ux, Fx, fExx);
       fEyy = fma(uy, Fy, fEyy);
       fEzz = fma(uz, Fz, fEzz);
@@ -945,8 +958,8 @@ __device__ __forceinline__ void collide_unit(const CollideConst<typename ScalarO
       d[5] = hs + ht;
       d[6] = hs - ht;
     }
-    auto plane = [](R f, R pr, R oi, R oj, R& Pp, R& Pm, R& Mp, R& Mm) {
-      const R a = f + pr, b = f - pr, c = oi + oj, e = oi - oj;
+    auto plane = [&](R f, R pr, R oi, R oj, R& Pp, R& Pm, R& Mp, R& Mm) {
+      const R a = fma(q4, pr, f), b = fma(-q4, pr, f), c = oi + oj, e = oi - oj;
       Pp = a + c;
       Pm = a - c;
       Mp = b + e;
