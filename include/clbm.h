@@ -248,7 +248,9 @@ int clbm_set_rounding(clbm_handle h, clbm_rounding mode);
  * lattices without body force and one over those with it, the two on two
  * streams at once (tiles from a device-side table), with each whole
  * check interval queued as one CUDA graph (or, after
- * clbm_batch_set_lattice_launch, one launch per lattice within that graph).  Lattices join and leave between
+ * clbm_batch_set_lattice_launch, one launch per lattice within that graph;
+ * so, too, while no launch was set or tuned and the attached lattices have
+ * 100,000 nodes or more on average).  Lattices join and leave between
  * clbm_batch_step() calls; each keeps its own buffers, parameters, step
  * count and residual.  While a lattice is in a batch, clbm_step() on it
  * fails; clbm_fields/get_state/residual/... on it first wait for the batch.

@@ -6,13 +6,16 @@
 // two streams (the two launches touch disjoint lattices).  Whole check
 // intervals run as one CUDA graph captured on first use: (check_interval - 1)
 // plain steps of alternating parity, then a check step whose per-lattice FP64
-// sums are copied to pinned host memory.  The kernel reads its tile table and lattice descriptors from device
-// memory, so the graph stays valid when lattices join or leave; only a change
-// of launch shape or of the table's capacity recaptures it.
+// sums are copied to pinned host memory.  The kernel reads its tile table and
+// lattice descriptors from device memory, so the graph stays valid when
+// lattices join or leave; only a change of launch shape or of the table's
+// capacity recaptures it.
 //
 // A second mode launches every lattice's own step kernel (kernels.cuh) once
 // per step instead, the lattices spread over a few streams that fork from the
-// batch's stream at the start of a check interval and join it at the end.
+// batch's stream at the start of a check interval and join it at the end.  A
+// batch whose launch was neither set nor tuned does the same with large
+// lattices (`spread`), for every form and rounding.
 // Each lattice then runs with its parameters as kernel arguments and no tile
 // table, and the streams fill each other's tails.  Its graph holds the
 // lattices' buffer addresses, so a change of membership recaptures it.
@@ -76,6 +79,14 @@ struct clbm_batch_ctx {
   std::vector<cudaStream_t> aux;      // mode 1: the streams besides `stream`
   std::vector<cudaEvent_t> ev;        // mode 1: fork event, then one join event per aux stream
   std::vector<int> stream_of;         // mode 1: slot -> stream (0 is `stream`)
+  // Until a launch is set or tuned, lattices that are large on average go one
+  // launch per lattice too (`spread`, decided with the tables): graphs of `sub`
+  // steps, the second one's last a check step.
+  bool auto_mode = true;
+  bool spread = false;
+  int sub = 2;
+  int64_t table_steps = 0;            // batch step at which the tables were written
+  cudaGraphExec_t sub_graph[2] = {nullptr, nullptr};
   cudaGraphExec_t graph = nullptr;
   cudaEvent_t check_done = nullptr;
   std::string err;
@@ -206,11 +217,36 @@ cudaError_t launch(clbm_batch_ctx* b, bool check) {
 }
 
 void drop_graph(clbm_batch_ctx* b) {
-  if (b->graph) cudaGraphExecDestroy(b->graph);
-  b->graph = nullptr;
+  for (cudaGraphExec_t* g : {&b->graph, &b->sub_graph[0], &b->sub_graph[1]}) {
+    if (*g) cudaGraphExecDestroy(*g);
+    *g = nullptr;
+  }
 }
 
-// ---- mode 1: one launch per lattice --------------------------------------
+// ---- mode 1 and `spread`: one launch per lattice --------------------------
+
+// Spread launches, from a mean of 100,000 nodes a lattice.  us a step, one
+// persistent kernel -> one launch each, 1 / 4 / 12 / 32 cavities:
+//   48^3 FP32  6.1 -> 5.1   16.4 -> 10.7   42.7 -> 39.2   111 -> 106
+//        F16S  9.5 -> 5.1   17.7 ->  9.1   40.0 -> 27.7    99 ->  74
+//        F16R 10.2 -> 5.9   22.2 -> 14.1   60.8 -> 45.3   154 -> 120
+//        FP64 65.5 -> 55.8   220 ->  199    626 ->  593  1643 -> 1578
+//   64^3 FP32 11.1 -> 7.6   36.8 -> 26.3    105 ->   78   272 -> 206
+// A launch costs the host 2 us, a node of FP32 0.035 ns in the other kernel, so
+// single steps lose below 60,000 nodes; graphs, too, with many lattices (64 of
+// 36^3, F16S: 116 -> 129).  More than 8 streams gave nothing.
+constexpr int SPREAD_STREAMS = 8;
+// Capturing a graph costs about 1 ms for 12 lattices and saves host time only,
+// so a batch whose members come and go is not captured at once.
+constexpr int64_t SPREAD_SETTLED = 100;
+constexpr double SPREAD_NODES = 100000.0;
+
+int pl_stream_count(const clbm_batch_ctx* b) { return b->spread ? SPREAD_STREAMS : b->pl_streams; }
+
+// The step count that seeds stochastic rounding in a replayed graph.
+__global__ void set_count_kernel(unsigned* p, unsigned v) { *p = v; }
+
+bool counts_steps(const clbm_batch_ctx* b) { return b->dtype == CLBM_F16R || any_sround(b); }
 
 cudaStream_t pl_stream(const clbm_batch_ctx* b, int k) {
   return k == 0 ? b->stream : b->aux[size_t(k - 1)];
@@ -244,7 +280,7 @@ void assign_streams(clbm_batch_ctx* b) {
     return double(h->g.nx) * h->g.ny * h->g.nz;
   };
   std::stable_sort(order.begin(), order.end(), [&](int a, int c) { return nodes(a) > nodes(c); });
-  std::vector<double> load(size_t(b->pl_streams), 0.0);
+  std::vector<double> load(size_t(pl_stream_count(b)), 0.0);
   b->stream_of.assign(size_t(b->capacity), 0);
   for (int s : order) {
     const size_t k = size_t(std::min_element(load.begin(), load.end()) - load.begin());
@@ -273,8 +309,11 @@ cudaError_t join_streams(clbm_batch_ctx* b, int n) {
 
 // One step of every lattice, each on its stream.  `flip` = 1 when the state
 // sits in the other buffer than h->cur says (inside a captured interval).
-// The check sums of slot s go to the batch's row s, as in mode 0.
-cudaError_t launch_lattices(clbm_batch_ctx* b, bool check, int flip) {
+// The check sums of slot s go to the batch's row s, as in mode 0.  `ahead`: steps
+// already launched since h->steps was current; `base`: in a captured graph,
+// the device-side count that holds the batch's steps at its start.
+cudaError_t launch_lattices(clbm_batch_ctx* b, bool check, int flip, int ahead = 0,
+                            const unsigned* base = nullptr) {
   for (int s = 0; s < b->capacity; ++s) {
     clbm_ctx* h = b->slots[size_t(s)];
     if (!h) continue;
@@ -284,7 +323,10 @@ cudaError_t launch_lattices(clbm_batch_ctx* b, bool check, int flip) {
     // the lattice's own block: the tile width of the persistent kernel's rule
     const int threads = int(b->pl_block.x * b->pl_block.y);
     const int tw = tile_width(h->g.nx, int(h->elem), int(b->pl_block.x), threads);
-    const dim3 blk(unsigned(tw), unsigned(threads / tw), 1);
+    const dim3 blk = b->spread ? default_block(h->g.nx, int(h->elem))
+                               : dim3(unsigned(tw), unsigned(threads / tw), 1);
+    const int npt = b->spread ? 1 : b->pl_npt;
+    const int64_t step = (base ? h->steps - b->steps : h->steps) + ahead;
     cudaError_t e;
     if (h->in_place) {  // one buffer, the layout alternating with the steps
       const int lay = h->layout ^ flip;
@@ -307,13 +349,18 @@ cudaError_t launch_lattices(clbm_batch_ctx* b, bool check, int flip) {
     void* dst = h->buf[1 - c];
     switch (b->dtype) {
       case CLBM_F64:
-        e = launch_step_f64(src, dst, h->g, h->P, cb, check, blk, b->pl_npt, st);
+        e = launch_step_f64(src, dst, h->g, h->P, cb, check, blk, npt, st);
         break;
       case CLBM_F32:
-        e = launch_step_f32(src, dst, h->g, h->P, cb, check, blk, b->pl_npt, st);
+        e = launch_step_f32(src, dst, h->g, h->P, cb, check, blk, npt, st);
+        break;
+      case CLBM_F16R:
+        e = launch_step_f16r(src, dst, h->ref[c], h->ref[1 - c], h->g, h->P, cb, check, blk, step,
+                             base, st);
         break;
       default:
-        e = launch_step_f16(src, dst, h->g, h->P, cb, check, blk, b->pl_npt, st);
+        e = h->sround ? launch_step_f16sr(src, dst, h->g, h->P, cb, check, blk, step, base, st)
+                      : launch_step_f16(src, dst, h->g, h->P, cb, check, blk, npt, st);
         break;
     }
     if (e != cudaSuccess) return e;
@@ -398,11 +445,21 @@ int upload(clbm_batch_ctx* b) {
                       cudaMemcpyHostToDevice));
   }
   BCK(b, cudaMemcpy(b->d_hdr, &hdr, sizeof(hdr), cudaMemcpyHostToDevice));
-  if (b->mode == 1) {
+  double nodes = 0.0;
+  int count = 0;
+  for (const clbm_ctx* h : b->slots)
+    if (h) {
+      nodes += double(h->g.nx) * h->g.ny * h->g.nz;
+      ++count;
+    }
+  b->spread = b->mode == 0 && b->auto_mode && count > 0 && nodes >= SPREAD_NODES * count;
+  if (b->spread) BCK(b, ensure_streams(b, SPREAD_STREAMS));
+  if (b->mode == 1 || b->spread) {
     assign_streams(b);
-    drop_graph(b);  // the graph holds the lattices' buffer addresses
+    drop_graph(b);  // the graphs hold the lattices' buffer addresses
   }
   b->parity = 0;
+  b->table_steps = b->steps;
   b->dirty = false;
   return CLBM_OK;
 }
@@ -441,6 +498,63 @@ int one_step(clbm_batch_ctx* b) {
       if (b->slots[s]) b->slot_checks[s] += 1;
   }
   advance(b, 1);
+  return CLBM_OK;
+}
+
+// n spread steps on the batch's stream (which may be capturing), the last one
+// a check step if `check`.
+cudaError_t launch_spread(clbm_batch_ctx* b, int n, bool check, const unsigned* base) {
+  cudaError_t e = cudaSuccess;
+  if (check) e = cudaMemsetAsync(b->d_acc, 0, acc_bytes(b), b->stream);
+  if (e == cudaSuccess) e = fork_streams(b, SPREAD_STREAMS);
+  for (int k = 0; k < n && e == cudaSuccess; ++k)
+    e = launch_lattices(b, check && k == n - 1, k & 1, k, base);
+  if (e == cudaSuccess) e = join_streams(b, SPREAD_STREAMS);
+  if (e == cudaSuccess && check) {
+    e = cudaMemcpyAsync(b->h_acc, b->d_acc, acc_bytes(b), cudaMemcpyDeviceToHost, b->stream);
+    if (e == cudaSuccess) e = cudaEventRecord(b->check_done, b->stream);
+  }
+  return e;
+}
+
+// Up to `left` spread steps, at most to the next multiple of `sub` (check steps
+// end one); returns a status, and the steps done in *done.  Whole runs of `sub`
+// steps replay a graph once the tables have stood for SPREAD_SETTLED steps.
+// `sub` is even, so the lattices' buffers are the same at each run's start.
+int spread_steps(clbm_batch_ctx* b, int64_t left, int64_t* done) {
+  const int n = int(std::min<int64_t>(left, b->sub - b->steps % b->sub));
+  const bool check = (b->steps + n) % b->check_interval == 0;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;  // the caller's own capture
+  BCK(b, cudaStreamIsCapturing(b->stream, &cap));
+  if (n < b->sub || b->steps - b->table_steps < SPREAD_SETTLED ||
+      cap != cudaStreamCaptureStatusNone) {
+    BCK(b, launch_spread(b, n, check, nullptr));
+  } else {
+    const unsigned* base = counts_steps(b) ? b->d_hdr->step : nullptr;
+    cudaGraphExec_t& exec = b->sub_graph[check ? 1 : 0];
+    if (!exec) {
+      cudaGraph_t g = nullptr;
+      BCK(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
+      cudaError_t e = launch_spread(b, n, check, base);
+      const cudaError_t e2 = cudaStreamEndCapture(b->stream, &g);
+      if (e == cudaSuccess) e = e2;
+      if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, g, 0);
+      if (g) cudaGraphDestroy(g);
+      if (e != cudaSuccess) {
+        exec = nullptr;
+        return bfail(b, CLBM_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(e));
+      }
+    }
+    if (base) {
+      set_count_kernel<<<1, 1, 0, b->stream>>>(b->d_hdr->step, unsigned(uint64_t(b->steps)));
+      BCK(b, cudaGetLastError());
+    }
+    BCK(b, cudaGraphLaunch(exec, b->stream));
+  }
+  for (int s = 0; s < b->capacity && check; ++s)
+    if (b->slots[s]) b->slot_checks[s] += 1;
+  advance(b, n);
+  *done = n;
   return CLBM_OK;
 }
 
@@ -550,6 +664,8 @@ int clbm_batch_create(clbm_dtype dtype, int capacity, int check_interval, void* 
   }
   b->capacity = capacity;
   b->check_interval = check_interval;
+  for (int k = 2; k <= 10; k += 2)  // the largest even divisor up to 10
+    if (check_interval % k == 0) b->sub = k;
   b->slots.assign(size_t(capacity), nullptr);
   b->slot_checks.assign(size_t(capacity), 0);
   b->slot_joined.assign(size_t(capacity), 0);
@@ -637,6 +753,12 @@ int clbm_batch_step(clbm_batch b, int64_t nsteps) {
       if (int r = upload(b)) return r;
     }
     const int64_t ci = b->check_interval;
+    if (b->spread) {
+      int64_t n = 0;
+      if (int r = spread_steps(b, left, &n)) return r;
+      left -= n;
+      continue;
+    }
     if (b->steps % ci == 0 && b->parity == 0 && left >= ci) {
       if (!b->graph) {
         if (int r = capture(b)) return r;
@@ -703,6 +825,7 @@ int clbm_batch_set_launch(clbm_batch b, int block_x, int block_y, int zc, int bl
   b->blocks_per_sm = blocks_per_sm;
   b->cap = cap;
   b->mode = 0;
+  b->auto_mode = false;
   b->dirty = true;
   drop_graph(b);
   return CLBM_OK;
@@ -726,6 +849,7 @@ int clbm_batch_set_lattice_launch(clbm_batch b, int block_x, int block_y, int np
   b->pl_npt = npt;
   b->pl_streams = streams;
   b->mode = 1;
+  b->auto_mode = false;
   b->dirty = true;
   drop_graph(b);
   return CLBM_OK;
@@ -760,6 +884,7 @@ int clbm_batch_autotune(clbm_batch b, int steps, int* block_x, int* block_y, int
     any_in_place = any_in_place || h->in_place;
   }
   const int64_t bsteps0 = b->steps;
+  b->auto_mode = false;  // the timing below chooses
   const dim3 block0 = b->block;
   const int zc0 = b->zc, bps0 = b->blocks_per_sm;
   const int shapes[][2] = {{16, 4}, {16, 8}, {32, 2}, {32, 4}, {32, 8}, {64, 4}};

@@ -187,10 +187,11 @@ CLBM_DECLARE_BATCH(f16r)
 
 // F16R form (step_f16r.cu): FP16 populations relative to each node's stored
 // first-order equilibrium reference, stored with stochastic rounding; `step`
-// is the lattice's count of steps done before this one (it seeds the rounding).
+// is the lattice's count of steps done before this one (it seeds the rounding),
+// relative to *base when base (device memory) is given.
 cudaError_t launch_step_f16r(const void* src, void* dst, const void* ref_src, void* ref_dst,
                              const Geom& g, const PhysParams& P, const CheckBufs& cb, bool check,
-                             dim3 block, int npt, int64_t step, cudaStream_t st);
+                             dim3 block, int64_t step, const unsigned* base, cudaStream_t st);
 cudaError_t launch_fields_f16r(const void* src, const void* ref, const Geom& g,
                                const PhysParams& P, double* rho, double* u, double* gd,
                                cudaStream_t st);

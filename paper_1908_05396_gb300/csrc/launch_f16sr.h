@@ -10,10 +10,10 @@
 namespace clbm {
 
 // One step of an F16S lattice from src into dst with stochastic rounding
-// seeded by (node, step); npt 1 or 5 (register-capped).
+// seeded by (node, step): step, or *base + step when base (device memory) is given.
 cudaError_t launch_step_f16sr(const void* src, void* dst, const Geom& g, const PhysParams& P,
-                              const CheckBufs& cb, bool check, dim3 block, int npt, int64_t step,
-                              cudaStream_t st);
+                              const CheckBufs& cb, bool check, dim3 block, int64_t step,
+                              const unsigned* base, cudaStream_t st);
 
 // Mark a filled F16S batch descriptor (fill_desc_f16) as rounding its
 // stores stochastically (batch.cuh, LatDesc::sround).

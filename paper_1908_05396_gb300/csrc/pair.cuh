@@ -332,12 +332,12 @@ __device__ __forceinline__ void check_pair(CheckSums& s, const NodeOut<V2>& o, f
   if (n1) check_node(s, lane1(o.rho), lane1(o.ux), lane1(o.uy), lane1(o.uz), rho0, up + 1, nst);
 }
 
-// F16R: reference buffers of a lone step; step: the lattice's steps done
+// F16R: reference buffers of a lone step; seed: the lattice's steps done
 // before this one.
 struct PairExtra {
   const uint2* ref_src;
   uint2* ref_dst;
-  unsigned step;
+  StepSeed seed;
 };
 
 // One time step of a lone lattice; the block is pair_width() threads along x.
@@ -358,7 +358,8 @@ __global__ void __launch_bounds__(256, pair_min_blocks(FORM == PAIR_REF))
     const LonePair p{a, FORM == PAIR_REF ? e.ref_src + i : nullptr, i};
     pull_pair<FORM == PAIR_REF>(p, x, y, z, d);
     collide_pair<FORM == PAIR_REF, FORCE>(a.C, d, o, e.ref_dst + i);
-    store_pair(d, FORM != PAIR_RN, [&](int q) { return a.dstq[q] + i; }, i, e.step);
+    store_pair(d, FORM != PAIR_RN, [&](int q) { return a.dstq[q] + i; }, i,
+               FORM != PAIR_RN ? e.seed.get() : 0u);
     if (CHECK)
       check_pair(sums, o, a.C.rho0, static_cast<float*>(a.cb.uprev) + i, int64_t(a.plane) * a.nz,
                  x + 1 < a.nx);

@@ -8,6 +8,15 @@
 
 namespace clbm {
 
+// The lattice's step count that seeds a step's rounding: a constant of the
+// launch, or relative to a count in device memory (a launch in a graph that
+// is replayed).
+struct StepSeed {
+  unsigned step = 0;
+  const unsigned* base = nullptr;
+  __device__ __forceinline__ unsigned get() const { return base ? *base + step : step; }
+};
+
 // Stochastic rounding of the stores: a value is rounded up in magnitude with
 // probability equal to the fraction of an FP16 ulp it carries, so increments
 // far below one ulp (a weak body force, a slow transient) survive on average

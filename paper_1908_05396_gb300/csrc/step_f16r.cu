@@ -61,7 +61,7 @@ struct RefArgs {
   const uint2* refq[Q];  // refq[q][i]: reference of the upwind neighbour of node i
   const uint2* ref_src;  // references of the source step
   uint2* ref_dst;        // references written by this step
-  unsigned step;         // the lattice's steps done before this one
+  StepSeed seed;         // the lattice's steps done before this one
 };
 
 // Pull of all 19 directions into node (x, y, z) with index i, for a node on
@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(256) step_ref_kernel(const StepArgs<__half, fl
     float d[Q];
     pull_node_ref(a, r, x, y, z, i, d);
     NodeOut<float> o;
-    collide_store_ref<FORCE, UNIT>(a, r, i, r.step, d, o);
+    collide_store_ref<FORCE, UNIT>(a, r, i, r.seed.get(), d, o);
     if (CHECK)
       check_node(sums, o.rho, o.ux, o.uy, o.uz, a.C.rho0, static_cast<float*>(a.cb.uprev) + i,
                  int64_t(a.plane) * a.nz);
@@ -243,24 +243,11 @@ __global__ void collide_nodes_ref_kernel(CollideConst<float> C, const double* __
   if (gd) gd[k] = double(o.gamma_dot);
 }
 
-RefArgs ref_args(const void* ref_src, void* ref_dst, const Geom& g, unsigned step) {
+RefArgs ref_args(const void* ref_src, void* ref_dst, const Geom& g, StepSeed seed) {
   RefArgs r;
-  r.step = step;
+  r.seed = seed;
   r.ref_src = static_cast<const uint2*>(ref_src);
   r.ref_dst = static_cast<uint2*>(ref_dst);
-  for (int q = 0; q < Q; ++q) {
-    const int64_t off = int64_t(cz(q)) * g.plane + int64_t(cy(q)) * g.pitch + cx(q);
-    r.refq[q] = reinterpret_cast<const uint2*>(reinterpret_cast<uintptr_t>(ref_src) -
-                                                off * int64_t(sizeof(uint2)));
-  }
-  return r;
-}
-
-RefArgs ref_args(const uint2* ref_src, uint2* ref_dst, const Geom& g, unsigned step) {
-  RefArgs r;
-  r.step = step;
-  r.ref_src = ref_src;
-  r.ref_dst = ref_dst;
   for (int q = 0; q < Q; ++q) {
     const int64_t off = int64_t(cz(q)) * g.plane + int64_t(cy(q)) * g.pitch + cx(q);
     r.refq[q] = reinterpret_cast<const uint2*>(reinterpret_cast<uintptr_t>(ref_src) -
@@ -305,15 +292,16 @@ __device__ void batch_node_ref(const LatDesc<float>& L, int parity, int x, int y
 
 cudaError_t launch_step_f16r(const void* src, void* dst, const void* ref_src, void* ref_dst,
                              const Geom& g, const PhysParams& P, const CheckBufs& cb, bool check,
-                             dim3 block, int npt, int64_t step, cudaStream_t st) {
+                             dim3 block, int64_t step, const unsigned* base, cudaStream_t st) {
   const StepArgs<__half, float> a = step_args<__half, float>(src, dst, g, P, cb);
   const uint2* rs = static_cast<const uint2*>(ref_src);
   uint2* rd = static_cast<uint2*>(ref_dst);
+  const StepSeed seed{unsigned(uint64_t(step)), base};
   const bool unit = unit_rates(P);
   if (unit && pair_pays(g, true))
-    return launch_step_pair<PAIR_REF>(a, PairExtra{rs, rd, unsigned(uint64_t(step))},
+    return launch_step_pair<PAIR_REF>(a, PairExtra{rs, rd, seed},
                                       P.has_force != 0, check, block, st);
-  const RefArgs r = ref_args(rs, rd, g, unsigned(uint64_t(step)));
+  const RefArgs r = ref_args(rs, rd, g, seed);
   const dim3 grid((g.nx + block.x - 1) / block.x, (g.ny + block.y - 1) / block.y, g.nz);
   void (*kernel)(const StepArgs<__half, float>, const RefArgs) = nullptr;
 #define CLBM_REF(F, C_) kernel = unit ? step_ref_kernel<F, C_, true> : step_ref_kernel<F, C_, false>
@@ -334,7 +322,7 @@ cudaError_t launch_fields_f16r(const void* src, const void* ref, const Geom& g,
   const dim3 block(32, 4);
   const dim3 grid((g.nx + 31) / 32, (g.ny + 3) / 4, g.nz);
   const StepArgs<__half, float> a = step_args<__half, float>(src, nullptr, g, P, CheckBufs{});
-  const RefArgs r = ref_args(static_cast<const uint2*>(ref), nullptr, g, 0u);
+  const RefArgs r = ref_args(static_cast<const uint2*>(ref), nullptr, g, StepSeed{});
   const FieldsOut f{rho, u, gd};
   if (P.has_force) fields_ref_kernel<true><<<grid, block, 0, st>>>(a, r, f);
   else fields_ref_kernel<false><<<grid, block, 0, st>>>(a, r, f);

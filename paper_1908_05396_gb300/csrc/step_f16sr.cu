@@ -18,7 +18,7 @@ namespace {
 // One node per thread.
 template <bool FORCE, bool CHECK, bool UNIT>
 __global__ void __launch_bounds__(256) step_sr_kernel(const StepArgs<__half, float> a,
-                                                      unsigned step) {
+                                                      const StepSeed seed) {
   pdl_enter();
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(256) step_sr_kernel(const StepArgs<__half, flo
     NodeOut<float> o;
     collide<float, FORCE, pair_out<__half>(), log2_scale<__half>(), UNIT>(a.C, d, o);
     // the deviations are carried scaled by 1024, as they are stored
-    store_sr1([&](int q) { return a.dstq[q] + i; }, d, uint32_t(i), step);
+    store_sr1([&](int q) { return a.dstq[q] + i; }, d, uint32_t(i), seed.get());
     if (CHECK)
       check_node(sums, o.rho, o.ux, o.uy, o.uz, a.C.rho0, static_cast<float*>(a.cb.uprev) + i,
                  int64_t(a.plane) * a.nz);
@@ -46,16 +46,16 @@ __global__ void __launch_bounds__(256) step_sr_kernel(const StepArgs<__half, flo
 // Lattices with the unit rates omega_9..18 take the pair kernel where it is
 // the faster one (pair_pays), the others one node per thread.
 cudaError_t launch_step_f16sr(const void* src, void* dst, const Geom& g, const PhysParams& P,
-                              const CheckBufs& cb, bool check, dim3 block, int npt, int64_t step,
-                              cudaStream_t st) {
+                              const CheckBufs& cb, bool check, dim3 block, int64_t step,
+                              const unsigned* base, cudaStream_t st) {
   const StepArgs<__half, float> a = step_args<__half, float>(src, dst, g, P, cb);
-  const unsigned sstep = unsigned(uint64_t(step));
+  const StepSeed seed{unsigned(uint64_t(step)), base};
   const bool unit = unit_rates(P);
   if (unit && pair_pays(g, false))
-    return launch_step_pair<PAIR_SR>(a, PairExtra{nullptr, nullptr, sstep}, P.has_force != 0,
+    return launch_step_pair<PAIR_SR>(a, PairExtra{nullptr, nullptr, seed}, P.has_force != 0,
                                      check, block, st);
   const dim3 grid((g.nx + block.x - 1) / block.x, (g.ny + block.y - 1) / block.y, g.nz);
-  void (*kernel)(const StepArgs<__half, float>, unsigned) = nullptr;
+  void (*kernel)(const StepArgs<__half, float>, const StepSeed) = nullptr;
 #define CLBM_SR(F, C_) kernel = unit ? step_sr_kernel<F, C_, true> : step_sr_kernel<F, C_, false>
   if (P.has_force) {
     if (check) CLBM_SR(true, true);
@@ -65,7 +65,7 @@ cudaError_t launch_step_f16sr(const void* src, void* dst, const Geom& g, const P
     else CLBM_SR(false, false);
   }
 #undef CLBM_SR
-  return pdl_launch(kernel, grid, block, st, a, sstep);
+  return pdl_launch(kernel, grid, block, st, a, seed);
 }
 
 }  // namespace clbm
