@@ -130,8 +130,8 @@ class Clocks:
                 "samples": len(sm)}
 
 
-STEP_KERNEL_SOURCES = ("d3q19.cuh", "v2.cuh", "collide.cuh", "launch.h", "kernels.cuh",
-                       "tma_step.cuh")
+STEP_KERNEL_SOURCES = ("d3q19.cuh", "v2.cuh", "collide.cuh", "log_table.h", "launch.h",
+                       "kernels.cuh", "tma_step.cuh")
 # translation unit of each storage form's step kernel
 STEP_TU = {"f64": "step_f64.cu", "f32": "step_f32.cu", "f16s": "step_f16.cu"}
 
@@ -366,8 +366,7 @@ def run_ours(args):
     achieved = bpn * N / per_launch_s / 1e9
     npt0 = tuned[0]["npt"]
     cap = "true" if npt0 & 4 else "false"
-    kern = (f"step2_kernel<float,false,false,{cap}>" if (npt0 & 3) == 2
-            else f"step_kernel<float,float,false,false,{cap}>")
+    kern = f"step_kernel<float,float,false,false,{cap},true>"
     traffic = _traffic_note(kern)
 
     # ---- the other forms ------------------------------------------------------
@@ -399,7 +398,7 @@ def run_ours(args):
     # ncu on the current kernel sources.
     if "f64" in forms:
         rate = clbm.probe_fma_rate("f64")
-        kern64 = "step_kernel<double,double,false,false,false>"
+        kern64 = "step_kernel<double,double,false,false,false,true>"
         ops = _fp64_ops_note(kern64)
         alu = {"bound": "alu", "unit": "FP64 instructions/s", "peak": rate / 2.0,
                "peak_kind": "measured (FMA probe: two FLOP per DFMA)", "kernel": kern64,

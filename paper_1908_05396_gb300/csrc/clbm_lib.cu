@@ -529,8 +529,7 @@ int clbm_autotune(clbm_handle h, int steps, int* block_x, int* block_y, int* npt
       return CLBM_OK;
     }
   }
-  // Candidates: block shapes up to 256 threads (128 for two nodes per thread,
-  // whose kernel is compiled for 128), x extent at most the padded row.
+  // Candidates: block shapes up to 256 threads, x extent at most the padded row.
   struct Cand { int bx, by, npt; };
   std::vector<Cand> cands;
   const int shapes[][2] = {{8, 4},  {8, 8},  {16, 2}, {16, 4}, {16, 8},  {32, 1}, {32, 2},
