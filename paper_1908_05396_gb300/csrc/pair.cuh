@@ -43,7 +43,7 @@ __device__ __forceinline__ RefT<float> ref_dec(uint2 v) {
   return {a.x, a.y, b.x, b.y};
 }
 __device__ __forceinline__ RefT<float> ref1(const uint2* p) { return ref_dec(*p); }
-// dr + e_q . v, the part of the reference term that w_q multiplies; the sums
+// dr + e_q . v, the part of the reference term that ref_wt(q) multiplies; the sums
 // are associated alike for a node and a pair, so that a reader forms the
 // value the writer subtracted.
 template <typename R>
@@ -130,7 +130,7 @@ __device__ __forceinline__ void pull_row(const P& p, int x, V2 (&d)[Q]) {
       const RefT<float> a = ref_dec(make_uint2(w.x, w.y)), b = ref_dec(make_uint2(w.z, w.w));
       const RefT<V2> r{V2(a.dr, b.dr), V2(a.vx, b.vx), V2(a.vy, b.vy), V2(a.vz, b.vz)};
       const V2 s = ref_sum(c, r);
-      d[c] = fma(V2(wt<float>(c)), s, d[c]);
+      d[c] = fma(V2(ref_wt(c)), s, d[c]);
       if (cy(c) != 0 && cz(c) != 0) continue;
       // left (x - 1) and right (x + 2, and where the pair's first node is the
       // last of the row, x + 1) neighbours, or what stands in for them
@@ -158,7 +158,7 @@ __device__ __forceinline__ void pull_row(const P& p, int x, V2 (&d)[Q]) {
         // e_x = 1: upwind nodes x - 1, x; e_x = -1: x + 1, x + 2
         const V2 t = cx(q) == 1 ? V2(sl, lane0(s)) + V2(l.vx, lane0(r.vx))
                                 : V2(s1, sn) - V2(x1, n.vx);
-        d[q] = fma(V2(wt<float>(q)), t, d[q]);
+        d[q] = fma(V2(ref_wt(q)), t, d[q]);
       }
     }
   }
@@ -241,7 +241,7 @@ __device__ __forceinline__ void pull_pair(const P& p, int x, int y, int z, V2 (&
       const RefT<float> rA = ref1(p.ref + jA), rB = ref1(p.ref + jB);
       const RefT<V2> r{V2(rA.dr, rB.dr), mulr(sgn, V2(rA.vx, rB.vx)), mulr(sgn, V2(rA.vy, rB.vy)),
                        mulr(sgn, V2(rA.vz, rB.vz))};
-      v = fma(V2(wt<float>(q)), ref_sum(q, r), v);
+      v = fma(V2(ref_wt(q)), ref_sum(q, r), v);
     }
     if (fA.lid & up_faces(q)) set0(v, lane0(v) + p.lid(q));
     if (fB.lid & up_faces(q)) set1(v, lane1(v) + p.lid(q));
@@ -300,7 +300,7 @@ __device__ __forceinline__ void collide_pair(const CollideConst<float>& C, V2 (&
     collide_unit<V2, true, false, L>(C, d, o);
     const RefT<V2> r = ref_store2(rdst, o, C.rho0, LAM);
 #pragma unroll
-    for (int q = 0; q < Q; ++q) d[q] = fma(V2(-wt<float>(q)), ref_sum(q, r), d[q]);
+    for (int q = 0; q < Q; ++q) d[q] = fma(V2(-ref_wt(q)), ref_sum(q, r), d[q]);
   } else {
     collide_unit<V2, false, true, L>(
         C, d, o, [&](const NodeOut<V2>& n) { return ref_store2(rdst, n, C.rho0, LAM); });

@@ -52,9 +52,10 @@ __device__ __forceinline__ float dec16(__half v) { return __half2float(v); }
 __device__ __forceinline__ __half enc16(float v) { return __float2half_rn(v); }
 
 // v plus (sgn = 1) or minus (sgn = -1) the first-order equilibrium deviation
-// of direction q about the reference, lam w_q [drho + 3 rho (e_q . u)].
+// of direction q about the reference, lam w_q [drho + 3 rho (e_q . u)],
+// with the weights ref_wt.
 __device__ __forceinline__ float plus_ref(float v, int q, const RefT<float>& r, float sgn = 1.0f) {
-  return fma(sgn * wt<float>(q), ref_sum(q, r), v);
+  return fma(sgn * ref_wt(q), ref_sum(q, r), v);
 }
 
 struct RefArgs {
