@@ -207,6 +207,14 @@ __device__ __forceinline__ bool below(double x, double bound) {
   return __double_as_longlong(x) < __double_as_longlong(bound);
 }
 
+// Tests on the bit patterns: 0 < x < infinity; x neither infinite nor NaN.
+__device__ __forceinline__ bool positive_finite(double x) {
+  return (unsigned long long)(__double_as_longlong(x)) - 1ull < 0x7fefffffffffffffull;
+}
+__device__ __forceinline__ bool finite_bits(double x) {
+  return (unsigned(__double2hiint(x)) & 0x7ff00000u) != 0x7ff00000u;
+}
+
 // 1/x for normal x: the FP32 reciprocal of the mantissa as the seed r0, then
 // r0 (1 + e + e^2) with e = 1 - x r0 (the cubically convergent iteration):
 // the seed's 2^-22 leaves 2^-66, below the rounding of the last operation.
@@ -293,7 +301,12 @@ __device__ __forceinline__ double omega_nu(const CollideConst<double>& C, double
   double t1 = fma(tau, d1 + widen(rest), tau);
   if (below(t1, C.tlo)) t1 = C.tlo;
   else if (below(C.thi, t1)) t1 = C.thi;
-  return rcp64(t1 + 0.5);
+  const double w1 = rcp64(t1 + 0.5);
+  // The logarithms and clamps work on bit patterns and turn anything into a
+  // rate.  A density that has none, and moments that are not finite, give NaN:
+  // a diverged node then spoils its lattice until the next check step reports it.
+  return positive_finite(rho) && finite_bits(d1) ? w1
+                                                 : __hiloint2double(0x7ff80000, 0);
 }
 
 // |gamma_dot| at the solved omega.

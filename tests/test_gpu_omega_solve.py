@@ -1,0 +1,48 @@
+"""The FP64 solve for omega_nu works on bit patterns in place of FP64
+comparisons and logarithms: what it does outside the positive, finite range."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def clbm():
+    from paper_1908_05396_gb300 import build
+    build.build()
+    from paper_1908_05396_gb300 import clbm as c
+    c.lib()
+    return c
+
+
+@pytest.mark.parametrize("n", [0.5, 0.9, 1.3, 1.8])
+def test_no_rate_without_a_valid_density_and_moments(clbm, n):
+    inf, nan = np.inf, np.nan
+    rho = np.array([1.0, 0.7, -0.27, -1e-3, 0.0, -0.0, nan, -nan, inf, -inf] + [1.0] * 4)
+    m = np.zeros((6, len(rho)))
+    m[0] = 1e-3
+    m[2, 10], m[5, 11], m[1, 12], m[5, 13] = nan, nan, inf, -inf
+    w, gd = clbm.omega_nodes(rho, m, 1e-3, n, "f64")
+    assert np.all(np.isfinite(w[:2]) & (w[:2] > 0) & (w[:2] < 2)) and np.all(gd[:2] > 0)
+    assert np.all(np.isnan(w[2:]))
+
+
+@pytest.mark.parametrize("in_place", [False, True])
+def test_negative_density_spreads_and_is_reported(clbm, in_place):
+    # one node of negative density: its collision leaves NaN, which its
+    # neighbours pull in the next step, and the check step reports it
+    kw = dict(face=(clbm.PERIODIC,) * 6, K=0.02, n=0.8, dtype="f64", check_interval=4)
+    with clbm.Lattice(9, 8, 7, in_place=in_place, **kw) as lat:
+        f = lat.get_state()
+        for q, (x, y, z) in enumerate(_E):      # what node (4, 4, 3) pulls
+            f[q, (3 - z) % 7, (4 - y) % 8, (4 - x) % 9] *= -0.27
+        lat.set_state(f)
+        lat.step(2)
+        assert np.isnan(lat.get_state()).any(axis=0).sum() >= 19
+        lat.step(2)
+        assert lat.residual()[1] == clbm.ERR_DIVERGED
+
+
+_E = [(0, 0, 0), (1, 0, 0), (-1, 0, 0), (0, 1, 0), (0, -1, 0), (0, 0, 1), (0, 0, -1),
+      (1, 1, 0), (-1, 1, 0), (1, -1, 0), (-1, -1, 0), (1, 0, 1), (-1, 0, 1), (1, 0, -1),
+      (-1, 0, -1), (0, 1, 1), (0, -1, 1), (0, 1, -1), (0, -1, -1)]
