@@ -309,10 +309,10 @@ __device__ __forceinline__ double omega_nu(const CollideConst<double>& C, double
                                                  : __hiloint2double(0x7ff80000, 0);
 }
 
-// |gamma_dot| at the solved omega.
+// |gamma_dot| at the solved omega (a diverged node's density may be negative).
 template <typename R>
 __device__ __forceinline__ R shear_rate(R rinv, R w, R A, R B) {
-  return mulr(mulr(R(3), rinv), sqrt(fma(mulr(w, w), A, B)));
+  return mulr(mulr(R(3), fabs(rinv)), sqrt(fma(mulr(w, w), A, B)));
 }
 
 // ---- pair space -------------------------------------------------------------

@@ -9,6 +9,7 @@
 namespace clbm {
 
 // Keep the scalar overloads visible next to the V2 ones below.
+using ::fabs;
 using ::fma;
 using ::fmax;
 using ::fmin;
@@ -45,6 +46,7 @@ __device__ __forceinline__ V2 fmax(V2 a, V2 b) {
 __device__ __forceinline__ V2 fmin(V2 a, V2 b) {
   return V2(fminf(a.v.x, b.v.x), fminf(a.v.y, b.v.y));
 }
+__device__ __forceinline__ V2 fabs(V2 a) { return V2(fabsf(a.v.x), fabsf(a.v.y)); }
 __device__ __forceinline__ V2 sqrt(V2 a) { return V2(sqrtf(a.v.x), sqrtf(a.v.y)); }
 
 __device__ __forceinline__ float lane0(V2 a) { return a.v.x; }

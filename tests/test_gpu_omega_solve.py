@@ -46,3 +46,13 @@ def test_negative_density_spreads_and_is_reported(clbm, in_place):
 _E = [(0, 0, 0), (1, 0, 0), (-1, 0, 0), (0, 1, 0), (0, -1, 0), (0, 0, 1), (0, 0, -1),
       (1, 1, 0), (-1, 1, 0), (1, -1, 0), (-1, -1, 0), (1, 0, 1), (-1, 0, 1), (1, 0, -1),
       (-1, 0, -1), (0, 1, 1), (0, -1, 1), (0, 1, -1), (0, -1, -1)]
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+@pytest.mark.parametrize("n", [0.7, 1.0, 1.4])
+def test_shear_rate_is_a_magnitude(clbm, n, dtype):
+    # gamma_dot is the root of an invariant: the density's sign is not its own
+    rho = np.array([-0.27, 0.27, -1.5, 1.5])
+    m = np.tile(np.array([1e-3, -2e-3, 5e-4, 1e-3, 0.0, 2e-4])[:, None], 4)
+    _, gd = clbm.omega_nodes(rho, m, 1e-3, n, dtype)
+    assert np.all((gd > 0) | np.isnan(gd)) and np.all(gd[[1, 3]] > 0)
