@@ -189,12 +189,16 @@ __device__ __forceinline__ double to64(float x) {
   return double(x);
 }
 
-// A non-negative double truncated to float; zero and values below 2^-125 give 2^-125.
+// A non-negative double truncated to float; zero and values below 2^-125 give
+// 2^-125, values from 2^110 on (beyond which the FP32 solve's products would
+// overflow) 2^110.
 __device__ __forceinline__ float narrow(double x) {
   const int hi = __double2hiint(x);
   const unsigned lo = unsigned(__double2loint(x));
   return hi < 0x38200000 ? 2.3509887e-38f
-                         : __uint_as_float((unsigned(hi - 0x38000000) << 3) | (lo >> 29));
+         : hi >= 0x46d00000
+             ? 1.2980742e33f
+             : __uint_as_float((unsigned(hi - 0x38000000) << 3) | (lo >> 29));
 }
 
 // The same for either sign.

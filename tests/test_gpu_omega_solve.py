@@ -56,3 +56,15 @@ def test_shear_rate_is_a_magnitude(clbm, n, dtype):
     m = np.tile(np.array([1e-3, -2e-3, 5e-4, 1e-3, 0.0, 2e-4])[:, None], 4)
     _, gd = clbm.omega_nodes(rho, m, 1e-3, n, dtype)
     assert np.all((gd > 0) | np.isnan(gd)) and np.all(gd[[1, 3]] > 0)
+
+
+@pytest.mark.parametrize("n", [0.4, 0.8, 1.6, 2.0])
+def test_shear_beyond_the_fp32_range_reaches_its_clamp(clbm, n):
+    # invariants around and past the largest FP32 value: the viscosity lies on
+    # the clamp that n decides, to the rounding of 1 / (3 nu + 1/2): a few 2^-53
+    mag = 10.0 ** np.arange(15, 61, 2.5)
+    rho = np.ones(len(mag))
+    m = mag * np.array([1.0, -0.5, 0.3, 0.2, 0.1, 0.4])[:, None]
+    w, _ = clbm.omega_nodes(rho, m, 1e-3, n, "f64")
+    nu = 5e-4 if n < 1 else 10.0
+    assert np.all(np.abs(w * (3 * nu + 0.5) - 1) <= 1e-15)
