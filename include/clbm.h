@@ -184,8 +184,9 @@ int clbm_set_allocator(clbm_alloc_fn alloc_fn, clbm_free_fn free_fn, void* user)
  * Each candidate runs `steps` steps (<= 0 -> 10) after two warm-up steps,
  * timed with CUDA events on the handle's stream; the state is saved first
  * and restored afterwards, and the step counter does not move.  The choice
- * is cached per (dtype, nx, ny, nz, force, Newtonian) for the process, so
- * later handles of the same kind reuse it without timing.  Any output
+ * is cached for the process per (dtype, in place or not, rounding, whether
+ * omega_9..18 are all 1, nx, ny, nz, force, Newtonian), so later handles of
+ * the same kind reuse it without timing.  Any output
  * pointer may be NULL.  Synchronises; temporarily needs one extra population
  * buffer of device memory. */
 int clbm_autotune(clbm_handle h, int steps, int* block_x, int* block_y, int* npt,

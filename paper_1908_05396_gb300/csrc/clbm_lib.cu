@@ -504,7 +504,8 @@ int clbm_sync(clbm_handle h) {
 }
 
 namespace {
-// Autotuner cache: (dtype, nx, ny, nz, force, newtonian) -> (bx, by, npt).
+// Autotuner cache: (kind, nx, ny, nz, force, newtonian) -> (bx, by, npt), the
+// kind being the storage form and what else decides which kernels run.
 std::mutex g_tune_mu;
 std::map<std::tuple<int, int, int, int, int, int>, std::tuple<int, int, int, double>> g_tune;
 }  // namespace
@@ -514,8 +515,10 @@ int clbm_autotune(clbm_handle h, int steps, int* block_x, int* block_y, int* npt
   if (bad(h)) return fail(h, CLBM_ERR_ARG, "invalid handle");
   if (int r = set_device(h)) return r;
   if (steps <= 0) steps = 10;
-  const auto key = std::make_tuple(int(h->dtype) + (h->in_place ? 16 : 0) + (h->sround ? 32 : 0), h->g.nx, h->g.ny,
-                                   h->g.nz, h->P.has_force, h->P.newtonian);
+  const bool unit = unit_rates(h->P);
+  const auto key = std::make_tuple(int(h->dtype) + (h->in_place ? 16 : 0) + (h->sround ? 32 : 0) +
+                                       (unit ? 0 : 64),
+                                   h->g.nx, h->g.ny, h->g.nz, h->P.has_force, h->P.newtonian);
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune.find(key);
@@ -536,10 +539,12 @@ int clbm_autotune(clbm_handle h, int steps, int* block_x, int* block_y, int* npt
                            {32, 4}, {32, 8}, {64, 1}, {64, 2}, {64, 4}, {128, 1}, {256, 1}};
   // FP16 forms with unit rates and two buffers: the pair kernel, which takes
   // from the block its thread count only
-  const bool pair = h->elem == 2 && !h->in_place && unit_rates(h->P);
+  const bool pair = h->elem == 2 && !h->in_place && unit;
   if (pair)
     for (int t : {32, 64, 128, 256}) cands.push_back({32, t / 32, 1});
-  for (int capped = 0; capped <= 1 && !pair; ++capped)
+  // other rates have neither a register-capped nor a TMA-staged kernel
+  const int caps = unit ? 1 : 0;
+  for (int capped = 0; capped <= caps && !pair; ++capped)
     for (auto& sh : shapes) {
       if (sh[0] > 32 && sh[0] > h->g.pitch) continue;
       cands.push_back({sh[0], sh[1], 1 + 4 * capped});
@@ -547,10 +552,10 @@ int clbm_autotune(clbm_handle h, int steps, int* block_x, int* block_y, int* npt
   // a lattice narrower than a warp: blocks as wide as its tile width
   const int tw = tile_width(h->g.nx, int(h->elem), 32, 64);
   if (tw < 32 && !pair)
-    for (int capped = 0; capped <= 1; ++capped)
+    for (int capped = 0; capped <= caps; ++capped)
       for (int t : {64, 128, 256}) cands.push_back({tw, t / tw, 1 + 4 * capped});
   // FP32 and FP16 storage: the TMA-staged kernel in each of its shapes
-  if ((h->dtype == CLBM_F32 || h->dtype == CLBM_F16S) && !h->in_place && !h->sround)
+  if ((h->dtype == CLBM_F32 || h->dtype == CLBM_F16S) && !h->in_place && !h->sround && unit)
     for (int v = 0; v < TMA_NVAR; ++v) cands.push_back({tma_bx(v), tma_by(v), TMA_NPT + 32 * v});
   // Save the state: tuning runs real steps.
   const size_t pop_bytes = size_t(NQ) * size_t(h->g.qstride) * h->elem;

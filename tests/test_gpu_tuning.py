@@ -1,0 +1,46 @@
+"""What the tuners time and keep."""
+import pytest
+
+from paper_1908_05396_gb300 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+CAVITY = wl.CAVITY_FACES
+
+
+@pytest.fixture(scope="module")
+def clbm():
+    from paper_1908_05396_gb300 import build
+    build.build()
+    from paper_1908_05396_gb300 import clbm as c
+    c.lib()
+    return c
+
+
+def _lattice(clbm, dims, form, **kw):
+    dtype, _, opt = form.partition("_")
+    lat = clbm.Lattice(*dims, face=CAVITY, K=0.02, n=0.7, U_lid=(0.05, 0.0, 0.0), dtype=dtype,
+                       in_place=opt == "inplace", **kw)
+    if opt == "sr":
+        lat.set_rounding("stochastic")
+    return lat
+
+
+# A choice handed on comes with its measured time, to the last bit; the two kinds
+# are timed over 53 and 59 steps, so that equal ticks do not give equal times.
+@pytest.mark.parametrize("rates_first", [False, True])
+@pytest.mark.parametrize("form", ["f64", "f32", "f16s", "f16s_sr", "f16r", "f32_inplace"])
+def test_unit_and_other_rates_are_tuned_apart(clbm, form, rates_first):
+    dims = (34, 22 + rates_first, 18)      # sizes no other test tunes
+    infos = {}
+    for rates in (rates_first, not rates_first, rates_first):
+        with _lattice(clbm, dims, form) as lat:
+            if rates:
+                lat.set_rates({9: 1.2, 12: 0.9})
+            info = lat.autotune(53 if rates else 59)
+        if rates:
+            assert info["npt"] == 1        # the one kernel that such lattices run
+        if rates in infos:
+            assert info == infos[rates]
+        infos[rates] = info
+    assert infos[False]["us_per_step"] != infos[True]["us_per_step"]
