@@ -178,9 +178,10 @@ typedef void (*clbm_free_fn)(void* ptr, size_t bytes, int device, void* stream, 
 int clbm_set_allocator(clbm_alloc_fn alloc_fn, clbm_free_fn free_fn, void* user);
 
 /* Pick the launch shape of h's step kernel by timing: thread-block shapes
- * from 8x4 to 256x1 with and without a 64-register cap; for the two-buffer
- * FP16 forms the block's thread count; for FP32 and F16S storage also the
- * TMA-staged kernel in each of its shapes (see clbm_set_launch).
+ * from 8x4 to 256x1, the untuned one among them, with and without a
+ * 64-register cap; for FP16 lattices that step two nodes per thread the block's
+ * thread count; for FP32 and F16S storage also the TMA-staged kernel in each
+ * of its shapes (see clbm_set_launch).
  * Each candidate runs `steps` steps (<= 0 -> 10) after two warm-up steps,
  * timed with CUDA events on the handle's stream; the state is saved first
  * and restored afterwards, and the step counter does not move.  The choice

@@ -537,13 +537,19 @@ int clbm_autotune(clbm_handle h, int steps, int* block_x, int* block_y, int* npt
   std::vector<Cand> cands;
   const int shapes[][2] = {{8, 4},  {8, 8},  {16, 2}, {16, 4}, {16, 8},  {32, 1}, {32, 2},
                            {32, 4}, {32, 8}, {64, 1}, {64, 2}, {64, 4}, {128, 1}, {256, 1}};
-  // FP16 forms with unit rates and two buffers: the pair kernel, which takes
-  // from the block its thread count only
-  const bool pair = h->elem == 2 && !h->in_place && unit;
+  // what an untuned lattice runs is always timed
+  const dim3 blkd = default_block(h->g.nx, int(h->elem));
+  cands.push_back({int(blkd.x), int(blkd.y), 1});
+  // FP16 lattices that step pairs take from the block its thread count only
+  // (smaller ones use its shape: 36^3 F16R took 8.0 us a step with the pairs'
+  // candidates, all 32 wide, against 4.7 untuned)
+  const bool pair = h->elem == 2 && !h->in_place && unit &&
+                    pair_pays(h->g, h->dtype == CLBM_F16R);
   if (pair)
     for (int t : {32, 64, 128, 256}) cands.push_back({32, t / 32, 1});
-  // other rates have neither a register-capped nor a TMA-staged kernel
-  const int caps = unit ? 1 : 0;
+  // other rates have neither a register-capped nor a TMA-staged kernel, and
+  // the two-buffer FP16 forms have one variant
+  const int caps = unit && (h->elem != 2 || h->in_place) ? 1 : 0;
   for (int capped = 0; capped <= caps && !pair; ++capped)
     for (auto& sh : shapes) {
       if (sh[0] > 32 && sh[0] > h->g.pitch) continue;

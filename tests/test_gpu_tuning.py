@@ -44,3 +44,12 @@ def test_unit_and_other_rates_are_tuned_apart(clbm, form, rates_first):
             assert info == infos[rates]
         infos[rates] = info
     assert infos[False]["us_per_step"] != infos[True]["us_per_step"]
+
+
+# FP16 lattices too small for pairs run one node per thread and use the block's
+# shape: 32-wide blocks leave three lanes in four, or seven rows in sixteen, idle
+@pytest.mark.parametrize("dims", [(8, 96, 40), (36, 36, 36)])
+@pytest.mark.parametrize("form", ["f16s", "f16s_sr", "f16r"])
+def test_small_fp16_lattices_are_tuned_by_shape(clbm, form, dims):
+    with _lattice(clbm, dims, form) as lat:
+        assert lat.autotune(40)["block"][0] < 32
