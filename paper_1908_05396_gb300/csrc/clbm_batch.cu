@@ -368,6 +368,25 @@ cudaError_t launch_lattices(clbm_batch_ctx* b, bool check, int flip, int ahead =
   return cudaSuccess;
 }
 
+// How a lattice is cut into tiles by the persistent kernel's launch shape.
+struct Tiling {
+  int threads, tw, tx, ty, tz;  // block size, threads along x of a tile, tiles per axis
+  bool fits() const { return tx <= 255 && ty <= 4095 && tz <= 4095; }  // the tile words
+};
+Tiling tiling(const clbm_batch_ctx* b, const clbm_ctx* h) {
+  Tiling t;
+  t.threads = int(b->block.x * b->block.y);
+  // FP16 forms with unit rates step two nodes along x per thread
+  const bool pair = h->elem == 2 && unit_rates(h->P);
+  t.tw = pair ? pair_width(h->g.nx, t.threads, int(b->block.x))
+              : tile_width(h->g.nx, int(h->elem), int(b->block.x), t.threads);
+  const int th = t.threads / t.tw, nodes_x = pair ? 2 * t.tw : t.tw;
+  t.tx = (h->g.nx + nodes_x - 1) / nodes_x;
+  t.ty = (h->g.ny + th - 1) / th;
+  t.tz = (h->g.nz + b->zc - 1) / b->zc;  // chunks of zc planes
+  return t;
+}
+
 // Rebuild and upload the tables from the attached lattices' current state.
 int upload(clbm_batch_ctx* b) {
   BCK(b, cudaStreamSynchronize(b->stream));  // staging buffers and tables are free
@@ -385,31 +404,23 @@ int upload(clbm_batch_ctx* b) {
       if (!h || h->in_place ||
           (h->P.has_force ? 2 : 0) + (unit_rates(h->P) ? 0 : 1) != pass)
         continue;
-      const int threads = int(b->block.x * b->block.y);
-      // FP16 forms with unit rates step two nodes along x per thread
-      const bool pair = h->elem == 2 && unit_rates(h->P);
-      const int tw = pair ? pair_width(h->g.nx, threads, int(b->block.x))
-                          : tile_width(h->g.nx, int(h->elem), int(b->block.x), threads);
+      const Tiling t = tiling(b, h);
       int twl = 0;
-      while ((1 << twl) < tw) ++twl;
-      const int th = threads / tw;
-      const int nodes_x = pair ? 2 * tw : tw;
-      const int tx = (h->g.nx + nodes_x - 1) / nodes_x;
-      const int ty = (h->g.ny + th - 1) / th;
-      const int tz = (h->g.nz + b->zc - 1) / b->zc;   // chunks of zc planes
-      if (tx > 255 || ty > 4095 || tz > 4095)
+      while ((1 << twl) < t.tw) ++twl;
+      if (!t.fits())
         return bfail(b, CLBM_ERR_UNSUPPORTED, "lattice has too many tiles for the batch table");
       // the lattice's step count minus the batch's: the kernels add the
       // batch's device-side count to recover the lattice's own
       const unsigned so = unsigned(uint64_t(h->steps) - uint64_t(b->steps));
-      fill_desc(b->dtype, stage + size_t(nlat) * b->desc_bytes, h, tx, ty, twl, s, so, threads);
-      for (int kz = 0; kz < tz; ++kz)
-        for (int ky = 0; ky < ty; ++ky)
-          for (int kx = 0; kx < tx; ++kx) {
+      fill_desc(b->dtype, stage + size_t(nlat) * b->desc_bytes, h, t.tx, t.ty, twl, s, so,
+                t.threads);
+      for (int kz = 0; kz < t.tz; ++kz)
+        for (int ky = 0; ky < t.ty; ++ky)
+          for (int kx = 0; kx < t.tx; ++kx) {
             b->h_owner.push_back(nlat);
             b->h_coord.push_back(unsigned(kx) | (unsigned(ky) << 8) | (unsigned(kz) << 20));
           }
-      ntiles += tx * ty * tz;
+      ntiles += t.tx * t.ty * t.tz;
       ++nlat;
     }
     tile_end[pass] = ntiles;
@@ -909,6 +920,11 @@ int clbm_batch_autotune(clbm_batch b, int steps, int* block_x, int* block_y, int
         b->block = dim3(sh[0], sh[1], 1);
         b->zc = z;
         b->blocks_per_sm = bp;
+        // a shape whose tile words cannot address some lattice (16-wide tiles of
+        // rows beyond 4080 nodes) is no candidate
+        bool fits = true;
+        for (const clbm_ctx* h : b->slots) fits = fits && (!h || tiling(b, h).fits());
+        if (!fits) continue;
         b->dirty = true;
         if (upload(b) != CLBM_OK) { err = cudaErrorUnknown; break; }
         err = fork_streams(b, 2);
@@ -940,6 +956,8 @@ int clbm_batch_autotune(clbm_batch b, int steps, int* block_x, int* block_y, int
   // One launch per lattice (not for F16R, nor with a stochastically rounding
   // lattice): block x kernel variant x streams.
   int bmode = 0, pbx = 32, pby = 2, pnpt = 5, pst = 4;
+  b->block = block0;  // (the tables are written in this mode too)
+  b->zc = zc0;
   if (b->dtype != CLBM_F16R && !any_sround(b)) {
     const int pshapes[][2] = {{16, 4}, {32, 2}, {32, 4}};
     const int pnpts[] = {5, 1};

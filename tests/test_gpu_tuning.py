@@ -1,4 +1,5 @@
 """What the tuners time and keep."""
+import numpy as np
 import pytest
 
 from paper_1908_05396_gb300 import workloads as wl
@@ -53,3 +54,22 @@ def test_unit_and_other_rates_are_tuned_apart(clbm, form, rates_first):
 def test_small_fp16_lattices_are_tuned_by_shape(clbm, form, dims):
     with _lattice(clbm, dims, form) as lat:
         assert lat.autotune(40)["block"][0] < 32
+
+
+# 16-wide tiles of these rows are more than a tile word can address: the batch's
+# tuner must pass over them, not give up (FP16 pairs are twice as wide)
+@pytest.mark.parametrize("form,nx", [("f64", 4200), ("f32", 4200), ("f32", 8160), ("f16s", 8200),
+                                     ("f16r", 8200)])
+def test_batch_tuner_passes_over_shapes_that_do_not_fit(clbm, form, nx):
+    with _lattice(clbm, (nx, 4, 4), form) as lat, _lattice(clbm, (nx, 4, 4), form) as lone:
+        with clbm.Batch(form, capacity=2) as b:
+            b.add(lat)
+            b.step(3)
+            f = lat.get_state()
+            info = b.autotune(2)
+            assert info["us_per_step"] < 1e4
+            assert np.array_equal(lat.get_state(), f) and lat.steps_done() == 3
+            b.step(4)
+        lone.step(7)
+        u, v = lat.fields()[1], lone.fields()[1]
+        assert np.linalg.norm(u - v) <= 2e-3 * np.linalg.norm(v)
