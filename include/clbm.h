@@ -304,15 +304,20 @@ int clbm_batch_set_launch(clbm_batch b, int block_x, int block_y, int zc, int bl
  * those of clbm_step on each lattice.  This mode also steps in-place
  * lattices.  clbm_batch_set_launch() returns to the persistent kernel. */
 int clbm_batch_set_lattice_launch(clbm_batch b, int block_x, int block_y, int npt, int streams);
+/* Back to the launch of a batch that was neither set nor tuned.
+ * CLBM_ERR_UNSUPPORTED while an in-place lattice is attached. */
+int clbm_batch_reset_launch(clbm_batch b);
 /* Time block shapes x zc x blocks-per-SM x register cap of the persistent
- * kernel and, except for F16R and stochastically rounding F16S lattices,
- * block shapes x kernel variant x streams of one
- * launch per lattice, on the attached lattices (states saved and restored),
- * and keep the fastest (only the latter while an in-place lattice is
- * attached).  Persistent kernel: *blocks_per_sm is negative when
+ * kernel, except for F16R and stochastically rounding F16S lattices block
+ * shapes x kernel variant x streams of one launch per lattice, and what the
+ * batch runs untuned, on the attached lattices (states saved and restored),
+ * and keep the fastest (while an in-place lattice is attached, of one launch
+ * per lattice only).  Persistent kernel: *blocks_per_sm is negative when
  * the capped variant won.  One launch per lattice: *zc is 0, *block_x and
  * *block_y are the lattices' block, |*blocks_per_sm| is the stream count,
- * negative for the register-capped kernel. */
+ * negative for the register-capped kernel; *block_x and *block_y are 0 when the
+ * untuned launch won, in which each lattice has its own block
+ * (clbm_batch_reset_launch sets it in another batch). */
 int clbm_batch_autotune(clbm_batch b, int steps, int* block_x, int* block_y, int* zc,
                         int* blocks_per_sm, double* us_per_step);
 int clbm_batch_sync(clbm_batch b);

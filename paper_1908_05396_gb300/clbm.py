@@ -391,6 +391,7 @@ class Batch:
                                                 ctypes.c_int]
             L.clbm_batch_set_lattice_launch.argtypes = [B, ctypes.c_int, ctypes.c_int,
                                                         ctypes.c_int, ctypes.c_int]
+            L.clbm_batch_reset_launch.argtypes = [B]
             L.clbm_batch_stats_all.argtypes = [B, _D, _D, ctypes.POINTER(ctypes.c_int),
                                                ctypes.POINTER(ctypes.c_int64)]
             L.clbm_batch_autotune.argtypes = [B, ctypes.c_int] + [ctypes.POINTER(ctypes.c_int)] * 4 + [_D]
@@ -400,7 +401,8 @@ class Batch:
             L.clbm_batch_last_error.restype = ctypes.c_char_p
             for n in ("clbm_batch_create", "clbm_batch_add", "clbm_batch_remove", "clbm_batch_detach",
                       "clbm_batch_step", "clbm_batch_stats", "clbm_batch_set_launch",
-                      "clbm_batch_set_lattice_launch", "clbm_batch_stats_all",
+                      "clbm_batch_set_lattice_launch", "clbm_batch_reset_launch",
+                      "clbm_batch_stats_all",
                       "clbm_batch_autotune", "clbm_batch_sync", "clbm_batch_destroy"):
                 getattr(L, n).restype = ctypes.c_int
             L._batch_ready = True
@@ -460,9 +462,14 @@ class Batch:
         self._bcheck(lib().clbm_batch_set_lattice_launch(self._b, int(block_x), int(block_y),
                                                          int(npt), int(streams)))
 
+    def reset_launch(self) -> None:
+        """Back to the launch of a batch that was neither set nor tuned."""
+        self._bcheck(lib().clbm_batch_reset_launch(self._b))
+
     def autotune(self, steps: int = 6) -> dict:
         """Time the launch choices and keep the fastest; the returned dict
-        can be given back to ``apply_launch``."""
+        can be given back to ``apply_launch`` (a per-lattice block of (0, 0) is
+        the untuned launch, in which each lattice has its own block)."""
         v = [ctypes.c_int() for _ in range(4)]
         us = ctypes.c_double()
         self._bcheck(lib().clbm_batch_autotune(self._b, int(steps), *[ctypes.byref(x) for x in v],
@@ -476,7 +483,9 @@ class Batch:
 
     def apply_launch(self, info: dict) -> None:
         """Set the launch an ``autotune`` result describes."""
-        if info["mode"] == "per_lattice":
+        if info["mode"] == "per_lattice" and info["block"] == (0, 0):
+            self.reset_launch()
+        elif info["mode"] == "per_lattice":
             self.set_lattice_launch(*info["block"], info["npt"], info["streams"])
         else:
             self.set_launch(*info["block"], info["zc"], info["blocks_per_sm"])

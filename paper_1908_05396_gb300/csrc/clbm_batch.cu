@@ -64,11 +64,7 @@ struct clbm_batch_ctx {
   bool dirty = true;
   dim3 block{32, 4, 1};
   int zc = 1;                         // planes per tile (autotuned)
-  // Until tuned (FP32-math forms): the register-capped kernel, eight CTAs
-  // per SM, which is within a few per cent of the tuned launch from 4 to 64
-  // small lattices and 1.8x faster than four uncapped CTAs once they fill the
-  // GPU.  FP64 keeps four uncapped CTAs (its registers are twice as wide).
-  int blocks_per_sm = 8;
+  int blocks_per_sm = 8;              // (see default_residency)
   bool cap = true;                    // register-capped kernel variant
   int sms = 1;
   bool rates = false;                 // some attached lattice has rates omega_9..18 other than 1
@@ -107,6 +103,15 @@ int bfail(clbm_batch_ctx* b, int code, const std::string& m) {
       return bfail(b, e_ == cudaErrorMemoryAllocation ? CLBM_ERR_OOM : CLBM_ERR_CUDA,        \
                    std::string(#expr) + ": " + cudaGetErrorString(e_));                      \
   } while (0)
+
+// Until tuned (FP32-math forms): the register-capped kernel, eight CTAs
+// per SM, which is within a few per cent of the tuned launch from 4 to 64
+// small lattices and 1.8x faster than four uncapped CTAs once they fill the
+// GPU.  FP64 keeps four uncapped CTAs (its registers are twice as wide).
+void default_residency(clbm_batch_ctx* b) {
+  b->cap = b->dtype != CLBM_F64;
+  b->blocks_per_sm = b->cap ? 8 : 4;
+}
 
 // Bytes of the check sums of all slots.
 size_t acc_bytes(const clbm_batch_ctx* b) {
@@ -669,10 +674,7 @@ int clbm_batch_create(clbm_dtype dtype, int capacity, int check_interval, void* 
   clbm_batch_ctx* b = new (std::nothrow) clbm_batch_ctx();
   if (!b) return bfail(nullptr, CLBM_ERR_OOM, "host allocation failed");
   b->dtype = dtype;
-  if (dtype == CLBM_F64) {
-    b->blocks_per_sm = 4;
-    b->cap = false;
-  }
+  default_residency(b);
   b->capacity = capacity;
   b->check_interval = check_interval;
   for (int k = 2; k <= 10; k += 2)  // the largest even divisor up to 10
@@ -842,6 +844,25 @@ int clbm_batch_set_launch(clbm_batch b, int block_x, int block_y, int zc, int bl
   return CLBM_OK;
 }
 
+int clbm_batch_reset_launch(clbm_batch b) {
+  if (!valid(b)) return bfail(b, CLBM_ERR_ARG, "invalid batch");
+  for (clbm_ctx* h : b->slots)
+    if (h && h->in_place)
+      return bfail(b, CLBM_ERR_UNSUPPORTED,
+                   "the batch holds in-place lattices: the persistent kernel needs two buffers");
+  BCK(b, cudaSetDevice(b->device));
+  BCK(b, cudaStreamSynchronize(b->stream));
+  const clbm_batch_ctx fresh;
+  b->block = fresh.block;
+  b->zc = fresh.zc;
+  default_residency(b);
+  b->mode = 0;
+  b->auto_mode = true;
+  b->dirty = true;
+  drop_graph(b);
+  return CLBM_OK;
+}
+
 int clbm_batch_set_lattice_launch(clbm_batch b, int block_x, int block_y, int npt, int streams) {
   if (!valid(b)) return bfail(b, CLBM_ERR_ARG, "invalid batch");
   if (b->dtype == CLBM_F16R)
@@ -895,9 +916,11 @@ int clbm_batch_autotune(clbm_batch b, int steps, int* block_x, int* block_y, int
     any_in_place = any_in_place || h->in_place;
   }
   const int64_t bsteps0 = b->steps;
-  b->auto_mode = false;  // the timing below chooses
-  const dim3 block0 = b->block;
+  const bool auto0 = b->auto_mode;
+  const int mode0 = b->mode, npt0 = b->pl_npt, st0 = b->pl_streams;
+  const dim3 block0 = b->block, plblock0 = b->pl_block;
   const int zc0 = b->zc, bps0 = b->blocks_per_sm;
+  b->auto_mode = false;  // the timing below chooses
   const int shapes[][2] = {{16, 4}, {16, 8}, {32, 2}, {32, 4}, {32, 8}, {64, 4}};
   const int zcs[] = {1, 2, 4};
   const int bpss[] = {4, 6, 8};
@@ -953,6 +976,28 @@ int clbm_batch_autotune(clbm_batch b, int steps, int* block_x, int* block_y, int
           bc = capped != 0;
         }
       }
+  // us a step of one launch per lattice over `streams` streams (sets err)
+  auto time_lattices = [&](int streams) {
+    b->dirty = true;
+    if (upload(b) != CLBM_OK) err = cudaErrorUnknown;
+    auto run = [&](int n) {
+      if (err == cudaSuccess) err = fork_streams(b, streams);
+      for (int k = 0; k < n && err == cudaSuccess; ++k) {
+        err = launch_lattices(b, false, b->parity);
+        b->parity ^= 1;
+      }
+      if (err == cudaSuccess) err = join_streams(b, streams);
+    };
+    run(2);
+    if (err == cudaSuccess) err = cudaEventRecord(e0, b->stream);
+    run(steps);
+    if (err == cudaSuccess) err = cudaEventRecord(e1, b->stream);
+    if (err == cudaSuccess) err = cudaEventSynchronize(e1);
+    float ms = 0.0f;
+    if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, e0, e1);
+    b->parity = 0;
+    return 1e3 * ms / steps;
+  };
   // One launch per lattice (not for F16R, nor with a stochastically rounding
   // lattice): block x kernel variant x streams.
   int bmode = 0, pbx = 32, pby = 2, pnpt = 5, pst = 4;
@@ -971,27 +1016,9 @@ int clbm_batch_autotune(clbm_batch b, int steps, int* block_x, int* block_y, int
           b->pl_block = dim3(sh[0], sh[1], 1);
           b->pl_npt = np;
           b->pl_streams = ns;
-          b->dirty = true;
-          if (upload(b) != CLBM_OK) { err = cudaErrorUnknown; break; }
-          err = fork_streams(b, b->pl_streams);
-          for (int k = 0; k < 2 && err == cudaSuccess; ++k) {
-            err = launch_lattices(b, false, b->parity);
-            b->parity ^= 1;
-          }
-          if (err == cudaSuccess) err = join_streams(b, b->pl_streams);
-          if (err == cudaSuccess) err = cudaEventRecord(e0, b->stream);
-          if (err == cudaSuccess) err = fork_streams(b, b->pl_streams);
-          for (int k = 0; k < steps && err == cudaSuccess; ++k) {
-            err = launch_lattices(b, false, b->parity);
-            b->parity ^= 1;
-          }
-          if (err == cudaSuccess) err = join_streams(b, b->pl_streams);
-          if (err == cudaSuccess) err = cudaEventRecord(e1, b->stream);
-          if (err == cudaSuccess) err = cudaEventSynchronize(e1);
-          float ms = 0.0f;
-          if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, e0, e1);
-          if (err == cudaSuccess && 1e3 * ms / steps < best) {
-            best = 1e3 * ms / steps;
+          const double us = time_lattices(ns);
+          if (err == cudaSuccess && us < best) {
+            best = us;
             bmode = 1;
             pbx = sh[0];
             pby = sh[1];
@@ -999,6 +1026,25 @@ int clbm_batch_autotune(clbm_batch b, int steps, int* block_x, int* block_y, int
             pst = ns;
           }
         }
+  }
+  // What the batch runs untuned, if that is one launch per lattice too (every
+  // form, each lattice with its own default block): without it, tuning lost F16R
+  // batches 1.4 to 1.7x and stochastic F16S ones 1.3 to 1.8x (4 and 12 cavities of
+  // 47^3 and 64^3; 12 of 47^3: 43.6 us a step untuned, 59.1 tuned).
+  bool untuned = false;
+  if (err == cudaSuccess && !any_in_place) {
+    b->mode = 0;
+    b->auto_mode = true;
+    b->dirty = true;
+    if (upload(b) != CLBM_OK) err = cudaErrorUnknown;
+    if (err == cudaSuccess && b->spread) {
+      const double us = time_lattices(SPREAD_STREAMS);
+      if (err == cudaSuccess && us < best) {
+        best = us;
+        bmode = 0;
+        untuned = true;
+      }
+    }
   }
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
@@ -1020,7 +1066,24 @@ int clbm_batch_autotune(clbm_batch b, int steps, int* block_x, int* block_y, int
     cudaFreeAsync(saved[s], b->stream);
   }
   b->steps = bsteps0;
-  b->block = dim3(bx, by, 1);
+  b->dirty = true;
+  drop_graph(b);
+  cudaError_t e3 = cudaStreamSynchronize(b->stream);
+  if (err == cudaSuccess) err = e3;
+  if (err != cudaSuccess) {  // the launch as it was
+    b->auto_mode = auto0;
+    b->mode = mode0;
+    b->block = block0;
+    b->zc = zc0;
+    b->blocks_per_sm = bps0;
+    b->cap = cap0;
+    b->pl_block = plblock0;
+    b->pl_npt = npt0;
+    b->pl_streams = st0;
+    return bfail(b, CLBM_ERR_CUDA, std::string("clbm_batch_autotune: ") + cudaGetErrorString(err));
+  }
+  b->auto_mode = untuned;
+  b->block = dim3(bx, by, 1);  // (also when members that leave end the launches per lattice)
   b->zc = bz;
   b->blocks_per_sm = bb;
   b->cap = bc;
@@ -1028,13 +1091,13 @@ int clbm_batch_autotune(clbm_batch b, int steps, int* block_x, int* block_y, int
   b->pl_block = dim3(pbx, pby, 1);
   b->pl_npt = pnpt;
   b->pl_streams = pst;
-  b->dirty = true;
-  drop_graph(b);
-  cudaError_t e3 = cudaStreamSynchronize(b->stream);
-  if (err == cudaSuccess) err = e3;
-  if (err != cudaSuccess)
-    return bfail(b, CLBM_ERR_CUDA, std::string("clbm_batch_autotune: ") + cudaGetErrorString(err));
-  if (bmode == 1) {
+  if (untuned) {
+    // zc = 0 and no block: one launch per lattice, each with its own
+    if (block_x) *block_x = 0;
+    if (block_y) *block_y = 0;
+    if (zc) *zc = 0;
+    if (blocks_per_sm) *blocks_per_sm = SPREAD_STREAMS;
+  } else if (bmode == 1) {
     // zc = 0: one launch per lattice; |blocks_per_sm| = streams, negative
     // for the register-capped kernel
     if (block_x) *block_x = pbx;
