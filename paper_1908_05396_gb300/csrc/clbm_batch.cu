@@ -248,8 +248,10 @@ constexpr double SPREAD_NODES = 100000.0;
 
 int pl_stream_count(const clbm_batch_ctx* b) { return b->spread ? SPREAD_STREAMS : b->pl_streams; }
 
-// The step count that seeds stochastic rounding in a replayed graph.
-__global__ void set_count_kernel(unsigned* p, unsigned v) { *p = v; }
+// The batch's step count in device memory, which seeds stochastic rounding: each
+// run of spread steps advances it, so that a graph, the batch's own or one that
+// a caller captured, rounds with new bits whenever it is replayed.
+__global__ void add_count_kernel(unsigned* p, unsigned n) { *p += n; }
 
 bool counts_steps(const clbm_batch_ctx* b) { return b->dtype == CLBM_F16R || any_sround(b); }
 
@@ -315,8 +317,8 @@ cudaError_t join_streams(clbm_batch_ctx* b, int n) {
 // One step of every lattice, each on its stream.  `flip` = 1 when the state
 // sits in the other buffer than h->cur says (inside a captured interval).
 // The check sums of slot s go to the batch's row s, as in mode 0.  `ahead`: steps
-// already launched since h->steps was current; `base`: in a captured graph,
-// the device-side count that holds the batch's steps at its start.
+// already launched since h->steps was current; `base`: the device-side count
+// that holds the batch's steps at the start of these, if the seeds come from it.
 cudaError_t launch_lattices(clbm_batch_ctx* b, bool check, int flip, int ahead = 0,
                             const unsigned* base = nullptr) {
   for (int s = 0; s < b->capacity; ++s) {
@@ -519,13 +521,18 @@ int one_step(clbm_batch_ctx* b) {
 
 // n spread steps on the batch's stream (which may be capturing), the last one
 // a check step if `check`.
-cudaError_t launch_spread(clbm_batch_ctx* b, int n, bool check, const unsigned* base) {
+cudaError_t launch_spread(clbm_batch_ctx* b, int n, bool check) {
+  unsigned* count = counts_steps(b) ? b->d_hdr->step : nullptr;
   cudaError_t e = cudaSuccess;
   if (check) e = cudaMemsetAsync(b->d_acc, 0, acc_bytes(b), b->stream);
   if (e == cudaSuccess) e = fork_streams(b, SPREAD_STREAMS);
   for (int k = 0; k < n && e == cudaSuccess; ++k)
-    e = launch_lattices(b, check && k == n - 1, k & 1, k, base);
+    e = launch_lattices(b, check && k == n - 1, k & 1, k, count);
   if (e == cudaSuccess) e = join_streams(b, SPREAD_STREAMS);
+  if (e == cudaSuccess && count) {
+    add_count_kernel<<<1, 1, 0, b->stream>>>(count, unsigned(n));
+    e = cudaGetLastError();
+  }
   if (e == cudaSuccess && check) {
     e = cudaMemcpyAsync(b->h_acc, b->d_acc, acc_bytes(b), cudaMemcpyDeviceToHost, b->stream);
     if (e == cudaSuccess) e = cudaEventRecord(b->check_done, b->stream);
@@ -544,14 +551,13 @@ int spread_steps(clbm_batch_ctx* b, int64_t left, int64_t* done) {
   BCK(b, cudaStreamIsCapturing(b->stream, &cap));
   if (n < b->sub || b->steps - b->table_steps < SPREAD_SETTLED ||
       cap != cudaStreamCaptureStatusNone) {
-    BCK(b, launch_spread(b, n, check, nullptr));
+    BCK(b, launch_spread(b, n, check));
   } else {
-    const unsigned* base = counts_steps(b) ? b->d_hdr->step : nullptr;
     cudaGraphExec_t& exec = b->sub_graph[check ? 1 : 0];
     if (!exec) {
       cudaGraph_t g = nullptr;
       BCK(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-      cudaError_t e = launch_spread(b, n, check, base);
+      cudaError_t e = launch_spread(b, n, check);
       const cudaError_t e2 = cudaStreamEndCapture(b->stream, &g);
       if (e == cudaSuccess) e = e2;
       if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, g, 0);
@@ -560,10 +566,6 @@ int spread_steps(clbm_batch_ctx* b, int64_t left, int64_t* done) {
         exec = nullptr;
         return bfail(b, CLBM_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(e));
       }
-    }
-    if (base) {
-      set_count_kernel<<<1, 1, 0, b->stream>>>(b->d_hdr->step, unsigned(uint64_t(b->steps)));
-      BCK(b, cudaGetLastError());
     }
     BCK(b, cudaGraphLaunch(exec, b->stream));
   }
