@@ -547,9 +547,10 @@ cudaError_t launch_spread(clbm_batch_ctx* b, int n, bool check) {
 int spread_steps(clbm_batch_ctx* b, int64_t left, int64_t* done) {
   const int n = int(std::min<int64_t>(left, b->sub - b->steps % b->sub));
   const bool check = (b->steps + n) % b->check_interval == 0;
+  const bool legacy = b->stream == cudaStreamLegacy;  // cannot be captured
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;  // the caller's own capture
-  BCK(b, cudaStreamIsCapturing(b->stream, &cap));
-  if (n < b->sub || b->steps - b->table_steps < SPREAD_SETTLED ||
+  if (!legacy) BCK(b, cudaStreamIsCapturing(b->stream, &cap));
+  if (n < b->sub || b->steps - b->table_steps < SPREAD_SETTLED || legacy ||
       cap != cudaStreamCaptureStatusNone) {
     BCK(b, launch_spread(b, n, check));
   } else {

@@ -1,6 +1,7 @@
 """Steps of an untuned batch of large lattices that a caller captures into a graph
 of its own: every replay advances the lattices as fresh steps would, with new
-random bits where stores are rounded stochastically."""
+random bits where stores are rounded stochastically.  And such a batch on the
+legacy default stream, which cannot be captured: it never replays a graph."""
 import numpy as np
 import pytest
 
@@ -52,3 +53,16 @@ def test_replays_continue_the_steps(clbm, form):
             assert np.array_equal(m.get_state(), lat.get_state())
     for lat in lone + mem:
         lat.close()
+
+
+@pytest.mark.parametrize("form", ["f32", "f16r"])
+def test_legacy_default_stream(clbm, form):
+    kw = dict(face=wl.CAVITY_FACES, K=0.02, n=0.7, U_lid=(0.05, 0.0, 0.0), dtype=form)
+    with clbm.Lattice(47, 46, 50, **kw) as lat, clbm.Lattice(47, 46, 50, **kw) as lone:
+        with clbm.Batch(form, capacity=1, stream=1) as b:      # cudaStreamLegacy
+            b.add(lat)
+            for _ in range(15):                  # past the steps launched singly
+                b.step(10)
+            b.sync()
+        lone.step(150)
+        assert np.array_equal(lat.get_state(), lone.get_state())
