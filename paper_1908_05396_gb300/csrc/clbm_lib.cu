@@ -48,10 +48,11 @@ clbm_alloc_fn g_alloc_fn = nullptr;
 clbm_free_fn g_free_fn = nullptr;
 void* g_alloc_user = nullptr;
 
-// Pinned copies of the check sums (CHECK_BYTES each): the first 64 lattices of
-// the process share one pinned slab, because a cudaMallocHost and cudaFreeHost
-// pair costs 0.33 ms, as much as the rest of a small lattice's creation.
-// Slots are handed back at destruction; the slab (130 KB) stays.
+// Pinned copies of the check sums (CHECK_BYTES each): up to 64 lattices of the
+// process share one pinned slab (130 KB), because a cudaMallocHost and
+// cudaFreeHost pair costs 0.33 ms, as much as the rest of a small lattice's
+// creation.  Slots are handed back at destruction, the slab with the last one:
+// nothing outlives the lattices (a program may reset the device between them).
 constexpr int PINNED_SLOTS = 64;
 constexpr size_t PINNED_STRIDE = (CHECK_BYTES + 63) / 64 * 64;
 std::mutex g_pinned_mu;
@@ -85,6 +86,10 @@ void pinned_give(double* p) {
     const char* c = reinterpret_cast<const char*>(p);
     if (g_pinned && c >= g_pinned && c < g_pinned + PINNED_SLOTS * PINNED_STRIDE) {
       g_pinned_used[size_t(c - g_pinned) / PINNED_STRIDE] = false;
+      for (bool used : g_pinned_used)
+        if (used) return;
+      cudaFreeHost(g_pinned);
+      g_pinned = nullptr;
       return;
     }
   }
