@@ -1013,14 +1013,13 @@ __device__ __forceinline__ void collide_unit(const CollideConst<typename ScalarO
     R bx = -p.Dxyy, cx_ = -p.Dxzz, by_ = -p.Dxxy, cy_ = -p.Dyzz, bz_ = -p.Dxxz, cz_ = -p.Dyyz;
     R dr9 = mulr(R(T(1.0 / 9.0)), drho);
     if (FORCE) {
-      const R fx = R(T(C.FS[0]) * T(1.0 / 6.0)), fy = R(T(C.FS[1]) * T(1.0 / 6.0)),
-              fz = R(T(C.FS[2]) * T(1.0 / 6.0));
-      bx = fx - p.Dxyy;
-      cx_ = fx - p.Dxzz;
-      by_ = fy - p.Dxxy;
-      cy_ = fy - p.Dyzz;
-      bz_ = fz - p.Dxxz;
-      cz_ = fz - p.Dyyz;
+      const R s6 = R(T(1.0 / 6.0));
+      bx = fma(Fx, s6, -p.Dxyy);
+      cx_ = fma(Fx, s6, -p.Dxzz);
+      by_ = fma(Fy, s6, -p.Dxxy);
+      cy_ = fma(Fy, s6, -p.Dyzz);
+      bz_ = fma(Fz, s6, -p.Dxxz);
+      cz_ = fma(Fz, s6, -p.Dyyz);
       nxy = fma(ux, Fy, fma(uy, Fx, mulr(nw, mxy)));
       nxz = fma(ux, Fz, fma(uz, Fx, mulr(nw, mxz)));
       nyz = fma(uy, Fz, fma(uz, Fy, mulr(nw, myz)));
