@@ -218,8 +218,8 @@ int clbm_set_launch(clbm_handle h, int block_x, int block_y, int npt);
  * can improve stability).  omega[k] is omega_(9+k); each must lie in (0, 2).
  * omega_9 also scales the isotropic part of the strain rate that sets
  * omega_nu.  Takes effect from the next step.  Lattices whose rates are not
- * all 1 run the plain one-node-per-thread kernel whatever launch shape is set
- * (its block is kept).  Not for a lattice in a batch
+ * all 1 run one node per thread in the block that is set, register-capped only
+ * if they are in-place FP32 or F16S lattices, without TMA.  Not for a lattice in a batch
  * (CLBM_ERR_ARG: detach it first).  Errors: CLBM_ERR_ARG. */
 int clbm_set_rates(clbm_handle h, const double omega[10]);
 

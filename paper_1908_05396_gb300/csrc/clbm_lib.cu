@@ -552,9 +552,9 @@ int clbm_autotune(clbm_handle h, int steps, int* block_x, int* block_y, int* npt
                     pair_pays(h->g, h->dtype == CLBM_F16R);
   if (pair)
     for (int t : {32, 64, 128, 256}) cands.push_back({32, t / 32, 1});
-  // other rates have neither a register-capped nor a TMA-staged kernel, and
-  // the two-buffer FP16 forms have one variant
-  const int caps = unit && (h->elem != 2 || h->in_place) ? 1 : 0;
+  // Other rates have no TMA-staged kernel, and a register-capped one in place
+  // and in FP32 math only; the two-buffer FP16 forms have one variant.
+  const int caps = h->in_place ? (unit || h->elem != 8) : (unit && h->elem != 2);
   for (int capped = 0; capped <= caps && !pair; ++capped)
     for (auto& sh : shapes) {
       if (sh[0] > 32 && sh[0] > h->g.pitch) continue;

@@ -40,11 +40,32 @@ def test_unit_and_other_rates_are_tuned_apart(clbm, form, rates_first):
                 lat.set_rates({9: 1.2, 12: 0.9})
             info = lat.autotune(53 if rates else 59)
         if rates:
-            assert info["npt"] == 1        # the one kernel that such lattices run
+            # two buffers: the one kernel that such lattices run
+            assert info["npt"] == 1 or form == "f32_inplace"
         if rates in infos:
             assert info == infos[rates]
         infos[rates] = info
     assert infos[False]["us_per_step"] != infos[True]["us_per_step"]
+
+
+# The register-capped in-place kernels of other rates against the plain
+# two-buffer one: FP32 roundings of 2^-24 at the scale of a deviation (0.05), under 20
+# of them a population and step, 1e-6 over 20 steps; F16S one ulp of the
+# deviation after one step (2^-10 of it, 1e-7 near zero)
+@pytest.mark.parametrize("form", ["f32", "f16s"])
+def test_capped_in_place_kernel_with_other_rates(clbm, form):
+    dims, states = (37, 19, 11), []
+    for opt, shape in (("", (32, 4, 1)), ("_inplace", (32, 8, 5))):
+        with _lattice(clbm, dims, form + opt, check_interval=10) as lat:
+            f = lat.get_state() * (1 + wl.noise((19,) + lat.shape, seed=3, amp=0.02))
+            lat.set_state(f)
+            lat.set_rates({9: 1.2, 12: 0.9, 17: 1.1})
+            lat.set_launch(*shape)
+            lat.step(20 if form == "f32" else 1)
+            states.append(lat.get_state())
+    w = np.array([1 / 3] + [1 / 18] * 6 + [1 / 36] * 12)[:, None, None, None]
+    tol = 1e-6 if form == "f32" else np.abs(states[0] - w) * 2.0 ** -10 + 1e-7
+    assert np.all(np.abs(states[1] - states[0]) <= tol)
 
 
 # FP16 lattices too small for pairs run one node per thread and use the block's
