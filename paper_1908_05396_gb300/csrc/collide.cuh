@@ -189,16 +189,19 @@ __device__ __forceinline__ double to64(float x) {
   return double(x);
 }
 
-// A non-negative double truncated to float; zero and values below 2^-125 give
-// 2^-125, values from 2^110 on (beyond which the FP32 solve's products would
-// overflow) 2^110.
+// A non-negative double below 2^128 truncated to float; zero and values below
+// 2^-125 give 2^-125.
 __device__ __forceinline__ float narrow(double x) {
   const int hi = __double2hiint(x);
   const unsigned lo = unsigned(__double2loint(x));
   return hi < 0x38200000 ? 2.3509887e-38f
-         : hi >= 0x46d00000
-             ? 1.2980742e33f
-             : __uint_as_float((unsigned(hi - 0x38000000) << 3) | (lo >> 29));
+                         : __uint_as_float((unsigned(hi - 0x38000000) << 3) | (lo >> 29));
+}
+
+// The same for any size: values from 2^110 on, beyond which the FP32 solve's
+// products would overflow, give about 2^110.
+__device__ __forceinline__ float narrow_any(double x) {
+  return narrow(__hiloint2double(min(__double2hiint(x), 0x46d00000), __double2loint(x)));
 }
 
 // The same for either sign.
@@ -211,9 +214,10 @@ __device__ __forceinline__ bool below(double x, double bound) {
   return __double_as_longlong(x) < __double_as_longlong(bound);
 }
 
-// Tests on the bit patterns: 0 < x < infinity; x neither infinite nor NaN.
+// Tests on the upper word's bits: x positive, finite and above 2^-1042; x neither
+// infinite nor NaN.
 __device__ __forceinline__ bool positive_finite(double x) {
-  return (unsigned long long)(__double_as_longlong(x)) - 1ull < 0x7fefffffffffffffull;
+  return unsigned(__double2hiint(x)) - 1u < 0x7fefffffu;
 }
 __device__ __forceinline__ bool finite_bits(double x) {
   return (unsigned(__double2hiint(x)) & 0x7ff00000u) != 0x7ff00000u;
@@ -272,7 +276,7 @@ __device__ __forceinline__ double omega_nu(const CollideConst<double>& C, double
     const double nu = fmin(fmax(mulr(C.K3 * (1.0 / 3.0), rinv), C.nu_min), C.nu_max);
     return rcp64(fma(3.0, nu, 0.5));
   }
-  const float Af = narrow(A), Bf = narrow(B);
+  const float Af = narrow_any(A), Bf = narrow_any(B);
   const float yf = solve_y2<float>(C.n, C.rn, C.ehalf, C.clog2, C.ylo2, C.yhi2, C.g2lo,
                                    narrow(rho), Af, Bf);
   const double tau = widen(ex2f(yf));
@@ -309,8 +313,9 @@ __device__ __forceinline__ double omega_nu(const CollideConst<double>& C, double
   // The logarithms and clamps work on bit patterns and turn anything into a
   // rate.  A density that has none, and moments that are not finite, give NaN:
   // a diverged node then spoils its lattice until the next check step reports it.
-  return positive_finite(rho) && finite_bits(d1) ? w1
-                                                 : __hiloint2double(0x7ff80000, 0);
+  return __hiloint2double(
+      positive_finite(rho) && finite_bits(d1) ? __double2hiint(w1) : 0x7ff80000,
+      __double2loint(w1));
 }
 
 // |gamma_dot| at the solved omega (a diverged node's density may be negative).
