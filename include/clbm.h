@@ -232,9 +232,10 @@ int clbm_set_rates(clbm_handle h, const double omega[10]);
  * value carries, from random bits that depend only on the node and the
  * lattice's step count (the same bits alone and in any run); such changes
  * then survive on average.  The stored layout does not change.  Stochastic
- * rounding runs the one-node-per-thread step kernel only (npt 1 or 5);
- * clbm_set_rounding resets another launch shape to npt 1, and a batch does
- * not take such a lattice (clbm_batch_add: CLBM_ERR_UNSUPPORTED).  Errors:
+ * rounding takes launch shapes with npt 1 or 5 (one or two nodes per thread by
+ * the lattice's size); clbm_set_rounding resets another to npt 1, and a batch set
+ * to one launch per lattice does not take such a lattice (clbm_batch_add:
+ * CLBM_ERR_UNSUPPORTED).  Errors:
  * CLBM_ERR_UNSUPPORTED for other storage forms (F16R always rounds
  * stochastically and accepts CLBM_ROUND_STOCHASTIC as a no-op; FP32 and FP64
  * accept CLBM_ROUND_NEAREST as a no-op) and for stochastic rounding of an
@@ -265,8 +266,8 @@ typedef struct clbm_batch_ctx* clbm_batch;
 int clbm_batch_create(clbm_dtype dtype, int capacity, int check_interval, void* stream,
                       clbm_batch* out);
 /* Attach h (same dtype and device, not in another batch, 19 x padded nodes
- * < 2^31; an in-place lattice only in the one-launch-per-lattice mode, an
- * F16S lattice with stochastic rounding only in the persistent mode, else
+ * < 2^31; an in-place lattice only, an F16S lattice with stochastic rounding
+ * never while clbm_batch_set_lattice_launch is in force, else
  * CLBM_ERR_UNSUPPORTED); its queued work is waited for; *slot receives its
  * slot. */
 int clbm_batch_add(clbm_batch b, clbm_handle h, int* slot);
@@ -294,8 +295,8 @@ int clbm_batch_stats_all(clbm_batch b, double* residual, double* mass, int* dive
 int clbm_batch_set_launch(clbm_batch b, int block_x, int block_y, int zc, int blocks_per_sm);
 /* One launch per lattice instead of the persistent kernel (FP64, FP32,
  * F16S; CLBM_ERR_UNSUPPORTED for F16R and while an F16S lattice with
- * stochastic rounding is attached, whose rounding is seeded by the batch's
- * device-side step count): every step launches each attached lattice's own
+ * stochastic rounding is attached: the launches of this mode hold their step
+ * counts, so a replayed graph would repeat the seeds): every step launches each attached lattice's own
  * step kernel (block_x x block_y threads, a multiple of 32 and <= 256; npt 1,
  * or 5 for the register-capped kernel), the lattices spread over `streams`
  * (1..16) streams, largest first onto the least-loaded one.  The streams fork
@@ -328,7 +329,7 @@ const char* clbm_batch_last_error(clbm_batch b);
  * Not in the paper: a worker thread owns a batch and repeatedly (1) admits
  * queued requests first come first served while a slot is free and the
  * request's device memory fits the HBM budget, (2) steps every admitted
- * lattice by one check interval in one graph launch, (3) retires lattices
+ * lattice by one check interval, (3) retires lattices
  * whose residual (as clbm_residual) is <= tol, that diverged, that reached
  * max_steps, or whose residual has not fallen by 10 % for plateau_checks
  * checks.  Requests join only at check-interval boundaries, so a request's

@@ -187,8 +187,9 @@ void fill_desc(clbm_dtype t, void* out, const clbm_ctx* h, int tx, int ty, int t
 }
 
 // Whether an attached lattice rounds its stores stochastically: its seeds
-// come from the batch's device-side step count, which only the persistent
-// kernel advances (a replayed graph of per-lattice launches would repeat them).
+// come from the batch's device-side step count, which the persistent kernel and
+// the spread launches advance; the launches of mode 1 do not read it (their
+// replayed graph would repeat its seeds), so that mode refuses such lattices.
 bool any_sround(const clbm_batch_ctx* b) {
   for (int s = 0; s < b->capacity; ++s)
     if (b->slots[s] && b->slots[s]->sround) return true;
@@ -730,8 +731,8 @@ int clbm_batch_add(clbm_batch b, clbm_handle h, int* slot) {
   if (h->device != b->device) return bfail(b, CLBM_ERR_ARG, "lattice lives on another device");
   if (h->sround && b->mode == 1)
     return bfail(b, CLBM_ERR_UNSUPPORTED,
-                 "lattices with stochastic rounding take the persistent kernel, not the "
-                 "one-launch-per-lattice mode");
+                 "lattices with stochastic rounding do not join a batch that is set to "
+                 "one launch per lattice");
   if (h->batch) return bfail(b, CLBM_ERR_ARG, "lattice is already in a batch");
   if (int64_t(NQ) * h->g.qstride >= (int64_t(1) << 31))
     return bfail(b, CLBM_ERR_UNSUPPORTED, "lattice too large to batch (19 x padded nodes >= 2^31)");
@@ -870,10 +871,12 @@ int clbm_batch_set_lattice_launch(clbm_batch b, int block_x, int block_y, int np
   if (!valid(b)) return bfail(b, CLBM_ERR_ARG, "invalid batch");
   if (b->dtype == CLBM_F16R)
     return bfail(b, CLBM_ERR_UNSUPPORTED,
-                 "F16R batches take the persistent kernel (its rounding is seeded by the step)");
+                 "F16R batches cannot be set to launches per lattice (replayed, they would repeat "
+                 "the seeds of the rounding)");
   if (any_sround(b))
     return bfail(b, CLBM_ERR_UNSUPPORTED,
-                 "a lattice rounds stochastically: the batch takes the persistent kernel");
+                 "a lattice rounds stochastically: the batch cannot be set to launches per lattice "
+                 "(replayed, they would repeat the seeds)");
   if (block_x < 1 || block_y < 1 || block_x * block_y > 256 || (block_x * block_y) % 32 ||
       (npt != 1 && npt != 5) || streams < 1 || streams > 16)
     return bfail(b, CLBM_ERR_ARG, "bad launch shape");

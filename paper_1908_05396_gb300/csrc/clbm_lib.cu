@@ -256,7 +256,7 @@ int clbm_create(const clbm_domain* d, double K, double n, const double U_lid[3],
   g.rho0 = rho0;
   fill_params(h->P, K, n, body_force, rho0, nu_min, nu_max, dtype);
   h->block = default_block(d->nx, int(h->elem));
-  h->npt = 1;  // the autotuner may switch to two nodes per thread
+  h->npt = 1;  // (FP16 lattices step one or two nodes per thread by their size: pair_pays)
 
   auto cleanup = [&](int code, const std::string& m) {
     g_create_err = m + (h->err.empty() ? "" : (": " + h->err));
@@ -657,7 +657,7 @@ int clbm_set_rounding(clbm_handle h, clbm_rounding mode) {
   if (sr && h->in_place)
     return fail(h, CLBM_ERR_UNSUPPORTED, "stochastic rounding takes two-buffer lattices");
   h->sround = sr;
-  // the stochastic kernel has one shape family: one node per thread
+  // the stochastic kernels choose one or two nodes per thread by the size only
   if (sr && ((h->npt & TMA_NPT) || (h->npt & 3) == 2)) h->npt = 1;
   return CLBM_OK;
 }
@@ -683,7 +683,7 @@ int clbm_set_launch(clbm_handle h, int block_x, int block_y, int npt) {
     if (h->dtype != CLBM_F32 && h->dtype != CLBM_F16S)
       return fail(h, CLBM_ERR_UNSUPPORTED, "the TMA-staged kernel takes FP32 or F16S storage");
     if (h->sround)
-      return fail(h, CLBM_ERR_UNSUPPORTED, "stochastic rounding runs one node per thread (npt 1 or 5)");
+      return fail(h, CLBM_ERR_UNSUPPORTED, "stochastic rounding takes npt 1 or 5");
     if (block_x != tma_bx(v) || block_y != tma_by(v))
       return fail(h, CLBM_ERR_ARG, "block does not match the TMA shape");
     h->block = dim3(block_x, block_y, 1);
@@ -700,7 +700,7 @@ int clbm_set_launch(clbm_handle h, int block_x, int block_y, int npt) {
   if (np == 2 && (h->dtype == CLBM_F64 || h->dtype == CLBM_F16R))
     return fail(h, CLBM_ERR_UNSUPPORTED, "two nodes per thread needs FP32 math");
   if (np == 2 && h->sround)
-    return fail(h, CLBM_ERR_UNSUPPORTED, "stochastic rounding runs one node per thread (npt 1 or 5)");
+    return fail(h, CLBM_ERR_UNSUPPORTED, "stochastic rounding takes npt 1 or 5");
   h->block = dim3(block_x, block_y, 1);
   h->npt = npt;
   return CLBM_OK;

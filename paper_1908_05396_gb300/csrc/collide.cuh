@@ -830,8 +830,10 @@ struct NoRef {};
 // per population), counted with every possible multiply-add fused.  What it
 // gave: the FP64 step is bound by the FP64 pipe and went from 2030 to 978 us
 // on 128^3 (with the solve above); on 256^3 FP32 went from 431 to 379 us a
-// step (6.7 TB/s), F16S from 395 to 323 and F16R from 792 to 753 us, and no
-// register-capped FP32 or FP16 kernel spills any more.
+// step (6.7 TB/s), F16S from 395 to 323 and F16R from 792 to 753 us, and the
+// register-capped two-buffer FP32 and FP16 kernels of a lone lattice no longer spill
+// (of unit rates, the batch's kernels spill 4 to 56 bytes, the capped FP32
+// in-place check step 4, F16R's forced check step 8).
 //
 // PAIR_OUT, LOG2LAM and the body force's symmetric split are as in
 // collide_rates.  With PAIR_OUT the populations are rebuilt from the raw

@@ -48,7 +48,8 @@ inline int tile_width(int nx, int elem, int bx, int threads) {
 // a step, in place 58.5 -> 54.1, 80^3 15.4 -> 12.7, 40^3 5.2 -> 3.5).  FP64
 // is bound by the FP64 pipe, which a warp occupies whatever its idle lanes:
 // one warp per block, 8 x 4 (the finest spread over the SMs; 128^3 alike,
-// 80^3 304 -> 247 us, 48^3 78 -> 59, 36^3 58 -> 28).
+// 80^3 304 -> 247 us, 48^3 78 -> 59, 36^3 58 -> 28; 4 x 8 fills the warp of rows
+// of up to four nodes, in the same time: 4x64x4 11 us with 32 warps or 256).
 inline dim3 default_block(int nx, int elem) {
   if (elem == 8) return nx <= 4 ? dim3(4, 8, 1) : dim3(8, 4, 1);
   const int p16 = (nx + 15) / 16 * 16, p8 = (nx + 7) / 8 * 8;
