@@ -108,7 +108,7 @@ def test_batch_tuner_keeps_the_untuned_launch_where_it_wins(clbm, form):
         for lat in lats:
             b.add(lat)
         b.step(13)
-        info = b.autotune(10)
+        info = b.autotune(60)
         assert info["mode"] == "per_lattice" and info["block"] == (0, 0)
         b.step(130)
         b.apply_launch(info)
